@@ -1,9 +1,11 @@
-"""Thin ctypes binding over the C-ABI library (``include/prom.h``).
+"""Thin binding over the C-ABI library (``include/prom.h``).
 
 Argument marshalling only: every function hands device (or host) pointers of
 torch tensors to the entry point of the same name; all arithmetic runs in the
-library's CUDA kernels.  There is no fallback: if the library is missing, or a
-tensor lives on the wrong device, the call raises.
+library's CUDA kernels.  The calls a program makes per layer or per step go
+through the extension module ``_native`` (``csrc/native.cpp``), everything else
+through ctypes.  There is no fallback: if a library is missing, or a tensor
+lives on the wrong device, the call raises.
 """
 from __future__ import annotations
 
@@ -15,6 +17,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libprom.so")
+NATIVE_PATH = os.path.join(_HERE, "_native.so")
 
 PROM_OK = 0
 (PROM_ERR_NULL, PROM_ERR_SHAPE, PROM_ERR_ALIGN, PROM_ERR_BAD_WEIGHT, PROM_ERR_BAD_REQUANT,
@@ -163,6 +166,26 @@ def status_string(code: int) -> str:
     return lib().prom_status_string(int(code)).decode()
 
 
+_native = None
+
+
+def native():
+    """Loads the extension module ``_native`` (built in-tree like ``libprom.so``); raises if absent."""
+    global _native
+    if _native is None:
+        if not os.path.exists(NATIVE_PATH):
+            raise RuntimeError(f"{NATIVE_PATH} is missing: run paper_2505_03254_b200.build.build()")
+        lib()
+        from . import _native as module
+        _native = module
+    return _native
+
+
+def _handle(stream):
+    """The handle of a stream for ``_native``, which asks for the current stream itself (None)."""
+    return None if stream is None else int(stream.cuda_stream)
+
+
 def _check(code: int, what: str) -> None:
     if code != PROM_OK:
         raise PromError(code, what)
@@ -201,13 +224,10 @@ def last_device_status(stream=None) -> int:
 def dw_conv3x3_i8(x: torch.Tensor, w: torch.Tensor, rq: "PromRequant", stride: int = 1, y=None, stream=None):
     """prom_dw_conv3x3_i8: x int8 [batch, h, w, c], w int8 [c, 3, 3] on the device ->
     y int8 [batch, ho, wo, c]."""
-    b, h, wd, c = x.shape
-    ho, wo = (h - 1) // stride + 1, (wd - 1) // stride + 1
     if y is None:
-        y = torch.empty((b, ho, wo, c), dtype=torch.int8, device=x.device)
-    _check(lib().prom_dw_conv3x3_i8(_dev(x, torch.int8, "x"), b, h, wd, c, stride, _dev(w, torch.int8, "w"),
-                                    C.byref(rq), _dev(y, torch.int8, "y"), _stream(stream)),
-           "prom_dw_conv3x3_i8")
+        b, h, wd, c = x.shape
+        y = torch.empty((b, (h - 1) // stride + 1, (wd - 1) // stride + 1, c), dtype=torch.int8, device=x.device)
+    _check((_native or native()).dw_conv3x3_i8(x, w, rq, stride, y, _handle(stream)), "prom_dw_conv3x3_i8")
     return y
 
 
@@ -215,20 +235,13 @@ def pw_conv_i8_dyn(x: torch.Tensor, batch: int, w_packed: torch.Tensor, cout: in
                    gamma_x: torch.Tensor, out=None, stream=None):
     """prom_pw_conv_i8_dyn: x int8 [batch * rows_per_sample, cin], alpha float32 [cout], gamma_x
     float32 [batch], all on the device -> (q int8 [m, cout], gamma_y, scale_y float32 [batch])."""
-    m, cin = x.shape
-    if batch and m % batch:
-        raise ValueError("rows must divide evenly into samples")
-    rows = m // batch if batch else 1
     if out is None:
-        q = torch.empty((m, cout), dtype=torch.int8, device=x.device)
+        q = torch.empty((x.shape[0], cout), dtype=torch.int8, device=x.device)
         gy = torch.empty((batch,), dtype=torch.float32, device=x.device)
         sy = torch.empty((batch,), dtype=torch.float32, device=x.device)
     else:
         q, gy, sy = out
-    _check(lib().prom_pw_conv_i8_dyn(_dev(x, torch.int8, "x"), batch, rows, cin,
-                                     _dev(w_packed, torch.uint8, "w_packed"), cout,
-                                     _dev(alpha, torch.float32, "alpha"), _dev(gamma_x, torch.float32, "gamma_x"),
-                                     q.data_ptr(), gy.data_ptr(), sy.data_ptr(), _stream(stream)),
+    _check((_native or native()).pw_conv_i8_dyn(x, batch, w_packed, cout, alpha, gamma_x, q, gy, sy, _handle(stream)),
            "prom_pw_conv_i8_dyn")
     return q, gy, sy
 
@@ -236,21 +249,15 @@ def pw_conv_i8_dyn(x: torch.Tensor, batch: int, w_packed: torch.Tensor, cout: in
 def quantize_act_absmax(x: torch.Tensor, out=None, stream=None):
     """prom_quantize_act_absmax: float32 activations [batch, ...] on the device -> (q int8 like
     x, gamma float32 [batch], scale float32 [batch]); `out` may carry the three tensors."""
-    if not x.is_cuda or x.dtype != torch.float32 or not x.is_contiguous():
-        raise ValueError("x must be a contiguous float32 CUDA tensor")
-    batch = x.shape[0]
-    per = x.numel() // batch if batch else 1
     if out is None:
+        if not x.is_cuda or x.dtype != torch.float32 or not x.is_contiguous():
+            raise ValueError("x must be a contiguous float32 CUDA tensor")
         q = torch.empty(x.shape, dtype=torch.int8, device=x.device)
-        gamma = torch.empty((batch,), dtype=torch.float32, device=x.device)
-        scale = torch.empty((batch,), dtype=torch.float32, device=x.device)
+        gamma = torch.empty((x.shape[0],), dtype=torch.float32, device=x.device)
+        scale = torch.empty((x.shape[0],), dtype=torch.float32, device=x.device)
     else:
         q, gamma, scale = out
-        if q.shape != x.shape or q.dtype != torch.int8 or not q.is_cuda or gamma.numel() != batch or \
-                scale.numel() != batch or gamma.dtype != torch.float32 or scale.dtype != torch.float32:
-            raise ValueError("out must be (int8 like x, float32 [batch], float32 [batch]) on the device")
-    _check(lib().prom_quantize_act_absmax(x.data_ptr(), batch, per, q.data_ptr(), gamma.data_ptr(),
-                                          scale.data_ptr(), _stream(stream)), "prom_quantize_act_absmax")
+    _check((_native or native()).quantize_act_absmax(x, q, gamma, scale, _handle(stream)), "prom_quantize_act_absmax")
     return q, gamma, scale
 
 
@@ -417,7 +424,7 @@ def quantize_ternary_batch(ws: Optional[Sequence[torch.Tensor]] = None, out=None
     table marshalled earlier (then ws and out are not looked at)."""
     if jobs is None:
         jobs = QuantizeJobs(ws, out)
-    _check(lib().prom_quantize_ternary_batch(jobs.array, jobs.n, _stream(stream)), "prom_quantize_ternary_batch")
+    _check((_native or native()).quantize_ternary_batch(jobs.array, jobs.n, _handle(stream)), "prom_quantize_ternary_batch")
     return jobs.out
 
 
@@ -439,12 +446,9 @@ def make_requant(bias: torch.Tensor, mult: torch.Tensor, shift: torch.Tensor,
 def pw_conv_i8(x: torch.Tensor, w_packed: torch.Tensor, cout: int, rq: PromRequant,
                y: Optional[torch.Tensor] = None, variant="auto", stream=None) -> torch.Tensor:
     """prom_pw_conv_i8 on device tensors; x is [m, cin] int8."""
-    m, cin = x.shape
     if y is None:
-        y = torch.empty((m, cout), dtype=torch.int8, device=x.device)
-    _check(lib().prom_pw_conv_i8(_dev(x, torch.int8, "x"), m, cin,
-                                 _dev(w_packed, torch.uint8, "w_packed"), cout, C.byref(rq),
-                                 _dev(y, torch.int8, "y"), _variant(variant), _stream(stream)),
+        y = torch.empty((x.shape[0], cout), dtype=torch.int8, device=x.device)
+    _check((_native or native()).pw_conv_i8(x, w_packed, cout, rq, y, _variant(variant), _handle(stream)),
            "prom_pw_conv_i8")
     return y
 
@@ -464,12 +468,10 @@ def pw_prepare(m: int, cin: int, w_packed: torch.Tensor, cout: int, rq: PromRequ
 def pw_conv_i8_prepared(x: torch.Tensor, cout: int, prepared: torch.Tensor, act_min: int = 0, act_max: int = 127,
                         y: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
     """prom_pw_conv_i8_prepared on device tensors; x is [m, cin] int8."""
-    m, cin = x.shape
     if y is None:
-        y = torch.empty((m, cout), dtype=torch.int8, device=x.device)
-    _check(lib().prom_pw_conv_i8_prepared(_dev(x, torch.int8, "x"), m, cin, cout,
-                                          _dev(prepared, torch.uint8, "prepared"), act_min, act_max,
-                                          _dev(y, torch.int8, "y"), _stream(stream)), "prom_pw_conv_i8_prepared")
+        y = torch.empty((x.shape[0], cout), dtype=torch.int8, device=x.device)
+    _check((_native or native()).pw_conv_i8_prepared(x, cout, prepared, act_min, act_max, y, _handle(stream)),
+           "prom_pw_conv_i8_prepared")
     return y
 
 
@@ -478,15 +480,9 @@ def pw_conv_i8_res(x: torch.Tensor, w_packed: torch.Tensor, cout: int, rq: PromR
                    stream=None) -> torch.Tensor:
     """prom_pw_conv_i8_res: the layer plus the int8 tensor `res` ([m, cout]) with saturation;
     pass y=res to form the sum in place."""
-    m, cin = x.shape
-    if tuple(res.shape) != (m, cout):
-        raise ValueError("res must be [m, cout]")
     if y is None:
-        y = torch.empty((m, cout), dtype=torch.int8, device=x.device)
-    _check(lib().prom_pw_conv_i8_res(_dev(x, torch.int8, "x"), m, cin,
-                                     _dev(w_packed, torch.uint8, "w_packed"), cout, C.byref(rq),
-                                     _dev(res, torch.int8, "res"), _dev(y, torch.int8, "y"),
-                                     _variant(variant), _stream(stream)),
+        y = torch.empty((x.shape[0], cout), dtype=torch.int8, device=x.device)
+    _check((_native or native()).pw_conv_i8_res(x, w_packed, cout, rq, res, y, _variant(variant), _handle(stream)),
            "prom_pw_conv_i8_res")
     return y
 
@@ -567,14 +563,12 @@ class LayerSeq:
 def pw_layer_seq(seq: LayerSeq, x0: torch.Tensor, workspace: torch.Tensor,
                  y_out: Optional[torch.Tensor] = None, variant="auto", stream=None) -> torch.Tensor:
     """prom_pw_layer_seq on device tensors; x0 is [batch, h0, w0, cin0] int8."""
-    batch, h0, w0, _ = x0.shape
     if y_out is None:
+        batch, h0, w0, _ = x0.shape
         y_out = torch.empty((batch, h0 // seq.total_stride, w0 // seq.total_stride, seq.cout_last),
                             dtype=torch.int8, device=x0.device)
-    _check(lib().prom_pw_layer_seq(seq.array, seq.n, _dev(x0, torch.int8, "x0"), batch, h0, w0,
-                                   workspace.data_ptr(), workspace.numel(),
-                                   _dev(y_out, torch.int8, "y_out"), _variant(variant),
-                                   _stream(stream)), "prom_pw_layer_seq")
+    _check((_native or native()).pw_layer_seq(seq.array, seq.n, x0, workspace, y_out, _variant(variant), _handle(stream)),
+           "prom_pw_layer_seq")
     return y_out
 
 

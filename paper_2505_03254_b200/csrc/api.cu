@@ -39,27 +39,32 @@ struct DeviceInfo {
     int sms = 0;
     int smem_optin = 0;
     int smem_total = 0;   // shared memory per SM
+    int dev = 0;
     bool ok = false;
 };
 
+static DeviceInfo query_device(int dev)
+{
+    DeviceInfo d;
+    d.dev = dev;
+    d.ok = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&d.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
+           cudaDeviceGetAttribute(&d.smem_total, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) == cudaSuccess;
+    return d;
+}
+
+// The current device's limits; asked of the driver once per device.  A call is a few microseconds of
+// host time, so the look-up takes no lock once the entry is there.
 static DeviceInfo device_info()
 {
-    static std::mutex mu;
-    static std::unordered_map<int, DeviceInfo> cache;
+    constexpr int kDevices = 64;
+    static DeviceInfo cache[kDevices];
+    static std::once_flag once[kDevices];
     int dev = 0;
-    DeviceInfo d;
-    if (cudaGetDevice(&dev) != cudaSuccess) return d;
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = cache.find(dev);
-    if (it != cache.end()) return it->second;
-    if (cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&d.smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) ==
-            cudaSuccess &&
-        cudaDeviceGetAttribute(&d.smem_total, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) ==
-            cudaSuccess)
-        d.ok = true;
-    cache[dev] = d;
-    return d;
+    if (cudaGetDevice(&dev) != cudaSuccess) return DeviceInfo();
+    if (dev < 0 || dev >= kDevices) return query_device(dev);
+    std::call_once(once[dev], [dev] { cache[dev] = query_device(dev); });
+    return cache[dev];
 }
 
 // ---- the layer as the host sees it -----------------------------------------------
@@ -171,8 +176,12 @@ static TcTune g_tune = {0, 0, 0, 0, 0};
 static std::mutex g_shape_tune_mu;
 static std::map<std::array<long long, 4>, TcTune> g_shape_tune;
 
+// Whether any override is set (the look-up below takes a lock).
+static std::atomic<bool> g_tuned{false};
+
 static TcTune tune_for(long long m, int cin, int cout, int stride)
 {
+    if (!g_tuned.load()) return TcTune{0, 0, 0, 0, 0};
     std::lock_guard<std::mutex> lk(g_shape_tune_mu);
     auto it = g_shape_tune.find({m, cin, cout, stride});
     return it == g_shape_tune.end() ? g_tune : it->second;
@@ -385,28 +394,42 @@ static bool tc_search_plan(long long m, int cin, int cout, const RowMap &map, co
 
 
 // The search above costs tens of microseconds; its result depends only on the shape, the
-// device and the tuning override, so it is remembered.
-static bool tc_shape_plan(long long m, int cin, int cout, const RowMap &map, const DeviceInfo &d,
-                          TcPlan &best, int use = kPlanSingle)
+// device and the tuning override, so it is remembered: per process, and the last plans a thread has
+// used in a small table of its own in front of that, so that a repeated call takes no lock.
+typedef std::array<long long, 15> PlanKey;
+struct PlanEntry { PlanKey key; bool ok; TcPlan pl; };
+
+static void tc_find_plan(long long m, int cin, int cout, const RowMap &map, const DeviceInfo &d, int use,
+                         const PlanKey &key, PlanEntry &out)
 {
-    struct Entry { bool ok; TcPlan pl; };
     static std::mutex mu;
-    static std::map<std::array<long long, 15>, Entry> cache;
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const TcTune tn = tune_for(m, cin, cout, map.stride);
-    const std::array<long long, 15> key = {m, cin, cout, map.stride, map.ho, map.wo, map.hin, map.win,
-                                           tn.fold, tn.nt, tn.groups, tn.occ, tn.stages, dev, use};
+    static std::map<PlanKey, PlanEntry> cache;
     std::lock_guard<std::mutex> lk(mu);
     auto it = cache.find(key);
     if (it == cache.end()) {
-        Entry e;
+        PlanEntry e;
+        e.key = key;
         e.ok = tc_search_plan(m, cin, cout, map, d, use, e.pl);
         if (cache.size() > 4096) cache.clear();
         it = cache.emplace(key, e).first;
     }
-    if (it->second.ok) best = it->second.pl;
-    return it->second.ok;
+    out = it->second;
+}
+
+static bool tc_shape_plan(long long m, int cin, int cout, const RowMap &map, const DeviceInfo &d,
+                          TcPlan &best, int use = kPlanSingle)
+{
+    constexpr int kRecent = 128;
+    static thread_local std::vector<PlanEntry> recent(kRecent, PlanEntry{PlanKey{}, false, TcPlan()});
+    const TcTune tn = tune_for(m, cin, cout, map.stride);
+    const PlanKey key = {m, cin, cout, map.stride, map.ho, map.wo, map.hin, map.win,
+                         tn.fold, tn.nt, tn.groups, tn.occ, tn.stages, d.dev, use + 1};
+    const unsigned long long h = ((unsigned long long)m * 0x9E3779B1u + (unsigned)cin * 0x85EBCA6Bu +
+                                  (unsigned)cout * 0xC2B2AE35u + (unsigned)(map.stride * 8 + use) * 0x27D4EB2Fu);
+    PlanEntry &e = recent[(h ^ (h >> 17)) & (kRecent - 1)];
+    if (e.key != key) tc_find_plan(m, cin, cout, map, d, use, key, e);
+    if (e.ok) best = e.pl;
+    return e.ok;
 }
 
 static bool tc_make_maps(const Conv &c, TcPlan &pl)
@@ -456,6 +479,9 @@ static bool tc_make_maps(const Conv &c, TcPlan &pl)
 static prom_status tc_set_attr(const DeviceInfo &d)
 {
     // once per device: the limit is an attribute of the (function, device) pair
+    static std::atomic<unsigned long long> done{0};
+    const unsigned long long bit = d.dev >= 0 && d.dev < 64 ? 1ull << d.dev : 0ull;
+    if (done.load(std::memory_order_acquire) & bit) return PROM_OK;
     cudaError_t e = raise_smem_limit(tc::tc_conv_kernel<2>, d.smem_optin);
     if (e == cudaSuccess) e = raise_smem_limit(tc::tc_conv_kernel<3>, d.smem_optin);
     if (e == cudaSuccess) e = raise_smem_limit(tc::tc_conv_kernel<2, 1>, d.smem_optin);
@@ -463,7 +489,9 @@ static prom_status tc_set_attr(const DeviceInfo &d)
     if (e == cudaSuccess) e = raise_smem_limit(tc::tc_conv_kernel<2, 4>, d.smem_optin);
     if (e == cudaSuccess) e = raise_smem_limit(tc::tc_conv_kernel<2, 3>, d.smem_optin);
     if (e == cudaSuccess) e = raise_smem_limit(tc::tc_prep_kernel, d.smem_optin);
-    return e == cudaSuccess ? PROM_OK : PROM_ERR_CUDA;
+    if (e != cudaSuccess) return PROM_ERR_CUDA;
+    done.fetch_or(bit, std::memory_order_release);
+    return PROM_OK;
 }
 
 // Fills in the pointers of a planned layer (image: prepared operands, or null).
@@ -693,14 +721,6 @@ static prom_status launch_tc(const Conv &c)
     return tc_launch_planned(c, pl);
 }
 
-static bool tc_supported(const Conv &c)
-{
-    DeviceInfo d = device_info();
-    if (!d.ok) return false;
-    TcPlan pl;
-    return tc_shape_plan(c.m, c.cin, c.cout, c.map, d, pl);
-}
-
 // ---- variant choice --------------------------------------------------------------------------
 static prom_status run_conv(const Conv &c, prom_variant v)
 {
@@ -714,11 +734,13 @@ static prom_status run_conv(const Conv &c, prom_variant v)
                                                     c.st, g_launches);
     case PROM_VARIANT_ADDSUB: return addsub::launch(c.x, c.m, c.cin, c.map, c.w, c.cout, c.rq, c.y,
                                                     c.st, g_launches);
-    case PROM_VARIANT_AUTO:
-        if (tc_supported(c)) return launch_tc(c);
+    case PROM_VARIANT_AUTO: {
+        const prom_status e = launch_tc(c);
+        if (e != PROM_ERR_UNSUPPORTED) return e;
         if (!c.res && smallk::supported(c.cin, c.cout))
             return smallk::launch(c.x, c.m, c.cin, c.map, c.w, c.cout, c.rq, c.y, c.st, g_launches);
         return launch_naive(c, nullptr);
+    }
     default: return PROM_ERR_UNSUPPORTED;
     }
 }
@@ -2060,12 +2082,14 @@ void prom_debug_tc_plan_shape(int64_t m, int cin, int cout, int stride, int fold
     const std::array<long long, 4> key = {m, cin, cout, stride};
     if (!fold && !nt && !groups && !occ && !stages) g_shape_tune.erase(key);
     else g_shape_tune[key] = TcTune{fold, nt, groups, occ, stages};
+    g_tuned.store(true);
 }
 
 void prom_debug_tc_plan(int fold, int nt, int groups, int occ, int stages)
 {
     std::lock_guard<std::mutex> lk(g_shape_tune_mu);
     g_tune = TcTune{fold, nt, groups, occ, stages};
+    g_tuned.store(fold || nt || groups || occ || stages || !g_shape_tune.empty());
 }
 
 prom_status prom_debug_wait_timeout(uint64_t limit_ns, int *gave_up_dev, void *cuda_stream)
