@@ -112,6 +112,9 @@ act_quant_cluster_kernel(const float *__restrict__ x, int batch, long long per, 
     // every CTA of the cluster must be running before another one writes into its shared
     // memory: arrive now, wait just before the first exchange
     cluster.barrier_arrive();
+    // launched with programmatic dependent launch: x may be the previous kernel's output
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
 
     auto load_chunk = [&](int sample, int c) {      // thread 0 only
         const uint8_t *src = reinterpret_cast<const uint8_t *>(x + (long long)sample * per + first);
@@ -212,6 +215,8 @@ act_quant_reread_kernel(const float *__restrict__ x, int batch, long long per, l
     count = count < 0 ? 0 : (count > slice ? slice : count);
     const int n4 = (int)(count >> 2), n16 = (int)(count >> 4);
     cluster.barrier_arrive();
+    ptx::grid_dep_wait();           // as above
+    ptx::grid_dep_launch();
     bool first_exchange = true;
     for (int sample = cid, it = 0; sample < batch; sample += nclusters, ++it) {
         const float4 *src = reinterpret_cast<const float4 *>(x + (long long)sample * per + first);

@@ -78,8 +78,8 @@ struct Conv {
     prom_requant rq;
     int8_t *y;
     cudaStream_t st;
-    bool pdl;           // chain to the previous kernel with programmatic dependent launch
-    bool pdl_next;      // the next kernel of the sequence chains to this one
+    int pdl = tc::kPdlWait;    // how the kernel is chained to the previous one (tc.cuh: kPdl*, 0: plain launch)
+    bool pdl_next = true;      // the next kernel of the stream may chain to this one
     const int8_t *res = nullptr;   // added to the output with int8 saturation (may be y)
 };
 
@@ -121,6 +121,24 @@ static prom_status cuda_status(cudaError_t e)
     static const bool verbose = getenv("PROM_VERBOSE") != nullptr;
     if (verbose) fprintf(stderr, "prom: CUDA error %d: %s\n", (int)e, cudaGetErrorString(e));
     return PROM_ERR_CUDA;
+}
+
+// Launch configuration of a kernel that may be chained to its predecessor in the stream with
+// programmatic dependent launch (attr must outlive the launch call).
+static void fill_launch_cfg(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int grid, int threads, size_t smem,
+                            cudaStream_t st, bool pdl)
+{
+    memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    if (pdl) {
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+    }
 }
 
 // ---- naive -------------------------------------------------------------------------------
@@ -499,7 +517,7 @@ static void tc_bind(const Conv &c, TcPlan &pl, uint8_t *image)
 {
     tc::Params &p = pl.p;
     p.w_packed = c.w; p.bias = c.rq.bias; p.mult = c.rq.mult; p.shift = c.rq.shift;
-    p.act_min = c.rq.act_min; p.act_max = c.rq.act_max; p.y = c.y; p.pdl = c.pdl ? 1 : 0;
+    p.act_min = c.rq.act_min; p.act_max = c.rq.act_max; p.y = c.y; p.pdl = c.pdl;
     p.pdl_next = c.pdl_next ? 1 : 0;
     p.image = image;
     p.res = c.res;
@@ -509,18 +527,8 @@ static prom_status tc_launch_planned(const Conv &c, TcPlan &pl, int mode = 0)
 {
     if (!tc_make_maps(c, pl)) return PROM_ERR_CUDA;
     cudaLaunchConfig_t cfg;
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)pl.grid);
-    cfg.blockDim = dim3(tc::kThreads);
-    cfg.dynamicSmemBytes = pl.smem;
-    cfg.stream = c.st;
     cudaLaunchAttribute attr[1];
-    if (c.pdl) {
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-    }
+    fill_launch_cfg(cfg, attr, pl.grid, tc::kThreads, pl.smem, c.st, c.pdl != 0);
     cudaError_t e;
     if (mode == 1) e = cudaLaunchKernelEx(&cfg, tc::tc_conv_kernel<2, 1>, pl.xmap, pl.ymap, pl.p);
     else if (mode == 2) e = cudaLaunchKernelEx(&cfg, tc::tc_conv_kernel<2, 2>, pl.xmap, pl.ymap, pl.p);
@@ -588,7 +596,7 @@ struct WidePlan {
 // resident chunks.  `worth` says whether the library picks it by itself.
 static bool wide_plan(const Conv &c, const DeviceInfo &d, WidePlan &pl, bool &worth)
 {
-    if (c.map.stride != 1 || c.res || c.pdl || c.pdl_next) return false;
+    if (c.map.stride != 1 || c.res) return false;
     if ((c.cin & 15) || (c.cout & 15) || c.cin < wide::kChunk || c.cin > wide::kChunk * wide::kMaxKc) return false;
     if (c.cout < 64) return false;
     if (c.m >= (1ll << 31) - 256) return false;
@@ -1104,27 +1112,8 @@ static void seq_layout(const prom_layer *layers, int n, const SeqShape &s, const
 // 0: the library's choice, 1: CUDA cores only, 2: tensor cores or PROM_ERR_UNSUPPORTED
 static std::atomic<int> g_dw_variant{0};
 
-// Launch configuration of a kernel that may be chained to its predecessor in the stream with
-// programmatic dependent launch (attr must outlive the launch call).
-static void fill_launch_cfg(cudaLaunchConfig_t &cfg, cudaLaunchAttribute *attr, int grid, int threads, size_t smem,
-                            cudaStream_t st, bool pdl)
-{
-    memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    if (pdl) {
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-    }
-}
-
 static prom_status launch_dw_tc(const int8_t *x, int batch, int h, int w, int c, const int8_t *wt,
-                                const prom_requant *rq, int8_t *y, const DeviceInfo &d, cudaStream_t st,
-                                bool pdl, bool pdl_next)
+                                const prom_requant *rq, int8_t *y, const DeviceInfo &d, cudaStream_t st, int pdl)
 {
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return PROM_ERR_UNSUPPORTED;
@@ -1156,21 +1145,20 @@ static prom_status launch_dw_tc(const int8_t *x, int batch, int h, int w, int c,
     if (workers < 1) workers = 1;
     if (workers > p.tiles) workers = p.tiles;
     const int grid = (int)(workers * p.groups);
-    p.pdl = pdl ? 1 : 0;
-    p.pdl_next = pdl_next ? 1 : 0;
+    p.pdl = pdl;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    fill_launch_cfg(cfg, attr, grid, dwtc::kThreads, dwtc::kSmemBytes, st, pdl);
+    fill_launch_cfg(cfg, attr, grid, dwtc::kThreads, dwtc::kSmemBytes, st, pdl != 0);
     const cudaError_t e = cudaLaunchKernelEx(&cfg, dwtc::dw3x3_tc_kernel, map, p);
     ++g_launches;
     return cuda_status(e);
 }
 
-// pdl / pdl_next: the call is a link of a layer sequence (programmatic dependent launch behind the
-// kernel that writes x; the next kernel of the stream is launched that way)
+// pdl: how the kernel is chained to the previous one of the stream (tc.cuh: kPdl*); it may always
+// be chained to
 static prom_status dw_conv3x3(const int8_t *x_dev, int batch, int h, int w, int c, int stride,
                               const int8_t *w_dev, const prom_requant *rq, int8_t *y_dev, void *cuda_stream,
-                              bool pdl, bool pdl_next)
+                              int pdl)
 {
     if (batch < 0 || h < 1 || w < 1 || c < 1 || c > 4096 || (stride != 1 && stride != 2)) return PROM_ERR_SHAPE;
     if (c & 3) return PROM_ERR_UNSUPPORTED;
@@ -1192,7 +1180,7 @@ static prom_status dw_conv3x3(const int8_t *x_dev, int batch, int h, int w, int 
     if (dw_variant != 1 && stride == 1 && (c & 15) == 0 &&
         !(dw_variant == 0 && ((long long)batch * h * w < 128 || h * w < 100))) {
         const prom_status e = launch_dw_tc(x_dev, batch, h, w, c, w_dev, rq, y_dev, d,
-                                           static_cast<cudaStream_t>(cuda_stream), pdl, pdl_next);
+                                           static_cast<cudaStream_t>(cuda_stream), pdl);
         if (e != PROM_ERR_UNSUPPORTED) return e;
     }
     if (dw_variant == 2) return PROM_ERR_UNSUPPORTED;
@@ -1212,15 +1200,14 @@ static prom_status dw_conv3x3(const int8_t *x_dev, int batch, int h, int w, int 
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    fill_launch_cfg(cfg, attr, grid, dw::kThreads, 0, st, pdl);
-    const int f_pdl = pdl ? 1 : 0, f_next = pdl_next ? 1 : 0;
+    fill_launch_cfg(cfg, attr, grid, dw::kThreads, 0, st, pdl != 0);
     cudaError_t le;
     if (stride == 1)
         le = cudaLaunchKernelEx(&cfg, dw::dw3x3_kernel<1>, x_dev, batch, h, w, c, ho, wo, w_dev, rq->bias, rq->mult,
-                                rq->shift, rq->act_min, rq->act_max, y_dev, f_pdl, f_next);
+                                rq->shift, rq->act_min, rq->act_max, y_dev, pdl);
     else
         le = cudaLaunchKernelEx(&cfg, dw::dw3x3_kernel<2>, x_dev, batch, h, w, c, ho, wo, w_dev, rq->bias, rq->mult,
-                                rq->shift, rq->act_min, rq->act_max, y_dev, f_pdl, f_next);
+                                rq->shift, rq->act_min, rq->act_max, y_dev, pdl);
     ++g_launches;
     return cuda_status(le);
 }
@@ -1389,8 +1376,10 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
         c.y = (i == n - 1) ? y_out
               : (chained ? reinterpret_cast<int8_t *>(chain_base + lay.cbuf_off[i]) : reg[i & 1]);
         c.st = st;
-        c.pdl = i > 0;
-        c.pdl_next = i + 1 < n;
+        // the first kernel waits before it reads anything (the operands prepared below included) and
+        // before it releases its successor, so every later link finds weights and operands complete
+        c.pdl = i > 0 || layers[i].dw_w ? tc::kPdlChain : tc::kPdlWait;
+        c.pdl_next = true;
         // The block's input is the output of layer i-2, which sits where this layer's output
         // goes (unless a chain wrote it to a buffer of its own: then the sum reads from there).
         if (layers[i].add_block_input) c.res = i == 1 ? x0 : conv[i - 2].y;
@@ -1448,9 +1437,12 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
             }
             if (t.n == 0) break;
             t.first[t.n] = ctas;
-            tc::tc_prep_kernel<<<ctas, tc::kThreads, smem, st>>>(t);
+            cudaLaunchConfig_t cfg;
+            cudaLaunchAttribute attr[1];
+            fill_launch_cfg(cfg, attr, ctas, tc::kThreads, smem, st, true);
+            const cudaError_t e = cudaLaunchKernelEx(&cfg, tc::tc_prep_kernel, t);
             ++g_launches;
-            if (cudaGetLastError() != cudaSuccess) return PROM_ERR_CUDA;
+            if (e != cudaSuccess) return PROM_ERR_CUDA;
         }
     }
 
@@ -1499,7 +1491,8 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
             // chained like the pointwise kernels: behind layer i-1's kernel (which releases its
             // dependents at entry) and in front of layer i's, which waits for it before its loads
             prom_status de = dw_conv3x3(src, batch, s.h[i] * stride, s.w[i] * stride, layers[i].cin, stride,
-                                        layers[i].dw_w, &layers[i].dw_rq, dw_buf, st, i > 0, true);
+                                        layers[i].dw_w, &layers[i].dw_rq, dw_buf, st,
+                                        i > 0 ? tc::kPdlChain : tc::kPdlWait);
             if (de != PROM_OK) return de;
         }
         prom_status e = is_tc[i] ? tc_launch_planned(conv[i], plan[i]) : run_conv(conv[i], variant);
@@ -1590,10 +1583,13 @@ prom_status prom_quantize_ternary(const float *w_dev, int cout, int cin, uint8_t
     if (!d.ok) return PROM_ERR_CUDA;
     const int want = (cout + quant::kWarps - 1) / quant::kWarps;        // a warp per row
     const int grid = want < d.sms * 16 ? want : d.sms * 16;
-    quant::quantize_ternary_kernel<<<grid, quant::kThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-        w_dev, cout, cin, 1e-5, packed_dev, alpha_dev);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    fill_launch_cfg(cfg, attr, grid, quant::kThreads, 0, static_cast<cudaStream_t>(cuda_stream), true);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, quant::quantize_ternary_kernel, w_dev, cout, cin, 1e-5, packed_dev,
+                                             alpha_dev);
     ++g_launches;
-    return cuda_status(cudaGetLastError());
+    return cuda_status(e);
 }
 
 prom_status prom_quantize_ternary_batch(const prom_quantize_job *jobs, int n, void *cuda_stream)
@@ -1622,10 +1618,12 @@ prom_status prom_quantize_ternary_batch(const prom_quantize_job *jobs, int n, vo
         t.first_row[t.n] = rows;
         const int want = (rows + quant::kWarps - 1) / quant::kWarps;      // a warp per row
         const int grid = want < d.sms * 16 ? want : d.sms * 16;
-        quant::quantize_ternary_batch_kernel<<<grid, quant::kThreads, 0, static_cast<cudaStream_t>(cuda_stream)>>>(
-            t, 1e-5);
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr[1];
+        fill_launch_cfg(cfg, attr, grid, quant::kThreads, 0, static_cast<cudaStream_t>(cuda_stream), true);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, quant::quantize_ternary_batch_kernel, t, 1e-5);
         ++g_launches;
-        if (cudaGetLastError() != cudaSuccess) return PROM_ERR_CUDA;
+        if (e != cudaSuccess) return PROM_ERR_CUDA;
     }
     return PROM_OK;
 }
@@ -1634,7 +1632,7 @@ prom_status prom_dw_conv3x3_i8(const int8_t *x_dev, int batch, int h, int w, int
                                const int8_t *w_dev, const prom_requant *rq, int8_t *y_dev,
                                void *cuda_stream)
 {
-    return dw_conv3x3(x_dev, batch, h, w, c, stride, w_dev, rq, y_dev, cuda_stream, false, false);
+    return dw_conv3x3(x_dev, batch, h, w, c, stride, w_dev, rq, y_dev, cuda_stream, tc::kPdlWait);
 }
 
 prom_status prom_pw_conv_i8_dyn(const int8_t *x_dev, int batch, int64_t rows_per_sample, int cin,
@@ -1659,9 +1657,8 @@ prom_status prom_pw_conv_i8_dyn(const int8_t *x_dev, int batch, int64_t rows_per
     if (tc_set_attr(d) != PROM_OK) return PROM_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     Conv c;
-    memset(&c, 0, sizeof(c));
     c.x = x_dev; c.m = m; c.cin = cin; c.cout = cout; c.map = plain; c.in_rows = m;
-    c.w = w_packed_dev; c.y = q_dev; c.st = st; c.pdl = false; c.pdl_next = false;
+    c.w = w_packed_dev; c.y = q_dev; c.st = st;
     c.rq.bias = nullptr; c.rq.shift = nullptr;
     c.rq.mult = reinterpret_cast<const int32_t *>(alpha_dev);     // bit patterns of alpha
     c.rq.act_min = -128; c.rq.act_max = 127;                      // keeps the weights at +-1
@@ -1713,7 +1710,7 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
         cfg.blockDim = dim3(actq::kThreads);
         cfg.dynamicSmemBytes = (size_t)slice * 4;
         cfg.stream = st;
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = (unsigned)cluster;
         attr[0].val.clusterDim.y = 1;
@@ -1744,6 +1741,9 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
         if (resident > 0) {
             const int nclusters = resident < batch ? resident : batch;
             cfg.gridDim = dim3((unsigned)(nclusters * cluster));
+            attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[1].val.programmaticStreamSerializationAllowed = 1;
+            cfg.numAttrs = 2;
             cudaError_t e = cudaLaunchKernelEx(&cfg, actq::act_quant_cluster_kernel, x_dev, batch,
                                                (long long)per_sample, slice, eps, q_dev, gamma_dev,
                                                scale_dev);
@@ -1763,7 +1763,7 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
         cfg.gridDim = dim3((unsigned)c);
         cfg.blockDim = dim3(actq::kThreads);
         cfg.stream = st;
-        cudaLaunchAttribute attr[1];
+        cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = (unsigned)c;
         attr[0].val.clusterDim.y = 1;
@@ -1791,6 +1791,9 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
         if (resident > 0 && s * 4 <= (8ll << 20)) {
             const int nclusters = resident < batch ? resident : batch;
             cfg.gridDim = dim3((unsigned)(nclusters * c));
+            attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[1].val.programmaticStreamSerializationAllowed = 1;
+            cfg.numAttrs = 2;
             cudaError_t e = cudaLaunchKernelEx(&cfg, actq::act_quant_reread_kernel, x_dev, batch,
                                                (long long)per_sample, s, eps, q_dev, gamma_dev, scale_dev);
             ++g_launches;
@@ -1844,8 +1847,6 @@ prom_status prom_pw_conv_i8(const int8_t *x_dev, int64_t m, int cin, const uint8
     c.in_rows = m;
     c.w = w_packed_dev; c.rq = *rq; c.y = y_dev;
     c.st = static_cast<cudaStream_t>(cuda_stream);
-    c.pdl = false;
-    c.pdl_next = false;
     return run_conv(c, variant);
 }
 
@@ -1882,7 +1883,6 @@ prom_status prom_pw_prepare(int64_t m, int cin, const uint8_t *w_packed_dev, int
     Conv c;
     c.x = nullptr; c.m = m; c.cin = cin; c.cout = cout; c.map = RowMap{1, 1, 1, 1, 1}; c.in_rows = m;
     c.w = w_packed_dev; c.rq = *rq; c.y = nullptr; c.st = static_cast<cudaStream_t>(cuda_stream);
-    c.pdl = false; c.pdl_next = false;
     tc_bind(c, pl, static_cast<uint8_t *>(prepared_dev));
     tc::PrepTable t;
     memset(&t, 0, sizeof(t));
@@ -1890,9 +1890,12 @@ prom_status prom_pw_prepare(int64_t m, int cin, const uint8_t *w_packed_dev, int
     t.first[0] = 0;
     t.first[1] = pl.p.groups;
     t.layer[0] = pl.p;
-    tc::tc_prep_kernel<<<pl.p.groups, tc::kThreads, pl.smem, c.st>>>(t);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    fill_launch_cfg(cfg, attr, pl.p.groups, tc::kThreads, pl.smem, c.st, true);
+    const cudaError_t le = cudaLaunchKernelEx(&cfg, tc::tc_prep_kernel, t);
     ++g_launches;
-    return cuda_status(cudaGetLastError());
+    return cuda_status(le);
 }
 
 prom_status prom_pw_conv_i8_prepared(const int8_t *x_dev, int64_t m, int cin, int cout, const void *prepared_dev,
@@ -1912,7 +1915,6 @@ prom_status prom_pw_conv_i8_prepared(const int8_t *x_dev, int64_t m, int cin, in
     c.x = x_dev; c.m = m; c.cin = cin; c.cout = cout; c.map = RowMap{1, 1, 1, 1, 1}; c.in_rows = m;
     c.w = nullptr; c.rq = prom_requant{nullptr, nullptr, nullptr, act_min, act_max}; c.y = y_dev;
     c.st = static_cast<cudaStream_t>(cuda_stream);
-    c.pdl = false; c.pdl_next = false;
     tc_bind(c, pl, const_cast<uint8_t *>(static_cast<const uint8_t *>(prepared_dev)));
     return tc_launch_planned(c, pl);
 }
@@ -1933,8 +1935,6 @@ prom_status prom_pw_conv_i8_res(const int8_t *x_dev, int64_t m, int cin, const u
     c.in_rows = m;
     c.w = w_packed_dev; c.rq = *rq; c.y = y_dev;
     c.st = static_cast<cudaStream_t>(cuda_stream);
-    c.pdl = false;
-    c.pdl_next = false;
     c.res = res_dev;
     return run_conv(c, variant);
 }
@@ -1954,8 +1954,6 @@ prom_status prom_pw_conv_i8_acc32(const int8_t *x_dev, int64_t m, int cin,
     c.rq = prom_requant{nullptr, nullptr, nullptr, 0, 127};
     c.y = nullptr;
     c.st = static_cast<cudaStream_t>(cuda_stream);
-    c.pdl = false;
-    c.pdl_next = false;
     return launch_naive(c, acc_dev);
 }
 

@@ -49,8 +49,7 @@ struct Params {
     const int8_t *shift;
     int lo, hi;
     int8_t *y;
-    int pdl;                // launched with programmatic dependent launch behind the kernel that writes x
-    int pdl_next;           // the next kernel of the stream is launched that way
+    int pdl;                // how it is chained to the previous kernel of the stream (tc.cuh: kPdl*)
 };
 
 // Unswizzled K-major operand: core matrices of 8 rows x 16 bytes; `k_off` bytes from a core
@@ -83,7 +82,7 @@ __global__ void __launch_bounds__(kThreads, 2) dw3x3_tc_kernel(const __grid_cons
     const int ch0 = g * p.ns * 16;                        // its first channel
     const int nch = p.ns * 16;
 
-    if (p.pdl_next) ptx::grid_dep_launch();
+    if (p.pdl != tc::kPdlWait) ptx::grid_dep_launch();
 
     // ---- prologue (nothing here reads the previous kernel's output) -------------------------
     if (warp == 0) {
@@ -102,6 +101,10 @@ __global__ void __launch_bounds__(kThreads, 2) dw3x3_tc_kernel(const __grid_cons
         ptx::mbar_init_fence();
     }
     if (warp == 1) ptx::tmem_alloc(ptx::smem_u32((const void *)tmem_slot), 128u);
+    if (p.pdl == tc::kPdlWait) {
+        ptx::grid_dep_wait();
+        ptx::grid_dep_launch();
+    }
     // weights blocks: slice s, tap pair t: 16 rows (channel n) x 32 bytes, as four core matrices
     // {k half, n half}; row n holds tap 2t at byte n and tap 2t+1 at byte 16 + n
     for (int i = threadIdx.x; i < p.ns * 5 * 32; i += kThreads) {
@@ -137,7 +140,7 @@ __global__ void __launch_bounds__(kThreads, 2) dw3x3_tc_kernel(const __grid_cons
         if (lane == 0) {
             uint32_t slot = 0, ph = 0, issued = 0;
             bool ok = true;
-            if (p.pdl) ptx::grid_dep_wait();      // the loads are the only reads of x
+            if (p.pdl == tc::kPdlChain) ptx::grid_dep_wait();      // the loads are the only reads of x
             for (long long t = worker; t < p.tiles && ok; t += nworkers) {
                 const int b = (int)(t / tiles_img), r = (int)(t - (long long)b * tiles_img);
                 const int ty = r / p.tiles_x, tx = r - ty * p.tiles_x;
@@ -245,7 +248,7 @@ __global__ void __launch_bounds__(kThreads, 2) dw3x3_tc_kernel(const __grid_cons
 
     // ---- teardown -------------------------------------------------------------------------------
     // every CTA waits for the previous kernel before it ends, also one whose loader had no tile
-    if (p.pdl && threadIdx.x == 32) ptx::grid_dep_wait();
+    if (p.pdl == tc::kPdlChain && threadIdx.x == 32) ptx::grid_dep_wait();
     ptx::tc_fence_before_sync();
     __syncthreads();
     if (warp == 1) {

@@ -10,6 +10,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "ptx.cuh"
 
 namespace prom { namespace quant {
 
@@ -82,6 +83,8 @@ __global__ void __launch_bounds__(kThreads)
 quantize_ternary_kernel(const float *__restrict__ w, int cout, int cin, double eps,
                         uint8_t *__restrict__ packed, float *__restrict__ alpha)
 {
+    ptx::grid_dep_wait();           // launched with programmatic dependent launch
+    ptx::grid_dep_launch();
     const int rowb = (cin + 3) >> 2;
     const int warp = blockIdx.x * kWarps + (threadIdx.x >> 5), nwarps = gridDim.x * kWarps;
     for (int o = warp; o < cout; o += nwarps)
@@ -103,6 +106,8 @@ struct Jobs {
 __global__ void __launch_bounds__(kThreads)
 quantize_ternary_batch_kernel(const __grid_constant__ Jobs jobs, double eps)
 {
+    ptx::grid_dep_wait();           // launched with programmatic dependent launch
+    ptx::grid_dep_launch();
     const int warp = blockIdx.x * kWarps + (threadIdx.x >> 5), nwarps = gridDim.x * kWarps;
     int j = 0;
     for (int r = warp; r < jobs.first_row[jobs.n]; r += nwarps) {

@@ -46,6 +46,14 @@ constexpr int kBiasHiDigits = 30;        // A-const row: 1, 1, then 30 x 127
 constexpr int kBiasMax = 127 * 127 * kBiasHiDigits;
 constexpr int kNoColumn = -1000;        // marks a padding column (no int8 shift has this value)
 
+// What a kernel launched with programmatic dependent launch may read before it waits for its
+// predecessor.  kPdlChain: everything but activations (a link of a layer sequence, whose weights and
+// constants are complete before its first kernel starts).  kPdlWait: nothing (a call of its own, behind
+// whatever kernel the stream holds): barriers, tensor memory and constant tables are set up while that
+// kernel ends, and only behind the wait does it release its own successor, so that every kernel before
+// it is complete by the time the successor runs.
+constexpr int kPdlChain = 1, kPdlWait = 2;
+
 struct Params {
     long long m_rows;   // rows of the folded problem
     int k0, n0;         // layer cin, cout
@@ -75,8 +83,8 @@ struct Params {
     const int8_t *shift;
     int act_min, act_max;
     int8_t *y;
-    int pdl;            // launched with programmatic dependent launch
-    int pdl_next;       // the next kernel in the stream is launched that way
+    int pdl;            // launched with programmatic dependent launch: kPdl* below
+    int pdl_next;       // the next kernel in the stream may be launched that way
     int reverse;        // row tiles are taken from the last to the first
     // The dynamic layer (kernel modes 1 and 2): `mult` then holds the bit patterns of the
     // float per-channel factors alpha, bias and shift are not read, and rows belong to
@@ -492,13 +500,30 @@ __device__ __forceinline__ void build_aconst(uint8_t *aconst_smem, int tid, int 
     }
 }
 
+// Code tables: byte of four 2-bit codes -> four int8 of magnitude 1, 4, 8, .., 64.
+__device__ __forceinline__ void build_luts(uint32_t *lut, int tid, int nthreads)
+{
+    for (int i = tid; i < kLuts * 256; i += nthreads) {
+        const uint32_t t = (uint32_t)i >> 8, byte = (uint32_t)i & 255u;
+        const uint32_t mag = t == 0 ? 1u : (2u << t), neg = 256u - mag;
+        uint32_t w4 = 0;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const uint32_t code = (byte >> (2 * e)) & 3u;
+            const uint32_t val = code == 1u ? mag : (code == 3u ? neg : 0u);
+            w4 |= val << (8 * e);
+        }
+        lut[i] = w4;
+    }
+}
+
 // Builds the prepared operands of channel group g in shared memory: requantisation
 // constants checked and stored, the fast/exact decision, bias digits, and the 2-bit weights
 // expanded into the K-major swizzled int8 operand layout.  All kThreads threads take part
 // (three block-wide syncs inside); on return the header is written but not yet synchronised.
 // Thread 0 starts the bulk copy of the group's packed weights into the not yet used
-// activation stages; meanwhile every thread requests the constants of its channels and
-// builds the code tables.
+// activation stages; meanwhile every thread requests the constants of its channels.  The code tables
+// have been written by the caller (the first of the syncs is behind them).
 __device__ __forceinline__ void build_image(const Params &p, const int g, const View &vw)
 {
     uint8_t *const smem = vw.smem;
@@ -514,7 +539,7 @@ __device__ __forceinline__ void build_image(const Params &p, const int g, const 
     const uint32_t cw = (uint32_t)p.cw;
     // Thread 0 sets up the barriers and starts the bulk copy of this CTA's packed (2-bit)
     // weights into the not yet used activation stages; meanwhile every thread requests the
-    // constants of its channels and builds the code tables.  Three block-wide syncs in all.
+    // constants of its channels.  Three block-wide syncs in all.
     const int rowb = (p.k0 + 3) >> 2;
     const uint8_t *wq = smem;                    // packed weights: rows of rowb bytes
     if (threadIdx.x == 0) {
@@ -553,19 +578,6 @@ __device__ __forceinline__ void build_image(const Params &p, const int g, const 
                 cs_[u] = p.dyn ? 0 : (int)__ldg(p.shift + n);
             }
         }
-    }
-    // code tables: byte of four 2-bit codes -> four int8 of magnitude 1, 4, 8, .., 64
-    for (int i = threadIdx.x; i < kLuts * 256; i += kThreads) {
-        const uint32_t t = (uint32_t)i >> 8, byte = (uint32_t)i & 255u;
-        const uint32_t mag = t == 0 ? 1u : (2u << t), neg = 256u - mag;
-        uint32_t w4 = 0;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const uint32_t code = (byte >> (2 * e)) & 3u;
-            const uint32_t val = code == 1u ? mag : (code == 3u ? neg : 0u);
-            w4 |= val << (8 * e);
-        }
-        lut[i] = w4;
     }
     __syncthreads();                                        // barriers and flags are set up
 
@@ -756,17 +768,20 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
 
     // Let the next kernel of the stream start its own prologue as soon as there is room for
     // it; it waits for this grid to finish before it touches activations.
-    if (p.pdl_next) ptx::grid_dep_launch();
+    if (p.pdl_next && p.pdl != kPdlWait) ptx::grid_dep_launch();
 
     // ---- prologue: nothing here depends on the previous kernel's output -------------
-    if (threadIdx.x == 0 && p.image) {
-        // prepared by tc_prep_kernel: one bulk copy, started before anything else
-        ptx::mbar_init(bar_wload, 1);
-        ptx::mbar_init_fence();
+    // the image prepared by tc_prep_kernel: one bulk copy
+    auto load_image = [&] {
         ptx::mbar_expect_tx(bar_wload, p.image_bytes);
         ptx::bulk_load(smem_base + p.off_w, p.image + (size_t)g * p.image_stride, p.image_bytes,
                        bar_wload);
+    };
+    if (threadIdx.x == 0 && p.image) {
+        ptx::mbar_init(bar_wload, 1);
+        ptx::mbar_init_fence();
         flags[0] = 0;
+        if (p.pdl != kPdlWait) load_image();        // started before anything else
     }
     if (warp == 0) {
         // the pipeline's barriers, one lane each
@@ -785,6 +800,14 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     }
     if (warp == 1) ptx::tmem_alloc(ptx::smem_u32((const void *)tmem_slot), (uint32_t)p.tmem_cols);
     const View vw = make_view(p, smem, bars);
+    if (p.pdl == kPdlWait) {
+        if (!p.image) build_luts(vw.lut, (int)threadIdx.x, kThreads);
+        ptx::grid_dep_wait();
+        if (p.pdl_next) ptx::grid_dep_launch();
+        if (threadIdx.x == 0 && p.image) load_image();
+    } else if (!p.image) {
+        build_luts(vw.lut, (int)threadIdx.x, kThreads);
+    }
     // With a prepared image, warp 0 (the producer) does not take part in the rest of the
     // prologue: it announces the barriers and goes straight to its loads, which need neither
     // weights nor constants, while the other nine warps wait for the image.
@@ -845,7 +868,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 bool ok = true;
                 // Only this thread reads what the previous kernel wrote; everything else in the
                 // CTA follows from its loads, so it alone waits for that kernel to finish.
-                if (p.pdl) ptx::grid_dep_wait();
+                if (p.pdl == kPdlChain) ptx::grid_dep_wait();
                 for (int mt = worker; mt < p.n_mtiles && ok; mt += nworkers) {
                     const int mtx = p.reverse ? p.n_mtiles - 1 - mt : mt;
                     const int c_row = p.x3d ? mtx * p.box_r : mtx * p.tm;
@@ -965,7 +988,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
             const int q = warp & 3;                     // TMEM lane quarter of this warp
             if constexpr (MODE == 3) {
                 // the residual was written two kernels back: complete once the previous one is
-                if (p.pdl) ptx::grid_dep_wait();
+                if (p.pdl == kPdlChain) ptx::grid_dep_wait();
             }
             // Unit u goes to group u % 2 and accumulator u % nbuf; nbuf is even, so a group meets
             // each of its accumulators in cyclic order and never waits on a barrier that is more
@@ -1135,7 +1158,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     // ---- teardown -------------------------------------------------------------------------
     // A CTA whose roles were skipped has not waited for the previous kernel yet; it must, or
     // this grid could end (and release the next one) while that kernel is still running.
-    if (p.pdl && bad_consts && threadIdx.x == 0) ptx::grid_dep_wait();
+    if (p.pdl == kPdlChain && bad_consts && threadIdx.x == 0) ptx::grid_dep_wait();
     ptx::tc_fence_before_sync();
     __syncthreads();
     if (warp == 1) {
@@ -1186,6 +1209,10 @@ tc_prep_kernel(const __grid_constant__ PrepTable t)
     const int g = (int)blockIdx.x - t.first[l];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + p.off_bars);
     const View vw = make_view(p, smem, bars);
+    build_luts(vw.lut, (int)threadIdx.x, kThreads);
+    // a call of its own, like kPdlWait
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
     build_image(p, g, vw);
     ptx::fence_proxy_async_smem();
     __syncthreads();
