@@ -1111,45 +1111,64 @@ static void seq_layout(const prom_layer *layers, int n, const SeqShape &s, const
 // ---- depthwise 3x3 on the tensor cores (dwtc.cuh) ---------------------------------------------
 // 0: the library's choice, 1: CUDA cores only, 2: tensor cores or PROM_ERR_UNSUPPORTED
 static std::atomic<int> g_dw_variant{0};
+// Outputs from which the tensor-core kernel is the better one: a call of it costs about 6 us whatever its
+// size (tensor memory and weight blocks to set up, one CTA of 190 KB per SM, so that little of this
+// overlaps the kernel in front) against 3 us, and then 0.4 us per million outputs against 1.0 (stride 1)
+// and 0.8 against 1.8 (stride 2).  Measured alone the lines cross at 3.3 to 5.6 million, inside the
+// network's body at 3 to 6 million.
+constexpr long long kDwTcOutputs = 4ll << 20;
 
+template <int STRIDE>
 static prom_status launch_dw_tc(const int8_t *x, int batch, int h, int w, int c, const int8_t *wt,
                                 const prom_requant *rq, int8_t *y, const DeviceInfo &d, cudaStream_t st, int pdl)
 {
     EncodeTiledFn enc = encode_tiled_fn();
     if (!enc) return PROM_ERR_UNSUPPORTED;
-    const int slices = c / 16;
-    int ns = dwtc::kMaxSlices;
-    while (slices % ns) --ns;
     dwtc::Params p;
     memset(&p, 0, sizeof(p));
-    p.batch = batch; p.h = h; p.w = w; p.c = c; p.ns = ns; p.groups = slices / ns;
-    p.tiles_y = (h + dwtc::kTileH - 1) / dwtc::kTileH;
-    p.tiles_x = (w + dwtc::kTileW - 1) / dwtc::kTileW;
-    p.tiles = (long long)batch * p.tiles_y * p.tiles_x;
+    p.batch = batch; p.h = h; p.w = w; p.c = c;
+    p.ho = (h - 1) / STRIDE + 1; p.wo = (w - 1) / STRIDE + 1;
+    p.segs = (p.wo + 7) / 8;
+    const long long groups = (long long)batch * p.segs;
+    if (groups >= (1ll << 30) || h >= (1 << 30) || w >= (1 << 30)) return PROM_ERR_UNSUPPORTED;
+    p.groups = (int)groups;
+    p.blocks = (c + dwtc::kBlock - 1) / dwtc::kBlock;
+    p.rows = (groups + dwtc::kGroups - 1) / dwtc::kGroups * p.ho;
     p.wt = wt; p.bias = rq->bias; p.mult = rq->mult; p.shift = rq->shift; p.lo = rq->act_min; p.hi = rq->act_max;
-    p.y = y;
-    if (p.groups > 2 * d.sms || p.tiles >= (1ll << 31)) return PROM_ERR_UNSUPPORTED;
-    // {channel in slice, x, y, slice, image}: the slice is a dimension of its own (16 bytes apart),
-    // so that the patches of a group's slices land one after the other in shared memory
-    CUtensorMap map;
-    cuuint64_t dims[5] = {16, (cuuint64_t)w, (cuuint64_t)h, (cuuint64_t)slices, (cuuint64_t)batch};
-    cuuint64_t strides[4] = {(cuuint64_t)c, (cuuint64_t)w * c, 16, (cuuint64_t)h * w * c};
-    cuuint32_t box[5] = {16, (cuuint32_t)dwtc::kPatchW, (cuuint32_t)dwtc::kPatchH, (cuuint32_t)ns, 1};
-    cuuint32_t es[5] = {1, 1, 1, 1, 1};
-    if (enc(&map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 5, const_cast<int8_t *>(x), dims, strides, box, es,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return PROM_ERR_UNSUPPORTED;
-    if (raise_smem_limit(dwtc::dw3x3_tc_kernel, (int)dwtc::kSmemBytes) != cudaSuccess) return PROM_ERR_CUDA;
-    long long workers = (2ll * d.sms) / p.groups;
-    if (workers < 1) workers = 1;
-    if (workers > p.tiles) workers = p.tiles;
-    const int grid = (int)(workers * p.groups);
-    p.pdl = pdl;
+    p.y = y; p.pdl = pdl;
+    if (p.blocks > d.sms) return PROM_ERR_UNSUPPORTED;
+    // equal contiguous shares of the output rows; a share of a few rows would load mostly halo
+    const long long workers = d.sms / p.blocks;
+    long long per = (p.rows + workers - 1) / workers;
+    const int least = STRIDE == 1 ? 6 : 3;
+    if (per < least) per = least;
+    if (per >= (1ll << 31)) return PROM_ERR_UNSUPPORTED;
+    p.per_worker = (int)per;
+    const int grid = (int)((p.rows + per - 1) / per) * p.blocks;
+    // {channel, column, row, image}; with stride 2 one map of the odd and one of the even columns
+    auto map_of = [&](CUtensorMap *m, const int8_t *base, int cols, int step, int px) {
+        cuuint64_t dims[4] = {(cuuint64_t)c, (cuuint64_t)cols, (cuuint64_t)h, (cuuint64_t)batch};
+        cuuint64_t strides[3] = {(cuuint64_t)step * c, (cuuint64_t)w * c, (cuuint64_t)h * w * c};
+        cuuint32_t box[4] = {(cuuint32_t)dwtc::kBlock, (cuuint32_t)px, (cuuint32_t)dwtc::kBoxRows, 1};
+        cuuint32_t es[4] = {1, 1, 1, 1};
+        return enc(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<int8_t *>(base), dims, strides, box, es,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+    };
+    CUtensorMap xmap, emap;
+    if (STRIDE == 1) {
+        if (!map_of(&xmap, x, w, 1, dwtc::kPx)) return PROM_ERR_UNSUPPORTED;
+        emap = xmap;        // unused
+    } else {
+        if (w < 2 || !map_of(&xmap, x + c, w / 2, 2, dwtc::kPx) || !map_of(&emap, x, (w + 1) / 2, 2, 8))
+            return PROM_ERR_UNSUPPORTED;
+    }
+    const int smem = (int)dwtc::smem_bytes(STRIDE);
+    if (raise_smem_limit(dwtc::dw3x3_tc_kernel<STRIDE>, smem) != cudaSuccess) return PROM_ERR_CUDA;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    fill_launch_cfg(cfg, attr, grid, dwtc::kThreads, dwtc::kSmemBytes, st, pdl != 0);
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, dwtc::dw3x3_tc_kernel, map, p);
+    fill_launch_cfg(cfg, attr, grid, dwtc::kThreads, (size_t)smem, st, pdl != 0);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, dwtc::dw3x3_tc_kernel<STRIDE>, xmap, emap, p);
     ++g_launches;
     return cuda_status(e);
 }
@@ -1173,14 +1192,13 @@ static prom_status dw_conv3x3(const int8_t *x_dev, int batch, int h, int w, int 
     if ((long long)batch * h * w * c >= (1ll << 40)) return PROM_ERR_SHAPE;
     DeviceInfo d = device_info();
     if (!d.ok) return PROM_ERR_CUDA;
-    // stride 1 and whole slices of 16 channels: TMA patches and tensor-core taps
+    // whole slices of 16 channels and enough work: TMA patches and tensor-core taps
     const int dw_variant = g_dw_variant.load();
-    // (left to itself the library keeps images of fewer than 100 pixels on the CUDA cores: a 7 x 7
-    // image fills 49 of a tile's 128 rows, and [128,7,7,960] takes 18.6 us there against 14.8 us)
-    if (dw_variant != 1 && stride == 1 && (c & 15) == 0 &&
-        !(dw_variant == 0 && ((long long)batch * h * w < 128 || h * w < 100))) {
-        const prom_status e = launch_dw_tc(x_dev, batch, h, w, c, w_dev, rq, y_dev, d,
-                                           static_cast<cudaStream_t>(cuda_stream), pdl);
+    if (dw_variant != 1 && (c & 15) == 0 &&
+        (dw_variant == 2 || (long long)batch * ho * wo * c >= kDwTcOutputs)) {
+        cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+        const prom_status e = stride == 1 ? launch_dw_tc<1>(x_dev, batch, h, w, c, w_dev, rq, y_dev, d, st, pdl)
+                                          : launch_dw_tc<2>(x_dev, batch, h, w, c, w_dev, rq, y_dev, d, st, pdl);
         if (e != PROM_ERR_UNSUPPORTED) return e;
     }
     if (dw_variant == 2) return PROM_ERR_UNSUPPORTED;

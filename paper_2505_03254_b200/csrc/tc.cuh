@@ -136,6 +136,25 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity, volatile
     }
 }
 
+// The same wait by a whole converged warp, which leaves it converged: without that a lane that polls
+// late could be overtaken by the others and find its phase two completions in the past.  (A role that
+// runs warp-wide needs it; one lane alone, or a warp with a __syncwarp per phase, does not.)
+__device__ __forceinline__ bool wait_bar_warp(uint32_t bar, uint32_t parity, volatile int *abort_flag)
+{
+    return __all_sync(0xFFFFFFFFu, wait_bar(bar, parity, abort_flag));
+}
+
+// The loading thread's last act: the copies it has issued must have landed before its CTA may go away,
+// also when another role gives up.  `bar_full` are the barriers of a ring of `stages`, used in turn.
+__device__ __noinline__ void drain_copies(uint32_t bar_full, uint32_t stages, uint32_t issued)
+{
+    for (uint32_t j = issued > stages ? issued - stages : 0; j < issued; ++j) {
+        const unsigned long long t0 = ptx::globaltimer();
+        while (!ptx::mbar_try_wait(bar_full + 8 * (j % stages), (j / stages) & 1u) &&
+               ptx::globaltimer() - t0 < kWaitLimitNs) {}
+    }
+}
+
 // K-major operand with rows of `cw` bytes swizzled over a span of `cw` bytes:
 // 8-row atoms of 8*cw bytes, one after the other.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t cw)
@@ -887,16 +906,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         }
                     }
                 }
-                if (!ok) {
-                    // let the copies already issued land before the CTA goes away
-                    const uint32_t first = issued > (uint32_t)p.stages ? issued - p.stages : 0;
-                    for (uint32_t j = first; j < issued; ++j) {
-                        const unsigned long long t0 = ptx::globaltimer();
-                        while (!ptx::mbar_try_wait(bar_full + 8 * (j % p.stages),
-                                                   (j / p.stages) & 1u) &&
-                               ptx::globaltimer() - t0 < kWaitLimitNs) {}
-                    }
-                }
+                drain_copies(bar_full, (uint32_t)p.stages, issued);
             }
         } else if (warp == 1) {
             // ---- MMA issuer ---------------------------------------------------------
