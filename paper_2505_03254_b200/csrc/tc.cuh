@@ -758,7 +758,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     // access below a generic one)
     uint8_t *smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
     const uint32_t smem_base = ptx::smem_u32(smem);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
     constexpr int CH = MINB >= 3 ? 16 : 32;     // columns per tensor-memory load in the epilogue
 
     uint8_t *w_smem = smem + p.off_w;
@@ -880,7 +880,8 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         // descriptors are advanced by additions, never recomputed with divisions.
         if (warp == 0) {
             // ---- TMA producer ----------------------------------------------------
-            if (lane == 0) {
+            {
+                const bool leader = ptx::elect_one();      // warp-wide like the MMA issuer
                 uint32_t s = 0, ph = 0, issued = 0;
                 uint32_t dst = smem_base, bfull = bar_full, bempty = bar_empty;
                 const int cx_end = p.share_x ? p.cw : p.kc * p.cw;
@@ -893,10 +894,12 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     const int c_row = p.x3d ? mtx * p.box_r : mtx * p.tm;
                     int cx = 0;
                     for (int l = 0; l < loads_per_tile; ++l) {
-                        if (!wait_bar(bempty, ph ^ 1u, flags)) { ok = false; break; }
-                        ptx::mbar_expect_tx(bfull, p.tx_bytes);
-                        if (p.x3d) ptx::tma_load_3d(dst, &xmap, cx, 0, c_row, bfull);
-                        else ptx::tma_load_2d(dst, &xmap, cx, c_row, bfull);
+                        if (!wait_bar_warp(bempty, ph ^ 1u, flags)) { ok = false; break; }
+                        if (leader) {
+                            ptx::mbar_expect_tx(bfull, p.tx_bytes);
+                            if (p.x3d) ptx::tma_load_3d(dst, &xmap, cx, 0, c_row, bfull);
+                            else ptx::tma_load_2d(dst, &xmap, cx, c_row, bfull);
+                        }
                         ++issued;
                         cx += p.cw;
                         if (cx == cx_end) cx = 0;
@@ -906,11 +909,14 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         }
                     }
                 }
-                drain_copies(bar_full, (uint32_t)p.stages, issued);
+                if (leader) drain_copies(bar_full, (uint32_t)p.stages, issued);
             }
+            __syncwarp();
         } else if (warp == 1) {
             // ---- MMA issuer ---------------------------------------------------------
-            if (lane == 0) {
+            // (the whole warp, one lane issues: descriptors then stay in uniform registers)
+            {
+                const bool leader = ptx::elect_one();
                 bool ok = true;
                 // descriptors: constant high word, low word = (address >> 4) | LBO field
                 const uint64_t d_cw = smem_desc(0u, cw), d_32 = smem_desc(0u, 32u);
@@ -933,15 +939,16 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     const int nks = p.ksteps_last;
                     int left = (p.n_mtiles - worker + nworkers - 1) / nworkers;
                     for (; left > 0 && ok; --left) {
-                        if (!ptx::mbar_try_wait(btfull + tempty_off, tph ^ 1u) &&
-                            !wait_bar(btfull + tempty_off, tph ^ 1u, flags)) { ok = false; break; }
-                        if (!ptx::mbar_try_wait(bfull, ph) && !wait_bar(bfull, ph, flags)) { ok = false; break; }
+                        if (!wait_bar_warp(btfull + tempty_off, tph ^ 1u, flags)) { ok = false; break; }
+                        if (!wait_bar_warp(bfull, ph, flags)) { ok = false; break; }
                         ptx::tc_fence_after_sync();
-                        ptx::mma_i8(d_tmem, d_cw | (uint64_t)a_lo, b_desc, idesc, 0u);
-                        for (int ks = 1; ks < nks; ++ks)
-                            ptx::mma_i8(d_tmem, d_cw | (uint64_t)(a_lo + 2 * ks), b_desc + 2 * ks, idesc, 1u);
-                        if (fast) ptx::mma_i8(d_tmem, ac_desc, wb_desc, idesc, 1u);
-                        ptx::mma_commit(btfull);
+                        if (leader) {
+                            ptx::mma_i8<false>(d_tmem, d_cw | (uint64_t)a_lo, b_desc, idesc);
+                            for (int ks = 1; ks < nks; ++ks)
+                                ptx::mma_i8<true>(d_tmem, d_cw | (uint64_t)(a_lo + 2 * ks), b_desc + 2 * ks, idesc);
+                            if (fast) ptx::mma_i8<true>(d_tmem, ac_desc, wb_desc, idesc);
+                            ptx::mma_commit(btfull);
+                        }
                         a_lo += a_step; bfull += 8;
                         if (bfull == bfull_end) { ph ^= 1u; a_lo = a_lo0; bfull = bar_full; }
                         d_tmem += p.nt_pad; btfull += 8;
@@ -952,23 +959,24 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 for (int mt = worker; mt < p.n_mtiles && ok; mt += nworkers) {
                     uint32_t b_lo = b_lo0, wb_lo = wb_lo0;
                     for (int ls = 0; ls < p.subs_per_cta && ok; ++ls) {
-                        if (!wait_bar(btempty, tph ^ 1u, flags)) { ok = false; break; }
+                        if (!wait_bar_warp(btempty, tph ^ 1u, flags)) { ok = false; break; }
                         ptx::tc_fence_after_sync();
                         uint32_t acc = 0;
                         for (int chunk = 0; chunk < p.kc; ++chunk) {
                             if (!p.share_x || ls == 0) {
-                                if (!wait_bar(bfull, ph, flags)) { ok = false; break; }
+                                if (!wait_bar_warp(bfull, ph, flags)) { ok = false; break; }
                                 ptx::tc_fence_after_sync();
                             }
                             const int nks = (chunk == p.kc - 1) ? p.ksteps_last : ks_full;
                             for (int ks = 0; ks < nks; ++ks) {
-                                ptx::mma_i8(d_tmem, d_cw | (uint64_t)(a_lo + 2 * ks),
-                                            d_cw | (uint64_t)(b_lo + 2 * ks), idesc, acc);
+                                if (leader)
+                                    ptx::mma_i8(d_tmem, d_cw | (uint64_t)(a_lo + 2 * ks),
+                                                d_cw | (uint64_t)(b_lo + 2 * ks), idesc, acc);
                                 acc = 1;
                             }
                             b_lo += b_step;
                             if (!p.share_x || ls == p.subs_per_cta - 1) {
-                                if (!epi_frees) ptx::mma_commit(bempty);
+                                if (!epi_frees && leader) ptx::mma_commit(bempty);
                                 ++s; a_lo += a_step; bfull += 8; bempty += 8;
                                 if (s == (uint32_t)p.stages) {
                                     s = 0; ph ^= 1u; a_lo = a_lo0; bfull = bar_full; bempty = bar_empty;
@@ -976,9 +984,9 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                             }
                         }
                         if (!ok) break;
-                        if (fast) ptx::mma_i8(d_tmem, ac_desc, d_32 | (uint64_t)wb_lo, idesc, 1u);
+                        if (fast && leader) ptx::mma_i8<true>(d_tmem, ac_desc, d_32 | (uint64_t)wb_lo, idesc);
                         wb_lo += wb_step;
-                        ptx::mma_commit(btfull);
+                        if (leader) ptx::mma_commit(btfull);
                         ++b; d_tmem += p.nt_pad; btfull += 8; btempty += 8;
                         if (b == (uint32_t)p.nbuf) {
                             b = 0; tph ^= 1u; d_tmem = tmem_base; btfull = bar_tfull; btempty = bar_tempty;
@@ -986,7 +994,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     }
                 }
                 // every MMA has finished before tensor memory is released
-                ptx::mma_commit(bar_drain);
+                if (leader) ptx::mma_commit(bar_drain);
                 const unsigned long long t0 = ptx::globaltimer();
                 while (!ptx::mbar_try_wait(bar_drain, 0) && ptx::globaltimer() - t0 < kWaitLimitNs) {}
             }
