@@ -218,7 +218,7 @@ static int round_up(int v, int a) { return (v + a - 1) / a * a; }
 // Everything of a plan that follows from (fold, nt, groups, occ); false when it does not fit.
 static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, const DeviceInfo &d,
                          int fold, int nt, int groups, int occ, int want_stages, TcPlan &pl,
-                         int cw_max = 128)
+                         int cw_max = 128, int direct = 0)
 {
     tc::Params &p = pl.p;
     memset(&p, 0, sizeof(p));
@@ -261,11 +261,14 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
     if (tmem_cols / nt_pad < 2) return false;
     const int nbuf = tmem_cols / nt_pad >= 4 ? 4 : 2;
 
+    // outputs straight from registers: rows and subtiles of whole 32-byte sectors (a partial sector costs
+    // L2 a read-modify-write); three CTAs per SM have too few registers for it
+    if (direct && (nt % 32 || nf % 32 || occ == 4)) return false;
     const int ncols = subs * nt_pad;
     const size_t stage_bytes = (size_t)128 * cw;
     const size_t w_bytes = (size_t)subs * kc * nt_pad * cw;
     const size_t wbias_bytes = (size_t)subs * nt_pad * 32;
-    const size_t out_bytes = (size_t)tc::kEpiWarps * 32 * nt;
+    const size_t out_bytes = direct ? 0 : (size_t)tc::kEpiWarps * 32 * nt;
     const size_t fixed = w_bytes + wbias_bytes + tc::kAConstBytes + round_up((int)out_bytes, 128) +
                          (size_t)ncols * 12 + 16 + 256 + tc::kLuts * 1024 + 256 + 1024 /* alignment slack */;
     const size_t budget = share == 1 ? (size_t)d.smem_optin
@@ -292,7 +295,8 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
     p.ksteps_last = (kf - (kc - 1) * cw + 31) / 32;
     p.stages = stages; p.nbuf = nbuf; p.tmem_cols = tmem_cols;
     p.share_x = share_x;
-    p.store_2d = n_sub > 1 ? 1 : 0;
+    p.direct = direct;
+    p.store_2d = n_sub > 1 && !direct ? 1 : 0;
     p.x3d = x3d; p.box_r = box_r;
     p.tx_bytes = x3d ? (uint32_t)(cw * map.wo * box_r) : (uint32_t)stage_bytes;
 
@@ -333,19 +337,29 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
     const double epi_rate = 36e3 / ctas_per_sm;              // outputs per microsecond per CTA
     // an SM takes 58 bytes per clock from L2 (the copy-rate probe): 110 KB per microsecond
     const double load_rate = 110e3 / ctas_per_sm;            // bytes per microsecond per CTA
-    // subtile widths with a straight-line epilogue (tc.cuh: epi_fast_fixed); any other width that
-    // splits a row runs the looped epilogue, measured ~1 us per layer slower at 128 columns
+    // Staged subtile widths with a straight-line epilogue (tc.cuh: epi_fast_fixed); any other width that
+    // splits a row runs the looped epilogue, measured ~1 us per layer slower at 128 columns.
     const bool straight = nt == 96 || nt == 64 || nt == 48 || nt == 32 || nt == 80;
-    const double t_epi = (double)tm * nt / epi_rate * (straight || n_sub == 1 ? 1.0 : 1.5);
+    const double epi_cost = direct || straight ? 1.0 : (n_sub > 1 ? 1.5 : (nt <= 96 ? 1.0 : 1.2));
+    const double t_epi = (double)tm * nt / epi_rate * epi_cost;
     const double t_load = (double)kc * tm * (kf < cw ? kf : cw) / load_rate;
+    // Direct outputs want whole 64-column pieces: half of the stores of a last piece of 32 are short, which
+    // shows once L2 is busy (16 -> 96 at 1.6 M rows 53.9 us against 46.3 staged, 64 -> 384 at 25088 rows 6.6
+    // against 6.1; at 1176 rows, 160 -> 960, 4.3 against 4.8).  A bulk store runs beside the next unit, a
+    // direct one does not, so several units per CTA lose a little of what one gains.
+    const bool short_piece = direct && nt % 64 && nt > 32;
+    const double unit = short_piece ? 1.15 : (direct && rounds * subs > 1 ? 0.9 : 0.8);
     // 0.8 us per unit for the hand-overs around it (barrier waits, fences, store issue): fitted to
     // plans timed inside the chained step (32 -> 192 and 64 -> 384 prefer 96-column subtiles in
     // fewer channel groups to 64-column ones)
-    const double t_first = (t_epi > t_load ? t_epi : t_load) + 0.8;
-    const double t_next = share_x ? t_epi + 0.8 : t_first;
+    const double t_first = (t_epi > t_load ? t_epi : t_load) + unit;
+    const double t_next = share_x ? t_epi + unit : t_first;
     const double startup = 1.2 + (double)p.image_bytes / 80e3 * ctas_per_sm;
     const double fill = 1.0 + 0.1 * kc;                      // first load, first MMA
-    const double last = 0.45 * ((nt + 31) / 32) + 0.8;       // draining the last accumulator, store
+    // Draining the last accumulator, store.  A direct store saves the hand-over to the bulk-copy unit: at
+    // 392 rows, 64 -> 384 takes 3.1 / 3.4 / 3.9 us with 32 / 64 / 128 columns against 3.4 / 3.6 / 4.5 staged
+    // (and 3.5 with 16), 384 -> 64 3.8 against 4.2.
+    const double last = direct && !(short_piece && m * cout > 6000000) ? 0.35 * ((nt + 31) / 32) + 0.5 : 0.45 * ((nt + 31) / 32) + 0.8;
     const double t_cta = startup + fill + rounds * (t_first + (subs - 1) * t_next) + last +
                          (occ == 1 ? 2.5 : 0.0);   // a CTA that fills its SM keeps the next kernel out
     const double t_mem = ((double)m * cin * (groups == 1 ? 1.0 : 1.0 + 0.15 * (groups - 1)) +
@@ -400,10 +414,12 @@ static bool tc_search_plan(long long m, int cin, int cout, const RowMap &map, co
                 if (tn.occ > 0 && occ != tn.occ) continue;
                 if (dyn && occ > 2) continue;
                 if (tn.occ == 0 && occ >= 3) continue;      // only on request for now
-                TcPlan pl;
-                if (!tc_fill_plan(m, cin, cout, map, d, fold, nt, groups, occ, tn.stages, pl))
-                    continue;
-                if (!found || pl.est_us < best.est_us) { best = pl; found = true; }
+                for (int direct = dyn ? 0 : 1; direct >= 0; --direct) {
+                    TcPlan pl;
+                    if (!tc_fill_plan(m, cin, cout, map, d, fold, nt, groups, occ, tn.stages, pl, 128, direct))
+                        continue;
+                    if (!found || pl.est_us < best.est_us) { best = pl; found = true; }
+                }
             }
         }
     }
@@ -506,6 +522,9 @@ static prom_status tc_set_attr(const DeviceInfo &d)
     if (e == cudaSuccess) e = raise_smem_limit(tc::tc_conv_kernel<2, 2>, d.smem_optin);
     if (e == cudaSuccess) e = raise_smem_limit(tc::tc_conv_kernel<2, 4>, d.smem_optin);
     if (e == cudaSuccess) e = raise_smem_limit(tc::tc_conv_kernel<2, 3>, d.smem_optin);
+    if (e == cudaSuccess) e = raise_smem_limit(tc::tc_conv_kernel<2, 0, true>, d.smem_optin);
+    if (e == cudaSuccess) e = raise_smem_limit(tc::tc_conv_kernel<2, 3, true>, d.smem_optin);
+    if (e == cudaSuccess) e = raise_smem_limit(tc::tc_conv_kernel<2, 4, true>, d.smem_optin);
     if (e == cudaSuccess) e = raise_smem_limit(tc::tc_prep_kernel, d.smem_optin);
     if (e != cudaSuccess) return PROM_ERR_CUDA;
     done.fetch_or(bit, std::memory_order_release);
@@ -532,11 +551,15 @@ static prom_status tc_launch_planned(const Conv &c, TcPlan &pl, int mode = 0)
     cudaError_t e;
     if (mode == 1) e = cudaLaunchKernelEx(&cfg, tc::tc_conv_kernel<2, 1>, pl.xmap, pl.ymap, pl.p);
     else if (mode == 2) e = cudaLaunchKernelEx(&cfg, tc::tc_conv_kernel<2, 2>, pl.xmap, pl.ymap, pl.p);
-    else if (c.res) e = cudaLaunchKernelEx(&cfg, tc::tc_conv_kernel<2, 3>, pl.xmap, pl.ymap, pl.p);
-    else if (pl.p.act_min == -128 && pl.p.act_max == 127)
-        e = cudaLaunchKernelEx(&cfg, tc::tc_conv_kernel<2, 4>, pl.xmap, pl.ymap, pl.p);
-    else if (pl.per_sm == 3) e = cudaLaunchKernelEx(&cfg, tc::tc_conv_kernel<3>, pl.xmap, pl.ymap, pl.p);
-    else e = cudaLaunchKernelEx(&cfg, tc::tc_conv_kernel<2>, pl.xmap, pl.ymap, pl.p);
+    else {
+        const bool full_range = pl.p.act_min == -128 && pl.p.act_max == 127;
+        auto *kernel = pl.p.direct ? (c.res ? tc::tc_conv_kernel<2, 3, true>
+                                            : (full_range ? tc::tc_conv_kernel<2, 4, true> : tc::tc_conv_kernel<2, 0, true>))
+                                   : (c.res ? tc::tc_conv_kernel<2, 3>
+                                            : (full_range ? tc::tc_conv_kernel<2, 4>
+                                               : pl.per_sm == 3 ? tc::tc_conv_kernel<3> : tc::tc_conv_kernel<2, 0>));
+        e = cudaLaunchKernelEx(&cfg, kernel, pl.xmap, pl.ymap, pl.p);
+    }
     ++g_launches;
     return cuda_status(e);
 }

@@ -277,6 +277,15 @@ __device__ __forceinline__ void tmem_ld_x32(uint32_t taddr, uint32_t (&v)[32])
         : "memory");
 }
 
+// A 16-byte load from shared memory that stays where it is written (the compiler does not keep its
+// result in registers across a second use).
+__device__ __forceinline__ int4 lds_128(uint32_t addr)
+{
+    int4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr));
+    return v;
+}
+
 // ---- integer helpers -------------------------------------------------------------
 // hi32(a*b) + c
 __device__ __forceinline__ int mad_hi(int a, int b, int c)

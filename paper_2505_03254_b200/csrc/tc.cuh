@@ -68,6 +68,7 @@ struct Params {
     int ksteps_last;    // 32-wide MMA steps in the last chunk
     int stages, nbuf, tmem_cols;
     int share_x;        // kc == 1: one activation load serves all subtiles of the tile
+    int direct;         // outputs leave straight from registers; the rows of B are permuted (channel_of)
     int store_2d;       // 0: rows of a slab are contiguous in Y (one subtile), 1: tensor-map store
     int x3d, box_r;     // 3-D activation map (strided input); rows of dim 2 per tile
     uint32_t tx_bytes;
@@ -384,6 +385,173 @@ __device__ __noinline__ void store_partial_slab(int8_t *yp, const uint8_t *slab,
     }
 }
 
+// ---- outputs straight from registers (Params::direct) -------------------------------------------
+// tmem_ld_16x32 hands a thread two rows of the accumulator and, of 32 columns, four pairs.  With the rows
+// of B permuted those pairs are neighbouring channels, 16 of them out of 64 columns (8 out of a last 32):
+// four threads cover 64 (32) bytes of a row in one store instruction, eight rows at a time, whole
+// 32-byte sectors.  Against staging a slab in shared memory for a bulk store this saves the writes and
+// reads of the slab, the proxy fence and the wait for the previous store, and a thread needs the
+// multipliers of its own channels only (6 instead of 24 16-byte loads per 32 x 96 outputs).
+// Channel (inside its subtile of nt, a multiple of 32) that accumulator column n holds.
+__device__ __forceinline__ int channel_of(int n, int nt)
+{
+    const int base = n & ~63, r = n & 63;
+    const int c = (r >> 1) & 3, je = 2 * (r >> 3) + (r & 1);
+    return base + 64 <= nt ? base + 16 * c + je : base + 8 * c + je;
+}
+
+// The rows of one warp's slab as a thread sees them: its first row (row lane / 4 of the slab) and how
+// many of the slab's 32 rows exist.
+struct DirectRows {
+    int8_t *y;              // first output byte of this thread's first row, at the subtile's first column
+    const int8_t *res;      // the same place in the residual (mode 3)
+    long long step;         // bytes to eight rows further on
+    int valid;              // rows of the slab, counted from this thread's first one
+    __device__ __forceinline__ bool has(int i) const { return 8 * i < valid; }
+};
+
+__device__ __forceinline__ uint32_t add_sat(uint32_t w, uint32_t r) { return __vaddss4(w, r); }
+
+// Eight channels of one row (u: which of the load's two rows), fast epilogue.
+template <bool SIGNED>
+__device__ __forceinline__ uint2 direct_eight(const uint32_t (&v)[16], int u, const int4 &m0, const int4 &m1,
+                                              long long r64, int shmax)
+{
+    const int mu[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+    int q[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int a = (int)v[4 * (i >> 1) + 2 * u + (i & 1)];
+        q[i] = SIGNED ? fast_signed(a, mu[i], r64, shmax) : (int)(((long long)a * mu[i] + r64) >> 32) >> shmax;
+    }
+    if (SIGNED)
+        return make_uint2(ptx::pack_sat_s8(q[1], q[0], ptx::pack_sat_s8(q[3], q[2], 0u)),
+                          ptx::pack_sat_s8(q[5], q[4], ptx::pack_sat_s8(q[7], q[6], 0u)));
+    return make_uint2((ptx::pack_sat_u8(q[1], q[0], ptx::pack_sat_u8(q[3], q[2], 0u)) >> 1) & 0x7F7F7F7Fu,
+                      (ptx::pack_sat_u8(q[5], q[4], ptx::pack_sat_u8(q[7], q[6], 0u)) >> 1) & 0x7F7F7F7Fu);
+}
+
+// The fast epilogue over one subtile of 32 rows x nt columns; taddr is the warp's lane quarter.  The loads
+// of the next 32 columns are on their way while a piece is worked on, and the accumulator is released
+// once the last are in registers.
+template <bool SIGNED, bool RES>
+__device__ __forceinline__ void epi_direct(int nt, uint32_t taddr, const int *cm, int shmax, const DirectRows &d,
+                                           uint4 (&held)[4], uint32_t bar_release)
+{
+    constexpr uint32_t kHalf = 16u << 16;          // the upper 16 lanes of the quarter
+    const long long r64 = 1ll << (32 + shmax);
+    const int c = threadIdx.x & 3;
+    uint32_t va[16], vb[16];
+    ptx::tmem_ld_16x32(taddr, va);
+    ptx::tmem_ld_16x32(nt >= 64 ? taddr + 32 : taddr + kHalf, vb);
+    int col = 0;
+    for (; col + 64 <= nt; col += 64) {
+        const uint32_t mp = ptx::smem_u32(cm + col + 16 * c);
+        int4 m0, m1, m2, m3;
+        if constexpr (!RES) { m0 = ptx::lds_128(mp); m1 = ptx::lds_128(mp + 16); m2 = ptx::lds_128(mp + 32); m3 = ptx::lds_128(mp + 48); }
+        int8_t *y = d.y + col + 16 * c;
+        if constexpr (RES) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (col && d.has(i)) held[i] = __ldcg(reinterpret_cast<const uint4 *>(d.res + col + 16 * c + i * d.step));
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            ptx::tmem_wait_ld();
+            const int next = col + 64;
+            if (h == 1 && next == nt) release_acc(bar_release);
+            // (with the residual's bytes in registers too, the multipliers are fetched again for every half)
+            if constexpr (RES) { m0 = ptx::lds_128(mp); m1 = ptx::lds_128(mp + 16); }
+            const uint2 a0 = direct_eight<SIGNED>(va, 0, m0, m1, r64, shmax), a1 = direct_eight<SIGNED>(va, 1, m0, m1, r64, shmax);
+            if (h == 0) ptx::tmem_ld_16x32(taddr + col + kHalf, va);
+            else if (next < nt) ptx::tmem_ld_16x32(taddr + next, va);
+            if constexpr (RES) { m2 = ptx::lds_128(mp + 32); m3 = ptx::lds_128(mp + 48); }
+            const uint2 b0 = direct_eight<SIGNED>(vb, 0, m2, m3, r64, shmax), b1 = direct_eight<SIGNED>(vb, 1, m2, m3, r64, shmax);
+            if (h == 0) ptx::tmem_ld_16x32(taddr + col + 32 + kHalf, vb);
+            else if (next < nt) ptx::tmem_ld_16x32(next + 64 <= nt ? taddr + next + 32 : taddr + next + kHalf, vb);
+            uint4 o0 = make_uint4(a0.x, a0.y, b0.x, b0.y), o1 = make_uint4(a1.x, a1.y, b1.x, b1.y);
+            if constexpr (RES) {
+                const uint4 r0 = held[2 * h], r1 = held[2 * h + 1];
+                o0 = make_uint4(add_sat(o0.x, r0.x), add_sat(o0.y, r0.y), add_sat(o0.z, r0.z), add_sat(o0.w, r0.w));
+                o1 = make_uint4(add_sat(o1.x, r1.x), add_sat(o1.y, r1.y), add_sat(o1.z, r1.z), add_sat(o1.w, r1.w));
+            }
+            if (d.has(2 * h)) *reinterpret_cast<uint4 *>(y + 2 * h * d.step) = o0;
+            if (d.has(2 * h + 1)) *reinterpret_cast<uint4 *>(y + (2 * h + 1) * d.step) = o1;
+        }
+    }
+    if (col < nt) {
+        const int4 *mp = reinterpret_cast<const int4 *>(cm + col + 8 * c);
+        const int4 m0 = mp[0], m1 = mp[1];
+        int8_t *y = d.y + col + 8 * c;
+        if constexpr (RES) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (col && d.has(i)) {
+                    const uint2 r = __ldcg(reinterpret_cast<const uint2 *>(d.res + col + 8 * c + i * d.step));
+                    held[i].x = r.x; held[i].y = r.y;
+                }
+        }
+        ptx::tmem_wait_ld();
+        release_acc(bar_release);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            uint2 o = i < 2 ? direct_eight<SIGNED>(va, i & 1, m0, m1, r64, shmax) : direct_eight<SIGNED>(vb, i & 1, m0, m1, r64, shmax);
+            if constexpr (RES) o = make_uint2(add_sat(o.x, held[i].x), add_sat(o.y, held[i].y));
+            if (d.has(i)) *reinterpret_cast<uint2 *>(y + i * d.step) = o;
+        }
+    }
+}
+
+// The residual bytes of a subtile's first piece, asked for before the wait for its accumulator.
+__device__ __forceinline__ void direct_residual(int nt, const DirectRows &d, uint4 (&held)[4])
+{
+    const int c = threadIdx.x & 3;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        held[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (d.has(i)) {
+            if (nt >= 64) held[i] = __ldcg(reinterpret_cast<const uint4 *>(d.res + 16 * c + i * d.step));
+            else {
+                const uint2 r = __ldcg(reinterpret_cast<const uint2 *>(d.res + 8 * c + i * d.step));
+                held[i] = make_uint4(r.x, r.y, 0u, 0u);
+            }
+        }
+    }
+}
+
+// The 64-bit definition for the same layout (any clamp, any shifts), eight channels of a row at a time.
+__device__ __noinline__ void epi_exact_direct(int nt, int act_min, int act_max, uint32_t taddr, const int *cm,
+                                              const int2 *cbs, DirectRows d, uint32_t bar_release)
+{
+    const int c = threadIdx.x & 3;
+    for (int g = 0; g < nt; g += 32) {
+        const int ch = (g & ~63) + 64 <= nt ? (g & ~63) + 16 * c + ((g & 32) >> 2) : g + 8 * c;    // this thread's first channel
+        for (int h = 0; h < 2; ++h) {
+            uint32_t v[16];
+            ptx::tmem_ld_16x32(taddr + g + ((uint32_t)h << 20), v);
+            ptx::tmem_wait_ld();
+            if (g + 32 == nt && h == 1) release_acc(bar_release);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                uint32_t o[2] = {0u, 0u};
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int2 bs = cbs[ch + i];
+                    const int q = requant_exact((int)v[4 * (i >> 1) + 2 * u + (i & 1)] + bs.x, cm[ch + i], bs.y, act_min, act_max);
+                    o[i >> 2] |= ((uint32_t)q & 0xFFu) << (8 * (i & 3));
+                }
+                if (d.has(2 * h + u)) {
+                    if (d.res) {
+                        const uint2 r = __ldcg(reinterpret_cast<const uint2 *>(d.res + ch + (2 * h + u) * d.step));
+                        o[0] = add_sat(o[0], r.x); o[1] = add_sat(o[1], r.y);
+                    }
+                    *reinterpret_cast<uint2 *>(d.y + ch + (2 * h + u) * d.step) = make_uint2(o[0], o[1]);
+                }
+            }
+        }
+    }
+}
+
 // ---- the dynamic layer's epilogues ---------------------------------------------------------
 // y = acc * alpha[column] * dq[sample]: the int32 accumulator becomes a float exactly (the
 // magic-number form holds below 2^22; |acc| <= 4096 * 127), then two correctly rounded products
@@ -649,7 +817,7 @@ __device__ __forceinline__ void build_image(const Params &p, const int g, const 
     if (fast)
         for (int i = threadIdx.x; i < ncols_res; i += kThreads) {
             const int ls = i / p.nt_pad, c = i - ls * p.nt_pad;
-            const int2 bs = cbs[i];
+            const int2 bs = cbs[p.direct ? ls * p.nt_pad + channel_of(c, p.nt) : i];
             const int v = bs.x << (2 + shmax - bs.y);
             int h = (v >= 0 ? v + 63 : v - 63) / 127;        // nearest multiple of 127
             const int lo = v - 127 * h;                       // within [-63, 63]
@@ -690,8 +858,9 @@ __device__ __forceinline__ void build_image(const Params &p, const int g, const 
             uint8_t *dst_blk = w_smem + (size_t)blk * p.nt_pad * cw;
             const int jmax = (chunk == p.kc - 1) ? p.ksteps_last * 2 : cpr;   // pieces ever read
             for (int idx = threadIdx.x; idx < per_blk; idx += kThreads) {
-                const int n = idx >> cpr_log2, j = idx & (cpr - 1);
+                const int row_b = idx >> cpr_log2, j = idx & (cpr - 1);
                 if (j >= jmax) continue;
+                const int n = p.direct ? channel_of(row_b, p.nt) : row_b;     // the channel this row of B holds
                 const int nfold = sub * p.nt + n, kbase = chunk * p.cw + j * 16;
                 uint4 val = make_uint4(0, 0, 0, 0);
                 if (n < p.nt && nfold < p.nf && kbase < p.kf) {
@@ -730,7 +899,7 @@ __device__ __forceinline__ void build_image(const Params &p, const int g, const 
                         val = make_uint4(wd[0], wd[1], wd[2], wd[3]);
                     }
                 }
-                *reinterpret_cast<uint4 *>(dst_blk + swz_offset((uint32_t)n, (uint32_t)j, cw)) = val;
+                *reinterpret_cast<uint4 *>(dst_blk + swz_offset((uint32_t)row_b, (uint32_t)j, cw)) = val;
             }
         }
         if (invalid) raise_status(PROM_ERR_BAD_WEIGHT);
@@ -748,7 +917,9 @@ __device__ __forceinline__ void build_image(const Params &p, const int g, const 
 // MODE 3: mode 0 plus a residual tensor added to the output with int8 saturation.
 // MODE 4: mode 0 for the clamp [-128, 127] (the host launches it for exactly that clamp; the
 // kernel the benchmark step runs stays free of the second fast epilogue).
-template <int MINB, int MODE = 0>
+// DIRECT: Params::direct (a kernel of its own: the second epilogue's code and registers in the staged
+// kernel cost its loops 5 %).
+template <int MINB, int MODE = 0, bool DIRECT = false>
 __global__ void __launch_bounds__(kThreads, MINB)
 tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap ymap,
                const Params p)
@@ -1035,38 +1206,48 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
             int col = (g + ls * p.groups) * p.nt;       // first column of the subtile
             const int dcol = dls * p.groups * p.nt;
             const bool store_2d = p.store_2d != 0;
+            const uint32_t res_inv = MODE == 3 ? (65536u + (uint32_t)(p.nt >> 3) - 1u) / (uint32_t)(p.nt >> 3) : 0u;
             // accumulators of this group: grp alone (two in the ring) or grp and grp + 2 (four)
             const uint32_t btoggle = p.nbuf == 4 ? 2u : 0u;
             uint32_t b = (uint32_t)grp, tph = 0;
             uint32_t st = (uint32_t)grp % (uint32_t)p.stages;    // stage of this group's unit (epi_frees)
             while ((unsigned)(row0 - q * 32) < row_span && ok) {
-                // The residual (mode 3): the bytes that sit where this slab goes in Y, in 8-byte
-                // granules across the warp.  The first kResHeld granules of a lane are requested
+                DirectRows dr;
+                uint4 held[4];
+                if constexpr (DIRECT) {
+                    int rows_valid = p.tm - q * 32;
+                    if (m_rows - row0 < rows_valid) rows_valid = m_rows - row0;
+                    const long long at = (long long)(row0 + (lane >> 2)) * p.nf + col;
+                    dr.y = p.y + at;
+                    dr.res = MODE == 3 ? p.res + at : nullptr;
+                    dr.step = 8ll * p.nf;
+                    dr.valid = (rows_valid > 32 ? 32 : rows_valid) - (lane >> 2);
+                    if constexpr (MODE == 3) direct_residual(p.nt, dr, held);
+                }
+                // The residual of a staged slab (mode 3): the bytes that sit where the slab goes in Y, in
+                // 8-byte granules across the warp.  The first kResHeld granules of a lane are requested
                 // before the wait for the accumulator, so that their latency hides behind it.
                 constexpr int kResHeld = 6;
                 uint2 res_held[kResHeld];
-                int res_total = 0, res_g8 = 1;
+                int res_total = 0;
                 const int8_t *res_p = nullptr;
-                if constexpr (MODE == 3) {
+                // row and first byte of granule i (a row has nt / 8; the reciprocal is exact for i < 1024)
+                auto granule = [&](int i, int &r, int &c) { r = (int)((uint32_t)i * res_inv >> 16); c = 8 * (i - r * (p.nt >> 3)); };
+                if constexpr (MODE == 3 && !DIRECT) {
                     int rows_valid = p.tm - q * 32;
                     if (m_rows - row0 < rows_valid) rows_valid = m_rows - row0;
                     if (rows_valid > 32) rows_valid = 32;
-                    res_g8 = p.nt >> 3;
-                    res_total = rows_valid * res_g8;
+                    res_total = rows_valid * (p.nt >> 3);
                     res_p = p.res + (long long)row0 * p.nf + col;
 #pragma unroll
                     for (int j = 0; j < kResHeld; ++j) {
                         const int i = lane + 32 * j;
                         res_held[j] = make_uint2(0u, 0u);
                         if (i < res_total) {
-                            const int r = i / res_g8, c = (i - r * res_g8) * 8;
+                            int r, c;
+                            granule(i, r, c);
                             res_held[j] = __ldcg(reinterpret_cast<const uint2 *>(res_p + (long long)r * p.nf + c));
                         }
-                    }
-                    // the rest is asked into L2
-                    for (int i = lane + 32 * kResHeld; i < res_total; i += 32) {
-                        const int r = i / res_g8, c = (i - r * res_g8) * 8;
-                        asm volatile("prefetch.global.L2 [%0];" ::"l"(res_p + (long long)r * p.nf + c));
                     }
                 }
                 if (!wait_bar<true>(bar_tfull + 8 * b, tph, flags)) { ok = false; break; }
@@ -1076,12 +1257,24 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     if (st >= (uint32_t)p.stages) st -= p.stages;
                 }
                 ptx::tc_fence_after_sync();
-                // the previous bulk store must have read the slab before it is rewritten
-                ptx::bulk_wait_read0();
-                __syncwarp();
                 const uint32_t taddr = t_lane + b * p.nt_pad;
                 const int *cms = cmult + ls * p.nt_pad;
                 const uint32_t bar_rel = bar_tempty + 8 * b;
+                if constexpr (DIRECT) {
+                    // the fast epilogue's clamp: [0, 127] in mode 0, [-128, 127] in mode 4, either in mode 3
+                    if (!fast) epi_exact_direct(p.nt, p.act_min, p.act_max, taddr, cms, cbs + ls * p.nt_pad, dr, bar_rel);
+                    else if (MODE == 4 || (MODE == 3 && p.act_min < 0))
+                        epi_direct<true, MODE == 3>(p.nt, taddr, cms, shmax, dr, held, bar_rel);
+                    else epi_direct<false, MODE == 3>(p.nt, taddr, cms, shmax, dr, held, bar_rel);
+                    ls += dls; row0 += drow; col += dcol;
+                    if (ls >= subs) { ls -= subs; row0 += drow_wrap; col -= p.nf; }
+                    b ^= btoggle;
+                    if (b < (uint32_t)kEpiGroups) tph ^= 1u;
+                    continue;
+                }
+                // the previous bulk store must have read the slab before it is rewritten
+                ptx::bulk_wait_read0();
+                __syncwarp();
                 if constexpr (MODE == 0 || MODE == 3 || MODE == 4) {
                     // the fast epilogue's clamp: [0, 127] in mode 0, [-128, 127] in mode 4, either in mode 3
                     const bool full_range = MODE == 4 || (MODE == 3 && p.act_min < 0);
@@ -1098,21 +1291,18 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     else epi_exact_subtile<CH>(p.nt, p.act_min, p.act_max, taddr, cms, cbs + ls * p.nt_pad, my_row, bar_rel);
                     if constexpr (MODE == 3) {
                         __syncwarp();
-                        auto add_to_slab = [&](int i, uint2 rv) {
-                            const int r = i / res_g8, c = (i - r * res_g8) * 8;
+                        auto add_to_slab = [&](int i, bool have, uint2 rv) {
+                            int r, c;
+                            granule(i, r, c);
+                            if (!have) rv = __ldcg(reinterpret_cast<const uint2 *>(res_p + (long long)r * p.nf + c));
                             uint2 *sp = reinterpret_cast<uint2 *>(slab + r * p.nt + c);
-                            uint2 sv = *sp;
-                            sv.x = __vaddss4(sv.x, rv.x);
-                            sv.y = __vaddss4(sv.y, rv.y);
-                            *sp = sv;
+                            const uint2 sv = *sp;
+                            *sp = make_uint2(add_sat(sv.x, rv.x), add_sat(sv.y, rv.y));
                         };
 #pragma unroll
                         for (int j = 0; j < kResHeld; ++j)
-                            if (lane + 32 * j < res_total) add_to_slab(lane + 32 * j, res_held[j]);
-                        for (int i = lane + 32 * kResHeld; i < res_total; i += 32) {
-                            const int r = i / res_g8, c = (i - r * res_g8) * 8;
-                            add_to_slab(i, __ldcg(reinterpret_cast<const uint2 *>(res_p + (long long)r * p.nf + c)));
-                        }
+                            if (lane + 32 * j < res_total) add_to_slab(lane + 32 * j, true, res_held[j]);
+                        for (int i = lane + 32 * kResHeld; i < res_total; i += 32) add_to_slab(i, false, make_uint2(0u, 0u));
                     }
                 } else {
                     // this thread's row and its sample (rows past the end borrow the last sample's
