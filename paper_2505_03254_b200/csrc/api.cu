@@ -179,7 +179,7 @@ static EncodeTiledFn encode_tiled_fn()
 
 struct TcPlan {
     tc::Params p;
-    CUtensorMap xmap, ymap;
+    CUtensorMap xmap, ymap, tmap;
     int grid = 0;
     int per_sm = 2;        // CTAs of the launch that share an SM (picks the kernel build)
     size_t smem = 0;
@@ -218,7 +218,7 @@ static int round_up(int v, int a) { return (v + a - 1) / a * a; }
 // Everything of a plan that follows from (fold, nt, groups, occ); false when it does not fit.
 static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, const DeviceInfo &d,
                          int fold, int nt, int groups, int occ, int want_stages, TcPlan &pl,
-                         int cw_max = 128, int direct = 0)
+                         int cw_max = 128, int direct = 0, bool tail = false)
 {
     tc::Params &p = pl.p;
     memset(&p, 0, sizeof(p));
@@ -247,7 +247,7 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
     }
     const long long rows = m / fold;
     if ((nf & 15) && (tm & 1)) return false;     // slabs of the 1-D store start on 16-byte granules
-    const long long n_mtiles = (rows + tm - 1) / tm;
+    const long long n_mtiles = (rows + tm - 1) / tm + (tail ? 1 : 0);
     if (rows + 256 >= (1ll << 31)) return false;   // row coordinates are 32-bit in the kernel
 
     // tensor memory: the CTAs of an SM share its 512 columns
@@ -263,7 +263,7 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
 
     // outputs straight from registers: rows and subtiles of whole 32-byte sectors (a partial sector costs
     // L2 a read-modify-write); three CTAs per SM have too few registers for it
-    if (direct && (nt % 32 || nf % 32 || occ == 4)) return false;
+    if (direct && (nt % 32 || nf % 32 || occ == 4 || tail)) return false;
     const int ncols = subs * nt_pad;
     const size_t stage_bytes = (size_t)128 * cw;
     const size_t w_bytes = (size_t)subs * kc * nt_pad * cw;
@@ -288,7 +288,7 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
         if (packed > (size_t)stages * stage_bytes) return false;
     }
 
-    p.m_rows = rows; p.k0 = cin; p.n0 = cout; p.fold = fold; p.kf = kf; p.nf = nf;
+    p.m_rows = rows; p.tail = tail ? 1 : 0; p.k0 = cin; p.n0 = cout; p.fold = fold; p.kf = kf; p.nf = nf;
     p.tm = tm; p.n_mtiles = (int)n_mtiles; p.nt = nt; p.nt_pad = nt_pad;
     p.n_sub = n_sub; p.groups = groups; p.subs_per_cta = subs;
     p.cw = cw; p.kc = kc;
@@ -373,11 +373,15 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
 // use: kPlanSingle (one call: the kernel builds its operands itself), kPlanDynamic (the dynamic
 // layer: no row folding, a folded row could straddle two samples) or
 // kPlanPrepared (a layer of a sequence, whose operands tc_prep_kernel builds once)
-enum { kPlanSingle = 0, kPlanDynamic = 1, kPlanPrepared = 2 };
+// kPlanOdd, added to kPlanSingle or kPlanPrepared: an odd number of rows that have to be folded in pairs is
+// taken too, the last row as a tile of its own (the automatic choice; PROM_VARIANT_TC refuses such a shape)
+enum { kPlanSingle = 0, kPlanDynamic = 1, kPlanPrepared = 2, kPlanOdd = 4 };
 static bool tc_search_plan(long long m, int cin, int cout, const RowMap &map, const DeviceInfo &d,
                            int use, TcPlan &best)
 {
-    const bool dyn = use == kPlanDynamic;
+    const bool dyn = use == kPlanDynamic, odd_ok = (use & kPlanOdd) != 0;
+    use &= ~kPlanOdd;
+    bool tail = false;
     if (m <= 0 || (cin & 7) || (cout & 7)) return false;
     const TcTune tn = tune_for(m, cin, cout, map.stride);
     int fold = 1;
@@ -385,22 +389,25 @@ static bool tc_search_plan(long long m, int cin, int cout, const RowMap &map, co
         // Rows that are not 16-byte multiples cannot be described to TMA: two rows are folded into
         // one.  On the output side that is only needed when the row does not fit one subtile
         // (a slab of 32 whole rows is then one contiguous, 16-byte aligned range of Y anyway).
-        if ((cin & 15) || ((cout & 15) && cout > 256 && m % 2 == 0)) fold = 2;
-        if (m % fold) return false;
-        while (fold * 2 <= 8 && fold * 2 * cin <= 128 && fold * 2 * cout <= 128 &&
+        if ((cin & 15) || ((cout & 15) && cout > 256 && (m % 2 == 0 || odd_ok))) fold = 2;
+        tail = m % fold != 0;
+        if (tail && !odd_ok) return false;
+        while (!tail && fold * 2 <= 8 && fold * 2 * cin <= 128 && fold * 2 * cout <= 128 &&
                m % (fold * 2) == 0)
             fold *= 2;
         // rows of fewer than 32 bytes make poor TMA boxes (measured on the 16 -> 96 layer: 3 us
         // of 58): fold once more whatever the width, where the larger block-diagonal weights
         // are expanded once per sequence and not by every CTA
-        if (use == kPlanPrepared && cin * fold < 32 && fold * 2 <= 8 && m % (fold * 2) == 0) fold *= 2;
+        if (!tail && use == kPlanPrepared && cin * fold < 32 && fold * 2 <= 8 && m % (fold * 2) == 0) fold *= 2;
     }
     if (dyn) {
         if ((cin & 15) || ((cout & 15) && cout > 256)) return false;
         fold = 1;
     }
     if (tn.fold > 0) fold = tn.fold;
-    if (fold < 1 || fold > 8 || m % fold) return false;
+    if (fold < 1 || fold > 8) return false;
+    if (m % fold && !(tail && fold == 2)) return false;
+    if (fold == 1) tail = false;
     const int nf = cout * fold;
     bool found = false;
     for (int nt = 8; nt <= 256 && nt <= nf; nt += 8) {
@@ -416,7 +423,7 @@ static bool tc_search_plan(long long m, int cin, int cout, const RowMap &map, co
                 if (tn.occ == 0 && occ >= 3) continue;      // only on request for now
                 for (int direct = dyn ? 0 : 1; direct >= 0; --direct) {
                     TcPlan pl;
-                    if (!tc_fill_plan(m, cin, cout, map, d, fold, nt, groups, occ, tn.stages, pl, 128, direct))
+                    if (!tc_fill_plan(m, cin, cout, map, d, fold, nt, groups, occ, tn.stages, pl, 128, direct, tail))
                         continue;
                     if (!found || pl.est_us < best.est_us) { best = pl; found = true; }
                 }
@@ -459,7 +466,7 @@ static bool tc_shape_plan(long long m, int cin, int cout, const RowMap &map, con
     const PlanKey key = {m, cin, cout, map.stride, map.ho, map.wo, map.hin, map.win,
                          tn.fold, tn.nt, tn.groups, tn.occ, tn.stages, d.dev, use + 1};
     const unsigned long long h = ((unsigned long long)m * 0x9E3779B1u + (unsigned)cin * 0x85EBCA6Bu +
-                                  (unsigned)cout * 0xC2B2AE35u + (unsigned)(map.stride * 8 + use) * 0x27D4EB2Fu);
+                                  (unsigned)cout * 0xC2B2AE35u + (unsigned)(map.stride * 16 + use) * 0x27D4EB2Fu);
     PlanEntry &e = recent[(h ^ (h >> 17)) & (kRecent - 1)];
     if (e.key != key) tc_find_plan(m, cin, cout, map, d, use, key, e);
     if (e.ok) best = e.pl;
@@ -475,7 +482,7 @@ static bool tc_make_maps(const Conv &c, TcPlan &pl)
                                   : (p.cw == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B);
     CUresult r;
     if (!p.x3d) {
-        cuuint64_t dims[2] = {(cuuint64_t)p.kf, (cuuint64_t)p.m_rows};
+        cuuint64_t dims[2] = {(cuuint64_t)p.kf, (cuuint64_t)(p.m_rows > 0 ? p.m_rows : 1)};
         cuuint64_t strides[1] = {(cuuint64_t)p.kf};
         cuuint32_t box[2] = {(cuuint32_t)p.cw, 128};
         cuuint32_t es[2] = {1, 1};
@@ -496,7 +503,7 @@ static bool tc_make_maps(const Conv &c, TcPlan &pl)
     }
     if (r != CUDA_SUCCESS) return false;
     if (p.store_2d) {
-        cuuint64_t dims[2] = {(cuuint64_t)p.nf, (cuuint64_t)p.m_rows};
+        cuuint64_t dims[2] = {(cuuint64_t)p.nf, (cuuint64_t)(p.m_rows > 0 ? p.m_rows : 1)};
         cuuint64_t strides[1] = {(cuuint64_t)p.nf};
         cuuint32_t box[2] = {(cuuint32_t)p.nt, 32};
         cuuint32_t es[2] = {1, 1};
@@ -506,6 +513,18 @@ static bool tc_make_maps(const Conv &c, TcPlan &pl)
         if (r != CUDA_SUCCESS) return false;
     } else {
         pl.ymap = pl.xmap;      // unused by the kernel
+    }
+    pl.tmap = pl.xmap;          // unused by the kernel without a tail
+    if (p.tail) {
+        // the last row alone: columns past cin and the box's other rows arrive as zeros
+        cuuint64_t dims[2] = {(cuuint64_t)p.k0, 1};
+        cuuint64_t strides[1] = {(cuuint64_t)p.kf};
+        cuuint32_t box[2] = {(cuuint32_t)p.cw, 128};
+        cuuint32_t es[2] = {1, 1};
+        r = enc(&pl.tmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<int8_t *>(c.x) + p.m_rows * p.kf, dims, strides,
+                box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        if (r != CUDA_SUCCESS) return false;
     }
     return true;
 }
@@ -549,8 +568,8 @@ static prom_status tc_launch_planned(const Conv &c, TcPlan &pl, int mode = 0)
     cudaLaunchAttribute attr[1];
     fill_launch_cfg(cfg, attr, pl.grid, tc::kThreads, pl.smem, c.st, c.pdl != 0);
     cudaError_t e;
-    if (mode == 1) e = cudaLaunchKernelEx(&cfg, tc::tc_conv_kernel<2, 1>, pl.xmap, pl.ymap, pl.p);
-    else if (mode == 2) e = cudaLaunchKernelEx(&cfg, tc::tc_conv_kernel<2, 2>, pl.xmap, pl.ymap, pl.p);
+    if (mode == 1) e = cudaLaunchKernelEx(&cfg, tc::tc_conv_kernel<2, 1>, pl.xmap, pl.ymap, pl.tmap, pl.p);
+    else if (mode == 2) e = cudaLaunchKernelEx(&cfg, tc::tc_conv_kernel<2, 2>, pl.xmap, pl.ymap, pl.tmap, pl.p);
     else {
         const bool full_range = pl.p.act_min == -128 && pl.p.act_max == 127;
         auto *kernel = pl.p.direct ? (c.res ? tc::tc_conv_kernel<2, 3, true>
@@ -558,7 +577,7 @@ static prom_status tc_launch_planned(const Conv &c, TcPlan &pl, int mode = 0)
                                    : (c.res ? tc::tc_conv_kernel<2, 3>
                                             : (full_range ? tc::tc_conv_kernel<2, 4>
                                                : pl.per_sm == 3 ? tc::tc_conv_kernel<3> : tc::tc_conv_kernel<2, 0>));
-        e = cudaLaunchKernelEx(&cfg, kernel, pl.xmap, pl.ymap, pl.p);
+        e = cudaLaunchKernelEx(&cfg, kernel, pl.xmap, pl.ymap, pl.tmap, pl.p);
     }
     ++g_launches;
     return cuda_status(e);
@@ -730,7 +749,7 @@ static prom_status launch_wide(const Conv &c, const DeviceInfo &d, WidePlan &pl)
     return cuda_status(cudaGetLastError());
 }
 
-static prom_status launch_tc(const Conv &c)
+static prom_status launch_tc(const Conv &c, int use = kPlanSingle)
 {
     DeviceInfo d = device_info();
     if (!d.ok) return PROM_ERR_CUDA;
@@ -746,7 +765,7 @@ static prom_status launch_tc(const Conv &c)
         }
     }
     TcPlan pl;
-    if (!tc_shape_plan(c.m, c.cin, c.cout, c.map, d, pl)) return PROM_ERR_UNSUPPORTED;
+    if (!tc_shape_plan(c.m, c.cin, c.cout, c.map, d, pl, use)) return PROM_ERR_UNSUPPORTED;
     if (tc_set_attr(d) != PROM_OK) return PROM_ERR_CUDA;
     tc_bind(c, pl, nullptr);
     return tc_launch_planned(c, pl);
@@ -766,7 +785,7 @@ static prom_status run_conv(const Conv &c, prom_variant v)
     case PROM_VARIANT_ADDSUB: return addsub::launch(c.x, c.m, c.cin, c.map, c.w, c.cout, c.rq, c.y,
                                                     c.st, g_launches);
     case PROM_VARIANT_AUTO: {
-        const prom_status e = launch_tc(c);
+        const prom_status e = launch_tc(c, kPlanOdd);
         if (e != PROM_ERR_UNSUPPORTED) return e;
         if (!c.res && smallk::supported(c.cin, c.cout))
             return smallk::launch(c.x, c.m, c.cin, c.map, c.w, c.cout, c.rq, c.y, c.st, g_launches);
@@ -1115,7 +1134,7 @@ static void seq_layout(const prom_layer *layers, int n, const SeqShape &s, const
             continue;
         }
         TcPlan pl;
-        if (tc_shape_plan(s.m[i], layers[i].cin, layers[i].cout, s.map[i], d, pl, kPlanPrepared)) {
+        if (tc_shape_plan(s.m[i], layers[i].cin, layers[i].cout, s.map[i], d, pl, kPlanPrepared | kPlanOdd)) {
             L.img_off[i] = L.img_total;
             L.img_total += round256((size_t)pl.p.groups * pl.p.image_stride);
         }
@@ -1426,7 +1445,8 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
         if (layers[i].add_block_input) c.res = i == 1 ? x0 : conv[i - 2].y;
         if (chained) {
             chain_img[i] = chain_base + lay.cimg_off[i];
-        } else if (want_tc && c.m > 0 && tc_shape_plan(c.m, c.cin, c.cout, c.map, d, plan[i], kPlanPrepared)) {
+        } else if (want_tc && c.m > 0 && tc_shape_plan(c.m, c.cin, c.cout, c.map, d, plan[i],
+                                                               variant == PROM_VARIANT_AUTO ? kPlanPrepared | kPlanOdd : kPlanPrepared)) {
             is_tc[i] = 1;
             tc_bind(c, plan[i], img_base && lay.img_off[i] != (size_t)-1 ? img_base + lay.img_off[i] : nullptr);
         } else if (variant == PROM_VARIANT_TC && c.m > 0) {

@@ -56,6 +56,7 @@ constexpr int kPdlChain = 1, kPdlWait = 2;
 
 struct Params {
     long long m_rows;   // rows of the folded problem
+    int tail;           // one more row that fills half of a folded one (fold 2, odd row count): the last tile
     int k0, n0;         // layer cin, cout
     int fold;
     int kf, nf;         // folded cin, cout
@@ -382,6 +383,20 @@ __device__ __noinline__ void store_partial_slab(int8_t *yp, const uint8_t *slab,
         // the slab leaves row by row
         ptx::bulk_store(yp + (long long)lane * nf + col, slab_addr + (uint32_t)(lane * nt), (uint32_t)nt);
         ptx::bulk_commit();
+    }
+}
+
+// Stores the odd last row (Params::tail) of a folded matrix: `bytes` channels from the slab's first row,
+// with the residual if there is one.
+__device__ __noinline__ void store_tail_row(int8_t *y, const int8_t *res, const uint8_t *slab, int bytes, int lane)
+{
+    for (int i = 8 * lane; i < bytes; i += 8 * 32) {
+        uint2 v = *reinterpret_cast<const uint2 *>(slab + i);
+        if (res) {
+            const uint2 r = __ldcg(reinterpret_cast<const uint2 *>(res + i));
+            v = make_uint2(__vaddss4(v.x, r.x), __vaddss4(v.y, r.y));
+        }
+        *reinterpret_cast<uint2 *>(y + i) = v;
     }
 }
 
@@ -922,7 +937,7 @@ __device__ __forceinline__ void build_image(const Params &p, const int g, const 
 template <int MINB, int MODE = 0, bool DIRECT = false>
 __global__ void __launch_bounds__(kThreads, MINB)
 tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap ymap,
-               const Params p)
+               const __grid_constant__ CUtensorMap tmap, const Params p)
 {
     extern __shared__ uint8_t smem_raw[];
     // 1024-byte aligned base, by pointer arithmetic (a cast through an integer would make every
@@ -1062,14 +1077,16 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 if (p.pdl == kPdlChain) ptx::grid_dep_wait();
                 for (int mt = worker; mt < p.n_mtiles && ok; mt += nworkers) {
                     const int mtx = p.reverse ? p.n_mtiles - 1 - mt : mt;
-                    const int c_row = p.x3d ? mtx * p.box_r : mtx * p.tm;
+                    int c_row = p.x3d ? mtx * p.box_r : mtx * p.tm;
+                    const CUtensorMap *map = &xmap;
+                    if (p.tail && mtx == p.n_mtiles - 1) { map = &tmap; c_row = 0; }
                     int cx = 0;
                     for (int l = 0; l < loads_per_tile; ++l) {
                         if (!wait_bar_warp(bempty, ph ^ 1u, flags)) { ok = false; break; }
                         if (leader) {
                             ptx::mbar_expect_tx(bfull, p.tx_bytes);
                             if (p.x3d) ptx::tma_load_3d(dst, &xmap, cx, 0, c_row, bfull);
-                            else ptx::tma_load_2d(dst, &xmap, cx, c_row, bfull);
+                            else ptx::tma_load_2d(dst, map, cx, c_row, bfull);
                         }
                         ++issued;
                         cx += p.cw;
@@ -1201,6 +1218,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
             const int drow = subs == 1 ? dir * kEpiGroups * nworkers * p.tm : 0, drow_wrap = dir * nworkers * p.tm;
             const bool whole_tile = p.tm - q * 32 >= 32;     // a tile gives this warp 32 rows
             int row0 = (p.reverse ? p.n_mtiles - 1 - mt0 : mt0) * p.tm + q * 32;   // first row of this warp's slab
+            // (with an odd last row the tile behind the matrix is its tile)
             const unsigned row_span = (unsigned)(p.n_mtiles * p.tm);
             const uint32_t slab_bytes = 32u * (uint32_t)p.nf;
             int col = (g + ls * p.groups) * p.nt;       // first column of the subtile
@@ -1343,6 +1361,14 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         if (store_2d) ptx::tma_store_2d(&ymap, col, row0, slab_addr);
                         else ptx::bulk_store(p.y + (long long)row0 * p.nf, slab_addr, slab_bytes);
                         ptx::bulk_commit();
+                    }
+                } else if (p.tail && row0 - q * 32 >= m_rows) {
+                    // the tile of the odd last row
+                    // (the folded row holds n0 channels of a row that exists)
+                    if (q == 0) {
+                        const long long at = p.m_rows * p.nf + col;
+                        const int left = p.n0 - col;
+                        store_tail_row(p.y + at, MODE == 3 ? p.res + at : nullptr, slab, left < p.nt ? left : p.nt, lane);
                     }
                 } else {
                     // a short tile or the end of the matrix
