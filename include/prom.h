@@ -195,7 +195,7 @@ prom_status prom_dw_conv3x3_i8(const int8_t *x_dev, int batch, int h, int w, int
  *   q_dev        [batch * rows_per_sample][cout] int8, device, 16-byte aligned, not x_dev
  *   gamma_y_dev, scale_y_dev  [batch] float32 outputs
  * Tensor-core variant only: cin a multiple of 16, cout a multiple of 8 (of 16 above 256), else
- * PROM_ERR_UNSUPPORTED.  Asynchronous on the stream (one memset, three launches).  Other errors
+ * PROM_ERR_UNSUPPORTED.  Asynchronous on the stream (three launches).  Other errors
  * as for prom_pw_conv_i8; weights outside {-1,0,+1} surface as PROM_ERR_BAD_WEIGHT in
  * prom_last_device_status. */
 prom_status prom_pw_conv_i8_dyn(const int8_t *x_dev, int batch, int64_t rows_per_sample, int cin,

@@ -1586,15 +1586,14 @@ static uint8_t *static_scratch_address()
     return static_cast<uint8_t *>(p);
 }
 
-// scale_y[b] = 127 / max(gamma_y[b], eps): between the two passes of the dynamic layer
-__global__ void dyn_scale_kernel(const float *__restrict__ gamma_y, int batch, float eps,
-                                        float *__restrict__ scale_y)
+// Clears the maxima of the dynamic layer (a kernel and not a memset, which would keep the passes behind it
+// from being launched early).
+__global__ void dyn_clear_kernel(float *__restrict__ gamma_y, int batch)
 {
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < batch) {
-        const float g = gamma_y[b];
-        scale_y[b] = __fdiv_rn(127.0f, g < eps ? eps : g);
-    }
+    if (b < batch) gamma_y[b] = 0.0f;
 }
 
 }  // namespace prom
@@ -1720,6 +1719,10 @@ prom_status prom_pw_conv_i8_dyn(const int8_t *x_dev, int batch, int64_t rows_per
     Conv c;
     c.x = x_dev; c.m = m; c.cin = cin; c.cout = cout; c.map = plain; c.in_rows = m;
     c.w = w_packed_dev; c.y = q_dev; c.st = st;
+    // Links of a chain whose first kernel waits before it releases the passes: input, weights and factors
+    // are complete when a pass starts, only the maxima are not, so operands are built and the first tiles
+    // loaded and multiplied beside the kernel in front.
+    c.pdl = tc::kPdlChain;
     c.rq.bias = nullptr; c.rq.shift = nullptr;
     c.rq.mult = reinterpret_cast<const int32_t *>(alpha_dev);     // bit patterns of alpha
     c.rq.act_min = -128; c.rq.act_max = 127;                      // keeps the weights at +-1
@@ -1730,13 +1733,14 @@ prom_status prom_pw_conv_i8_dyn(const int8_t *x_dev, int batch, int64_t rows_per
     pl.p.gamma_x = gamma_x_dev;
     pl.p.gamma_y = gamma_y_dev;
     pl.p.scale_y = scale_y_dev;
-    if (cudaMemsetAsync(gamma_y_dev, 0, sizeof(float) * (size_t)batch, st) != cudaSuccess)
-        return PROM_ERR_CUDA;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    fill_launch_cfg(cfg, attr, (batch + 127) / 128, 128, 0, st, true);
+    const cudaError_t ce = cudaLaunchKernelEx(&cfg, dyn_clear_kernel, gamma_y_dev, batch);
+    ++g_launches;
+    if (ce != cudaSuccess) return PROM_ERR_CUDA;
     prom_status e = tc_launch_planned(c, pl, 1);
     if (e != PROM_OK) return e;
-    dyn_scale_kernel<<<(batch + 127) / 128, 128, 0, st>>>(gamma_y_dev, batch, 1e-5f, scale_y_dev);
-    ++g_launches;
-    if (cudaGetLastError() != cudaSuccess) return PROM_ERR_CUDA;
     return tc_launch_planned(c, pl, 2);
 }
 

@@ -286,6 +286,26 @@ __device__ __forceinline__ int4 lds_128(uint32_t addr)
     return v;
 }
 
+// ---- two floats per instruction (each lane rounded like the scalar operation) -------------------
+__device__ __forceinline__ unsigned long long pack_2(uint32_t lo, uint32_t hi)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(lo), "r"(hi));
+    return r;
+}
+__device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long mul_f32x2(unsigned long long a, unsigned long long b)
+{
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
 // ---- integer helpers -------------------------------------------------------------
 // hi32(a*b) + c
 __device__ __forceinline__ int mad_hi(int a, int b, int c)

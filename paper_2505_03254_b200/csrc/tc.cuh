@@ -96,7 +96,7 @@ struct Params {
     int batch;
     const float *gamma_x;       // [batch] per-sample maximum behind the int8 input
     float *gamma_y;             // [batch] mode 1: maxima of the dequantised output (as bit patterns)
-    const float *scale_y;       // [batch] mode 2: 127 / max(gamma_y, eps)
+    float *scale_y;             // [batch] mode 2: 127 / max(gamma_y, eps), written for the caller
     // Kernel mode 3: an int8 tensor of Y's shape added to the requantised output with
     // saturation.  It may be Y itself: a warp reads the bytes of a slab before it stores there.
     const int8_t *res;
@@ -578,7 +578,7 @@ __device__ __forceinline__ float dyn_value(uint32_t acc, int alpha_bits, float d
 }
 
 // NC accumulator columns of this thread's row, already in registers.
-// Mode 1: the largest |y| among them joins m.
+// Mode 1, rows of several samples in a slab: the largest |y| among them joins m.
 template <int NC>
 __device__ __forceinline__ float dyn_piece_max(const uint32_t (&v)[NC], const int *__restrict__ cm, float dq,
                                                float m)
@@ -594,30 +594,60 @@ __device__ __forceinline__ float dyn_piece_max(const uint32_t (&v)[NC], const in
     return m;
 }
 
-// Mode 2: y quantised with the sample's scale (ties to even through the magic-number add,
-// saturating packs clip to [-128, 127]) and staged like the static epilogue's bytes.
+// Mode 1, all 32 rows of the warp's slab in one sample.  Rounded products are monotone, so the largest |y| is
+// fl(fl(max |acc| * |alpha|) * dq): the maximum over a channel's rows is taken on the integers, and the
+// factors are applied once per channel (alpha) and once per slab (dq).  With the 16x256b read-out a thread
+// has four rows of a channel.  Returns the warp's largest fl(|acc| * alpha).
+__device__ __forceinline__ float dyn_slab_max(int nt, uint32_t taddr, const int *cm, uint32_t bar_release)
+{
+    const int c = threadIdx.x & 3;
+    float m = 0.0f;
+    for (int col = 0; col < nt; col += 32) {
+        uint32_t va[16], vb[16];
+        ptx::tmem_ld_16x32(taddr + col, va);
+        ptx::tmem_ld_16x32(taddr + col + (16u << 16), vb);     // (columns past nt are read and not used)
+        ptx::tmem_wait_ld();
+        if (col + 32 >= nt) release_acc(bar_release);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (col + 8 * j >= nt) break;
+            const int2 al = *reinterpret_cast<const int2 *>(cm + col + 8 * j + 2 * c);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int r0 = (int)va[4 * j + e], r1 = (int)va[4 * j + 2 + e], r2 = (int)vb[4 * j + e], r3 = (int)vb[4 * j + 2 + e];
+                const int hi = max(max(max(r0, r1), r2), r3), lo = min(min(min(r0, r1), r2), r3);
+                const float f = __fadd_rn(__int_as_float(max(hi, -lo) + 0x4B400000), -12582912.0f);
+                m = fmaxf(m, __fmul_rn(f, fabsf(__int_as_float(e ? al.y : al.x))));
+            }
+        }
+    }
+    // non-negative floats are ordered like their bit patterns
+    return __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(m)));
+}
+
+// Mode 2: y quantised with the sample's scale (ties to even through the magic-number add) and staged like
+// the static epilogue's bytes, two outputs per instruction.  |y| <= gamma, so |y * scale| <= 127 up to two
+// roundings and the rounded value is within [-127, 127]: the clip of the definition never acts, and the code
+// is the low byte of the sum's bit pattern.
 template <int NC>
-__device__ __forceinline__ void dyn_piece_quant(const uint32_t (&v)[NC], const int *__restrict__ cm, float dq,
-                                                float sc, uint8_t *dst, bool wide)
+__device__ __forceinline__ void dyn_piece_quant(const uint32_t (&v)[NC], const int *__restrict__ cm, unsigned long long dq2,
+                                                unsigned long long sc2, uint8_t *dst, bool wide)
 {
     uint32_t out[NC / 4];
 #pragma unroll
     for (int e = 0; e < NC; e += 4) {
         const int4 mu = *reinterpret_cast<const int4 *>(cm + e);
-        const int a4[4] = {mu.x, mu.y, mu.z, mu.w};
-        int r[4];
+        uint32_t r[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float y = dyn_value(v[e + j], a4[j], dq);
-            r[j] = __float_as_int(__fadd_rn(__fmul_rn(y, sc), 12582912.0f)) - 0x4B400000;
+        for (int h = 0; h < 2; ++h) {
+            unsigned long long t = ptx::pack_2(v[e + 2 * h] + 0x4B400000u, v[e + 2 * h + 1] + 0x4B400000u);
+            t = ptx::add_f32x2(t, ptx::pack_2(0xCB400000u, 0xCB400000u));            // the accumulators as floats
+            t = ptx::mul_f32x2(t, ptx::pack_2((uint32_t)(h ? mu.z : mu.x), (uint32_t)(h ? mu.w : mu.y)));
+            t = ptx::mul_f32x2(ptx::mul_f32x2(t, dq2), sc2);
+            t = ptx::add_f32x2(t, ptx::pack_2(0x4B400000u, 0x4B400000u));
+            r[2 * h] = (uint32_t)t; r[2 * h + 1] = (uint32_t)(t >> 32);
         }
-        uint32_t w;
-        asm("{\n\t.reg .b32 t;\n\t"
-            "cvt.pack.sat.s8.s32.b32 t, %4, %3, 0;\n\t"
-            "cvt.pack.sat.s8.s32.b32 %0, %2, %1, t;\n\t}"
-            : "=r"(w)
-            : "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]));
-        out[e / 4] = w;
+        out[e / 4] = __byte_perm(__byte_perm(r[0], r[1], 0x0040), __byte_perm(r[2], r[3], 0x0040), 0x5410);
     }
     put_row<NC>(dst, out, wide);
 }
@@ -630,6 +660,8 @@ __device__ __forceinline__ float epi_dyn_subtile(const Params &p, uint32_t taddr
 {
     const bool wide = (p.nt & 15) == 0;
     const int tail = p.nt & (CH - 1);
+    const unsigned long long dq2 = ptx::pack_2(__float_as_uint(dq), __float_as_uint(dq)),
+                             sc2 = ptx::pack_2(__float_as_uint(sc), __float_as_uint(sc));
     float m = 0.0f;
     int c = 0;
     for (; c + CH <= p.nt; c += CH) {
@@ -637,7 +669,7 @@ __device__ __forceinline__ float epi_dyn_subtile(const Params &p, uint32_t taddr
         tmem_ld<CH>(taddr + c, v);
         ptx::tmem_wait_ld();
         if (tail == 0 && c + CH == p.nt) release_acc(bar_release);
-        if constexpr (QUANT) dyn_piece_quant<CH>(v, cm + c, dq, sc, dst_row + c, wide);
+        if constexpr (QUANT) dyn_piece_quant<CH>(v, cm + c, dq2, sc2, dst_row + c, wide);
         else m = dyn_piece_max<CH>(v, cm + c, dq, m);
     }
     if (CH > 16 && c + 16 <= p.nt) {
@@ -645,7 +677,7 @@ __device__ __forceinline__ float epi_dyn_subtile(const Params &p, uint32_t taddr
         ptx::tmem_ld_x16(taddr + c, v);
         ptx::tmem_wait_ld();
         if (c + 16 == p.nt) release_acc(bar_release);
-        if constexpr (QUANT) dyn_piece_quant<16>(v, cm + c, dq, sc, dst_row + c, wide);
+        if constexpr (QUANT) dyn_piece_quant<16>(v, cm + c, dq2, sc2, dst_row + c, wide);
         else m = dyn_piece_max<16>(v, cm + c, dq, m);
         c += 16;
     }
@@ -654,11 +686,41 @@ __device__ __forceinline__ float epi_dyn_subtile(const Params &p, uint32_t taddr
         ptx::tmem_ld_x8(taddr + c, v);
         ptx::tmem_wait_ld();
         release_acc(bar_release);
-        if constexpr (QUANT) dyn_piece_quant<8>(v, cm + c, dq, sc, dst_row + c, wide);
+        if constexpr (QUANT) dyn_piece_quant<8>(v, cm + c, dq2, sc2, dst_row + c, wide);
         else m = dyn_piece_max<8>(v, cm + c, dq, m);
     }
     return m;
 }
+
+// Mode 2 over a subtile of a width known at compile time (a multiple of 16): straight-line code.
+template <int NT>
+__device__ __forceinline__ void epi_dyn_fixed(uint32_t taddr, const int *cm, float dq, float sc, uint8_t *dst_row,
+                                              uint32_t bar_release)
+{
+    const unsigned long long dq2 = ptx::pack_2(__float_as_uint(dq), __float_as_uint(dq)),
+                             sc2 = ptx::pack_2(__float_as_uint(sc), __float_as_uint(sc));
+    constexpr int full = NT & ~31;
+#pragma unroll
+    for (int c = 0; c < full; c += 32) {
+        uint32_t v[32];
+        ptx::tmem_ld_x32(taddr + c, v);
+        ptx::tmem_wait_ld();
+        if (c + 32 == NT) release_acc(bar_release);
+        dyn_piece_quant<32>(v, cm + c, dq2, sc2, dst_row + c, true);
+    }
+    if constexpr ((NT & 16) != 0) {
+        uint32_t v[16];
+        ptx::tmem_ld_x16(taddr + full, v);
+        ptx::tmem_wait_ld();
+        release_acc(bar_release);
+        dyn_piece_quant<16>(v, cm + full, dq2, sc2, dst_row + full, true);
+    }
+}
+
+// The factor between a sample's accumulators and its dequantised outputs (besides alpha), and the scale of
+// its codes; both guarded like the figure's clamp.
+__device__ __forceinline__ float dyn_dequant(float gamma_x) { return __fdiv_rn(gamma_x < 1e-5f ? 1e-5f : gamma_x, 127.0f); }
+__device__ __forceinline__ float dyn_scale(float gamma_y) { return __fdiv_rn(127.0f, gamma_y < 1e-5f ? 1e-5f : gamma_y); }
 
 // Where the parts of a CTA's shared memory are.
 struct View {
@@ -1074,7 +1136,8 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 bool ok = true;
                 // Only this thread reads what the previous kernel wrote; everything else in the
                 // CTA follows from its loads, so it alone waits for that kernel to finish.
-                if (p.pdl == kPdlChain) ptx::grid_dep_wait();
+                // (The dynamic layer's passes share their input, which the kernel in front has not written.)
+                if (MODE != 1 && MODE != 2 && p.pdl == kPdlChain) ptx::grid_dep_wait();
                 for (int mt = worker; mt < p.n_mtiles && ok; mt += nworkers) {
                     const int mtx = p.reverse ? p.n_mtiles - 1 - mt : mt;
                     int c_row = p.x3d ? mtx * p.box_r : mtx * p.tm;
@@ -1196,6 +1259,14 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 // the residual was written two kernels back: complete once the previous one is
                 if (p.pdl == kPdlChain) ptx::grid_dep_wait();
             }
+            if constexpr (MODE == 1 || MODE == 2) {
+                // the maxima: cleared by the kernel in front of the first pass, complete behind that pass
+                if (p.pdl == kPdlChain) ptx::grid_dep_wait();
+            }
+            if constexpr (MODE == 2) {
+                for (int i = blockIdx.x * (kThreads - 64) + (int)threadIdx.x - 64; i < p.batch; i += gridDim.x * (kThreads - 64))
+                    p.scale_y[i] = dyn_scale(__ldcg(p.gamma_y + i));
+            }
             // Unit u goes to group u % 2 and accumulator u % nbuf; nbuf is even, so a group meets
             // each of its accumulators in cyclic order and never waits on a barrier that is more
             // than one phase away.
@@ -1268,6 +1339,19 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         }
                     }
                 }
+                // Modes 1 and 2: this thread's row and its sample, and the samples of the slab's first and last
+                // row (rows past the end borrow the last sample's factors; they are neither counted nor
+                // stored); what the sample's factors come from is asked for before the wait.
+                int smp = 0, smp_a = 0, smp_b = 0;
+                float gx = 0.0f, gy = 0.0f;
+                if constexpr (MODE == 1 || MODE == 2) {
+                    smp_a = min(row0 / p.rows_per_sample, p.batch - 1);
+                    smp_b = row0 + 31 < (smp_a + 1) * (long long)p.rows_per_sample ? smp_a
+                                                                                   : min((row0 + 31) / p.rows_per_sample, p.batch - 1);
+                    smp = smp_a == smp_b ? smp_a : min((row0 + lane) / p.rows_per_sample, p.batch - 1);
+                    gx = __ldg(p.gamma_x + smp);
+                    if constexpr (MODE == 2) gy = __ldcg(p.gamma_y + smp);
+                }
                 if (!wait_bar<true>(bar_tfull + 8 * b, tph, flags)) { ok = false; break; }
                 if (epi_frees) {
                     if (q == 0 && lane == 0) ptx::mbar_arrive(bar_empty + 8 * st);
@@ -1323,25 +1407,16 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         for (int i = lane + 32 * kResHeld; i < res_total; i += 32) add_to_slab(i, false, make_uint2(0u, 0u));
                     }
                 } else {
-                    // this thread's row and its sample (rows past the end borrow the last sample's
-                    // factors; they are neither counted nor stored)
-                    const int row = row0 + lane;
-                    int smp = row / p.rows_per_sample;
-                    smp = smp < p.batch ? smp : p.batch - 1;
-                    const float gx = __ldg(p.gamma_x + smp);
-                    const float dq = __fdiv_rn(gx < 1e-5f ? 1e-5f : gx, 127.0f);
                     if constexpr (MODE == 1) {
-                        float mx = epi_dyn_subtile<CH, false>(p, taddr, cms, dq, 0.0f, nullptr, bar_rel);
-                        if (row >= m_rows || p.tm - q * 32 <= lane) mx = 0.0f;
-                        // one atomic per warp when its 32 rows share a sample, else one per row
-                        const int smp0 = __shfl_sync(0xFFFFFFFFu, smp, 0);
-                        if (__all_sync(0xFFFFFFFFu, smp == smp0)) {
-#pragma unroll
-                            for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xFFFFFFFFu, mx, d));
+                        if (smp_a == smp_b) {
+                            // (rows past the end are zeros)
+                            const float mx = __fmul_rn(dyn_slab_max(p.nt, taddr, cms, bar_rel), dyn_dequant(gx));
                             if (lane == 0 && mx > 0.0f)
-                                atomicMax(reinterpret_cast<unsigned int *>(p.gamma_y + smp0), __float_as_uint(mx));
-                        } else if (mx > 0.0f) {
-                            atomicMax(reinterpret_cast<unsigned int *>(p.gamma_y + smp), __float_as_uint(mx));
+                                atomicMax(reinterpret_cast<unsigned int *>(p.gamma_y + smp_a), __float_as_uint(mx));
+                        } else {
+                            const float mx = epi_dyn_subtile<CH, false>(p, taddr, cms, dyn_dequant(gx), 0.0f, nullptr, bar_rel);
+                            if (mx > 0.0f && row0 + lane < m_rows)
+                                atomicMax(reinterpret_cast<unsigned int *>(p.gamma_y + smp), __float_as_uint(mx));
                         }
                         // nothing is stored in this pass
                         ls += dls; row0 += drow; col += dcol;
@@ -1350,7 +1425,13 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         if (b < (uint32_t)kEpiGroups) tph ^= 1u;
                         continue;
                     } else {
-                        epi_dyn_subtile<CH, true>(p, taddr, cms, dq, __ldg(p.scale_y + smp), my_row, bar_rel);
+                        const float dq = dyn_dequant(gx), sc = dyn_scale(gy);
+                        if (p.nt == 96) epi_dyn_fixed<96>(taddr, cms, dq, sc, my_row, bar_rel);
+                        else if (p.nt == 64) epi_dyn_fixed<64>(taddr, cms, dq, sc, my_row, bar_rel);
+                        else if (p.nt == 48) epi_dyn_fixed<48>(taddr, cms, dq, sc, my_row, bar_rel);
+                        else if (p.nt == 32) epi_dyn_fixed<32>(taddr, cms, dq, sc, my_row, bar_rel);
+                        else if (p.nt == 80) epi_dyn_fixed<80>(taddr, cms, dq, sc, my_row, bar_rel);
+                        else epi_dyn_subtile<CH, true>(p, taddr, cms, dq, sc, my_row, bar_rel);
                     }
                 }
                 ptx::fence_proxy_async_smem();
