@@ -340,7 +340,11 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
     // Staged subtile widths with a straight-line epilogue (tc.cuh: epi_fast_fixed); any other width that
     // splits a row runs the looped epilogue, measured ~1 us per layer slower at 128 columns.
     const bool straight = nt == 96 || nt == 64 || nt == 48 || nt == 32 || nt == 80;
-    const double epi_cost = direct || straight ? 1.0 : (n_sub > 1 ? 1.5 : (nt <= 96 ? 1.0 : 1.2));
+    // Subtiles that split 32-byte sectors: another CTA writes the rest of the sector, and once the output is
+    // larger than L2 that comes too late (802816 rows, 16 -> 1280: 848 us with 80 columns, 334 with 64;
+    // 921600 rows, 16 -> 320: 151 and 106; 64 MB outputs show no difference).
+    const bool torn = n_sub > 1 && nt % 32 && (double)m * cout > 1e8;
+    const double epi_cost = (direct || straight ? 1.0 : (n_sub > 1 ? 1.5 : (nt <= 96 ? 1.0 : 1.2))) * (torn ? 2.5 : 1.0);
     const double t_epi = (double)tm * nt / epi_rate * epi_cost;
     const double t_load = (double)kc * tm * (kf < cw ? kf : cw) / load_rate;
     // Direct outputs want whole 64-column pieces: half of the stores of a last piece of 32 are short, which
@@ -398,7 +402,9 @@ static bool tc_search_plan(long long m, int cin, int cout, const RowMap &map, co
         // rows of fewer than 32 bytes make poor TMA boxes (measured on the 16 -> 96 layer: 3 us
         // of 58): fold once more whatever the width, where the larger block-diagonal weights
         // are expanded once per sequence and not by every CTA
-        if (!tail && use == kPlanPrepared && cin * fold < 32 && fold * 2 <= 8 && m % (fold * 2) == 0) fold *= 2;
+        // (a single call expands them in every CTA, which pays when the CTA then has many tiles)
+        const bool many = m >= 128ll * 16 * 2 * d.sms;
+        if (!tail && (use == kPlanPrepared || many) && cin * fold < 32 && fold * 2 <= 8 && m % (fold * 2) == 0) fold *= 2;
     }
     if (dyn) {
         if ((cin & 15) || ((cout & 15) && cout > 256)) return false;

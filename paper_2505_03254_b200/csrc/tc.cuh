@@ -596,16 +596,57 @@ __device__ __forceinline__ float dyn_piece_max(const uint32_t (&v)[NC], const in
 
 // Mode 1, all 32 rows of the warp's slab in one sample.  Rounded products are monotone, so the largest |y| is
 // fl(fl(max |acc| * |alpha|) * dq): the maximum over a channel's rows is taken on the integers, and the
-// factors are applied once per channel (alpha) and once per slab (dq).  With the 16x256b read-out a thread
-// has four rows of a channel.  Returns the warp's largest fl(|acc| * alpha).
-__device__ __forceinline__ float dyn_slab_max(int nt, uint32_t taddr, const int *cm, uint32_t bar_release)
+// factors are applied once per channel (alpha) and once per sample (dq).  With the 16x256b read-out a thread
+// has four rows of a channel.
+__device__ __forceinline__ int abs_max(int m, int r0, int r1, int r2, int r3)
+{
+    const int hi = __vimax3_s32(__vimax3_s32(r0, r1, r2), r3, m), lo = min(__vimin3_s32(r0, r1, r2), r3);
+    return max(hi, -lo);
+}
+__device__ __forceinline__ float dyn_channel(float m, int acc, int alpha_bits)
+{
+    const float f = __fadd_rn(__int_as_float(acc + 0x4B400000), -12582912.0f);
+    return fmaxf(m, __fmul_rn(f, fabsf(__int_as_float(alpha_bits))));
+}
+// Subtiles of up to kDynHeld columns, one per CTA: the channels' maxima stay in registers from tile to tile
+// (nt / 4 of them per thread) until the sample ends.
+constexpr int kDynHeld = 96;
+__device__ __forceinline__ void dyn_hold_max(int nt, uint32_t taddr, int (&held)[kDynHeld / 4], uint32_t bar_release)
+{
+#pragma unroll
+    for (int p = 0; p < kDynHeld / 32; ++p) {
+        if (32 * p >= nt) break;
+        uint32_t va[16], vb[16];
+        ptx::tmem_ld_16x32(taddr + 32 * p, va);
+        ptx::tmem_ld_16x32(taddr + 32 * p + (16u << 16), vb);     // (columns past nt are read and not used)
+        ptx::tmem_wait_ld();
+        if (32 * p + 32 >= nt) release_acc(bar_release);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int j = 4 * (i >> 1) + (i & 1);
+            held[8 * p + i] = abs_max(held[8 * p + i], (int)va[j], (int)va[j + 2], (int)vb[j], (int)vb[j + 2]);
+        }
+    }
+}
+__device__ __forceinline__ float dyn_held_value(int nt, const int *cm, int (&held)[kDynHeld / 4])
+{
+    float m = 0.0f;
+#pragma unroll
+    for (int i = 0; i < kDynHeld / 4; ++i) {
+        const int col = 8 * (i >> 1) + 2 * (threadIdx.x & 3) + (i & 1);
+        if (8 * (i >> 1) < nt) m = dyn_channel(m, held[i], cm[col]);
+        held[i] = 0;
+    }
+    return m;
+}
+// Any subtile: the factors per tile; returns this thread's largest fl(|acc| * alpha) so far.
+__device__ __forceinline__ float dyn_slab_max(int nt, uint32_t taddr, const int *cm, float m, uint32_t bar_release)
 {
     const int c = threadIdx.x & 3;
-    float m = 0.0f;
     for (int col = 0; col < nt; col += 32) {
         uint32_t va[16], vb[16];
         ptx::tmem_ld_16x32(taddr + col, va);
-        ptx::tmem_ld_16x32(taddr + col + (16u << 16), vb);     // (columns past nt are read and not used)
+        ptx::tmem_ld_16x32(taddr + col + (16u << 16), vb);
         ptx::tmem_wait_ld();
         if (col + 32 >= nt) release_acc(bar_release);
 #pragma unroll
@@ -613,16 +654,12 @@ __device__ __forceinline__ float dyn_slab_max(int nt, uint32_t taddr, const int 
             if (col + 8 * j >= nt) break;
             const int2 al = *reinterpret_cast<const int2 *>(cm + col + 8 * j + 2 * c);
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int r0 = (int)va[4 * j + e], r1 = (int)va[4 * j + 2 + e], r2 = (int)vb[4 * j + e], r3 = (int)vb[4 * j + 2 + e];
-                const int hi = max(max(max(r0, r1), r2), r3), lo = min(min(min(r0, r1), r2), r3);
-                const float f = __fadd_rn(__int_as_float(max(hi, -lo) + 0x4B400000), -12582912.0f);
-                m = fmaxf(m, __fmul_rn(f, fabsf(__int_as_float(e ? al.y : al.x))));
-            }
+            for (int e = 0; e < 2; ++e)
+                m = dyn_channel(m, abs_max(0, (int)va[4 * j + e], (int)va[4 * j + 2 + e], (int)vb[4 * j + e], (int)vb[4 * j + 2 + e]),
+                                e ? al.y : al.x);
         }
     }
-    // non-negative floats are ordered like their bit patterns
-    return __uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(m)));
+    return m;
 }
 
 // Mode 2: y quantised with the sample's scale (ties to even through the magic-number add) and staged like
@@ -1032,6 +1069,12 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     const int nworkers = gridDim.x / p.groups;
     const uint32_t cw = (uint32_t)p.cw;
     const uint32_t stage_bytes = 128u * cw;
+    // Row tiles mt_first, + mt_step, ... below mt_end.  The passes of the dynamic layer take a contiguous
+    // range each, so that a CTA stays within a sample for many tiles.
+    constexpr bool kDyn = MODE == 1 || MODE == 2;
+    const int share = kDyn ? (p.n_mtiles + nworkers - 1) / nworkers : 1;
+    const int mt_first = worker * share, mt_step = kDyn ? 1 : nworkers;
+    const int mt_end = kDyn ? min(mt_first + share, p.n_mtiles) : p.n_mtiles;
 
     // Let the next kernel of the stream start its own prologue as soon as there is room for
     // it; it waits for this grid to finish before it touches activations.
@@ -1138,7 +1181,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 // CTA follows from its loads, so it alone waits for that kernel to finish.
                 // (The dynamic layer's passes share their input, which the kernel in front has not written.)
                 if (MODE != 1 && MODE != 2 && p.pdl == kPdlChain) ptx::grid_dep_wait();
-                for (int mt = worker; mt < p.n_mtiles && ok; mt += nworkers) {
+                for (int mt = mt_first; mt < mt_end && ok; mt += mt_step) {
                     const int mtx = p.reverse ? p.n_mtiles - 1 - mt : mt;
                     int c_row = p.x3d ? mtx * p.box_r : mtx * p.tm;
                     const CUtensorMap *map = &xmap;
@@ -1188,7 +1231,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     const uint32_t btfull_end = bar_tfull + 8u * (uint32_t)p.nbuf;
                     const uint32_t tempty_off = bar_tempty - bar_tfull;
                     const int nks = p.ksteps_last;
-                    int left = (p.n_mtiles - worker + nworkers - 1) / nworkers;
+                    int left = (mt_end - mt_first + mt_step - 1) / mt_step;
                     for (; left > 0 && ok; --left) {
                         if (!wait_bar_warp(btfull + tempty_off, tph ^ 1u, flags)) { ok = false; break; }
                         if (!wait_bar_warp(bfull, ph, flags)) { ok = false; break; }
@@ -1207,7 +1250,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     }
                     (void)a_end;
                 } else
-                for (int mt = worker; mt < p.n_mtiles && ok; mt += nworkers) {
+                for (int mt = mt_first; mt < mt_end && ok; mt += mt_step) {
                     uint32_t b_lo = b_lo0, wb_lo = wb_lo0;
                     for (int ls = 0; ls < p.subs_per_cta && ok; ++ls) {
                         if (!wait_bar_warp(btempty, tph ^ 1u, flags)) { ok = false; break; }
@@ -1259,14 +1302,6 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 // the residual was written two kernels back: complete once the previous one is
                 if (p.pdl == kPdlChain) ptx::grid_dep_wait();
             }
-            if constexpr (MODE == 1 || MODE == 2) {
-                // the maxima: cleared by the kernel in front of the first pass, complete behind that pass
-                if (p.pdl == kPdlChain) ptx::grid_dep_wait();
-            }
-            if constexpr (MODE == 2) {
-                for (int i = blockIdx.x * (kThreads - 64) + (int)threadIdx.x - 64; i < p.batch; i += gridDim.x * (kThreads - 64))
-                    p.scale_y[i] = dyn_scale(__ldcg(p.gamma_y + i));
-            }
             // Unit u goes to group u % 2 and accumulator u % nbuf; nbuf is even, so a group meets
             // each of its accumulators in cyclic order and never waits on a barrier that is more
             // than one phase away.
@@ -1278,19 +1313,19 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
             const int subs = p.subs_per_cta;
             const int m_rows = (int)p.m_rows;           // the planner keeps rows below 2^31
             bool ok = true;
-            int mt0 = worker, ls = grp;                 // this group's first unit
-            while (ls >= subs) { ls -= subs; mt0 += nworkers; }
+            int mt0 = mt_first, ls = grp;               // this group's first unit
+            while (ls >= subs) { ls -= subs; mt0 += mt_step; }
             // the next unit of the group is two further on: with one subtile per CTA that is two
             // tiles on, otherwise two subtiles on and at most one step to the next tile
             const int dls = subs == 1 ? 0 : kEpiGroups;
             // (in a sequence every second layer walks its tiles backwards: what the layer before
             // wrote last, and is still in L2, is read first)
             const int dir = p.reverse ? -1 : 1;
-            const int drow = subs == 1 ? dir * kEpiGroups * nworkers * p.tm : 0, drow_wrap = dir * nworkers * p.tm;
+            const int drow = subs == 1 ? dir * kEpiGroups * mt_step * p.tm : 0, drow_wrap = dir * mt_step * p.tm;
             const bool whole_tile = p.tm - q * 32 >= 32;     // a tile gives this warp 32 rows
             int row0 = (p.reverse ? p.n_mtiles - 1 - mt0 : mt0) * p.tm + q * 32;   // first row of this warp's slab
             // (with an odd last row the tile behind the matrix is its tile)
-            const unsigned row_span = (unsigned)(p.n_mtiles * p.tm);
+            const unsigned row_span = (unsigned)((kDyn ? mt_end : p.n_mtiles) * p.tm);
             const uint32_t slab_bytes = 32u * (uint32_t)p.nf;
             int col = (g + ls * p.groups) * p.nt;       // first column of the subtile
             const int dcol = dls * p.groups * p.nt;
@@ -1300,6 +1335,38 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
             const uint32_t btoggle = p.nbuf == 4 ? 2u : 0u;
             uint32_t b = (uint32_t)grp, tph = 0;
             uint32_t st = (uint32_t)grp % (uint32_t)p.stages;    // stage of this group's unit (epi_frees)
+            // Modes 1 and 2: the sample of the rows at hand, up to row smp_end; its factors; its maxima so far
+            int smp = 0, smp_end = 0;
+            float gx = 0.0f, dq = 0.0f, sc = 0.0f, lane_max = 0.0f;
+            auto look_up = [&] {
+                smp = min(row0 / p.rows_per_sample, p.batch - 1);
+                smp_end = smp + 1 == p.batch ? 0x7FFFFFFF : (smp + 1) * p.rows_per_sample;
+                gx = __ldg(p.gamma_x + smp);
+                if constexpr (MODE == 2) dq = dyn_dequant(gx);
+            };
+            if constexpr (kDyn) {
+                look_up();
+                // the maxima: cleared by the kernel in front of the first pass, complete behind that pass
+                if (p.pdl == kPdlChain) ptx::grid_dep_wait();
+            }
+            if constexpr (MODE == 2) {
+                sc = dyn_scale(__ldcg(p.gamma_y + smp));
+                for (int i = blockIdx.x * (kThreads - 64) + (int)threadIdx.x - 64; i < p.batch; i += gridDim.x * (kThreads - 64))
+                    p.scale_y[i] = dyn_scale(__ldcg(p.gamma_y + i));
+            }
+            int held_max[kDynHeld / 4];
+            const bool hold = MODE == 1 && subs == 1 && p.nt <= kDynHeld;
+            if constexpr (MODE == 1) {
+#pragma unroll
+                for (int i = 0; i < kDynHeld / 4; ++i) held_max[i] = 0;
+            }
+            auto flush_max = [&] {
+                if (hold) lane_max = dyn_held_value(p.nt, cmult, held_max);
+                // non-negative floats are ordered like their bit patterns
+                const float mx = __fmul_rn(__uint_as_float(__reduce_max_sync(0xFFFFFFFFu, __float_as_uint(lane_max))), dyn_dequant(gx));
+                if (lane == 0 && mx > 0.0f) atomicMax(reinterpret_cast<unsigned int *>(p.gamma_y + smp), __float_as_uint(mx));
+                lane_max = 0.0f;
+            };
             while ((unsigned)(row0 - q * 32) < row_span && ok) {
                 DirectRows dr;
                 uint4 held[4];
@@ -1339,18 +1406,26 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         }
                     }
                 }
-                // Modes 1 and 2: this thread's row and its sample, and the samples of the slab's first and last
-                // row (rows past the end borrow the last sample's factors; they are neither counted nor
-                // stored); what the sample's factors come from is asked for before the wait.
-                int smp = 0, smp_a = 0, smp_b = 0;
-                float gx = 0.0f, gy = 0.0f;
-                if constexpr (MODE == 1 || MODE == 2) {
-                    smp_a = min(row0 / p.rows_per_sample, p.batch - 1);
-                    smp_b = row0 + 31 < (smp_a + 1) * (long long)p.rows_per_sample ? smp_a
-                                                                                   : min((row0 + 31) / p.rows_per_sample, p.batch - 1);
-                    smp = smp_a == smp_b ? smp_a : min((row0 + lane) / p.rows_per_sample, p.batch - 1);
-                    gx = __ldg(p.gamma_x + smp);
-                    if constexpr (MODE == 2) gy = __ldcg(p.gamma_y + smp);
+                // Modes 1 and 2: the sample of the slab's first row, and whether the slab ends in another one (then
+                // every thread looks up its own row's; rows past the end borrow the last sample's factors,
+                // they are neither counted nor stored).
+                bool split_slab = false;
+                float dq_row = 0.0f, sc_row = 0.0f;
+                int smp_row = 0;
+                if constexpr (kDyn) {
+                    if (row0 >= smp_end) {
+                        if constexpr (MODE == 1) flush_max();
+                        look_up();
+                        if constexpr (MODE == 2) sc = dyn_scale(__ldcg(p.gamma_y + smp));
+                    }
+                    dq_row = dq;
+                    sc_row = sc;
+                    split_slab = row0 + 31 >= smp_end;
+                    if (split_slab) {
+                        smp_row = min((row0 + lane) / p.rows_per_sample, p.batch - 1);
+                        dq_row = dyn_dequant(__ldg(p.gamma_x + smp_row));
+                        if constexpr (MODE == 2) sc_row = dyn_scale(__ldcg(p.gamma_y + smp_row));
+                    }
                 }
                 if (!wait_bar<true>(bar_tfull + 8 * b, tph, flags)) { ok = false; break; }
                 if (epi_frees) {
@@ -1408,15 +1483,14 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     }
                 } else {
                     if constexpr (MODE == 1) {
-                        if (smp_a == smp_b) {
+                        if (!split_slab) {
                             // (rows past the end are zeros)
-                            const float mx = __fmul_rn(dyn_slab_max(p.nt, taddr, cms, bar_rel), dyn_dequant(gx));
-                            if (lane == 0 && mx > 0.0f)
-                                atomicMax(reinterpret_cast<unsigned int *>(p.gamma_y + smp_a), __float_as_uint(mx));
+                            if (hold) dyn_hold_max(p.nt, taddr, held_max, bar_rel);
+                            else lane_max = dyn_slab_max(p.nt, taddr, cms, lane_max, bar_rel);
                         } else {
-                            const float mx = epi_dyn_subtile<CH, false>(p, taddr, cms, dyn_dequant(gx), 0.0f, nullptr, bar_rel);
+                            const float mx = epi_dyn_subtile<CH, false>(p, taddr, cms, dq_row, 0.0f, nullptr, bar_rel);
                             if (mx > 0.0f && row0 + lane < m_rows)
-                                atomicMax(reinterpret_cast<unsigned int *>(p.gamma_y + smp), __float_as_uint(mx));
+                                atomicMax(reinterpret_cast<unsigned int *>(p.gamma_y + smp_row), __float_as_uint(mx));
                         }
                         // nothing is stored in this pass
                         ls += dls; row0 += drow; col += dcol;
@@ -1425,13 +1499,12 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         if (b < (uint32_t)kEpiGroups) tph ^= 1u;
                         continue;
                     } else {
-                        const float dq = dyn_dequant(gx), sc = dyn_scale(gy);
-                        if (p.nt == 96) epi_dyn_fixed<96>(taddr, cms, dq, sc, my_row, bar_rel);
-                        else if (p.nt == 64) epi_dyn_fixed<64>(taddr, cms, dq, sc, my_row, bar_rel);
-                        else if (p.nt == 48) epi_dyn_fixed<48>(taddr, cms, dq, sc, my_row, bar_rel);
-                        else if (p.nt == 32) epi_dyn_fixed<32>(taddr, cms, dq, sc, my_row, bar_rel);
-                        else if (p.nt == 80) epi_dyn_fixed<80>(taddr, cms, dq, sc, my_row, bar_rel);
-                        else epi_dyn_subtile<CH, true>(p, taddr, cms, dq, sc, my_row, bar_rel);
+                        if (p.nt == 96) epi_dyn_fixed<96>(taddr, cms, dq_row, sc_row, my_row, bar_rel);
+                        else if (p.nt == 64) epi_dyn_fixed<64>(taddr, cms, dq_row, sc_row, my_row, bar_rel);
+                        else if (p.nt == 48) epi_dyn_fixed<48>(taddr, cms, dq_row, sc_row, my_row, bar_rel);
+                        else if (p.nt == 32) epi_dyn_fixed<32>(taddr, cms, dq_row, sc_row, my_row, bar_rel);
+                        else if (p.nt == 80) epi_dyn_fixed<80>(taddr, cms, dq_row, sc_row, my_row, bar_rel);
+                        else epi_dyn_subtile<CH, true>(p, taddr, cms, dq_row, sc_row, my_row, bar_rel);
                     }
                 }
                 ptx::fence_proxy_async_smem();
@@ -1465,6 +1538,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 b ^= btoggle;
                 if (b < (uint32_t)kEpiGroups) tph ^= 1u;
             }
+            if constexpr (MODE == 1) flush_max();
             // the stores complete with the grid; only their reads of the slab must be over
             ptx::bulk_wait_read0();
         }
