@@ -177,19 +177,17 @@ act_quant_cluster_kernel(const float *__restrict__ x, int batch, long long per, 
             scale[sample] = sc;
         }
 
-        // ---- quantise from shared memory, 16 codes per store; refill each chunk at once ----
+        // ---- quantise from shared memory; refill each chunk at once ----
         int8_t *dst = q + (long long)sample * per + first;
         const int next = sample + nclusters;
         for (int c = 0; c < nchunks; ++c) {
             if (ok) {
-                const int lo = c * (int)(kCopyBytes / 64);
-                const int hi = min((int)(count >> 4), lo + (int)(kCopyBytes / 64));
-                for (int i = lo + threadIdx.x; i < hi; i += kThreads) {
-                    uint32_t w[4];
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) w[j] = quantise_four(b4[4 * i + j], sc);
-                    *reinterpret_cast<uint4 *>(dst + 16 * (size_t)i) = make_uint4(w[0], w[1], w[2], w[3]);
-                }
+                // (four codes per thread: neighbouring lanes on neighbouring 16-byte words, no bank conflicts)
+                const int lo = c * (int)(kCopyBytes / 16);
+                const int hi = min((int)(count >> 2), lo + (int)(kCopyBytes / 16));
+                uint32_t *dst4 = reinterpret_cast<uint32_t *>(dst);
+#pragma unroll 4
+                for (int i = lo + threadIdx.x; i < hi; i += kThreads) dst4[i] = quantise_four(b4[i], sc);
             }
             __syncthreads();              // the chunk has been read by everyone
             if (threadIdx.x == 0 && ok && next < batch) load_chunk(next, c);
@@ -198,63 +196,94 @@ act_quant_cluster_kernel(const float *__restrict__ x, int batch, long long per, 
     if (first_exchange) cluster.barrier_wait();     // a cluster without a sample still pairs its arrive
 }
 
-// Fused route without staging: the same clusters and slices, but a CTA reads its slice from
-// global memory twice, first for the maximum, then (from L2, where the slice of a few hundred
-// kilobytes still sits) to quantise it.  No shared-memory limit on the slice, several CTAs per SM.
-__global__ void __launch_bounds__(kThreads)
-act_quant_reread_kernel(const float *__restrict__ x, int batch, long long per, long long slice, float eps,
-                        int8_t *__restrict__ q, float *__restrict__ gamma, float *__restrict__ scale)
+// Grouped route.  The samples are taken in groups of a few ten megabytes, kernel k of the call takes the
+// maxima of group k and quantises group k - 1, which L2 still holds: HBM reads a float once, every SM works
+// on every group whatever the number and size of the samples, and a kernel's first half needs nothing of the
+// kernel in front, so that it runs beside that kernel's second half (programmatic dependent launch).  A warp
+// takes a contiguous run of pieces of kPiece floats, a piece lies in one sample; per is a multiple of 4.
+constexpr int kGroupThreads = 512;
+constexpr int kPieceVec = 8;                        // float4 loads of a lane in flight
+constexpr int kPiece = 32 * 4 * kPieceVec;
+struct GroupArgs {
+    const float *x;
+    long long per;
+    long long pieces;           // of a sample
+    int max_first, max_count;   // samples whose maxima are taken
+    int q_first, q_count;       // samples that are quantised
+    int first;                  // the first kernel of the call
+    float eps;
+    int8_t *q;
+    float *gamma, *scale;
+};
+
+// This warp's run [p, end) of `total` pieces.
+__device__ __forceinline__ void warp_run(long long total, long long &p, long long &end)
 {
-    __shared__ float part[kThreads / 32];
-    __shared__ float peer_max[2][kMaxCluster];
-    cg::cluster_group cluster = cg::this_cluster();
-    const unsigned rank = cluster.block_rank(), csize = cluster.num_blocks();
-    const int cid = blockIdx.x / csize, nclusters = gridDim.x / csize;
-    const long long first = (long long)rank * slice;
-    long long count = per - first;
-    count = count < 0 ? 0 : (count > slice ? slice : count);
-    const int n4 = (int)(count >> 2), n16 = (int)(count >> 4);
-    cluster.barrier_arrive();
-    ptx::grid_dep_wait();           // as above
+    const long long warps = (long long)gridDim.x * (kGroupThreads / 32);
+    const long long w = (long long)blockIdx.x * (kGroupThreads / 32) + (threadIdx.x >> 5);
+    const long long each = total / warps, more = total % warps;
+    p = w * each + (w < more ? w : more);
+    end = p + each + (w < more ? 1 : 0);
+}
+
+__global__ void __launch_bounds__(kGroupThreads, 2) act_group_kernel(const GroupArgs a)
+{
+    // The first kernel waits for what wrote x (and for the cleared maxima) before it releases the others; they
+    // wait for the kernel in front only where its maxima are needed.
+    if (a.first) ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    bool first_exchange = true;
-    for (int sample = cid, it = 0; sample < batch; sample += nclusters, ++it) {
-        const float4 *src = reinterpret_cast<const float4 *>(x + (long long)sample * per + first);
+    const int lane = threadIdx.x & 31;
+    const long long per4 = a.per >> 2;
+    long long p, end;
+    warp_run(a.pieces * a.max_count, p, end);
+    if (p < end) {
+        long long s = p / a.pieces, r = p - s * a.pieces;
         float m = 0.0f;
-        int i = threadIdx.x;
-        for (; i + 3 * kThreads < n4; i += 4 * kThreads) {
-            const float4 v0 = src[i], v1 = src[i + kThreads], v2 = src[i + 2 * kThreads], v3 = src[i + 3 * kThreads];
-            float a;
-            a = fmaxf(fmaxf(fabsf(v0.x), fabsf(v0.y)), fmaxf(fabsf(v0.z), fabsf(v0.w))); m = a > m ? a : m;
-            a = fmaxf(fmaxf(fabsf(v1.x), fabsf(v1.y)), fmaxf(fabsf(v1.z), fabsf(v1.w))); m = a > m ? a : m;
-            a = fmaxf(fmaxf(fabsf(v2.x), fabsf(v2.y)), fmaxf(fabsf(v2.z), fabsf(v2.w))); m = a > m ? a : m;
-            a = fmaxf(fmaxf(fabsf(v3.x), fabsf(v3.y)), fmaxf(fabsf(v3.z), fabsf(v3.w))); m = a > m ? a : m;
-        }
-        for (; i < n4; i += kThreads) {
-            const float4 v = src[i];
-            const float a = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
-            m = a > m ? a : m;
-        }
-        m = block_absmax(m, part);
-        if (first_exchange) { cluster.barrier_wait(); first_exchange = false; }
-        if (threadIdx.x < csize) *cluster.map_shared_rank(&peer_max[it & 1][rank], threadIdx.x) = m;
-        cluster.sync();
-        float g = 0.0f;
-        for (unsigned r = 0; r < csize; ++r) g = peer_max[it & 1][r] > g ? peer_max[it & 1][r] : g;
-        const float sc = scale_of(g, eps);
-        if (rank == 0 && threadIdx.x == 0) {
-            gamma[sample] = g;
-            scale[sample] = sc;
-        }
-        int8_t *dst = q + (long long)sample * per + first;
-        for (int j = threadIdx.x; j < n16; j += kThreads) {
-            uint32_t w[4];
+        for (; p < end; ++p) {
+            const float4 *src = reinterpret_cast<const float4 *>(a.x + (a.max_first + s) * a.per) + r * (kPiece / 4);
+            const int left = (int)(per4 - r * (kPiece / 4) < kPiece / 4 ? per4 - r * (kPiece / 4) : kPiece / 4);
+            float4 v[kPieceVec];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) w[e] = quantise_four(src[4 * j + e], sc);
-            *reinterpret_cast<uint4 *>(dst + 16 * (size_t)j) = make_uint4(w[0], w[1], w[2], w[3]);
+            for (int j = 0; j < kPieceVec; ++j)
+                v[j] = lane + 32 * j < left ? __ldg(src + lane + 32 * j) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+            for (int j = 0; j < kPieceVec; ++j)       // (fmaxf drops NaNs)
+                m = fmaxf(fmaxf(m, fmaxf(fabsf(v[j].x), fabsf(v[j].y))), fmaxf(fabsf(v[j].z), fabsf(v[j].w)));
+            if (++r == a.pieces || p + 1 == end) {
+                // non-negative floats are ordered like their bit patterns
+                const uint32_t g = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(m));
+                if (lane == 0 && g) atomicMax(reinterpret_cast<unsigned int *>(a.gamma + a.max_first + s), g);
+                m = 0.0f;
+                if (r == a.pieces) { r = 0; ++s; }
+            }
         }
     }
-    if (first_exchange) cluster.barrier_wait();
+    if (!a.first) ptx::grid_dep_wait();
+    warp_run(a.pieces * a.q_count, p, end);
+    if (p < end) {
+        long long s = p / a.pieces, r = p - s * a.pieces;
+        float sc = 0.0f;
+        bool fresh = true;
+        for (; p < end; ++p) {
+            const long long sample = a.q_first + s, at = r * (kPiece / 4);
+            const float4 *src = reinterpret_cast<const float4 *>(a.x + sample * a.per) + at;
+            uint32_t *dst = reinterpret_cast<uint32_t *>(a.q + sample * a.per) + at;
+            const int left = (int)(per4 - at < kPiece / 4 ? per4 - at : kPiece / 4);
+            float4 v[kPieceVec];
+#pragma unroll
+            for (int j = 0; j < kPieceVec; ++j)
+                if (lane + 32 * j < left) v[j] = __ldcs(src + lane + 32 * j);
+            if (fresh) {
+                sc = scale_of(__ldcg(a.gamma + sample), a.eps);
+                if (r == 0 && lane == 0) a.scale[sample] = sc;
+                fresh = false;
+            }
+#pragma unroll
+            for (int j = 0; j < kPieceVec; ++j)
+                if (lane + 32 * j < left) __stcs(dst + lane + 32 * j, quantise_four(v[j], sc));
+            if (++r == a.pieces) { r = 0; ++s; fresh = true; }
+        }
+    }
 }
 
 // Two-pass route, pass 1: gamma (zeroed beforehand) takes the maxima; |x| >= 0, so the order of

@@ -1750,6 +1750,8 @@ prom_status prom_pw_conv_i8_dyn(const int8_t *x_dev, int batch, int64_t rows_per
     return tc_launch_planned(c, pl, 2);
 }
 
+static std::atomic<long long> g_act_group{32ll << 20}; extern "C" __attribute__((visibility("default"))) void act_grp(long long v) { g_act_group.store(v); }
+static std::atomic<long long> g_act_max{1ll << 40}; extern "C" __attribute__((visibility("default"))) void act_mx(long long v) { g_act_max.store(v); }
 prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_sample,
                                      int8_t *q_dev, float *gamma_dev, float *scale_dev,
                                      void *cuda_stream)
@@ -1766,7 +1768,7 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
     // fused route: the smallest cluster whose slices fit shared memory
     const size_t room = (size_t)d.smem_optin - 4096;
     int cluster = 0, slice = 0;
-    if (per_sample % 16 == 0) {
+    if (per_sample % 16 == 0 && (long long)batch * per_sample * 4 <= g_act_max.load()) {
         for (int c = 1; c <= actq::kMaxCluster; c *= 2) {
             const long long s = ((per_sample + c - 1) / c + 15) / 16 * 16;
             if ((size_t)s * 4 <= room) { cluster = c; slice = (int)s; break; }
@@ -1823,53 +1825,36 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
         }
     }
 
-    // the same clusters reading their slices twice (the second time from L2): samples whose
-    // slices do not fit shared memory (as fast as the staged route at the bench's size, but the
-    // second read is from HBM again whenever L2 has lost the slice)
-    if (per_sample % 16 == 0) {
-        const int c = actq::kMaxCluster;
-        const long long s = ((per_sample + c - 1) / c + 15) / 16 * 16;
+    // groups of samples, maxima of one beside the codes of the one before
+    if (per_sample % 4 == 0) {
+        actq::GroupArgs a;
+        memset(&a, 0, sizeof(a));
+        a.x = x_dev; a.per = per_sample; a.pieces = (per_sample + actq::kPiece - 1) / actq::kPiece;
+        a.eps = eps; a.q = q_dev; a.gamma = gamma_dev; a.scale = scale_dev;
+        const long long group_bytes = g_act_group.load();
+        long long per_group = group_bytes / (per_sample * 4);
+        if (per_group < 1) per_group = 1;
+        const long long groups = (batch + per_group - 1) / per_group;
+        per_group = (batch + groups - 1) / groups;
         cudaLaunchConfig_t cfg;
-        memset(&cfg, 0, sizeof(cfg));
-        cfg.gridDim = dim3((unsigned)c);
-        cfg.blockDim = dim3(actq::kThreads);
-        cfg.stream = st;
-        cudaLaunchAttribute attr[2];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)c;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        static std::mutex mu;
-        static std::map<int, int> known;
-        int dev = 0;
-        cudaGetDevice(&dev);
-        int resident = 0;
-        {
-            std::lock_guard<std::mutex> lk(mu);
-            auto it = known.find(dev);
-            if (it == known.end()) {
-                if (cudaOccupancyMaxActiveClusters(&resident, actq::act_quant_reread_kernel, &cfg) !=
-                    cudaSuccess)
-                    resident = 0;
-                cudaGetLastError();
-                known[dev] = resident;
-            } else {
-                resident = it->second;
-            }
-        }
-        if (resident > 0 && s * 4 <= (8ll << 20)) {
-            const int nclusters = resident < batch ? resident : batch;
-            cfg.gridDim = dim3((unsigned)(nclusters * c));
-            attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[1].val.programmaticStreamSerializationAllowed = 1;
-            cfg.numAttrs = 2;
-            cudaError_t e = cudaLaunchKernelEx(&cfg, actq::act_quant_reread_kernel, x_dev, batch,
-                                               (long long)per_sample, s, eps, q_dev, gamma_dev, scale_dev);
+        cudaLaunchAttribute attr[1];
+        fill_launch_cfg(cfg, attr, (batch + 127) / 128, 128, 0, st, true);
+        cudaError_t e = cudaLaunchKernelEx(&cfg, dyn_clear_kernel, gamma_dev, batch);
+        ++g_launches;
+        for (long long k = 0; k * per_group < batch + per_group && e == cudaSuccess; ++k) {
+            auto count = [&](long long first) { return (int)(first < 0 || first >= batch ? 0 : (batch - first < per_group ? batch - first : per_group)); };
+            a.first = k == 0;
+            a.max_first = (int)(k * per_group < batch ? k * per_group : 0); a.max_count = count(k * per_group);
+            a.q_first = k ? (int)((k - 1) * per_group) : 0; a.q_count = k ? count((k - 1) * per_group) : 0;
+            // blocks for about two pieces per warp and pass, at most two per SM
+            const long long most = a.pieces * (a.max_count > a.q_count ? a.max_count : a.q_count);
+            long long blocks = (most + 31) / 32;
+            if (blocks > 2 * d.sms) blocks = 2 * d.sms;
+            fill_launch_cfg(cfg, attr, (int)blocks, actq::kGroupThreads, 0, st, true);
+            e = cudaLaunchKernelEx(&cfg, actq::act_group_kernel, a);
             ++g_launches;
-            return cuda_status(e);
         }
+        return cuda_status(e);
     }
 
     // two passes

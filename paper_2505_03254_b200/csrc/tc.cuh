@@ -236,10 +236,13 @@ __device__ __forceinline__ void epi_exact(uint32_t taddr, const int *__restrict_
 }
 
 // One output of the fast epilogue for the full int8 range: the rounding term loses one unit
-// when the product is negative (ties go away from zero), and the shift drops the extra bit.
+// when the product is negative (ties go away from zero), and the shift drops the extra bit.  r64 = 2^(32 + shmax)
+// has an empty low word, so r64 - 1 is the sign in the low word and added to the high one.
 __device__ __forceinline__ int fast_signed(int v, int mu, long long r64, int shmax)
 {
-    return (int)(((long long)v * mu + (r64 + (long long)(v >> 31))) >> 32) >> (shmax + 1);
+    const int sign = v >> 31;
+    const unsigned long long add = ptx::pack_2((uint32_t)sign, (uint32_t)((int)(r64 >> 32) + sign));
+    return (int)(((long long)v * mu + (long long)add) >> 32) >> (shmax + 1);
 }
 
 // NC accumulator columns of this thread's row, already in registers: the high word of a
@@ -1464,7 +1467,10 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         else if (CH == 32 && p.nt == 80) epi_fast_fixed<80>(taddr, cms, shmax, my_row, bar_rel);
                         else epi_fast_subtile<CH>(p, taddr, cms, shmax, my_row, bar_rel);
                     }
-                    else if (fast) epi_fast_subtile<CH, true>(p, taddr, cms, shmax, my_row, bar_rel);
+                    // (a straight line for 96 columns only: more of them made the kernel longer, which small
+                    // layers pay for in instruction fetches, 4 % of a body at batch 8)
+                    else if (MODE == 4 && fast && p.nt == 96) epi_fast_fixed<96, true>(taddr, cms, shmax, my_row, bar_rel);
+                    else if (MODE != 0 && fast) epi_fast_subtile<CH, true>(p, taddr, cms, shmax, my_row, bar_rel);
                     else epi_exact_subtile<CH>(p.nt, p.act_min, p.act_max, taddr, cms, cbs + ls * p.nt_pad, my_row, bar_rel);
                     if constexpr (MODE == 3) {
                         __syncwarp();
