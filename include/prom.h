@@ -213,11 +213,13 @@ prom_status prom_pw_conv_i8_dyn(const int8_t *x_dev, int batch, int64_t rows_per
  *   x_dev      [batch][per_sample] float32, device, 16-byte aligned
  *   q_dev      [batch][per_sample] int8, device, 16-byte aligned
  *   gamma_dev, scale_dev  [batch] float32, device (Eq. 6's gamma and the factor applied)
- * Asynchronous on the stream.  When per_sample is a multiple of 16 a thread-block cluster of
- * up to 8 CTAs works on each sample and exchanges the maxima through distributed shared
- * memory: if the sample fits the shared memory of 8 SMs (per_sample <= about 450 000) it is
- * staged there and read from HBM once, larger samples are read twice (the second time from L2
- * while it still holds them).  Other sizes take two kernels and read every value twice.
+ * Asynchronous on the stream.  When per_sample is a multiple of 16 and the sample fits the
+ * shared memory of 8 SMs (per_sample <= about 450 000) a thread-block cluster of up to 8 CTAs
+ * works on each sample, exchanges the maxima through distributed shared memory and reads the
+ * sample from HBM once.  Larger samples, and batches of which clusters would take several
+ * rounds, are taken in groups of a few ten megabytes (one kernel per group and one more) and
+ * read twice, the second time from L2.  Sizes that are not a multiple of 4 take two kernels and
+ * read every value twice.
  * Errors: PROM_ERR_NULL, PROM_ERR_SHAPE (batch < 0, per_sample < 1, batch > 65535 on the
  * two-pass route), PROM_ERR_ALIGN, PROM_ERR_CUDA; a copy that does not land within 0.1 s sets
  * PROM_ERR_TIMEOUT in prom_last_device_status.  batch == 0 is a no-op. */

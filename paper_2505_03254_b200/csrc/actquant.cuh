@@ -8,12 +8,16 @@
 // __fmul_rn: no contraction, no approximate division), the precision the paper's framework
 // computes in, so the codes do not depend on how the work is split.
 //
-// Two routes.  Fused: a thread-block cluster per sample; every CTA copies its slice of the
+// Three routes.  Fused: a thread-block cluster per sample; every CTA copies its slice of the
 // sample into shared memory once (bulk copies), the CTAs exchange their maxima through
 // distributed shared memory, and the slice is quantised from shared memory: each float is read
-// from HBM once (5 bytes per element).  Two-pass: one kernel takes the maxima with atomicMax
-// on the bit pattern, a second one quantises (9 bytes per element; for samples whose slice
-// does not fit shared memory or whose size is not a multiple of 4).
+// from HBM once (5 bytes per element).  Grouped: the maxima of one group of samples beside the codes of
+// the group before, which L2 still holds (samples that do not fit eight SMs' shared memory, and batches
+// of which clusters would take several rounds).  Two-pass, for sizes that are not a multiple of 4: one kernel
+// takes the maxima with atomicMax on the bit pattern, a second one quantises.
+// Measured, calls back to back (floor: 5 bytes per value at the copy bandwidth): [128,112,112,32] 64 us (39; 74.5
+// before, when a lane quantised 64 neighbouring bytes and met four-way bank conflicts); [1,112,112,320] 8 us
+// (3; 60 on one cluster); [60,112,112,96] 96 us (55; 107); [192,7,7,960] 11 us (7; 19).
 #pragma once
 
 #include <cooperative_groups.h>

@@ -1750,8 +1750,6 @@ prom_status prom_pw_conv_i8_dyn(const int8_t *x_dev, int batch, int64_t rows_per
     return tc_launch_planned(c, pl, 2);
 }
 
-static std::atomic<long long> g_act_group{32ll << 20}; extern "C" __attribute__((visibility("default"))) void act_grp(long long v) { g_act_group.store(v); }
-static std::atomic<long long> g_act_max{1ll << 40}; extern "C" __attribute__((visibility("default"))) void act_mx(long long v) { g_act_max.store(v); }
 prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_sample,
                                      int8_t *q_dev, float *gamma_dev, float *scale_dev,
                                      void *cuda_stream)
@@ -1765,15 +1763,34 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const float eps = 1e-5f;
 
-    // fused route: the smallest cluster whose slices fit shared memory
+    // Fused route: a cluster of CTAs per sample, its slices in shared memory.  The cluster size follows a time
+    // model fitted to a B200: every round of resident clusters costs an exchange that grows with the
+    // cluster, and the load of an SM's slices at about 100 KB per us.  (190 samples of 125 KB: 7.7 us with
+    // clusters of 2, which all fit at once, 10.1 and 11.1 with 1 and 4; 3 samples of 358 KB: 4.3 us with 8,
+    // 6.8 with 2.)
     const size_t room = (size_t)d.smem_optin - 4096;
     int cluster = 0, slice = 0;
-    if (per_sample % 16 == 0 && (long long)batch * per_sample * 4 <= g_act_max.load()) {
-        for (int c = 1; c <= actq::kMaxCluster; c *= 2) {
+    long long rounds = 0;
+    const long long total_bytes = (long long)batch * per_sample * 4;
+    if (per_sample % 16 == 0) {
+        double best = 0;
+        for (int c = 1, log2c = 0; c <= actq::kMaxCluster; c *= 2, ++log2c) {
             const long long s = ((per_sample + c - 1) / c + 15) / 16 * 16;
-            if ((size_t)s * 4 <= room) { cluster = c; slice = (int)s; break; }
+            if ((size_t)s * 4 > room) continue;
+            long long per_sm = (d.smem_total - 1024) / (s * 4 + 2048);
+            if (per_sm > 2048 / actq::kThreads) per_sm = 2048 / actq::kThreads;
+            if (per_sm < 1) per_sm = 1;
+            const long long at_once = per_sm * d.sms / c > 0 ? per_sm * d.sms / c : 1;
+            const long long r = (batch + at_once - 1) / at_once;
+            const long long used = ((long long)batch * c + d.sms - 1) / d.sms;
+            const double t = (double)r * (2.2 + 0.2 * log2c + (double)(s * 4 * (used < per_sm ? used : per_sm)) / 100e3);
+            if (!cluster || t < best) { best = t; cluster = c; slice = (int)s; rounds = r; }
         }
     }
+    // Several rounds of clusters run in step, each with its loads exposed; what fits one group of the grouped
+    // route below is faster there (192 x 188 KB: 11.3 us against 14.9; 128 x 301 KB: 11.5 against 13.5)
+    constexpr long long kOneGroup = 64ll << 20, kGroup = 40ll << 20;
+    if (rounds > 1 && total_bytes > (24ll << 20) && total_bytes <= kOneGroup) cluster = 0;
     if (cluster) {
         const cudaError_t attr_err = raise_smem_limit(actq::act_quant_cluster_kernel, d.smem_optin - 4096);
         if (attr_err != cudaSuccess) return cuda_status(attr_err);
@@ -1831,8 +1848,8 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
         memset(&a, 0, sizeof(a));
         a.x = x_dev; a.per = per_sample; a.pieces = (per_sample + actq::kPiece - 1) / actq::kPiece;
         a.eps = eps; a.q = q_dev; a.gamma = gamma_dev; a.scale = scale_dev;
-        const long long group_bytes = g_act_group.load();
-        long long per_group = group_bytes / (per_sample * 4);
+        // groups of about 40 MB (32 to 64 are alike, 16 cost 20 % more launches' worth); up to 64 MB in one
+        long long per_group = total_bytes <= kOneGroup ? batch : kGroup / (per_sample * 4);
         if (per_group < 1) per_group = 1;
         const long long groups = (batch + per_group - 1) / per_group;
         per_group = (batch + groups - 1) / groups;
