@@ -180,7 +180,7 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
     const uint32_t smem_base = ptx::smem_u32(smem);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
 
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + p.off_bars);
     const uint32_t bar_afull = ptx::smem_u32(bars);               // a resident chunk has landed
@@ -244,15 +244,16 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
         // Per pair of column tiles (one for each issuing thread): their constants, then chunk by
         // chunk {the row tile's chunk for the first pair of a row tile, the chunk of either tile's
         // weights into its thread's half of the ring}, then the two tiles' bias digits.
-        if (lane == 0) {
+        {
+            const bool leader = ptx::elect_one();
             uint32_t hs[2] = {0u, 0u}, hph[2] = {0u, 0u}, k[2] = {0u, 0u}, aph = 0;
             bool ok = true;
             // next stage of thread t's half ring, armed for tx bytes; 0 when a wait gave up
             auto w_slot = [&](int t, uint32_t tx, uint32_t &bar) -> uint32_t {
                 const uint32_t st = 2u * hs[t] + (uint32_t)t;
-                if (!tc::wait_bar(bar_wempty + 8 * st, hph[t] ^ 1u, flags)) { ok = false; return 0u; }
+                if (!tc::wait_bar_warp(bar_wempty + 8 * st, hph[t] ^ 1u, flags)) { ok = false; return 0u; }
                 bar = bar_wfull + 8 * st;
-                ptx::mbar_expect_tx(bar, tx);
+                if (leader) ptx::mbar_expect_tx(bar, tx);
                 if (++hs[t] == half) { hs[t] = 0; hph[t] ^= 1u; }
                 return smem_base + p.off_w + st * w_stage;
             };
@@ -263,28 +264,32 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
                     for (int t = 0; t < nu && ok; ++t) {
                         ct[t] = g + (lc0 + t) * p.groups;
                         const uint32_t slot = slot_of((uint32_t)t, k[t]);
-                        if (!tc::wait_bar(bar_cempty + 8 * slot, phase_of(k[t]) ^ 1u, flags)) { ok = false; break; }
-                        ptx::mbar_expect_tx(bar_cfull + 8 * slot, nb * kConstBytes);
-                        ptx::bulk_load(smem_base + p.off_const + slot * nb * kConstBytes,
-                                       p.consts + (size_t)ct[t] * nb * kConstBytes, nb * kConstBytes, bar_cfull + 8 * slot);
+                        if (!tc::wait_bar_warp(bar_cempty + 8 * slot, phase_of(k[t]) ^ 1u, flags)) { ok = false; break; }
+                        if (leader) {
+                            ptx::mbar_expect_tx(bar_cfull + 8 * slot, nb * kConstBytes);
+                            ptx::bulk_load(smem_base + p.off_const + slot * nb * kConstBytes,
+                                           p.consts + (size_t)ct[t] * nb * kConstBytes, nb * kConstBytes, bar_cfull + 8 * slot);
+                        }
                         ++k[t];
                     }
                     for (int c = 0; c < p.kc && ok; ++c) {
                         if (lc0 == 0) {
-                            if (!tc::wait_bar(bar_aempty + 8 * c, aph ^ 1u, flags)) { ok = false; break; }
-                            ptx::mbar_expect_tx(bar_afull + 8 * c, kStageBytes);
-                            ptx::tma_load_2d(smem_base + c * kStageBytes, &xmap, c * kChunk, mt * 128, bar_afull + 8 * c);
+                            if (!tc::wait_bar_warp(bar_aempty + 8 * c, aph ^ 1u, flags)) { ok = false; break; }
+                            if (leader) {
+                                ptx::mbar_expect_tx(bar_afull + 8 * c, kStageBytes);
+                                ptx::tma_load_2d(smem_base + c * kStageBytes, &xmap, c * kChunk, mt * 128, bar_afull + 8 * c);
+                            }
                         }
                         for (int t = 0; t < nu && ok; ++t) {
                             uint32_t bar = 0;
                             const uint32_t dst = w_slot(t, w_stage, bar);
-                            if (ok) ptx::tma_load_2d(dst, &wmap, c * kChunk, ct[t] * (int)nt, bar);
+                            if (ok && leader) ptx::tma_load_2d(dst, &wmap, c * kChunk, ct[t] * (int)nt, bar);
                         }
                     }
                     for (int t = 0; t < nu && ok; ++t) {
                         uint32_t bar = 0;
                         const uint32_t dst = w_slot(t, nb * kWbiasBytes, bar);
-                        if (ok) ptx::bulk_load(dst, p.wbias + (size_t)ct[t] * nb * kWbiasBytes, nb * kWbiasBytes, bar);
+                        if (ok && leader) ptx::bulk_load(dst, p.wbias + (size_t)ct[t] * nb * kWbiasBytes, nb * kWbiasBytes, bar);
                     }
                 }
             }
@@ -294,9 +299,12 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
                 while (ptx::globaltimer() - t0 < 20000ull) {}
             }
         }
+        __syncwarp();
     } else if (warp == 1 || warp == kIssuer2) {
         // ---- MMA issuers ------------------------------------------------------------------------------
-        if (lane == 0) {
+        // (the whole warp, one lane issues: descriptors then stay in uniform registers)
+        {
+            const bool leader = ptx::elect_one();
             const uint32_t t = warp == 1 ? 0u : 1u;
             // s8 x s8 -> s32, both K-major, M = 128, N = 128 or 256
             const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((nt >> 3) << 17) | ((128u >> 4) << 24);
@@ -309,38 +317,43 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
             for (int mt = worker; mt < p.n_mtiles && ok; mt += nworkers, aph ^= 1u) {
                 for (int lc = (int)t; lc < cols && ok; lc += 2, ++k) {
                     const uint32_t acc = slot_of(t, k);
-                    if (!tc::wait_bar(bar_tempty + 8 * acc, phase_of(k) ^ 1u, flags)) { ok = false; break; }
+                    if (!tc::wait_bar_warp(bar_tempty + 8 * acc, phase_of(k) ^ 1u, flags)) { ok = false; break; }
                     ptx::tc_fence_after_sync();
                     const uint32_t d_tmem = tmem_base + acc * nt;
                     const bool first = lc == (int)t, last = lc + 2 >= cols;     // of this thread in the row tile
-                    uint32_t accum = 0;
                     for (int c = 0; c < p.kc; ++c) {
                         const uint32_t st = 2u * hs + t;
-                        if (first && !tc::wait_bar(bar_afull + 8 * c, aph, flags)) { ok = false; break; }
-                        if (!tc::wait_bar(bar_wfull + 8 * st, hph, flags)) { ok = false; break; }
+                        if (first && !tc::wait_bar_warp(bar_afull + 8 * c, aph, flags)) { ok = false; break; }
+                        if (!tc::wait_bar_warp(bar_wfull + 8 * st, hph, flags)) { ok = false; break; }
                         ptx::tc_fence_after_sync();
                         const uint32_t a_lo = a_lo0 + (uint32_t)c * a_step, w_lo = w_lo0 + st * w_step;
                         const int nks = c == p.kc - 1 ? p.ksteps_last : 4;
-                        for (int ks = 0; ks < nks; ++ks) {
-                            ptx::mma_i8(d_tmem, d_128 | (uint64_t)(a_lo + 2 * ks), d_128 | (uint64_t)(w_lo + 2 * ks), idesc, accum);
-                            accum = 1;
+                        if (leader) {
+                            if (c == 0) ptx::mma_i8<false>(d_tmem, d_128 | (uint64_t)a_lo, d_128 | (uint64_t)w_lo, idesc);
+                            else ptx::mma_i8<true>(d_tmem, d_128 | (uint64_t)a_lo, d_128 | (uint64_t)w_lo, idesc);
+#pragma unroll
+                            for (int ks = 1; ks < 4; ++ks)
+                                if (ks < nks)
+                                    ptx::mma_i8<true>(d_tmem, d_128 | (uint64_t)(a_lo + 2 * ks), d_128 | (uint64_t)(w_lo + 2 * ks), idesc);
+                            ptx::mma_commit(bar_wempty + 8 * st);
+                            if (last) ptx::mma_commit(bar_aempty + 8 * c);
                         }
-                        ptx::mma_commit(bar_wempty + 8 * st);
-                        if (last) ptx::mma_commit(bar_aempty + 8 * c);
                         if (++hs == half) { hs = 0; hph ^= 1u; }
                     }
                     if (!ok) break;
                     // the bias step: the constant block of 1s and 127s against the tile's digits
                     const uint32_t st = 2u * hs + t;
-                    if (!tc::wait_bar(bar_wfull + 8 * st, hph, flags)) { ok = false; break; }
+                    if (!tc::wait_bar_warp(bar_wfull + 8 * st, hph, flags)) { ok = false; break; }
                     ptx::tc_fence_after_sync();
-                    ptx::mma_i8(d_tmem, ac_desc, d_32 | (uint64_t)(w_lo0 + st * w_step), idesc, 1u);
-                    ptx::mma_commit(bar_wempty + 8 * st);
+                    if (leader) {
+                        ptx::mma_i8<true>(d_tmem, ac_desc, d_32 | (uint64_t)(w_lo0 + st * w_step), idesc);
+                        ptx::mma_commit(bar_wempty + 8 * st);
+                        ptx::mma_commit(bar_tfull + 8 * acc);
+                    }
                     if (++hs == half) { hs = 0; hph ^= 1u; }
-                    ptx::mma_commit(bar_tfull + 8 * acc);
                 }
             }
-            ptx::mma_commit(bar_drain);
+            if (leader) ptx::mma_commit(bar_drain);
             const unsigned long long t0 = ptx::globaltimer();
             while (!ptx::mbar_try_wait(bar_drain, 0) && ptx::globaltimer() - t0 < tc::kWaitLimitNs) {}
         }
