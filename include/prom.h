@@ -31,10 +31,11 @@
  *   - The library allocates nothing the caller must free.  It keeps small
  *     internal caches (tensor-map plans; per device and stream, the index
  *     lists of the add/sub variant and the expanded weight matrix of the
- *     row-resident tensor-core kernel, which single calls with Cin >= 512 and
+ *     row-resident tensor-core kernel, which single calls with Cin >= 640 and
  *     Cout >= 256 on many rows use: device memory obtained with cudaMalloc on
- *     first use, so the first such call on a stream should not be made while
- *     that stream is being captured) that prom_shutdown() releases.
+ *     first use; while a stream is being captured the add/sub variant must
+ *     already have its own, and the row-resident kernel gives way to the
+ *     weight-resident one when it has not) that prom_shutdown() releases.
  *   - `cuda_stream` is a cudaStream_t passed as void* (NULL = default stream).
  *     Convolution calls are asynchronous on that stream.
  *   - Errors are return codes; nothing aborts or traps.  Argument errors are

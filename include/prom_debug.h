@@ -71,8 +71,8 @@ void prom_debug_dw_variant(int variant);
 /* Which kernel the tensor-core variant of a single pointwise call runs: 0 = the
  * library's choice (the row-resident kernel, which keeps 128 rows with all their
  * input channels in shared memory and streams the weight matrix past them, for
- * layers with Cin >= 512, Cout >= 256 (nearly a multiple of 128 unless Cin >= 768)
- * and at least four tiles of 128 rows per SM;
+ * layers with Cin >= 640, Cout >= 256 (nearly a multiple of 128, or at least 640), the clamp
+ * [0, 127] and at least one tile of 128 rows per SM;
  * the weight-resident kernel otherwise), 1 = the weight-resident kernel only, 2 = the row-resident kernel
  * or PROM_ERR_UNSUPPORTED (it takes plain matrices with Cin and Cout multiples
  * of 16, 128 <= Cin <= 1024, Cout >= 64, no residual).  blocks: 128-channel

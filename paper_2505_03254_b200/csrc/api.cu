@@ -607,20 +607,31 @@ struct WideBuf { uint8_t *p = nullptr; size_t bytes = 0; };
 static std::mutex g_wide_mu;
 static std::map<WideKey, WideBuf> g_wide_cache;
 
-static uint8_t *wide_scratch_for(cudaStream_t st, size_t bytes)
+static std::vector<uint8_t *> g_wide_retired;
+
+// null: no memory, or (sets *capturing) none yet and the stream is being captured.  A buffer that has become
+// too small is kept until prom_shutdown(): earlier calls and captured graphs may still use it.  Sizes are
+// powers of two, so a stream's buffers add up to less than twice its largest.
+static uint8_t *wide_scratch_for(cudaStream_t st, size_t bytes, bool *capturing)
 {
+    *capturing = false;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
     std::lock_guard<std::mutex> lk(g_wide_mu);
     WideBuf &b = g_wide_cache[WideKey{dev, st}];
     if (b.bytes < bytes) {
-        if (b.p) {
-            cudaStreamSynchronize(st);      // an earlier call may still be reading it
-            cudaFree(b.p);
-            b.p = nullptr; b.bytes = 0;
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+            *capturing = true;
+            return nullptr;
         }
-        if (cudaMalloc(reinterpret_cast<void **>(&b.p), bytes) != cudaSuccess) return nullptr;
-        b.bytes = bytes;
+        size_t want = 1 << 20;
+        while (want < bytes) want *= 2;
+        uint8_t *p = nullptr;
+        if (cudaMalloc(reinterpret_cast<void **>(&p), want) != cudaSuccess) return nullptr;
+        if (b.p) g_wide_retired.push_back(b.p);
+        b.p = p;
+        b.bytes = want;
     }
     return b.p;
 }
@@ -631,6 +642,8 @@ static void wide_release_cache()
     for (auto &kv : g_wide_cache)
         if (kv.second.p) cudaFree(kv.second.p);
     g_wide_cache.clear();
+    for (uint8_t *p : g_wide_retired) cudaFree(p);
+    g_wide_retired.clear();
 }
 
 struct WidePlan {
@@ -690,12 +703,14 @@ static bool wide_plan(const Conv &c, const DeviceInfo &d, WidePlan &pl, bool &wo
     if (workers < 1) workers = 1;
     pl.grid = (int)(workers * groups);
     p.act_min = c.rq.act_min; p.act_max = c.rq.act_max;
-    // measured on B200: it beats the weight-resident kernel from Cin = 512 on when there are
-    // several row tiles per SM (1.4 to 1.7 times at Cin = 960); below that both are bound by the
-    // cost of issuing tcgen05 instructions and the weight-resident kernel issues fewer per output
-    // (a last column tile that is mostly padding costs it that margin unless Cin is large)
+    // Measured on B200, time as a share of the weight-resident kernel's: from Cin = 640 on it is the faster one
+    // where the column tiles are nearly full (802816 rows: 960 -> 1280 0.64, 960 -> 512 0.62, 768 -> 768 0.81,
+    // 640 -> 256 0.78; 25088 rows: 960 -> 512 0.80, 640 -> 1280 0.99), but 960 -> 320 1.06 and 640 -> 320 1.26
+    // (a sixth of its columns is padding), 512 -> 512 1.19, 384 -> 960 1.08.  Its one-multiply epilogue
+    // is for the clamp [0, 127].
     const bool full_cols = 10 * c.cout > 9 * p.n_ctiles * nb * wide::kNt;
-    worth = c.cin >= 512 && c.cout >= 256 && p.n_mtiles >= 4 * d.sms && (full_cols || c.cin >= 768);
+    worth = c.cin >= 640 && c.cout >= 256 && (full_cols || c.cout >= 640) && p.n_mtiles >= d.sms &&
+            c.rq.act_min == 0 && c.rq.act_max == 127;
     return true;
 }
 
@@ -708,8 +723,9 @@ static prom_status launch_wide(const Conv &c, const DeviceInfo &d, WidePlan &pl)
     const size_t w8_bytes = (size_t)blocks * wide::kNt * pl.k_pad;
     const size_t wb_bytes = (size_t)blocks * wide::kWbiasBytes;
     const size_t cs_bytes = round256((size_t)blocks * wide::kConstBytes);
-    uint8_t *scratch = wide_scratch_for(c.st, w8_bytes + wb_bytes + cs_bytes);
-    if (!scratch) return PROM_ERR_CUDA;
+    bool capturing = false;
+    uint8_t *scratch = wide_scratch_for(c.st, w8_bytes + wb_bytes + cs_bytes, &capturing);
+    if (!scratch) return capturing ? PROM_ERR_UNSUPPORTED : PROM_ERR_CUDA;
     wide::PrepParams pp;
     memset(&pp, 0, sizeof(pp));
     pp.cin = c.cin; pp.cout = c.cout; pp.k_pad = pl.k_pad; pp.w_packed = c.w;
@@ -747,12 +763,16 @@ static prom_status launch_wide(const Conv &c, const DeviceInfo &d, WidePlan &pl)
             return PROM_ERR_UNSUPPORTED;
     }
     if (raise_smem_limit(wide::wide_conv_kernel, d.smem_optin) != cudaSuccess) return PROM_ERR_CUDA;
-    wide::wide_prep_kernel<<<blocks, 256, 0, c.st>>>(pp);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    fill_launch_cfg(cfg, attr, blocks * wide::kPrepParts, 256, 0, c.st, true);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, wide::wide_prep_kernel, pp);
     ++g_launches;
-    if (cudaGetLastError() != cudaSuccess) return PROM_ERR_CUDA;
-    wide::wide_conv_kernel<<<pl.grid, wide::kThreads, pl.smem, c.st>>>(xmap, wmap, ymap, p);
+    if (e != cudaSuccess) return cuda_status(e);
+    fill_launch_cfg(cfg, attr, pl.grid, wide::kThreads, pl.smem, c.st, true);
+    e = cudaLaunchKernelEx(&cfg, wide::wide_conv_kernel, xmap, wmap, ymap, p);
     ++g_launches;
-    return cuda_status(cudaGetLastError());
+    return cuda_status(e);
 }
 
 static prom_status launch_tc(const Conv &c, int use = kPlanSingle)

@@ -67,8 +67,9 @@ struct PrepParams {
     uint8_t *wbias, *consts;
 };
 
-// The operands of column tile `tile` of one layer; all 256 threads of the CTA take part.
-__device__ __forceinline__ void prep_tile(const PrepParams &p, const int tile)
+// The operands of column tile `tile` of one layer; all 256 threads of the CTA take part.  `parts` CTAs share
+// the expansion of the tile's weights (each checks the constants; the first writes them).
+__device__ __forceinline__ void prep_tile(const PrepParams &p, const int tile, const int part = 0, const int parts = 1)
 {
     __shared__ int s_mult[kNt], s_bias[kNt], s_shift[kNt];
     __shared__ int s_flags[4];      // shmin, shmax, bad, slow
@@ -100,7 +101,7 @@ __device__ __forceinline__ void prep_tile(const PrepParams &p, const int tile)
     // constants and bias digits
     uint8_t *cst = p.consts + (size_t)tile * kConstBytes;
     uint8_t *wb = p.wbias + (size_t)tile * kWbiasBytes;
-    if (threadIdx.x < kNt) {
+    if (threadIdx.x < kNt && part == 0) {
         const int c = threadIdx.x;
         reinterpret_cast<int *>(cst)[c] = s_mult[c];
         reinterpret_cast<int2 *>(cst + kNt * 4)[c] = make_int2(s_bias[c], s_shift[c]);
@@ -120,7 +121,7 @@ __device__ __forceinline__ void prep_tile(const PrepParams &p, const int tile)
         *reinterpret_cast<uint4 *>(wb + tc::swz_offset((uint32_t)c, 0u, 32u)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
         *reinterpret_cast<uint4 *>(wb + tc::swz_offset((uint32_t)c, 1u, 32u)) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
     }
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && part == 0) {
         int *hdr = reinterpret_cast<int *>(cst + kNt * 12);
         hdr[0] = shmax; hdr[1] = fast ? 1 : 0; hdr[2] = bad ? 1 : 0; hdr[3] = 0;
     }
@@ -128,7 +129,7 @@ __device__ __forceinline__ void prep_tile(const PrepParams &p, const int tile)
     // the tile's rows of the int8 matrix, 16 bytes (16 codes = one 32-bit word) per step
     const int rowb = (p.cin + 3) >> 2, pieces = p.k_pad >> 4;
     uint32_t invalid = 0;
-    for (int i = threadIdx.x; i < kNt * pieces; i += blockDim.x) {
+    for (int i = part * blockDim.x + threadIdx.x; i < kNt * pieces; i += parts * blockDim.x) {
         const int c = i / pieces, j = i - c * pieces, n = n0 + c;
         uint4 val = make_uint4(0u, 0u, 0u, 0u);
         if (n < p.cout && j * 16 < p.cin && !bad) {
@@ -149,8 +150,16 @@ __device__ __forceinline__ void prep_tile(const PrepParams &p, const int tile)
     if (invalid) raise_status(PROM_ERR_BAD_WEIGHT);
 }
 
-// One CTA per column tile.
-__global__ void __launch_bounds__(256, 1) wide_prep_kernel(const PrepParams p) { prep_tile(p, (int)blockIdx.x); }
+// kPrepParts CTAs per column tile (one per tile kept 138 SMs idle for 15 us).
+constexpr int kPrepParts = 8;
+__global__ void __launch_bounds__(256, 1) wide_prep_kernel(const PrepParams p)
+{
+    // launched with programmatic dependent launch: the weights may be the previous kernel's output, and the
+    // scratch it fills may still be read by an earlier call
+    ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    prep_tile(p, (int)blockIdx.x / kPrepParts, (int)blockIdx.x % kPrepParts, kPrepParts);
+}
 
 // The same for several layers in one launch: CTA b belongs to the layer l with first[l] <= b < first[l + 1].
 constexpr int kMaxPrepLayers = 16;
@@ -207,6 +216,8 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
     auto slot_of = [&](uint32_t t, uint32_t k) { return nb == 1u ? t + 2u * (k & 1u) : t; };
     auto phase_of = [&](uint32_t k) { return nb == 1u ? (k >> 1) & 1u : k & 1u; };
 
+    // the next call's kernel may start its set-up; it waits before it reads or writes anything
+    ptx::grid_dep_launch();
     // ---- prologue -----------------------------------------------------------------------------
     if (warp == 0) {
         if (lane < kMaxKc) {
@@ -246,6 +257,7 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
         // weights into its thread's half of the ring}, then the two tiles' bias digits.
         {
             const bool leader = ptx::elect_one();
+            ptx::grid_dep_wait();           // for wide_prep_kernel, which waited for what wrote x
             uint32_t hs[2] = {0u, 0u}, hph[2] = {0u, 0u}, k[2] = {0u, 0u}, aph = 0;
             bool ok = true;
             // next stage of thread t's half ring, armed for tx bytes; 0 when a wait gave up
