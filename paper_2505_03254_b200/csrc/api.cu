@@ -1270,8 +1270,16 @@ static prom_status dw_conv3x3(const int8_t *x_dev, int batch, int h, int w, int 
         if (e != PROM_ERR_UNSUPPORTED) return e;
     }
     if (dw_variant == 2) return PROM_ERR_UNSUPPORTED;
-    const int rows = dw::rows_per_unit(stride);
-    const long long units = (long long)batch * ((ho + rows - 1) / rows) * ((wo + dw::kStrip - 1) / dw::kStrip);
+    // Units (dw3x3_kernel's ROWS x STRIP pixels of four channels, one per thread at a time): large ones read
+    // fewer pixels twice, small ones give a small layer more threads and each of them less to do.
+    int rows = stride == 1 ? 2 : 1, strip = 4;
+    auto units_of = [&] { return (long long)batch * ((ho + rows - 1) / rows) * ((wo + strip - 1) / strip); };
+    // (Inside a sequence the next layer waits for the slowest thread: body of the network at batch 9 and width
+    // 0.75 285 -> 264 us, at batch 1 219 -> 200.  Calls of their own overlap, and there the work counts:
+    // [9,28,28,144] 4.1 us against 5.7 with small units, [1,28,28,192] 3.5 against 2.8.)
+    const bool small = units_of() * (c >> 2) < (pdl == tc::kPdlChain ? 300ll : 40ll) * d.sms;
+    if (small) { rows = 1; strip = 2; }
+    const long long units = units_of();
     if (units >= (1ll << 31)) return PROM_ERR_SHAPE;
     const long long total = units * (c >> 2);
     // a multiple of c / 4 threads, so that a thread keeps its channels: blocks in multiples of
@@ -1282,18 +1290,13 @@ static prom_status dw_conv3x3(const int8_t *x_dev, int batch, int h, int w, int 
     const long long cap = (long long)d.sms * 16;
     if (blocks > cap) blocks = cap;
     blocks = (blocks + step - 1) / step * step;
-    const int grid = (int)blocks;
-    cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    fill_launch_cfg(cfg, attr, grid, dw::kThreads, 0, st, pdl != 0);
-    cudaError_t le;
-    if (stride == 1)
-        le = cudaLaunchKernelEx(&cfg, dw::dw3x3_kernel<1>, x_dev, batch, h, w, c, ho, wo, w_dev, rq->bias, rq->mult,
-                                rq->shift, rq->act_min, rq->act_max, y_dev, pdl);
-    else
-        le = cudaLaunchKernelEx(&cfg, dw::dw3x3_kernel<2>, x_dev, batch, h, w, c, ho, wo, w_dev, rq->bias, rq->mult,
-                                rq->shift, rq->act_min, rq->act_max, y_dev, pdl);
+    fill_launch_cfg(cfg, attr, (int)blocks, dw::kThreads, 0, static_cast<cudaStream_t>(cuda_stream), pdl != 0);
+    auto *kernel = stride == 1 ? (small ? dw::dw3x3_kernel<1, 1, 2> : dw::dw3x3_kernel<1, 2, 4>)
+                               : (small ? dw::dw3x3_kernel<2, 1, 2> : dw::dw3x3_kernel<2, 1, 4>);
+    const cudaError_t le = cudaLaunchKernelEx(&cfg, kernel, x_dev, batch, h, w, c, ho, wo, w_dev, rq->bias, rq->mult,
+                                              rq->shift, rq->act_min, rq->act_max, y_dev, pdl);
     ++g_launches;
     return cuda_status(le);
 }

@@ -4,8 +4,10 @@
 // with one pixel of zero padding, then the same per-channel fixed-point requantisation as the
 // pointwise layers.  NHWC, so a pixel's channels are contiguous.
 //
-// A thread owns 4 channels (one 32-bit word per pixel) and a strip of kStrip output pixels of
-// kRows output rows (two rows at stride 1, one at stride 2).  It loads the words of the input rows
+// A thread owns 4 channels (one 32-bit word per pixel) and a strip of STRIP output pixels of
+// ROWS output rows: four pixels of two rows at stride 1 (of one at stride 2) where there are threads enough,
+// two pixels of one row where the layer is small and a thread's own chain of a thousand instructions is what
+// takes the time (the host's rule says when).  It loads the words of the input rows
 // and columns under the strip once.  Every input column is transposed with byte permutes into
 // one word per channel that holds the column's values of all the input rows, and an output's sum
 // is three dp4a instructions, one per tap column, against words that hold that column's three
@@ -21,7 +23,6 @@
 namespace prom { namespace dw {
 
 constexpr int kThreads = 256;
-constexpr int kStrip = 4;
 
 // 4 x 4 byte transpose: words a, b, c, d hold one input row each (byte k = channel k); o[k] gets
 // the four rows of channel k.
@@ -41,11 +42,9 @@ __device__ __forceinline__ void transpose3(uint32_t a, uint32_t b, uint32_t c, u
     o[2] = __byte_perm(t1, c, 0x6610); o[3] = __byte_perm(t1, c, 0x7732);
 }
 
-__host__ __device__ constexpr int rows_per_unit(int stride) { return stride == 1 ? 2 : 1; }
-
 // The launch has a multiple of c / 4 threads, so a thread keeps its four channels for all the
 // units it works on: filters and constants are fetched once.
-template <int STRIDE>
+template <int STRIDE, int ROWS, int STRIP>
 __global__ void __launch_bounds__(kThreads, 3)
 dw3x3_kernel(const int8_t *__restrict__ x, int batch, int h, int w, int c, int ho, int wo,
              const int8_t *__restrict__ wt, const int32_t *__restrict__ bias,
@@ -55,7 +54,7 @@ dw3x3_kernel(const int8_t *__restrict__ x, int batch, int h, int w, int c, int h
     // pdl: how this kernel is chained to the previous one of the stream (tc.cuh: kPdl*)
     if (pdl == tc::kPdlWait) ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    constexpr int kRows = rows_per_unit(STRIDE);          // output rows of a unit
+    constexpr int kRows = ROWS, kStrip = STRIP;           // output rows and pixels of a unit
     constexpr int kRowsIn = STRIDE * (kRows - 1) + 3;     // input rows under them (3 or 4)
     constexpr int kCols = STRIDE * (kStrip - 1) + 3;      // input columns under a strip
     const int cw = c >> 2;                                // channel words per pixel
@@ -71,12 +70,23 @@ dw3x3_kernel(const int8_t *__restrict__ x, int batch, int h, int w, int c, int h
     uint32_t wk[kRows][3][4];
     int cb[4], cm[4], cs[4];
     bool bad = false;
+    // the nine weights of each of the four channels are 36 neighbouring bytes: nine words where they are aligned
+    uint32_t ww[9];
+    if ((reinterpret_cast<uintptr_t>(wt) & 3u) == 0) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) ww[i] = __ldg(reinterpret_cast<const uint32_t *>(wt + (size_t)ch * 9) + i);
+    } else {
+        const uint8_t *wp = reinterpret_cast<const uint8_t *>(wt) + (size_t)ch * 9;
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+            ww[i] = (uint32_t)wp[4 * i] | ((uint32_t)wp[4 * i + 1] << 8) | ((uint32_t)wp[4 * i + 2] << 16) | ((uint32_t)wp[4 * i + 3] << 24);
+    }
+    auto byte_of = [&](int i) { return (ww[i >> 2] >> (8 * (i & 3))) & 0xFFu; };
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const uint8_t *wp = reinterpret_cast<const uint8_t *>(wt) + (size_t)(ch + k) * 9;
 #pragma unroll
         for (int dj = 0; dj < 3; ++dj) {
-            const uint32_t col = (uint32_t)wp[dj] | ((uint32_t)wp[3 + dj] << 8) | ((uint32_t)wp[6 + dj] << 16);
+            const uint32_t col = byte_of(9 * k + dj) | (byte_of(9 * k + 3 + dj) << 8) | (byte_of(9 * k + 6 + dj) << 16);
 #pragma unroll
             for (int rr = 0; rr < kRows; ++rr) wk[rr][dj][k] = col << (8 * rr * STRIDE);
         }

@@ -50,3 +50,23 @@ def test_the_librarys_choice_for_a_large_layer(stride):
         binding.debug_dw_variant(0)
     assert torch.equal(y, want)
     assert binding.last_device_status() == binding.PROM_OK
+
+
+@pytest.mark.parametrize("stride", [1, 2])
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("b,h,w,c", [(1, 1, 1, 4), (1, 2, 3, 8), (2, 7, 7, 64), (1, 28, 28, 192), (9, 28, 30, 144)])
+def test_units_of_the_cuda_core_kernel(oracle, stride, b, h, w, c, offset):
+    """Small and large units on both sides of the rule, filters on a word boundary and one byte off it."""
+    x, wt, bias, mult, shift = _case(47, b, h, w, c)
+    store = torch.empty(c * 9 + 4, dtype=torch.int8, device="cuda")
+    wd = store[offset:offset + c * 9].view(c, 3, 3)
+    wd.copy_(torch.from_numpy(wt))
+    try:
+        binding.debug_dw_variant(1)
+        for lo in (0, -128):
+            rq = binding.make_requant(torch.from_numpy(bias).cuda(), torch.from_numpy(mult).cuda(), torch.from_numpy(shift).cuda(), lo, 127)
+            y = binding.dw_conv3x3_i8(torch.from_numpy(x).cuda(), wd, rq, stride=stride)
+            torch.cuda.synchronize()
+            assert np.array_equal(y.cpu().numpy(), oracle.dw3x3(x, wt, bias, mult, shift, stride=stride, act_min=lo, act_max=127))
+    finally:
+        binding.debug_dw_variant(0)
