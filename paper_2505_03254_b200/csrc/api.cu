@@ -550,7 +550,6 @@ static prom_status tc_set_attr(const DeviceInfo &d)
     if (e == cudaSuccess) e = raise_smem_limit(tc::tc_conv_kernel<2, 0, true>, d.smem_optin);
     if (e == cudaSuccess) e = raise_smem_limit(tc::tc_conv_kernel<2, 3, true>, d.smem_optin);
     if (e == cudaSuccess) e = raise_smem_limit(tc::tc_conv_kernel<2, 4, true>, d.smem_optin);
-    if (e == cudaSuccess) e = raise_smem_limit(tc::tc_prep_kernel, d.smem_optin);
     if (e != cudaSuccess) return PROM_ERR_CUDA;
     done.fetch_or(bit, std::memory_order_release);
     return PROM_OK;
@@ -587,6 +586,26 @@ static prom_status tc_launch_planned(const Conv &c, TcPlan &pl, int mode = 0)
     }
     ++g_launches;
     return cuda_status(e);
+}
+
+// Adds a planned layer with an image to a preparation launch.
+static void prep_add(tc::PrepTable &t, const tc::Params &p, int &ctas, size_t &smem)
+{
+    tc::PrepLayer &q = t.layer[t.n];
+    q.w_packed = p.w_packed; q.bias = p.bias; q.mult = p.mult; q.shift = p.shift;
+    q.image = p.image; q.image_stride = p.image_stride;
+    q.off_wbias = p.off_wbias - p.off_w; q.off_mult = p.off_mult - p.off_w;
+    q.off_bs = p.off_bs - p.off_w; q.off_hdr = p.off_hdr - p.off_w;
+    q.k0 = p.k0; q.n0 = p.n0; q.fold = p.fold; q.kf = p.kf; q.nf = p.nf; q.nt = p.nt; q.nt_pad = p.nt_pad;
+    q.groups = p.groups; q.subs = p.subs_per_cta; q.cw = p.cw; q.kc = p.kc; q.ksteps_last = p.ksteps_last;
+    q.direct = p.direct; q.act_min = p.act_min; q.act_max = p.act_max;
+    const int pieces = p.subs_per_cta * p.kc * p.nt_pad * (p.cw >> 4);
+    q.parts = (pieces + tc::kPrepPieces - 1) / tc::kPrepPieces;
+    t.first[t.n] = ctas;
+    ctas += p.groups * q.parts;
+    t.first[++t.n] = ctas;
+    const size_t bytes = (size_t)p.subs_per_cta * p.nt_pad * sizeof(int2);
+    if (bytes > smem) smem = bytes;
 }
 
 static size_t round256(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -1506,30 +1525,20 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
             size_t smem = 0;
             int ctas = 0;
             for (; i < n && t.n < tc::kMaxPrepLayers; ++i) {
-                const TcPlan *pl = nullptr;
                 if (lay.chain_of[i] >= 0) {
                     const ChainPlan &c = lay.chains[lay.chain_of[i]];
                     if (c.kind == 1) continue;          // prepared by the batch below
                     TcPlan tmp = c.prep[i - c.first];
                     tc_bind(conv[i], tmp, chain_img[i]);
-                    t.layer[t.n] = tmp.p;
-                    pl = &c.prep[i - c.first];
+                    prep_add(t, tmp.p, ctas, smem);
                 } else if (is_tc[i] && plan[i].p.image) {
-                    t.layer[t.n] = plan[i].p;
-                    pl = &plan[i];
-                } else {
-                    continue;
+                    prep_add(t, plan[i].p, ctas, smem);
                 }
-                t.first[t.n] = ctas;
-                ctas += pl->p.groups;
-                if (pl->smem > smem) smem = pl->smem;
-                ++t.n;
             }
             if (t.n == 0) break;
-            t.first[t.n] = ctas;
             cudaLaunchConfig_t cfg;
             cudaLaunchAttribute attr[1];
-            fill_launch_cfg(cfg, attr, ctas, tc::kThreads, smem, st, true);
+            fill_launch_cfg(cfg, attr, ctas, tc::kPrepThreads, smem, st, true);
             const cudaError_t e = cudaLaunchKernelEx(&cfg, tc::tc_prep_kernel, t);
             ++g_launches;
             if (e != cudaSuccess) return PROM_ERR_CUDA;
@@ -1982,13 +1991,12 @@ prom_status prom_pw_prepare(int64_t m, int cin, const uint8_t *w_packed_dev, int
     tc_bind(c, pl, static_cast<uint8_t *>(prepared_dev));
     tc::PrepTable t;
     memset(&t, 0, sizeof(t));
-    t.n = 1;
-    t.first[0] = 0;
-    t.first[1] = pl.p.groups;
-    t.layer[0] = pl.p;
+    int ctas = 0;
+    size_t smem = 0;
+    prep_add(t, pl.p, ctas, smem);
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    fill_launch_cfg(cfg, attr, pl.p.groups, tc::kThreads, pl.smem, c.st, true);
+    fill_launch_cfg(cfg, attr, ctas, tc::kPrepThreads, smem, c.st, true);
     const cudaError_t le = cudaLaunchKernelEx(&cfg, tc::tc_prep_kernel, t);
     ++g_launches;
     return cuda_status(le);

@@ -1582,40 +1582,158 @@ __global__ void __launch_bounds__(32, 1) wait_timeout_probe_kernel(unsigned long
     }
 }
 
-// Prepared operands for a whole layer sequence in one launch: CTA b builds the image of
-// (layer, channel group) = the b-th entry of the table and writes it to that layer's
-// `image` buffer.  Shared-memory offsets are those of the layer's convolution launch.
+// Prepared operands for a whole layer sequence in one launch.  An image (build_image's layout) is written
+// straight to global memory by several CTAs, kPrepPieces 16-byte pieces of its weights each; the first of
+// them also writes the bias digits, the constants and the header.  (One CTA per image, built in shared memory
+// and copied out, took 7 us of every sequence call: the largest image decided, and a CTA with the layout of a
+// convolution's shared memory kept the first layer off its SM.)
 constexpr int kMaxPrepLayers = 48;
+constexpr int kPrepThreads = 256;
+constexpr int kPrepPieces = 4 * kPrepThreads;
+struct PrepLayer {
+    const uint8_t *w_packed;
+    const int32_t *bias, *mult;
+    const int8_t *shift;
+    uint8_t *image;
+    uint32_t image_stride, off_wbias, off_mult, off_bs, off_hdr;    // offsets inside an image
+    int k0, n0, fold, kf, nf, nt, nt_pad, groups, subs, cw, kc, ksteps_last, direct, act_min, act_max;
+    int parts;                                                      // CTAs per image
+};
 struct PrepTable {
     int n;
     int first[kMaxPrepLayers + 1];     // first CTA of each layer; first[n] = grid size
-    Params layer[kMaxPrepLayers];
+    PrepLayer layer[kMaxPrepLayers];
 };
 
-__global__ void __launch_bounds__(kThreads, 1)
-tc_prep_kernel(const __grid_constant__ PrepTable t)
+// Four 2-bit codes (the low byte of b) as four int8 of magnitude mag (1..64), without a table: the codes are
+// spread to bytes, 01 becomes mag and 11 its two's complement (mag ^ 0xFF) + 1, which does not carry.
+__device__ __forceinline__ uint32_t expand_four(uint32_t b, uint32_t mag)
 {
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>(
-        (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    int l = 0;
-    while (l + 1 < t.n && (int)blockIdx.x >= t.first[l + 1]) ++l;
-    const Params &p = t.layer[l];
-    const int g = (int)blockIdx.x - t.first[l];
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + p.off_bars);
-    const View vw = make_view(p, smem, bars);
-    build_luts(vw.lut, (int)threadIdx.x, kThreads);
+    uint32_t c = (b | (b << 12)) & 0x000F000Fu;
+    c = (c | (c << 6)) & 0x03030303u;
+    const uint32_t neg = (c >> 1) & 0x01010101u;
+    return (((c & 0x01010101u) * mag) ^ (neg * 0xFFu)) + neg;
+}
+
+__global__ void __launch_bounds__(kPrepThreads) tc_prep_kernel(const __grid_constant__ PrepTable t)
+{
+    extern __shared__ int2 prep_bs[];              // {bias, shift} per column of the group
+    __shared__ int flags[4];                       // shmin, shmax, bad constants, slow path
+    const int tid = (int)threadIdx.x;
+    int l = 0, end = t.n;
+    while (end - l > 1) {
+        const int mid = (l + end) >> 1;
+        if ((int)blockIdx.x >= t.first[mid]) l = mid; else end = mid;
+    }
+    const PrepLayer &p = t.layer[l];
+    const int local = (int)blockIdx.x - t.first[l], g = local / p.parts, part = local - g * p.parts;
+    uint8_t *const image = p.image + (size_t)g * p.image_stride;
+    const int ncols = p.subs * p.nt_pad;
+    if (tid == 0) { flags[0] = 31; flags[1] = 0; flags[2] = 0; flags[3] = 0; }
+    __syncthreads();
     // a call of its own, like kPdlWait
     ptx::grid_dep_wait();
     ptx::grid_dep_launch();
-    build_image(p, g, vw);
-    ptx::fence_proxy_async_smem();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        ptx::bulk_store(p.image + (size_t)g * p.image_stride, vw.smem_base + p.off_w, p.image_bytes);
-        ptx::bulk_commit();
-        ptx::bulk_wait_all();
+
+    // range check, shift span, and whether every channel can take the fast epilogue (see build_image)
+    int mn = 31, mx = 0, bad = 0, slow = 0;
+    for (int i = tid; i < ncols; i += kPrepThreads) {
+        const int ls = i / p.nt_pad, c = i - ls * p.nt_pad, nfold = (g + ls * p.groups) * p.nt + c;
+        int b = 0, mu = 0, sh = 0;
+        if (c < p.nt && nfold < p.nf) {
+            const int n = nfold % p.n0;
+            b = __ldg(p.bias + n); mu = __ldg(p.mult + n); sh = __ldg(p.shift + n);
+            if (!requant_ok(b, mu, sh)) { bad = 1; b = 0; mu = 0; sh = 0; }
+            mn = min(mn, sh); mx = max(mx, sh);
+            const long long ab = b < 0 ? -(long long)b : b;
+            if ((((long long)128 * p.k0 + ab) << 6) >= (1ll << 31) || (ab << 6) > kBiasMax) slow = 1;
+        }
+        prep_bs[i] = make_int2(b, sh);
+        if (part == 0) {
+            reinterpret_cast<int *>(image + p.off_mult)[i] = mu;
+            reinterpret_cast<int2 *>(image + p.off_bs)[i] = make_int2(b, sh);
+        }
     }
+    mn = __reduce_min_sync(0xFFFFFFFFu, mn); mx = __reduce_max_sync(0xFFFFFFFFu, mx);
+    if ((tid & 31) == 0) { atomicMin(&flags[0], mn); atomicMax(&flags[1], mx); }
+    if (bad) flags[2] = 1;
+    if (slow) flags[3] = 1;
+    __syncthreads();
+    const int shmax = flags[1];
+    const bool fast = flags[3] == 0 && (p.act_min == 0 || p.act_min == -128) && p.act_max == 127 &&
+                      shmax - flags[0] <= 4 && shmax <= 24;
+
+    if (part == 0) {
+        // bias digits, a thread writes four; without the fast epilogue the block is all zeros
+        for (int i = tid; i < ncols * 8; i += kPrepThreads) {
+            const int col = i >> 3, w = i & 7, ls = col / p.nt_pad, c = col - ls * p.nt_pad;
+            const int2 bs = prep_bs[p.direct ? ls * p.nt_pad + channel_of(c, p.nt) : col];
+            const int v = fast ? bs.x << (2 + shmax - bs.y) : 0;
+            const int h = (v >= 0 ? v + 63 : v - 63) / 127;        // nearest multiple of 127
+            uint32_t wd = 0;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int d = 4 * w + e - 2;                        // digit of weight 127, or below 0
+                int dig = 0;
+                if (d == -2) dig = v - 127 * h;
+                else if (d >= 0) dig = h >= 0 ? min(127, max(0, h - 127 * d)) : max(-127, min(0, h + 127 * d));
+                wd |= ((uint32_t)dig & 0xFFu) << (8 * e);
+            }
+            uint8_t *blk = image + p.off_wbias + (size_t)ls * p.nt_pad * 32;
+            *reinterpret_cast<uint32_t *>(blk + swz_offset((uint32_t)c, (uint32_t)w >> 2, 32u) + 4 * (w & 3)) = wd;
+        }
+        if (tid == 0) {
+            int *hdr = reinterpret_cast<int *>(image + p.off_hdr);
+            hdr[0] = shmax; hdr[1] = fast ? 1 : 0; hdr[2] = flags[2];
+            hdr[3] = ((p.act_min & 0xFF) << 8) | (p.act_max & 0xFF);
+            if (flags[2]) raise_status(PROM_ERR_BAD_REQUANT);
+        }
+    }
+
+    // this CTA's pieces of the expanded weights
+    const uint32_t cw = (uint32_t)p.cw;
+    const int rowb = (p.k0 + 3) >> 2, cpr = p.cw >> 4, cpr_log2 = cpr == 8 ? 3 : (cpr == 4 ? 2 : 1);
+    const int per_blk = p.nt_pad * cpr, total = p.subs * p.kc * per_blk;
+    const bool quick = (p.k0 & 15) == 0;
+    uint32_t invalid = 0;
+    for (int idx = part * kPrepPieces + tid; idx < total && idx < (part + 1) * kPrepPieces; idx += kPrepThreads) {
+        const int blk = idx / per_blk, r = idx - blk * per_blk, ls = blk / p.kc, chunk = blk - ls * p.kc;
+        const int row_b = r >> cpr_log2, j = r & (cpr - 1);
+        if (chunk == p.kc - 1 && j >= p.ksteps_last * 2) continue;         // never read
+        const int n = p.direct ? channel_of(row_b, p.nt) : row_b;           // the channel this row of B holds
+        const int nfold = (g + ls * p.groups) * p.nt + n, kbase = chunk * p.cw + j * 16;
+        uint4 val = make_uint4(0u, 0u, 0u, 0u);
+        if (n < p.nt && nfold < p.nf && kbase < p.kf) {
+            const uint32_t mag = fast ? 4u << (shmax - prep_bs[ls * p.nt_pad + n].y) : 1u;
+            const int pn = nfold / p.n0, pk = kbase / p.k0;                 // diagonal blocks of the folded weights
+            const uint8_t *row = p.w_packed + (size_t)(nfold - pn * p.n0) * rowb;
+            if (quick) {
+                if (pn == pk) {
+                    const uint32_t w = __ldg(reinterpret_cast<const uint32_t *>(row + ((kbase - pk * p.k0) >> 2)));
+                    invalid |= (w >> 1) & ~w & 0x55555555u;
+                    val = make_uint4(expand_four(w & 0xFFu, mag), expand_four((w >> 8) & 0xFFu, mag),
+                                     expand_four((w >> 16) & 0xFFu, mag), expand_four(w >> 24, mag));
+                }
+            } else {
+                // cin is 8 modulo 16: a piece may straddle two diagonal blocks; the part of it that lies in
+                // this channel's block pn is the K range [pn k0, (pn + 1) k0), in units of 8 values = 2 bytes
+                uint32_t wd[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int k = kbase + 8 * h - pn * p.k0;
+                    if (k >= 0 && k < p.k0) {
+                        const uint32_t w = __ldg(reinterpret_cast<const uint16_t *>(row + (k >> 2)));
+                        invalid |= (w >> 1) & ~w & 0x5555u;
+                        wd[2 * h] = expand_four(w & 0xFFu, mag);
+                        wd[2 * h + 1] = expand_four(w >> 8, mag);
+                    }
+                }
+                val = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+            }
+        }
+        *reinterpret_cast<uint4 *>(image + (size_t)blk * p.nt_pad * cw + swz_offset((uint32_t)row_b, (uint32_t)j, cw)) = val;
+    }
+    if (invalid) raise_status(PROM_ERR_BAD_WEIGHT);
 }
 
 }}  // namespace prom::tc
