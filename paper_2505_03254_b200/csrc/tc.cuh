@@ -821,6 +821,16 @@ __device__ __forceinline__ void build_luts(uint32_t *lut, int tid, int nthreads)
     }
 }
 
+// Four 2-bit codes (the low byte of b) as four int8 of magnitude mag (1..64), without a table: the codes are
+// spread to bytes, 01 becomes mag and 11 its two's complement (mag ^ 0xFF) + 1, which does not carry.
+__device__ __forceinline__ uint32_t expand_four(uint32_t b, uint32_t mag)
+{
+    uint32_t c = (b | (b << 12)) & 0x000F000Fu;
+    c = (c | (c << 6)) & 0x03030303u;
+    const uint32_t neg = (c >> 1) & 0x01010101u;
+    return (((c & 0x01010101u) * mag) ^ (neg * 0xFFu)) + neg;
+}
+
 // Builds the prepared operands of channel group g in shared memory: requantisation
 // constants checked and stored, the fast/exact decision, bias digits, and the 2-bit weights
 // expanded into the K-major swizzled int8 operand layout.  All kThreads threads take part
@@ -1002,16 +1012,19 @@ __device__ __forceinline__ void build_image(const Params &p, const int g, const 
                         }
                     } else {
                         // cin is 8 modulo 16: a piece may straddle two diagonal blocks; the part of
-                        // it that lies in this channel's block pn is the K range [pn k0, (pn + 1) k0)
-                        const uint32_t mag = t == 0 ? 1u : (2u << t), neg = 256u - mag;
+                        // it that lies in this channel's block pn is the K range [pn k0, (pn + 1) k0), in
+                        // units of 8 values = 2 bytes
+                        const uint32_t mag = t == 0 ? 1u : (2u << t);
                         uint32_t wd[4] = {0, 0, 0, 0};
-                        const int k_lo = pn * p.k0, k_hi = min(k_lo + p.k0, p.kf);
-                        const int e_lo = max(0, k_lo - kbase), e_hi = min(16, k_hi - kbase);
-                        for (int e = e_lo; e < e_hi; ++e) {
-                            int wv = weight_at(wq, rowb, row, kbase + e - k_lo);
-                            if (wv == -2) { invalid = 1; wv = 0; }
-                            const uint32_t byte = wv == 0 ? 0u : (wv > 0 ? mag : neg);
-                            wd[e >> 2] |= byte << (8 * (e & 3));
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int k = kbase + 8 * h - pn * p.k0;
+                            if (k >= 0 && k < p.k0) {
+                                const uint32_t w = *reinterpret_cast<const uint16_t *>(wq + (size_t)row * rowb + (k >> 2));
+                                invalid |= (w >> 1) & ~w & 0x5555u;
+                                wd[2 * h] = expand_four(w & 0xFFu, mag);
+                                wd[2 * h + 1] = expand_four(w >> 8, mag);
+                            }
                         }
                         val = make_uint4(wd[0], wd[1], wd[2], wd[3]);
                     }
@@ -1604,16 +1617,6 @@ struct PrepTable {
     int first[kMaxPrepLayers + 1];     // first CTA of each layer; first[n] = grid size
     PrepLayer layer[kMaxPrepLayers];
 };
-
-// Four 2-bit codes (the low byte of b) as four int8 of magnitude mag (1..64), without a table: the codes are
-// spread to bytes, 01 becomes mag and 11 its two's complement (mag ^ 0xFF) + 1, which does not carry.
-__device__ __forceinline__ uint32_t expand_four(uint32_t b, uint32_t mag)
-{
-    uint32_t c = (b | (b << 12)) & 0x000F000Fu;
-    c = (c | (c << 6)) & 0x03030303u;
-    const uint32_t neg = (c >> 1) & 0x01010101u;
-    return (((c & 0x01010101u) * mag) ^ (neg * 0xFFu)) + neg;
-}
 
 __global__ void __launch_bounds__(kPrepThreads) tc_prep_kernel(const __grid_constant__ PrepTable t)
 {
