@@ -218,7 +218,7 @@ static int round_up(int v, int a) { return (v + a - 1) / a * a; }
 // Everything of a plan that follows from (fold, nt, groups, occ); false when it does not fit.
 static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, const DeviceInfo &d,
                          int fold, int nt, int groups, int occ, int want_stages, TcPlan &pl,
-                         int cw_max = 128, int direct = 0, bool tail = false)
+                         int cw_max = 128, int direct = 0, bool tail = false, bool any_width = false)
 {
     tc::Params &p = pl.p;
     memset(&p, 0, sizeof(p));
@@ -226,7 +226,10 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
     if (kf > 4096 || nf % nt) return false;
     const int n_sub = nf / nt;
     if (n_sub % groups) return false;
-    if (n_sub > 1 && ((nt & 15) || (nf & 15))) return false;     // tensor-map stores
+    // tensor-map stores want rows and subtiles of whole 16-byte pieces; a small layer may store its rows in
+    // 8-byte pieces instead, which lets it use more than one channel group (720 -> 120 on 441 rows)
+    const bool rows_8 = n_sub > 1 && ((nt & 15) || (nf & 15));
+    if (rows_8 && (!any_width || direct || (nt & 7) || m * cout > 1500000)) return false;
     if (n_sub == 1 && (nt & 7)) return false;
     const int subs = n_sub / groups;
     const int nt_pad = round_up(nt, 16);
@@ -296,7 +299,7 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
     p.stages = stages; p.nbuf = nbuf; p.tmem_cols = tmem_cols;
     p.share_x = share_x;
     p.direct = direct;
-    p.store_2d = n_sub > 1 && !direct ? 1 : 0;
+    p.store_2d = rows_8 ? 2 : (n_sub > 1 && !direct ? 1 : 0);
     p.x3d = x3d; p.box_r = box_r;
     p.tx_bytes = x3d ? (uint32_t)(cw * map.wo * box_r) : (uint32_t)stage_bytes;
 
@@ -352,7 +355,7 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
     // against 6.1; at 1176 rows, 160 -> 960, 4.3 against 4.8).  A bulk store runs beside the next unit, a
     // direct one does not, so several units per CTA lose a little of what one gains.
     const bool short_piece = direct && nt % 64 && nt > 32;
-    const double unit = short_piece ? 1.15 : (direct && rounds * subs > 1 ? 0.9 : 0.8);
+    const double unit = short_piece ? 1.15 : (direct && rounds * subs > 1 ? 0.9 : 0.8) + (rows_8 ? 0.3 : 0.0);
     // 0.8 us per unit for the hand-overs around it (barrier waits, fences, store issue): fitted to
     // plans timed inside the chained step (32 -> 192 and 64 -> 384 prefer 96-column subtiles in
     // fewer channel groups to 64-column ones)
@@ -377,8 +380,9 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
 // use: kPlanSingle (one call: the kernel builds its operands itself), kPlanDynamic (the dynamic
 // layer: no row folding, a folded row could straddle two samples) or
 // kPlanPrepared (a layer of a sequence, whose operands tc_prep_kernel builds once)
-// kPlanOdd, added to kPlanSingle or kPlanPrepared: an odd number of rows that have to be folded in pairs is
-// taken too, the last row as a tile of its own (the automatic choice; PROM_VARIANT_TC refuses such a shape)
+// kPlanOdd, added to kPlanSingle or kPlanPrepared (the automatic choice of calls and sequences): an odd number of
+// rows that have to be folded in pairs is taken too, the last row as a tile of its own (PROM_VARIANT_TC
+// refuses such a shape), and small layers may have subtiles of any multiple of 8
 enum { kPlanSingle = 0, kPlanDynamic = 1, kPlanPrepared = 2, kPlanOdd = 4 };
 static bool tc_search_plan(long long m, int cin, int cout, const RowMap &map, const DeviceInfo &d,
                            int use, TcPlan &best)
@@ -429,7 +433,7 @@ static bool tc_search_plan(long long m, int cin, int cout, const RowMap &map, co
                 if (tn.occ == 0 && occ >= 3) continue;      // only on request for now
                 for (int direct = dyn ? 0 : 1; direct >= 0; --direct) {
                     TcPlan pl;
-                    if (!tc_fill_plan(m, cin, cout, map, d, fold, nt, groups, occ, tn.stages, pl, 128, direct, tail))
+                    if (!tc_fill_plan(m, cin, cout, map, d, fold, nt, groups, occ, tn.stages, pl, 128, direct, tail, odd_ok))
                         continue;
                     if (!found || pl.est_us < best.est_us) { best = pl; found = true; }
                 }
@@ -508,7 +512,7 @@ static bool tc_make_maps(const Conv &c, TcPlan &pl)
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     }
     if (r != CUDA_SUCCESS) return false;
-    if (p.store_2d) {
+    if (p.store_2d == 1) {
         cuuint64_t dims[2] = {(cuuint64_t)p.nf, (cuuint64_t)(p.m_rows > 0 ? p.m_rows : 1)};
         cuuint64_t strides[1] = {(cuuint64_t)p.nf};
         cuuint32_t box[2] = {(cuuint32_t)p.nt, 32};

@@ -70,7 +70,8 @@ struct Params {
     int stages, nbuf, tmem_cols;
     int share_x;        // kc == 1: one activation load serves all subtiles of the tile
     int direct;         // outputs leave straight from registers; the rows of B are permuted (channel_of)
-    int store_2d;       // 0: rows of a slab are contiguous in Y (one subtile), 1: tensor-map store
+    int store_2d;       // 0: rows of a slab are contiguous in Y (one subtile), 1: tensor-map store, 2: row by
+                        // row in 8-byte pieces (subtiles of widths that are 8 modulo 16)
     int x3d, box_r;     // 3-D activation map (strided input); rows of dim 2 per tile
     uint32_t tx_bytes;
     uint32_t off_w, off_wbias, off_mult, off_bs, off_hdr, off_aconst, off_out, off_lut, off_bars;
@@ -400,6 +401,17 @@ __device__ __noinline__ void store_tail_row(int8_t *y, const int8_t *res, const 
             v = make_uint2(__vaddss4(v.x, r.x), __vaddss4(v.y, r.y));
         }
         *reinterpret_cast<uint2 *>(y + i) = v;
+    }
+}
+
+// Stores the first rows_valid rows of a warp's 32 x nt slab in 8-byte pieces (Params::store_2d == 2); yp points
+// at the slab's first byte in Y.
+__device__ __noinline__ void store_rows_8(int8_t *yp, const uint8_t *slab, int rows_valid, int nf, int nt, int lane)
+{
+    const int g8 = nt >> 3, total = rows_valid * g8;
+    for (int i = lane; i < total; i += 32) {
+        const int r = i / g8, c = 8 * (i - r * g8);
+        *reinterpret_cast<uint2 *>(yp + (long long)r * nf + c) = *reinterpret_cast<const uint2 *>(slab + r * nt + c);
     }
 }
 
@@ -1120,7 +1132,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         } else if (lane == 31) {
             ptx::mbar_init(bar_drain, 1);
             ptx::tma_prefetch_desc(&xmap);
-            if (p.store_2d) ptx::tma_prefetch_desc(&ymap);
+            if (p.store_2d == 1) ptx::tma_prefetch_desc(&ymap);
         }
         ptx::mbar_init_fence();
     }
@@ -1345,7 +1357,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
             const uint32_t slab_bytes = 32u * (uint32_t)p.nf;
             int col = (g + ls * p.groups) * p.nt;       // first column of the subtile
             const int dcol = dls * p.groups * p.nt;
-            const bool store_2d = p.store_2d != 0;
+            const bool store_2d = p.store_2d != 0, rows_8 = p.store_2d == 2;
             const uint32_t res_inv = MODE == 3 ? (65536u + (uint32_t)(p.nt >> 3) - 1u) / (uint32_t)(p.nt >> 3) : 0u;
             // accumulators of this group: grp alone (two in the ring) or grp and grp + 2 (four)
             const uint32_t btoggle = p.nbuf == 4 ? 2u : 0u;
@@ -1528,7 +1540,7 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 }
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
-                if (whole_tile && row0 + 32 <= m_rows) {
+                if (whole_tile && row0 + 32 <= m_rows && !rows_8) {
                     // a whole slab: one copy
                     if (lane == 0) {
                         if (store_2d) ptx::tma_store_2d(&ymap, col, row0, slab_addr);
@@ -1548,7 +1560,8 @@ tc_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     int rows_valid = p.tm - q * 32;
                     if (m_rows - row0 < rows_valid) rows_valid = m_rows - row0;
                     if (rows_valid > 32) rows_valid = 32;
-                    store_partial_slab(p.y + (long long)row0 * p.nf, slab, rows_valid, p.nf, p.nt, col,
+                    if (rows_8) store_rows_8(p.y + (long long)row0 * p.nf + col, slab, rows_valid, p.nf, p.nt, lane);
+                    else store_partial_slab(p.y + (long long)row0 * p.nf, slab, rows_valid, p.nf, p.nt, col,
                                        store_2d, lane);
                 }
                 // this group's next unit and accumulator
