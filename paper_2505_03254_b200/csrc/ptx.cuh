@@ -299,6 +299,8 @@ __device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, un
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
     return r;
 }
+// (Not to be added to afterwards with add_f32x2: the pair is then fused and the product reaches the sum
+// unrounded, although for scalars the .rn of both keeps them apart.)
 __device__ __forceinline__ unsigned long long mul_f32x2(unsigned long long a, unsigned long long b)
 {
     unsigned long long r;

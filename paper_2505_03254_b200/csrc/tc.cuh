@@ -696,8 +696,9 @@ __device__ __forceinline__ void dyn_piece_quant(const uint32_t (&v)[NC], const i
             t = ptx::add_f32x2(t, ptx::pack_2(0xCB400000u, 0xCB400000u));            // the accumulators as floats
             t = ptx::mul_f32x2(t, ptx::pack_2((uint32_t)(h ? mu.z : mu.x), (uint32_t)(h ? mu.w : mu.y)));
             t = ptx::mul_f32x2(ptx::mul_f32x2(t, dq2), sc2);
-            t = ptx::add_f32x2(t, ptx::pack_2(0x4B400000u, 0x4B400000u));
-            r[2 * h] = (uint32_t)t; r[2 * h + 1] = (uint32_t)(t >> 32);
+            // (one at a time: a packed addition would take the packed product unrounded)
+            r[2 * h] = __float_as_uint(__fadd_rn(__uint_as_float((uint32_t)t), 12582912.0f));
+            r[2 * h + 1] = __float_as_uint(__fadd_rn(__uint_as_float((uint32_t)(t >> 32)), 12582912.0f));
         }
         out[e / 4] = __byte_perm(__byte_perm(r[0], r[1], 0x0040), __byte_perm(r[2], r[3], 0x0040), 0x5410);
     }
