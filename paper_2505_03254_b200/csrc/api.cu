@@ -676,6 +676,27 @@ struct WidePlan {
     int k_pad;
 };
 
+// Pairs of CTAs that are resident at once, one CTA per SM (asked once per device: the query takes tens of
+// microseconds).
+static int wide_pairs(const DeviceInfo &d)
+{
+    static std::atomic<int> known[64];
+    const bool keep = d.dev >= 0 && d.dev < 64;
+    int n = keep ? known[d.dev].load() : 0;
+    if (n == 0) {
+        if (raise_smem_limit(wide::wide_conv_kernel, d.smem_optin) != cudaSuccess) return 0;
+        cudaLaunchConfig_t cfg;
+        fill_launch_cfg(cfg, nullptr, 2 * (d.sms / 2), wide::kThreads, (size_t)d.smem_optin, nullptr, false);
+        if (cudaOccupancyMaxActiveClusters(&n, wide::wide_conv_kernel, &cfg) != cudaSuccess) {
+            cudaGetLastError();
+            n = 0;
+        }
+        if (n > d.sms / 2) n = d.sms / 2;
+        if (keep) known[d.dev].store(n);
+    }
+    return n;
+}
+
 // Shapes the variant takes: a plain matrix, whole 16-channel slices on both sides, K within the
 // resident chunks.  `worth` says whether the library picks it by itself.
 static bool wide_plan(const Conv &c, const DeviceInfo &d, WidePlan &pl, bool &worth)
@@ -689,42 +710,33 @@ static bool wide_plan(const Conv &c, const DeviceInfo &d, WidePlan &pl, bool &wo
     p.m = c.m; p.cin = c.cin; p.cout = c.cout;
     p.kc = (c.cin + wide::kChunk - 1) / wide::kChunk;
     p.ksteps_last = (c.cin - (p.kc - 1) * wide::kChunk + 31) / 32;
-    p.n_mtiles = (int)((c.m + 127) / 128);
+    p.n_mtiles = (int)((c.m + 255) / 256);
     pl.k_pad = p.kc * wide::kChunk;
+    // 256-channel column tiles; the tests ask for 128, or for 256 where a CTA of its own could hold them
+    const int forced = g_wide_nb.load();
+    if (forced == 2 && c.cin > 512) return false;
+    const int nb = forced ? forced : 2;
+    p.nb = nb;
     // shared memory: resident chunks, weight ring, constants, staging slabs, the bias step's A block, barriers
-    const uint32_t a_bytes = (uint32_t)p.kc * wide::kStageBytes;
-    const uint32_t const_bytes = (wide::kAccs * wide::kConstBytes + 1023u) & ~1023u;
+    const uint32_t a_bytes = (uint32_t)p.kc * wide::kAChunkBytes, w_stage = (uint32_t)nb * (wide::kNt / 2) * wide::kChunk;
+    const uint32_t const_bytes = ((uint32_t)(wide::kAccs * nb) * wide::kConstBytes + 1023u) & ~1023u;
     const uint32_t fixed = const_bytes + wide::kEpiWarps * wide::kSlabBytes + tc::kAConstBytes + 1024;
     const long long room = (long long)d.smem_optin - 1024 - a_bytes - fixed;
-    // 128-channel column tiles.  256-channel tiles (half as many tcgen05 instructions per output;
-    // on request, where four stages of 32 KB fit beside the resident rows) measured slower: tensor
-    // memory then holds one accumulator per issuing thread, so a thread's MMAs cannot overlap the
-    // read-out of its previous tile (1.6 M x 384 -> 1280: 1416 against 1090 us, x 512 -> 256: 490
-    // against 300 us).
-    int nb = g_wide_nb.load();
-    if (nb == 0) nb = 1;
-    p.nb = nb;
-    int stages = (int)(room / (nb * wide::kStageBytes));
+    int stages = (int)(room / w_stage);
     if (stages > wide::kMaxStages) stages = wide::kMaxStages;
-    stages &= ~1;                       // one half of the ring per issuing thread
-    if (stages < 4) return false;
+    if (stages < 3) return false;
     p.stages = stages;
     p.n_ctiles = (c.cout + nb * wide::kNt - 1) / (nb * wide::kNt);
     p.off_w = a_bytes;
-    p.off_aconst = p.off_w + (uint32_t)stages * nb * wide::kStageBytes;
+    p.off_aconst = p.off_w + (uint32_t)stages * w_stage;
     p.off_const = p.off_aconst + tc::kAConstBytes;
     p.off_out = p.off_const + const_bytes;
     p.off_bars = p.off_out + wide::kEpiWarps * wide::kSlabBytes;
     pl.smem = p.off_bars + 1024 + 1024;
-    // few row tiles: CTAs share a row tile's columns
-    int groups = 1;
-    for (int g = 1; g <= p.n_ctiles; ++g)
-        if (p.n_ctiles % g == 0 && (long long)p.n_mtiles * g <= d.sms) groups = g;
-    p.groups = groups;
-    long long workers = d.sms / groups;
-    if (workers > p.n_mtiles) workers = p.n_mtiles;
-    if (workers < 1) workers = 1;
-    pl.grid = (int)(workers * groups);
+    long long pairs = wide_pairs(d);
+    if (pairs < 1) return false;
+    if (pairs > (long long)p.n_mtiles * p.n_ctiles) pairs = (long long)p.n_mtiles * p.n_ctiles;
+    pl.grid = (int)(2 * pairs);
     p.act_min = c.rq.act_min; p.act_max = c.rq.act_max;
     // Measured on B200, time as a share of the weight-resident kernel's: from Cin = 640 on it is the faster one
     // where the column tiles are nearly full (802816 rows: 960 -> 1280 0.64, 960 -> 512 0.62, 768 -> 768 0.81,
@@ -732,7 +744,7 @@ static bool wide_plan(const Conv &c, const DeviceInfo &d, WidePlan &pl, bool &wo
     // (a sixth of its columns is padding), 512 -> 512 1.19, 384 -> 960 1.08.  Its one-multiply epilogue
     // is for the clamp [0, 127].
     const bool full_cols = 10 * c.cout > 9 * p.n_ctiles * nb * wide::kNt;
-    worth = c.cin >= 640 && c.cout >= 256 && (full_cols || c.cout >= 640) && p.n_mtiles >= d.sms &&
+    worth = c.cin >= 640 && c.cout >= 256 && (full_cols || c.cout >= 640) && c.m > 128ll * (d.sms - 1) &&
             c.rq.act_min == 0 && c.rq.act_max == 127;
     return true;
 }
@@ -755,8 +767,8 @@ static prom_status launch_wide(const Conv &c, const DeviceInfo &d, WidePlan &pl)
     pp.bias = c.rq.bias; pp.mult = c.rq.mult; pp.shift = c.rq.shift;
     pp.act_min = c.rq.act_min; pp.act_max = c.rq.act_max;
     pp.w8 = reinterpret_cast<int8_t *>(scratch); pp.wbias = scratch + w8_bytes; pp.consts = scratch + w8_bytes + wb_bytes;
-    p.wbias = pp.wbias; p.consts = pp.consts;
-    CUtensorMap xmap, wmap, ymap;
+    p.consts = pp.consts;
+    CUtensorMap xmap, wmap, bmap, ymap;
     cuuint32_t es[2] = {1, 1};
     {
         cuuint64_t dims[2] = {(cuuint64_t)c.cin, (cuuint64_t)c.m};
@@ -770,10 +782,18 @@ static prom_status launch_wide(const Conv &c, const DeviceInfo &d, WidePlan &pl)
     {
         cuuint64_t dims[2] = {(cuuint64_t)pl.k_pad, (cuuint64_t)blocks * wide::kNt};
         cuuint64_t strides[1] = {(cuuint64_t)pl.k_pad};
-        cuuint32_t box[2] = {(cuuint32_t)wide::kChunk, (cuuint32_t)(p.nb * wide::kNt)};
+        cuuint32_t box[2] = {(cuuint32_t)wide::kChunk, (cuuint32_t)(p.nb * wide::kNt / 2)};      // one CTA's half
         if (enc(&wmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, pp.w8, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
             CUDA_SUCCESS)
+            return PROM_ERR_UNSUPPORTED;
+    }
+    {
+        cuuint64_t dims[2] = {32, (cuuint64_t)blocks * wide::kNt};
+        cuuint64_t strides[1] = {32};
+        cuuint32_t box[2] = {32, (cuuint32_t)(p.nb * wide::kNt / 2)};
+        if (enc(&bmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, pp.wbias, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return PROM_ERR_UNSUPPORTED;
     }
     {
@@ -785,7 +805,6 @@ static prom_status launch_wide(const Conv &c, const DeviceInfo &d, WidePlan &pl)
             CUDA_SUCCESS)
             return PROM_ERR_UNSUPPORTED;
     }
-    if (raise_smem_limit(wide::wide_conv_kernel, d.smem_optin) != cudaSuccess) return PROM_ERR_CUDA;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     fill_launch_cfg(cfg, attr, blocks * wide::kPrepParts, 256, 0, c.st, true);
@@ -793,7 +812,7 @@ static prom_status launch_wide(const Conv &c, const DeviceInfo &d, WidePlan &pl)
     ++g_launches;
     if (e != cudaSuccess) return cuda_status(e);
     fill_launch_cfg(cfg, attr, pl.grid, wide::kThreads, pl.smem, c.st, true);
-    e = cudaLaunchKernelEx(&cfg, wide::wide_conv_kernel, xmap, wmap, ymap, p);
+    e = cudaLaunchKernelEx(&cfg, wide::wide_conv_kernel, xmap, wmap, bmap, ymap, p);
     ++g_launches;
     return cuda_status(e);
 }

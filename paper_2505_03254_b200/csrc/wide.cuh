@@ -4,12 +4,14 @@
 // tc_conv_kernel keeps the weights of a channel group resident and streams the activations
 // past them once per group; with Cin x Cout in the hundreds of thousands a group is only a few
 // dozen channels wide, the MMAs are narrow and the activations cross the SM many times.  Here
-// the roles are swapped: a CTA (one per SM) keeps a tile of 128 rows resident, all of its K
-// (up to 8 chunks of 128 bytes), and streams the expanded weights of one 128-channel column
-// tile after the other through a ring, so that every MMA is 128 x 128 x 32 (the tensor pipe's
-// full rate) and an activation byte enters the SM once.  What an SM then has to pull from L2 is
-// the weight matrix once per row tile: Cin * Cout bytes per 128 * Cin * Cout MACs, i.e. 64 bytes
-// per clock at the pipe's 8192 MACs per clock, which is what one SM can take (61.5 measured).
+// the roles are swapped: a pair of CTAs (one per SM) keeps a tile of 256 rows resident, all of its K
+// (up to 8 chunks of 128 bytes, 128 rows in each CTA), and streams the expanded weights of one
+// 256-channel column tile after the other through a ring.  The MMAs span the pair (cta_group::2,
+// 256 x 256 x 32): each CTA holds half of a column tile's weights, so that per 128 clocks of the tensor
+// pipe a CTA's shared memory is read for 4 KB of rows and 4 KB of weights and written with 4 KB, 96 of the
+// 128 bytes per clock that it can take, and 32 bytes per clock come from L2.  (One CTA alone with 128 x 128 x 32
+// MMAs needs 128 + 64 bytes per clock, and 64 of the 61.5 measured from L2.)
+// 1.6 M x 960 -> 1280: 1615-1670 us with single CTAs, 1460-1480 with pairs, under the power cap in both.
 //
 // wide_prep_kernel (one CTA per column tile) expands the 2-bit weights into an int8 matrix
 // [Cout padded to 128][Cin padded to 128] in global scratch, scaled for the one-multiply
@@ -18,26 +20,25 @@
 // tensor map (128-byte swizzle, like the activations), the bias digits as the last "chunk" of a
 // column tile, and the constants into a small ring of their own.
 //
-// Warp 0 issues the loads, warps 1 and 18 the MMAs, warps 2..17 are four epilogue groups, one per
-// accumulator, that requantise 32 columns at a time and store through the
-// output's tensor map (rows and columns outside the matrix are not written).
+// Warp 0 of each CTA issues its loads, warp 1 of the first CTA the MMAs of both, warps 2..17 requantise the
+// CTA's own 128 rows, 32 columns at a time, and store through the output's tensor map (rows and columns outside
+// the matrix are not written).
 #pragma once
 
 #include "tc.cuh"
 
 namespace prom { namespace wide {
 
-constexpr int kEpiWarps = 16;                     // four groups, one per accumulator
-constexpr int kIssuer2 = 2 + kEpiWarps;           // warp of the second MMA issuer
-constexpr int kThreads = 32 * (kIssuer2 + 1);     // loader, MMA issuer, sixteen epilogue warps, MMA issuer
-constexpr int kNt = 128;                          // columns of a column tile = MMA N
+constexpr int kEpiWarps = 16;                     // four groups of four
+constexpr int kThreads = 32 * (2 + kEpiWarps);    // loader, MMA issuer, epilogue warps
+constexpr int kNt = 128;                          // channels of a block of constants
 constexpr int kChunk = 128;                       // bytes of K per chunk = swizzle span
 constexpr int kMaxKc = 8;                         // resident K chunks: Cin <= 1024
 constexpr int kMaxStages = 8;
-constexpr int kAccs = 4;                          // accumulators of 128 columns: all 512 of tensor memory
-constexpr uint32_t kStageBytes = kNt * kChunk;    // 16 KB, also one resident chunk of the row tile
-constexpr uint32_t kWbiasBytes = kNt * 32;        // bias digits of a column tile (32-byte swizzled rows)
-// constants of a column tile: mult[128], {bias, shift}[128], header {shmax, fast, bad, 0}
+constexpr int kAccs = 2;                          // accumulators of up to 256 columns
+constexpr uint32_t kAChunkBytes = 128 * kChunk;   // one resident chunk of a CTA's 128 rows
+constexpr uint32_t kWbiasBytes = kNt * 32;        // bias digits of a block (32-byte swizzled rows)
+// constants of a block: mult[128], {bias, shift}[128], header {shmax, fast, bad, 0}
 constexpr uint32_t kConstBytes = kNt * 4 + kNt * 8 + 16 + 112;
 constexpr uint32_t kEpiCols = 32;                 // columns an epilogue warp stages per store
 constexpr uint32_t kSlabBytes = 32 * kEpiCols;
@@ -47,12 +48,10 @@ struct Params {
     long long m;
     int cin, cout;
     int kc, ksteps_last;        // chunks of K; 32-byte MMA steps in the last one
-    int n_mtiles, n_ctiles;     // row tiles, column tiles
-    int nb;                     // 128-channel blocks per column tile: 1 (MMA N = 128) or 2 (N = 256)
-    int groups;                 // CTAs that share a row tile's columns; n_ctiles % groups == 0
+    int n_mtiles, n_ctiles;     // tiles of 256 rows, column tiles
+    int nb;                     // 128-channel blocks per column tile: 1 or 2
     int stages;                 // of the weight ring
     uint32_t off_w, off_const, off_out, off_aconst, off_bars;
-    const uint8_t *wbias;       // [n_ctiles * nb][kWbiasBytes]
     const uint8_t *consts;      // [n_ctiles * nb][kConstBytes]
     int act_min, act_max;
 };
@@ -176,21 +175,21 @@ __global__ void __launch_bounds__(256, 1) wide_prep_batch_kernel(const __grid_co
     prep_tile(t.layer[l], (int)blockIdx.x - t.first[l]);
 }
 
-// Two threads issue MMAs (warps 1 and 18), each with half of the weight ring (stages t, t + 2, ..),
-// two of the four accumulators (t and t + 2) and every second column tile of a row tile: the
-// k-th unit of thread t uses accumulator t + 2 (k & 1).  One thread alone cannot keep the pipe busy
-// with 128-column MMAs: between the four MMAs of a chunk it spends more cycles on the barrier
-// wait, the commit and its own bookkeeping than the pipe needs for them.  Epilogue group a takes
-// the units of accumulator a.
-__global__ void __launch_bounds__(kThreads, 1)
+// One pair of CTAs per two SMs takes a contiguous range of units (row tile of 256, column tile), column tiles
+// of a row tile one after the other; the range's first unit in a row tile loads the tile's rows, the last one
+// lets go of them.  (Ranges instead of whole row tiles: 98 row tiles on 74 pairs are 1.3 rounds instead of 2.)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap wmap,
-                 const __grid_constant__ CUtensorMap ymap, const Params p)
+                 const __grid_constant__ CUtensorMap bmap, const __grid_constant__ CUtensorMap ymap, const Params p)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
     const uint32_t smem_base = ptx::smem_u32(smem);
     const int warp = ptx::warp_index(), lane = threadIdx.x & 31;
+    const uint32_t rank = ptx::cluster_rank();
 
+    // Barriers of the first CTA count both CTAs' loads (afull, wfull) and read-outs (tempty); the MMAs'
+    // completions arrive in both (aempty, wempty, tfull); constants are each CTA's own.
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + p.off_bars);
     const uint32_t bar_afull = ptx::smem_u32(bars);               // a resident chunk has landed
     const uint32_t bar_aempty = bar_afull + 8 * kMaxKc;           // ... has been read for the last time
@@ -204,107 +203,107 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(bars + kBars);
     volatile int *flags = reinterpret_cast<volatile int *>(bars + kBars + 1);     // [0] abort
 
-    const int g = blockIdx.x % p.groups;
-    const int worker = blockIdx.x / p.groups;
-    const int nworkers = gridDim.x / p.groups;
-    const int cols = p.n_ctiles / p.groups;                       // column tiles g, g + groups, ...
-    const uint32_t half = (uint32_t)p.stages >> 1;                // stages per issuing thread
-    // With 128-channel tiles the k-th unit of thread t uses slot t + 2 (k & 1) of four (accumulator,
-    // constants); with 256-channel tiles a thread has the one slot t, twice as wide.
-    const uint32_t nb = (uint32_t)p.nb, nt = nb * (uint32_t)kNt;
-    const uint32_t w_stage = nb * kStageBytes;
-    auto slot_of = [&](uint32_t t, uint32_t k) { return nb == 1u ? t + 2u * (k & 1u) : t; };
-    auto phase_of = [&](uint32_t k) { return nb == 1u ? (k >> 1) & 1u : k & 1u; };
+    const int pair = (int)blockIdx.x >> 1, pairs = (int)gridDim.x >> 1;
+    const long long units = (long long)p.n_mtiles * p.n_ctiles;
+    const long long u0 = units * pair / pairs, u1 = units * (pair + 1) / pairs;
+    const int mt0 = (int)(u0 / p.n_ctiles), ct0 = (int)(u0 % p.n_ctiles), n_units = (int)(u1 - u0);
+    const int nt = p.nb * kNt;
+    const uint32_t w_stage = (uint32_t)(nt / 2) * kChunk;
+    // columns of column tile ct that exist, in the MMA's steps of 32
+    auto width = [&](int ct) { const int left = p.cout - ct * nt; return left >= nt ? nt : (left + 31) & ~31; };
 
-    // the next call's kernel may start its set-up; it waits before it reads or writes anything
-    ptx::grid_dep_launch();
     // ---- prologue -----------------------------------------------------------------------------
     if (warp == 0) {
         if (lane < kMaxKc) {
             ptx::mbar_init(bar_afull + 8 * lane, 1);
-            // the last unit of each issuing thread in a row tile lets go of the chunk
-            ptx::mbar_init(bar_aempty + 8 * lane, cols >= 2 ? 2 : 1);
+            ptx::mbar_init(bar_aempty + 8 * lane, 1);
         } else if (lane < kMaxKc + kMaxStages) {
             ptx::mbar_init(bar_wfull + 8 * (lane - kMaxKc), 1);
             ptx::mbar_init(bar_wempty + 8 * (lane - kMaxKc), 1);
         } else if (lane < kMaxKc + kMaxStages + kAccs) {
             const int b = lane - kMaxKc - kMaxStages;
             ptx::mbar_init(bar_tfull + 8 * b, 1);
-            ptx::mbar_init(bar_tempty + 8 * b, 4 * p.nb);      // the warps that read the slot
+            ptx::mbar_init(bar_tempty + 8 * b, 2 * kEpiWarps);
             ptx::mbar_init(bar_cfull + 8 * b, 1);
-            ptx::mbar_init(bar_cempty + 8 * b, 4 * p.nb);
+            ptx::mbar_init(bar_cempty + 8 * b, kEpiWarps);
         } else if (lane == 31) {
-            ptx::mbar_init(bar_drain, 2);
+            ptx::mbar_init(bar_drain, 1);
             flags[0] = 0;
             ptx::tma_prefetch_desc(&xmap);
             ptx::tma_prefetch_desc(&wmap);
+            ptx::tma_prefetch_desc(&bmap);
             ptx::tma_prefetch_desc(&ymap);
         }
         ptx::mbar_init_fence();
     }
-    if (warp == 1) ptx::tmem_alloc(ptx::smem_u32((const void *)tmem_slot), 128u * kAccs);
+    if (warp == 1) ptx::tmem_alloc_pair(ptx::smem_u32((const void *)tmem_slot), 512u);
     tc::build_aconst(smem + p.off_aconst, (int)threadIdx.x, kThreads);
     ptx::fence_proxy_async_smem();
     ptx::tc_fence_before_sync();
     __syncthreads();
+    ptx::cluster_sync();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
+    // The next call's kernel may start its set-up; it waits before it reads or writes anything.  (Not before the
+    // tensor memory is held, which that kernel may want too.)
+    ptx::grid_dep_launch();
 
     if (warp == 0) {
         // ---- producer -----------------------------------------------------------------------------
-        // Per pair of column tiles (one for each issuing thread): their constants, then chunk by
-        // chunk {the row tile's chunk for the first pair of a row tile, the chunk of either tile's
-        // weights into its thread's half of the ring}, then the two tiles' bias digits.
+        // Per unit: its constants, then chunk by chunk {this CTA's rows for the first unit of a row tile, its
+        // half of the column tile's weights}, then its half of the bias digits.
         {
             const bool leader = ptx::elect_one();
             ptx::grid_dep_wait();           // for wide_prep_kernel, which waited for what wrote x
-            uint32_t hs[2] = {0u, 0u}, hph[2] = {0u, 0u}, k[2] = {0u, 0u}, aph = 0;
+            const uint32_t afull = ptx::map_to_rank(bar_afull, 0), wfull = ptx::map_to_rank(bar_wfull, 0);
+            uint32_t st = 0, ph = 0, aph = 0;
+            int mt = mt0, ct = ct0;
             bool ok = true;
-            // next stage of thread t's half ring, armed for tx bytes; 0 when a wait gave up
-            auto w_slot = [&](int t, uint32_t tx, uint32_t &bar) -> uint32_t {
-                const uint32_t st = 2u * hs[t] + (uint32_t)t;
-                if (!tc::wait_bar_warp(bar_wempty + 8 * st, hph[t] ^ 1u, flags)) { ok = false; return 0u; }
-                bar = bar_wfull + 8 * st;
-                if (leader) ptx::mbar_expect_tx(bar, tx);
-                if (++hs[t] == half) { hs[t] = 0; hph[t] ^= 1u; }
-                return smem_base + p.off_w + st * w_stage;
+            // the ring's next stage, armed for both CTAs' loads
+            auto next_stage = [&](uint32_t tx, uint32_t &bar) -> uint32_t {
+                if (!tc::wait_bar_warp(bar_wempty + 8 * st, ph ^ 1u, flags)) { ok = false; return 0u; }
+                if (leader && rank == 0) ptx::mbar_expect_tx(bar_wfull + 8 * st, 2u * tx);
+                bar = wfull + 8 * st;
+                const uint32_t dst = smem_base + p.off_w + st * w_stage;
+                if (++st == (uint32_t)p.stages) { st = 0; ph ^= 1u; }
+                return dst;
             };
-            for (int mt = worker; mt < p.n_mtiles && ok; mt += nworkers, aph ^= 1u) {
-                for (int lc0 = 0; lc0 < cols && ok; lc0 += 2) {
-                    const int nu = lc0 + 1 < cols ? 2 : 1;
-                    int ct[2];
-                    for (int t = 0; t < nu && ok; ++t) {
-                        ct[t] = g + (lc0 + t) * p.groups;
-                        const uint32_t slot = slot_of((uint32_t)t, k[t]);
-                        if (!tc::wait_bar_warp(bar_cempty + 8 * slot, phase_of(k[t]) ^ 1u, flags)) { ok = false; break; }
-                        if (leader) {
-                            ptx::mbar_expect_tx(bar_cfull + 8 * slot, nb * kConstBytes);
-                            ptx::bulk_load(smem_base + p.off_const + slot * nb * kConstBytes,
-                                           p.consts + (size_t)ct[t] * nb * kConstBytes, nb * kConstBytes, bar_cfull + 8 * slot);
-                        }
-                        ++k[t];
-                    }
-                    for (int c = 0; c < p.kc && ok; ++c) {
-                        if (lc0 == 0) {
-                            if (!tc::wait_bar_warp(bar_aempty + 8 * c, aph ^ 1u, flags)) { ok = false; break; }
-                            if (leader) {
-                                ptx::mbar_expect_tx(bar_afull + 8 * c, kStageBytes);
-                                ptx::tma_load_2d(smem_base + c * kStageBytes, &xmap, c * kChunk, mt * 128, bar_afull + 8 * c);
-                            }
-                        }
-                        for (int t = 0; t < nu && ok; ++t) {
-                            uint32_t bar = 0;
-                            const uint32_t dst = w_slot(t, w_stage, bar);
-                            if (ok && leader) ptx::tma_load_2d(dst, &wmap, c * kChunk, ct[t] * (int)nt, bar);
-                        }
-                    }
-                    for (int t = 0; t < nu && ok; ++t) {
-                        uint32_t bar = 0;
-                        const uint32_t dst = w_slot(t, nb * kWbiasBytes, bar);
-                        if (ok && leader) ptx::bulk_load(dst, p.wbias + (size_t)ct[t] * nb * kWbiasBytes, nb * kWbiasBytes, bar);
-                    }
+            for (int k = 0; k < n_units && ok; ++k) {
+                const uint32_t slot = (uint32_t)k & 1u;
+                const int w_row = ct * nt + (int)rank * (width(ct) / 2);
+                const bool first = k == 0 || ct == 0;
+                if (!tc::wait_bar_warp(bar_cempty + 8 * slot, (((uint32_t)k >> 1) & 1u) ^ 1u, flags)) { ok = false; break; }
+                if (leader) {
+                    const uint32_t bytes = (uint32_t)p.nb * kConstBytes;
+                    ptx::mbar_expect_tx(bar_cfull + 8 * slot, bytes);
+                    ptx::bulk_load(smem_base + p.off_const + slot * bytes, p.consts + (size_t)ct * bytes, bytes, bar_cfull + 8 * slot);
                 }
+                for (int c = 0; c < p.kc && ok; ++c) {
+                    if (first) {
+                        if (!tc::wait_bar_warp(bar_aempty + 8 * c, aph ^ 1u, flags)) { ok = false; break; }
+                        if (leader) {
+                            if (rank == 0) ptx::mbar_expect_tx(bar_afull + 8 * c, 2u * kAChunkBytes);
+                            ptx::tma_load_2d_pair(smem_base + c * kAChunkBytes, &xmap, c * kChunk, mt * 256 + (int)rank * 128, afull + 8 * c);
+                        }
+                    }
+                    uint32_t bar = 0;
+                    const uint32_t dst = next_stage(w_stage, bar);
+                    if (ok && leader) ptx::tma_load_2d_pair(dst, &wmap, c * kChunk, w_row, bar);
+                }
+                if (ok) {
+                    uint32_t bar = 0;
+                    const uint32_t dst = next_stage((uint32_t)(nt / 2) * 32u, bar);
+                    if (ok && leader) ptx::tma_load_2d_pair(dst, &bmap, 0, w_row, bar);
+                }
+                if (first) aph ^= 1u;
+                if (++ct == p.n_ctiles) { ct = 0; ++mt; }
             }
+            // The completions of the last MMAs must have arrived here before the CTA may go away.
+            for (int s = 0; s < p.stages && ok; ++s) {
+                ok = tc::wait_bar_warp(bar_wempty + 8 * st, ph ^ 1u, flags);
+                if (++st == (uint32_t)p.stages) { st = 0; ph ^= 1u; }
+            }
+            for (int c = 0; c < p.kc && ok; ++c) ok = tc::wait_bar_warp(bar_aempty + 8 * c, aph ^ 1u, flags);
             if (!ok) {
                 // let the copies in flight land before the CTA goes away
                 const unsigned long long t0 = ptx::globaltimer();
@@ -312,131 +311,135 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
             }
         }
         __syncwarp();
-    } else if (warp == 1 || warp == kIssuer2) {
-        // ---- MMA issuers ------------------------------------------------------------------------------
+    } else if (warp == 1) {
+        // ---- MMA issuer: the first CTA's, for both --------------------------------------------------
         // (the whole warp, one lane issues: descriptors then stay in uniform registers)
-        {
+        if (rank == 0) {
             const bool leader = ptx::elect_one();
-            const uint32_t t = warp == 1 ? 0u : 1u;
-            // s8 x s8 -> s32, both K-major, M = 128, N = 128 or 256
-            const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((nt >> 3) << 17) | ((128u >> 4) << 24);
             const uint64_t d_128 = tc::smem_desc(0u, 128u), d_32 = tc::smem_desc(0u, 32u);
             const uint64_t ac_desc = d_32 | (uint64_t)((smem_base + p.off_aconst) >> 4);
             const uint32_t a_lo0 = smem_base >> 4, w_lo0 = (smem_base + p.off_w) >> 4;
-            const uint32_t a_step = kStageBytes >> 4, w_step = w_stage >> 4;
-            uint32_t hs = 0, hph = 0, k = 0, aph = 0;
+            const uint32_t a_step = kAChunkBytes >> 4, w_step = w_stage >> 4;
+            uint32_t st = 0, ph = 0, aph = 0;
+            int ct = ct0, k = 0;
             bool ok = true;
-            for (int mt = worker; mt < p.n_mtiles && ok; mt += nworkers, aph ^= 1u) {
-                for (int lc = (int)t; lc < cols && ok; lc += 2, ++k) {
-                    const uint32_t acc = slot_of(t, k);
-                    if (!tc::wait_bar_warp(bar_tempty + 8 * acc, phase_of(k) ^ 1u, flags)) { ok = false; break; }
+            for (; k < n_units && ok; ++k) {
+                const uint32_t acc = (uint32_t)k & 1u;
+                // s8 x s8 -> s32, both K-major, M = 256
+                const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | (((uint32_t)width(ct) >> 3) << 17) | ((256u >> 4) << 24);
+                if (!tc::wait_bar_warp(bar_tempty + 8 * acc, (((uint32_t)k >> 1) & 1u) ^ 1u, flags)) { ok = false; break; }
+                ptx::tc_fence_after_sync();
+                const uint32_t d_tmem = tmem_base + acc * 256u;
+                const bool first = k == 0 || ct == 0, last = k + 1 == n_units || ct + 1 == p.n_ctiles;     // of the row tile
+                for (int c = 0; c < p.kc; ++c) {
+                    if (first && !tc::wait_bar_warp(bar_afull + 8 * c, aph, flags)) { ok = false; break; }
+                    if (!tc::wait_bar_warp(bar_wfull + 8 * st, ph, flags)) { ok = false; break; }
                     ptx::tc_fence_after_sync();
-                    const uint32_t d_tmem = tmem_base + acc * nt;
-                    const bool first = lc == (int)t, last = lc + 2 >= cols;     // of this thread in the row tile
-                    for (int c = 0; c < p.kc; ++c) {
-                        const uint32_t st = 2u * hs + t;
-                        if (first && !tc::wait_bar_warp(bar_afull + 8 * c, aph, flags)) { ok = false; break; }
-                        if (!tc::wait_bar_warp(bar_wfull + 8 * st, hph, flags)) { ok = false; break; }
-                        ptx::tc_fence_after_sync();
-                        const uint32_t a_lo = a_lo0 + (uint32_t)c * a_step, w_lo = w_lo0 + st * w_step;
-                        const int nks = c == p.kc - 1 ? p.ksteps_last : 4;
-                        if (leader) {
-                            if (c == 0) ptx::mma_i8<false>(d_tmem, d_128 | (uint64_t)a_lo, d_128 | (uint64_t)w_lo, idesc);
-                            else ptx::mma_i8<true>(d_tmem, d_128 | (uint64_t)a_lo, d_128 | (uint64_t)w_lo, idesc);
-#pragma unroll
-                            for (int ks = 1; ks < 4; ++ks)
-                                if (ks < nks)
-                                    ptx::mma_i8<true>(d_tmem, d_128 | (uint64_t)(a_lo + 2 * ks), d_128 | (uint64_t)(w_lo + 2 * ks), idesc);
-                            ptx::mma_commit(bar_wempty + 8 * st);
-                            if (last) ptx::mma_commit(bar_aempty + 8 * c);
-                        }
-                        if (++hs == half) { hs = 0; hph ^= 1u; }
-                    }
-                    if (!ok) break;
-                    // the bias step: the constant block of 1s and 127s against the tile's digits
-                    const uint32_t st = 2u * hs + t;
-                    if (!tc::wait_bar_warp(bar_wfull + 8 * st, hph, flags)) { ok = false; break; }
-                    ptx::tc_fence_after_sync();
+                    const uint32_t a_lo = a_lo0 + (uint32_t)c * a_step, w_lo = w_lo0 + st * w_step;
+                    const int nks = c == p.kc - 1 ? p.ksteps_last : 4;
                     if (leader) {
-                        ptx::mma_i8<true>(d_tmem, ac_desc, d_32 | (uint64_t)(w_lo0 + st * w_step), idesc);
-                        ptx::mma_commit(bar_wempty + 8 * st);
-                        ptx::mma_commit(bar_tfull + 8 * acc);
+                        if (c == 0) ptx::mma_i8_pair<false>(d_tmem, d_128 | (uint64_t)a_lo, d_128 | (uint64_t)w_lo, idesc);
+                        else ptx::mma_i8_pair<true>(d_tmem, d_128 | (uint64_t)a_lo, d_128 | (uint64_t)w_lo, idesc);
+#pragma unroll
+                        for (int ks = 1; ks < 4; ++ks)
+                            if (ks < nks)
+                                ptx::mma_i8_pair<true>(d_tmem, d_128 | (uint64_t)(a_lo + 2 * ks), d_128 | (uint64_t)(w_lo + 2 * ks), idesc);
+                        ptx::mma_commit_pair(bar_wempty + 8 * st);
+                        if (last) ptx::mma_commit_pair(bar_aempty + 8 * c);
                     }
-                    if (++hs == half) { hs = 0; hph ^= 1u; }
+                    if (++st == (uint32_t)p.stages) { st = 0; ph ^= 1u; }
                 }
+                if (!ok) break;
+                // the bias step: the constant block of 1s and 127s against the tile's digits
+                if (!tc::wait_bar_warp(bar_wfull + 8 * st, ph, flags)) { ok = false; break; }
+                ptx::tc_fence_after_sync();
+                if (leader) {
+                    ptx::mma_i8_pair<true>(d_tmem, ac_desc, d_32 | (uint64_t)(w_lo0 + st * w_step), idesc);
+                    ptx::mma_commit_pair(bar_wempty + 8 * st);
+                    ptx::mma_commit_pair(bar_tfull + 8 * acc);
+                }
+                if (++st == (uint32_t)p.stages) { st = 0; ph ^= 1u; }
+                if (first) aph ^= 1u;
+                if (++ct == p.n_ctiles) ct = 0;
             }
-            if (leader) ptx::mma_commit(bar_drain);
+            // the second CTA's read-outs arrive here
+            for (int e = 0; e < 2 && ok; ++e, ++k)
+                ok = tc::wait_bar_warp(bar_tempty + 8 * ((uint32_t)k & 1u), (((uint32_t)k >> 1) & 1u) ^ 1u, flags);
+            // nothing of the pair's MMAs is outstanding (the second CTA learns of it at the teardown)
+            if (leader) ptx::mma_commit_own(bar_drain);
             const unsigned long long t0 = ptx::globaltimer();
             while (!ptx::mbar_try_wait(bar_drain, 0) && ptx::globaltimer() - t0 < tc::kWaitLimitNs) {}
         }
+        __syncwarp();
     } else {
         // ---- epilogue ---------------------------------------------------------------------------------
-        // Group grp follows issuing thread grp & 1.  With 128-channel tiles it takes that thread's
-        // units with k & 1 == grp >> 1 (slot grp); with 256-channel tiles it takes every unit of the
-        // thread and the half grp >> 1 of its 256 columns.
+        // Four groups of four warps: group grp takes the pieces grp, grp + 4 of 32 columns of every unit.
         const int q = warp & 3, grp = (warp - 2) >> 2;
-        const int t = grp & 1, h = grp >> 1;
         uint8_t *slab = smem + p.off_out + (size_t)(warp - 2) * kSlabBytes;
         uint8_t *my_row = slab + lane * kEpiCols;
         const uint32_t slab_addr = ptx::smem_u32(slab);
         const uint32_t t_lane = tmem_base + ((uint32_t)(q * 32) << 16);
-        const uint32_t acc = nb == 1u ? (uint32_t)grp : (uint32_t)t;          // slot: barriers, accumulator
-        const uint32_t blk = nb == 1u ? (uint32_t)grp : 2u * (uint32_t)t + (uint32_t)h;   // 128-column block of constants
-        const uint32_t tcol = blk * 128u;                                       // its accumulator columns
-        const int col_in_tile = nb == 1u ? 0 : h * kNt;
-        const uint8_t *cst = smem + p.off_const + blk * kConstBytes;
-        const int *cm = reinterpret_cast<const int *>(cst);
-        const int2 *cbs = reinterpret_cast<const int2 *>(cst + kNt * 4);
-        const int *hdr = reinterpret_cast<const int *>(cst + kNt * 12);
-        uint32_t k = 0;
-        bool ok = true;
-        for (int mt = worker; mt < p.n_mtiles && ok; mt += nworkers) {
-            const int row0 = mt * 128 + q * 32;
-            for (int lc = t; lc < cols && ok; lc += 2, ++k) {
-                if (nb == 1u && (int)(k & 1u) != h) continue;
-                const int col0 = (g + lc * p.groups) * (int)nt + col_in_tile;
-                const uint32_t ph = phase_of(k);
-                if (!tc::wait_bar<true>(bar_cfull + 8 * acc, ph, flags)) { ok = false; break; }
-                if (!tc::wait_bar<true>(bar_tfull + 8 * acc, ph, flags)) { ok = false; break; }
-                ptx::tc_fence_after_sync();
-                const int shmax = hdr[0];
-                const bool fast = hdr[1] != 0, bad = hdr[2] != 0;
-#pragma unroll 1
-                for (int pc = 0; pc < kNt / (int)kEpiCols; ++pc) {
-                    const int col = col0 + pc * (int)kEpiCols;
-                    const uint32_t rel = pc == kNt / (int)kEpiCols - 1 ? bar_tempty + 8 * acc : 0u;
-                    if (col >= p.cout || bad) {                 // nothing of this piece exists
-                        tc::release_acc(rel);
-                        continue;
-                    }
-                    // the previous store has read the slab
-                    ptx::bulk_wait_read0();
-                    __syncwarp();
-                    const uint32_t taddr = t_lane + tcol + pc * kEpiCols;
-                    if (fast) tc::epi_fast_fixed<32>(taddr, cm + pc * kEpiCols, shmax, my_row, rel);
-                    else tc::epi_exact_subtile<32>(32, p.act_min, p.act_max, taddr, cm + pc * kEpiCols,
-                                                   cbs + pc * kEpiCols, my_row, rel);
-                    ptx::fence_proxy_async_smem();
-                    __syncwarp();
-                    if (lane == 0 && row0 < p.m) {
-                        ptx::tma_store_2d(&ymap, col, row0, slab_addr);
-                        ptx::bulk_commit();
-                    }
-                }
-                // the unit's constants are free for this group's next unit
+        const uint32_t tempty = ptx::map_to_rank(bar_tempty, 0);
+        int mt = mt0, ct = ct0;
+        for (int k = 0; k < n_units; ++k) {
+            const uint32_t acc = (uint32_t)k & 1u, ph = ((uint32_t)k >> 1) & 1u;
+            const int row0 = mt * 256 + (int)rank * 128 + q * 32, pieces = width(ct) / (int)kEpiCols;
+            if (!tc::wait_bar<true>(bar_cfull + 8 * acc, ph, flags)) break;
+            if (!tc::wait_bar<true>(bar_tfull + 8 * acc, ph, flags)) break;
+            ptx::tc_fence_after_sync();
+            // the accumulator is free for the MMAs once every warp has read its last piece
+            auto release = [&] {
+                ptx::tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(bar_cempty + 8 * acc);
+                if (lane == 0) ptx::mbar_arrive_cluster(tempty + 8 * acc);
+            };
+            if (grp >= pieces) release();
+#pragma unroll 1
+            for (int pc = grp; pc < pieces; pc += 4) {
+                const int at = pc * (int)kEpiCols;
+                const uint8_t *cst = smem + p.off_const + (acc * (uint32_t)p.nb + (uint32_t)(at / kNt)) * kConstBytes;
+                const int *cm = reinterpret_cast<const int *>(cst) + (at & (kNt - 1));
+                const int2 *cbs = reinterpret_cast<const int2 *>(cst + kNt * 4) + (at & (kNt - 1));
+                const int *hdr = reinterpret_cast<const int *>(cst + kNt * 12);
+                const int shmax = hdr[0];
+                const bool fast = hdr[1] != 0, bad = hdr[2] != 0, last = pc + 4 >= pieces;
+                const uint32_t taddr = t_lane + acc * 256u + (uint32_t)at;
+                // the previous store has read the slab
+                ptx::bulk_wait_read0();
+                __syncwarp();
+                if (fast) {
+                    uint32_t v[32];
+                    ptx::tmem_ld_x32(taddr, v);
+                    ptx::tmem_wait_ld();
+                    if (last) release();
+                    tc::fast_piece<32, false>(v, cm, 1ll << (32 + shmax), shmax, my_row, true);
+                } else {
+                    if (!bad) tc::epi_exact_subtile<32>(32, p.act_min, p.act_max, taddr, cm, cbs, my_row, 0u);
+                    if (last) release();
+                }
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0 && row0 < p.m && !bad) {
+                    ptx::tma_store_2d(&ymap, ct * nt + at, row0, slab_addr);
+                    ptx::bulk_commit();
+                }
             }
+            // the unit's constants are free for the unit after next
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive(bar_cempty + 8 * acc);
+            if (++ct == p.n_ctiles) { ct = 0; ++mt; }
         }
         ptx::bulk_wait_read0();
     }
 
     // ---- teardown ---------------------------------------------------------------------------------
+    // (neither CTA may go while the other can still reach its shared memory)
     ptx::tc_fence_before_sync();
     __syncthreads();
+    ptx::cluster_sync();
     if (warp == 1) {
         ptx::tc_fence_after_sync();
-        ptx::tmem_dealloc(tmem_base, 128u * kAccs);
+        ptx::tmem_dealloc_pair(tmem_base, 512u);
     }
 }
 
