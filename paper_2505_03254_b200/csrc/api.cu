@@ -738,14 +738,18 @@ static bool wide_plan(const Conv &c, const DeviceInfo &d, WidePlan &pl, bool &wo
     if (pairs > (long long)p.n_mtiles * p.n_ctiles) pairs = (long long)p.n_mtiles * p.n_ctiles;
     pl.grid = (int)(2 * pairs);
     p.act_min = c.rq.act_min; p.act_max = c.rq.act_max;
-    // Measured on B200, time as a share of the weight-resident kernel's: from Cin = 640 on it is the faster one
-    // where the column tiles are nearly full (802816 rows: 960 -> 1280 0.64, 960 -> 512 0.62, 768 -> 768 0.81,
-    // 640 -> 256 0.78; 25088 rows: 960 -> 512 0.80, 640 -> 1280 0.99), but 960 -> 320 1.06 and 640 -> 320 1.26
-    // (a sixth of its columns is padding), 512 -> 512 1.19, 384 -> 960 1.08.  Its one-multiply epilogue
-    // is for the clamp [0, 127].
-    const bool full_cols = 10 * c.cout > 9 * p.n_ctiles * nb * wide::kNt;
-    worth = c.cin >= 640 && c.cout >= 256 && (full_cols || c.cout >= 640) && c.m > 128ll * (d.sms - 1) &&
-            c.rq.act_min == 0 && c.rq.act_max == 127;
+    // Measured on B200, time as a share of the weight-resident kernel's (rows: 12544 / 50176 / 401408):
+    //   Cin 576, Cout 256: 0.88 0.79 0.86, 512: 1.01 0.78 0.76, 1280: 0.89 0.80 0.74; linear layers alike
+    //   Cin 640, Cout 320: 1.10 1.02 1.25 (a column tile and a quarter), from Cin 768 on 1.06 0.96 0.92
+    //   Cin 960, Cout 144: 0.85 0.88 0.65, 160: 0.82 0.84 0.96, but 96: 0.87 0.91 1.22; 512: 0.80 0.66 0.55
+    //   Cin 512, Cout 512: 1.02 0.88 1.2, 1280: 0.85 0.96 1.1
+    // and on 6272 rows Cin 672, Cout 256: 0.94, 512: 0.81, 1280: 0.86, but Cin 576: 1.01 0.88 0.94; on 3136 rows
+    // 1.14 0.95 0.97.  Its one-multiply epilogue is for the clamps [0, 127] and [-128, 127].
+    const bool tiles_full = c.cout >= 240 && (c.cout <= 256 || c.cout >= 480 || c.cin >= 768);
+    const long long rows_per_sm = c.m / d.sms;
+    worth = ((c.cin >= 576 && tiles_full && rows_per_sm >= 80) || (c.cin >= 672 && tiles_full && rows_per_sm >= 40) ||
+             (c.cin >= 960 && c.cout >= 144 && rows_per_sm >= 80)) &&
+            (c.rq.act_min == 0 || c.rq.act_min == -128) && c.rq.act_max == 127;
     return true;
 }
 
@@ -765,7 +769,7 @@ static prom_status launch_wide(const Conv &c, const DeviceInfo &d, WidePlan &pl)
     memset(&pp, 0, sizeof(pp));
     pp.cin = c.cin; pp.cout = c.cout; pp.k_pad = pl.k_pad; pp.w_packed = c.w;
     pp.bias = c.rq.bias; pp.mult = c.rq.mult; pp.shift = c.rq.shift;
-    pp.act_min = c.rq.act_min; pp.act_max = c.rq.act_max;
+    pp.act_min = c.rq.act_min; pp.act_max = c.rq.act_max; pp.signed_fast = 1;
     pp.w8 = reinterpret_cast<int8_t *>(scratch); pp.wbias = scratch + w8_bytes; pp.consts = scratch + w8_bytes + wb_bytes;
     p.consts = pp.consts;
     CUtensorMap xmap, wmap, bmap, ymap;

@@ -62,6 +62,7 @@ struct PrepParams {
     const int32_t *bias, *mult;
     const int8_t *shift;
     int act_min, act_max;
+    int signed_fast;            // the reader of the constants has the one-multiply form for [-128, 127] too
     int8_t *w8;                 // [n_ctiles * 128][k_pad]
     uint8_t *wbias, *consts;
 };
@@ -93,7 +94,7 @@ __device__ __forceinline__ void prep_tile(const PrepParams &p, const int tile, c
     __syncthreads();
     const int shmax = s_flags[1];
     const bool bad = s_flags[2] != 0;
-    const bool fast = !bad && s_flags[3] == 0 && p.act_min == 0 && p.act_max == 127 && shmax - s_flags[0] <= 4 &&
+    const bool fast = !bad && s_flags[3] == 0 && (p.act_min == 0 || (p.signed_fast && p.act_min == -128)) && p.act_max == 127 && shmax - s_flags[0] <= 4 &&
                       shmax <= 24 && s_flags[0] <= shmax;
     if (bad && threadIdx.x == 0) raise_status(PROM_ERR_BAD_REQUANT);
 
@@ -412,7 +413,8 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
                     ptx::tmem_ld_x32(taddr, v);
                     ptx::tmem_wait_ld();
                     if (last) release();
-                    tc::fast_piece<32, false>(v, cm, 1ll << (32 + shmax), shmax, my_row, true);
+                    if (p.act_min == 0) tc::fast_piece<32, false>(v, cm, 1ll << (32 + shmax), shmax, my_row, true);
+                    else tc::fast_piece<32, true>(v, cm, 1ll << (32 + shmax), shmax, my_row, true);
                 } else {
                     if (!bad) tc::epi_exact_subtile<32>(32, p.act_min, p.act_max, taddr, cm, cbs, my_row, 0u);
                     if (last) release();

@@ -1,0 +1,30 @@
+"""The row-resident kernel over pairs of CTAs: row counts around its 256-row tiles (a second CTA with no rows, one
+row, all but one), last column tiles of 32 to 256 columns, one and several units per pair, K up to its limit, and
+the one-multiply epilogue for both clamps beside the 64-bit one."""
+import numpy as np
+import pytest
+
+from paper_2505_03254_b200 import binding
+from gpu_util import first_mismatch, make_case, run_variant, to_device
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("lo,hi", [(0, 127), (-128, 127), (-7, 100)])
+@pytest.mark.parametrize("m,cin,cout", [(1, 128, 64), (127, 640, 288), (128, 960, 272), (129, 576, 496), (255, 1024, 512),
+                                        (257, 720, 240), (4999, 1024, 1280), (20225, 592, 336), (37889, 960, 144)])
+def test_tiles_and_clamps(oracle, m, cin, cout, lo, hi):
+    x, lay = make_case(m + cin + cout, m, cin, cout, 0.5, act="i8")
+    xd, wp, consts = to_device(x, lay)
+    binding.debug_tc_wide(2)
+    try:
+        y = run_variant(xd, wp, consts, cout, "tc", lo, hi)
+    finally:
+        binding.debug_tc_wide(0)
+    assert binding.last_device_status() == binding.PROM_OK
+    rows = np.unique(np.r_[0:min(m, 300), m // 2:min(m, m // 2 + 300), max(0, m - 300):m])
+    want = oracle.conv_mul(x.numpy()[rows], lay["w"].numpy(), lay["bias"].numpy(), lay["mult"].numpy(), lay["shift"].numpy(), lo, hi)
+    assert first_mismatch(np.asarray(y)[rows], want) is None
+    # the rest against the plain kernel
+    naive = run_variant(xd, wp, consts, cout, "naive", lo, hi)
+    assert np.array_equal(np.asarray(y), np.asarray(naive))
