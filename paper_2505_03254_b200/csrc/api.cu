@@ -718,7 +718,7 @@ static bool wide_plan(const Conv &c, const DeviceInfo &d, WidePlan &pl, bool &wo
     const int nb = forced ? forced : 2;
     p.nb = nb;
     // shared memory: resident chunks, weight ring, constants, staging slabs, the bias step's A block, barriers
-    const uint32_t a_bytes = (uint32_t)p.kc * wide::kAChunkBytes, w_stage = (uint32_t)nb * (wide::kNt / 2) * wide::kChunk;
+    const uint32_t a_bytes = (uint32_t)wide::kASlots * wide::kAChunkBytes, w_stage = (uint32_t)nb * (wide::kNt / 2) * wide::kChunk;
     const uint32_t const_bytes = ((uint32_t)(wide::kAccs * nb) * wide::kConstBytes + 1023u) & ~1023u;
     const uint32_t fixed = const_bytes + wide::kEpiWarps * wide::kSlabBytes + tc::kAConstBytes + 1024;
     const long long room = (long long)d.smem_optin - 1024 - a_bytes - fixed;

@@ -20,7 +20,11 @@
 // tensor map (128-byte swizzle, like the activations), the bias digits as the last "chunk" of a
 // column tile, and the constants into a small ring of their own.
 //
-// Warp 0 of each CTA issues its loads, warp 1 of the first CTA the MMAs of both, warps 2..17 requantise the
+// Warp 0 of each CTA loads its weights, warp 18 its rows and constants, each waiting only for room of its own (one
+// loader for all three held the weights back until the constants of the unit before last had been read, which put
+// half of every read-out on the MMAs' path).  The chunks of rows go through a ring of eight, so that with K of less
+// than eight chunks the next tile's first ones are there before this tile's last unit has ended.
+// Warp 1 of the first CTA issues the MMAs of both, warps 2..17 requantise the
 // CTA's own 128 rows, 32 columns at a time, and store through the output's tensor map (rows and columns outside
 // the matrix are not written).
 #pragma once
@@ -30,10 +34,12 @@
 namespace prom { namespace wide {
 
 constexpr int kEpiWarps = 16;                     // four groups of four
-constexpr int kThreads = 32 * (2 + kEpiWarps);    // loader, MMA issuer, epilogue warps
+constexpr int kLoader2 = 2 + kEpiWarps;           // warp of the second loader
+constexpr int kThreads = 32 * (kLoader2 + 1);     // weight loader, MMA issuer, epilogue warps, loader of rows and constants
 constexpr int kNt = 128;                          // channels of a block of constants
 constexpr int kChunk = 128;                       // bytes of K per chunk = swizzle span
 constexpr int kMaxKc = 8;                         // resident K chunks: Cin <= 1024
+constexpr int kASlots = kMaxKc;                   // their ring (a power of two)
 constexpr int kMaxStages = 8;
 constexpr int kAccs = 2;                          // accumulators of up to 256 columns
 constexpr uint32_t kAChunkBytes = 128 * kChunk;   // one resident chunk of a CTA's 128 rows
@@ -42,7 +48,7 @@ constexpr uint32_t kWbiasBytes = kNt * 32;        // bias digits of a block (32-
 constexpr uint32_t kConstBytes = kNt * 4 + kNt * 8 + 16 + 112;
 constexpr uint32_t kEpiCols = 32;                 // columns an epilogue warp stages per store
 constexpr uint32_t kSlabBytes = 32 * kEpiCols;
-constexpr int kBars = 2 * kMaxKc + 2 * kMaxStages + 4 * kAccs + 1;
+constexpr int kBars = 2 * kASlots + 2 * kMaxStages + 4 * kAccs + 1;
 
 struct Params {
     long long m;
@@ -193,8 +199,8 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
     // completions arrive in both (aempty, wempty, tfull); constants are each CTA's own.
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + p.off_bars);
     const uint32_t bar_afull = ptx::smem_u32(bars);               // a resident chunk has landed
-    const uint32_t bar_aempty = bar_afull + 8 * kMaxKc;           // ... has been read for the last time
-    const uint32_t bar_wfull = bar_aempty + 8 * kMaxKc;           // weight ring
+    const uint32_t bar_aempty = bar_afull + 8 * kASlots;           // ... has been read for the last time
+    const uint32_t bar_wfull = bar_aempty + 8 * kASlots;           // weight ring
     const uint32_t bar_wempty = bar_wfull + 8 * kMaxStages;
     const uint32_t bar_tfull = bar_wempty + 8 * kMaxStages;       // accumulators
     const uint32_t bar_tempty = bar_tfull + 8 * kAccs;
@@ -215,14 +221,14 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
 
     // ---- prologue -----------------------------------------------------------------------------
     if (warp == 0) {
-        if (lane < kMaxKc) {
+        if (lane < kASlots) {
             ptx::mbar_init(bar_afull + 8 * lane, 1);
             ptx::mbar_init(bar_aempty + 8 * lane, 1);
-        } else if (lane < kMaxKc + kMaxStages) {
-            ptx::mbar_init(bar_wfull + 8 * (lane - kMaxKc), 1);
-            ptx::mbar_init(bar_wempty + 8 * (lane - kMaxKc), 1);
-        } else if (lane < kMaxKc + kMaxStages + kAccs) {
-            const int b = lane - kMaxKc - kMaxStages;
+        } else if (lane < kASlots + kMaxStages) {
+            ptx::mbar_init(bar_wfull + 8 * (lane - kASlots), 1);
+            ptx::mbar_init(bar_wempty + 8 * (lane - kASlots), 1);
+        } else if (lane < kASlots + kMaxStages + kAccs) {
+            const int b = lane - kASlots - kMaxStages;
             ptx::mbar_init(bar_tfull + 8 * b, 1);
             ptx::mbar_init(bar_tempty + 8 * b, 2 * kEpiWarps);
             ptx::mbar_init(bar_cfull + 8 * b, 1);
@@ -250,15 +256,14 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
     ptx::grid_dep_launch();
 
     if (warp == 0) {
-        // ---- producer -----------------------------------------------------------------------------
-        // Per unit: its constants, then chunk by chunk {this CTA's rows for the first unit of a row tile, its
-        // half of the column tile's weights}, then its half of the bias digits.
+        // ---- loader of weights ----------------------------------------------------------------------
+        // Per unit this CTA's half of the column tile's weights, chunk by chunk, then of the bias digits.
         {
             const bool leader = ptx::elect_one();
             ptx::grid_dep_wait();           // for wide_prep_kernel, which waited for what wrote x
-            const uint32_t afull = ptx::map_to_rank(bar_afull, 0), wfull = ptx::map_to_rank(bar_wfull, 0);
-            uint32_t st = 0, ph = 0, aph = 0;
-            int mt = mt0, ct = ct0;
+            const uint32_t wfull = ptx::map_to_rank(bar_wfull, 0);
+            uint32_t st = 0, ph = 0;
+            int ct = ct0;
             bool ok = true;
             // the ring's next stage, armed for both CTAs' loads
             auto next_stage = [&](uint32_t tx, uint32_t &bar) -> uint32_t {
@@ -270,23 +275,8 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
                 return dst;
             };
             for (int k = 0; k < n_units && ok; ++k) {
-                const uint32_t slot = (uint32_t)k & 1u;
                 const int w_row = ct * nt + (int)rank * (width(ct) / 2);
-                const bool first = k == 0 || ct == 0;
-                if (!tc::wait_bar_warp(bar_cempty + 8 * slot, (((uint32_t)k >> 1) & 1u) ^ 1u, flags)) { ok = false; break; }
-                if (leader) {
-                    const uint32_t bytes = (uint32_t)p.nb * kConstBytes;
-                    ptx::mbar_expect_tx(bar_cfull + 8 * slot, bytes);
-                    ptx::bulk_load(smem_base + p.off_const + slot * bytes, p.consts + (size_t)ct * bytes, bytes, bar_cfull + 8 * slot);
-                }
                 for (int c = 0; c < p.kc && ok; ++c) {
-                    if (first) {
-                        if (!tc::wait_bar_warp(bar_aempty + 8 * c, aph ^ 1u, flags)) { ok = false; break; }
-                        if (leader) {
-                            if (rank == 0) ptx::mbar_expect_tx(bar_afull + 8 * c, 2u * kAChunkBytes);
-                            ptx::tma_load_2d_pair(smem_base + c * kAChunkBytes, &xmap, c * kChunk, mt * 256 + (int)rank * 128, afull + 8 * c);
-                        }
-                    }
                     uint32_t bar = 0;
                     const uint32_t dst = next_stage(w_stage, bar);
                     if (ok && leader) ptx::tma_load_2d_pair(dst, &wmap, c * kChunk, w_row, bar);
@@ -296,17 +286,54 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
                     const uint32_t dst = next_stage((uint32_t)(nt / 2) * 32u, bar);
                     if (ok && leader) ptx::tma_load_2d_pair(dst, &bmap, 0, w_row, bar);
                 }
-                if (first) aph ^= 1u;
-                if (++ct == p.n_ctiles) { ct = 0; ++mt; }
+                if (++ct == p.n_ctiles) ct = 0;
             }
             // The completions of the last MMAs must have arrived here before the CTA may go away.
             for (int s = 0; s < p.stages && ok; ++s) {
                 ok = tc::wait_bar_warp(bar_wempty + 8 * st, ph ^ 1u, flags);
                 if (++st == (uint32_t)p.stages) { st = 0; ph ^= 1u; }
             }
-            for (int c = 0; c < p.kc && ok; ++c) ok = tc::wait_bar_warp(bar_aempty + 8 * c, aph ^ 1u, flags);
             if (!ok) {
                 // let the copies in flight land before the CTA goes away
+                const unsigned long long t0 = ptx::globaltimer();
+                while (ptx::globaltimer() - t0 < 20000ull) {}
+            }
+        }
+        __syncwarp();
+    } else if (warp == kLoader2) {
+        // ---- loader of rows and constants -------------------------------------------------------------
+        // Per unit: this CTA's rows, for the first unit of a row tile, then the constants.
+        {
+            const bool leader = ptx::elect_one();
+            ptx::grid_dep_wait();
+            const uint32_t afull = ptx::map_to_rank(bar_afull, 0);
+            uint32_t n = 0;                 // chunks of rows so far
+            int mt = mt0, ct = ct0;
+            bool ok = true;
+            for (int k = 0; k < n_units && ok; ++k) {
+                if (k == 0 || ct == 0) {
+                    for (int c = 0; c < p.kc; ++c, ++n) {
+                        const uint32_t s = n % kASlots;
+                        if (!tc::wait_bar_warp(bar_aempty + 8 * s, ((n / kASlots) & 1u) ^ 1u, flags)) { ok = false; break; }
+                        if (leader) {
+                            if (rank == 0) ptx::mbar_expect_tx(bar_afull + 8 * s, 2u * kAChunkBytes);
+                            ptx::tma_load_2d_pair(smem_base + s * kAChunkBytes, &xmap, c * kChunk, mt * 256 + (int)rank * 128, afull + 8 * s);
+                        }
+                    }
+                    if (!ok) break;
+                }
+                const uint32_t slot = (uint32_t)k & 1u;
+                if (!tc::wait_bar_warp(bar_cempty + 8 * slot, (((uint32_t)k >> 1) & 1u) ^ 1u, flags)) { ok = false; break; }
+                if (leader) {
+                    const uint32_t bytes = (uint32_t)p.nb * kConstBytes;
+                    ptx::mbar_expect_tx(bar_cfull + 8 * slot, bytes);
+                    ptx::bulk_load(smem_base + p.off_const + slot * bytes, p.consts + (size_t)ct * bytes, bytes, bar_cfull + 8 * slot);
+                }
+                if (++ct == p.n_ctiles) { ct = 0; ++mt; }
+            }
+            for (int s = 0; s < kASlots && ok; ++s, ++n)
+                ok = tc::wait_bar_warp(bar_aempty + 8 * (n % kASlots), ((n / kASlots) & 1u) ^ 1u, flags);
+            if (!ok) {
                 const unsigned long long t0 = ptx::globaltimer();
                 while (ptx::globaltimer() - t0 < 20000ull) {}
             }
@@ -321,7 +348,7 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
             const uint64_t ac_desc = d_32 | (uint64_t)((smem_base + p.off_aconst) >> 4);
             const uint32_t a_lo0 = smem_base >> 4, w_lo0 = (smem_base + p.off_w) >> 4;
             const uint32_t a_step = kAChunkBytes >> 4, w_step = w_stage >> 4;
-            uint32_t st = 0, ph = 0, aph = 0;
+            uint32_t st = 0, ph = 0, n0 = 0;          // n0: chunks of rows before this row tile's
             int ct = ct0, k = 0;
             bool ok = true;
             for (; k < n_units && ok; ++k) {
@@ -333,10 +360,11 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
                 const uint32_t d_tmem = tmem_base + acc * 256u;
                 const bool first = k == 0 || ct == 0, last = k + 1 == n_units || ct + 1 == p.n_ctiles;     // of the row tile
                 for (int c = 0; c < p.kc; ++c) {
-                    if (first && !tc::wait_bar_warp(bar_afull + 8 * c, aph, flags)) { ok = false; break; }
+                    const uint32_t s = (n0 + (uint32_t)c) % kASlots;
+                    if (first && !tc::wait_bar_warp(bar_afull + 8 * s, ((n0 + (uint32_t)c) / kASlots) & 1u, flags)) { ok = false; break; }
                     if (!tc::wait_bar_warp(bar_wfull + 8 * st, ph, flags)) { ok = false; break; }
                     ptx::tc_fence_after_sync();
-                    const uint32_t a_lo = a_lo0 + (uint32_t)c * a_step, w_lo = w_lo0 + st * w_step;
+                    const uint32_t a_lo = a_lo0 + s * a_step, w_lo = w_lo0 + st * w_step;
                     const int nks = c == p.kc - 1 ? p.ksteps_last : 4;
                     if (leader) {
                         if (c == 0) ptx::mma_i8_pair<false>(d_tmem, d_128 | (uint64_t)a_lo, d_128 | (uint64_t)w_lo, idesc);
@@ -346,7 +374,7 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
                             if (ks < nks)
                                 ptx::mma_i8_pair<true>(d_tmem, d_128 | (uint64_t)(a_lo + 2 * ks), d_128 | (uint64_t)(w_lo + 2 * ks), idesc);
                         ptx::mma_commit_pair(bar_wempty + 8 * st);
-                        if (last) ptx::mma_commit_pair(bar_aempty + 8 * c);
+                        if (last) ptx::mma_commit_pair(bar_aempty + 8 * s);
                     }
                     if (++st == (uint32_t)p.stages) { st = 0; ph ^= 1u; }
                 }
@@ -360,7 +388,7 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
                     ptx::mma_commit_pair(bar_tfull + 8 * acc);
                 }
                 if (++st == (uint32_t)p.stages) { st = 0; ph ^= 1u; }
-                if (first) aph ^= 1u;
+                if (last) n0 += (uint32_t)p.kc;
                 if (++ct == p.n_ctiles) ct = 0;
             }
             // the second CTA's read-outs arrive here
