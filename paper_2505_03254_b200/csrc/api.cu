@@ -738,17 +738,18 @@ static bool wide_plan(const Conv &c, const DeviceInfo &d, WidePlan &pl, bool &wo
     if (pairs > (long long)p.n_mtiles * p.n_ctiles) pairs = (long long)p.n_mtiles * p.n_ctiles;
     pl.grid = (int)(2 * pairs);
     p.act_min = c.rq.act_min; p.act_max = c.rq.act_max;
-    // Measured on B200, time as a share of the weight-resident kernel's (rows: 12544 / 50176 / 401408):
-    //   Cin 576, Cout 256: 0.88 0.79 0.86, 512: 1.01 0.78 0.76, 1280: 0.89 0.80 0.74; linear layers alike
-    //   Cin 640, Cout 320: 1.10 1.02 1.25 (a column tile and a quarter), from Cin 768 on 1.06 0.96 0.92
-    //   Cin 960, Cout 144: 0.85 0.88 0.65, 160: 0.82 0.84 0.96, but 96: 0.87 0.91 1.22; 512: 0.80 0.66 0.55
-    //   Cin 512, Cout 512: 1.02 0.88 1.2, 1280: 0.85 0.96 1.1
-    // and on 6272 rows Cin 672, Cout 256: 0.94, 512: 0.81, 1280: 0.86, but Cin 576: 1.01 0.88 0.94; on 3136 rows
-    // 1.14 0.95 0.97.  Its one-multiply epilogue is for the clamps [0, 127] and [-128, 127].
-    const bool tiles_full = c.cout >= 240 && (c.cout <= 256 || c.cout >= 480 || c.cin >= 768);
+    // Measured on B200, time as a share of the weight-resident kernel's (rows: 12544 / 50176 / 802816):
+    //   Cin 960, Cout 1280: 0.65 0.54 0.47, 320: 0.97 0.79 0.69, 160: 0.80 0.81 0.83, 64: 0.82 0.92 0.97
+    //   Cin 576, Cout 1280: 0.76 0.64 0.53, 320: 0.97 0.85 0.75, 160: 0.85 0.87 0.91, but 64: 0.93 0.96 1.20
+    //   Cin 512, Cout 1280: 0.74 0.74 0.78, 240: 0.86 0.85 0.65, but 160: 0.86 0.94 1.02
+    //   Cin 320, Cout 1280: 0.89 0.88 0.86, 320: 0.98 0.97 0.88, 256: 0.77 0.89 0.91, but 192: 0.86 0.95 1.08
+    //   Cin 256, Cout 1280: 0.97 0.93 1.00, 320: 1.01 1.01 1.01
+    // and on 6272 rows Cin 512, Cout 240 0.91, 1280 0.89, but Cin 320, Cout 720 1.11; on 3136 rows Cin 576,
+    // Cout 320 0.95, 720 0.84, but 256 1.05.  Its one-multiply epilogue is for the clamps [0, 127] and [-128, 127].
     const long long rows_per_sm = c.m / d.sms;
-    worth = ((c.cin >= 576 && tiles_full && rows_per_sm >= 80) || (c.cin >= 672 && tiles_full && rows_per_sm >= 40) ||
-             (c.cin >= 960 && c.cout >= 144 && rows_per_sm >= 80)) &&
+    worth = ((rows_per_sm >= 80 && ((c.cin >= 320 && c.cout >= 256) || c.cin >= 960)) ||
+             (rows_per_sm >= 40 && ((c.cin >= 512 && c.cout >= 240) || (c.cin >= 576 && c.cout >= 160))) ||
+             (rows_per_sm >= 20 && c.cin >= 576 && c.cout >= 320)) &&
             (c.rq.act_min == 0 || c.rq.act_min == -128) && c.rq.act_max == 127;
     return true;
 }
