@@ -754,25 +754,54 @@ static bool wide_plan(const Conv &c, const DeviceInfo &d, WidePlan &pl, bool &wo
     return true;
 }
 
-static prom_status launch_wide(const Conv &c, const DeviceInfo &d, WidePlan &pl)
+// The same question for operands prepared ahead of the call, which spares the weight-resident kernel more than
+// this one (whose operands take a kernel of their own, 4 us).  Time as a share of the other's (rows: 12544 / 25088 /
+// 401408): Cin 960, Cout 160: 0.76 0.92 0.87, 1280: 0.57 0.56 0.51; Cin 576, Cout 240: 0.85 0.74 0.49, but 160: 0.81
+// 0.95 1.06; Cin 320, Cout 576: 0.99 0.95 0.97, 1280: 0.92 0.91 0.83, but 384: 1.11 1.06 0.91; Cin 192, Cout 1280:
+// 1.01 0.99 1.00.  On 6272 rows Cin 960, Cout 320 0.99, 576 0.85, but Cin 576: 1.02 1.07; on 3136 rows Cin 576,
+// Cout 960 0.97, 1280 0.82.
+static bool wide_prepared_worth(const Conv &c, const DeviceInfo &d)
 {
-    EncodeTiledFn enc = encode_tiled_fn();
-    if (!enc) return PROM_ERR_UNSUPPORTED;
-    wide::Params &p = pl.p;
-    const int blocks = p.n_ctiles * p.nb;           // of 128 channels
-    const size_t w8_bytes = (size_t)blocks * wide::kNt * pl.k_pad;
-    const size_t wb_bytes = (size_t)blocks * wide::kWbiasBytes;
-    const size_t cs_bytes = round256((size_t)blocks * wide::kConstBytes);
-    bool capturing = false;
-    uint8_t *scratch = wide_scratch_for(c.st, w8_bytes + wb_bytes + cs_bytes, &capturing);
-    if (!scratch) return capturing ? PROM_ERR_UNSUPPORTED : PROM_ERR_CUDA;
+    const long long rows_per_sm = c.m / d.sms;
+    return (rows_per_sm >= 80 && ((c.cin >= 320 && c.cout >= 512) || (c.cin >= 576 && c.cout >= 240) ||
+                                  (c.cin >= 960 && c.cout >= 160))) ||
+           (rows_per_sm >= 40 && c.cin >= 960 && c.cout >= 320) ||
+           (rows_per_sm >= 20 && c.cin >= 576 && c.cout >= 960);
+}
+
+// The kernel's operands in global memory: int8 weights, bias digits, constants.
+static size_t wide_w8_bytes(const WidePlan &pl) { return (size_t)pl.p.n_ctiles * pl.p.nb * wide::kNt * pl.k_pad; }
+static size_t wide_wbias_bytes(const WidePlan &pl) { return (size_t)pl.p.n_ctiles * pl.p.nb * wide::kWbiasBytes; }
+static size_t wide_operand_bytes(const WidePlan &pl)
+{
+    return wide_w8_bytes(pl) + wide_wbias_bytes(pl) + round256((size_t)pl.p.n_ctiles * pl.p.nb * wide::kConstBytes);
+}
+
+static prom_status launch_wide_prep(const Conv &c, const WidePlan &pl, uint8_t *operands)
+{
     wide::PrepParams pp;
     memset(&pp, 0, sizeof(pp));
     pp.cin = c.cin; pp.cout = c.cout; pp.k_pad = pl.k_pad; pp.w_packed = c.w;
     pp.bias = c.rq.bias; pp.mult = c.rq.mult; pp.shift = c.rq.shift;
     pp.act_min = c.rq.act_min; pp.act_max = c.rq.act_max; pp.signed_fast = 1;
-    pp.w8 = reinterpret_cast<int8_t *>(scratch); pp.wbias = scratch + w8_bytes; pp.consts = scratch + w8_bytes + wb_bytes;
-    p.consts = pp.consts;
+    pp.w8 = reinterpret_cast<int8_t *>(operands); pp.wbias = operands + wide_w8_bytes(pl);
+    pp.consts = pp.wbias + wide_wbias_bytes(pl);
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[1];
+    fill_launch_cfg(cfg, attr, pl.p.n_ctiles * pl.p.nb * wide::kPrepParts, 256, 0, c.st, true);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, wide::wide_prep_kernel, pp);
+    ++g_launches;
+    return cuda_status(e);
+}
+
+static prom_status launch_wide_conv(const Conv &c, WidePlan &pl, uint8_t *operands)
+{
+    EncodeTiledFn enc = encode_tiled_fn();
+    if (!enc) return PROM_ERR_UNSUPPORTED;
+    wide::Params &p = pl.p;
+    const int blocks = p.n_ctiles * p.nb;           // of 128 channels
+    uint8_t *wbias = operands + wide_w8_bytes(pl);
+    p.consts = wbias + wide_wbias_bytes(pl);
     CUtensorMap xmap, wmap, bmap, ymap;
     cuuint32_t es[2] = {1, 1};
     {
@@ -788,7 +817,7 @@ static prom_status launch_wide(const Conv &c, const DeviceInfo &d, WidePlan &pl)
         cuuint64_t dims[2] = {(cuuint64_t)pl.k_pad, (cuuint64_t)blocks * wide::kNt};
         cuuint64_t strides[1] = {(cuuint64_t)pl.k_pad};
         cuuint32_t box[2] = {(cuuint32_t)wide::kChunk, (cuuint32_t)(p.nb * wide::kNt / 2)};      // one CTA's half
-        if (enc(&wmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, pp.w8, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        if (enc(&wmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, operands, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) !=
             CUDA_SUCCESS)
             return PROM_ERR_UNSUPPORTED;
@@ -797,7 +826,7 @@ static prom_status launch_wide(const Conv &c, const DeviceInfo &d, WidePlan &pl)
         cuuint64_t dims[2] = {32, (cuuint64_t)blocks * wide::kNt};
         cuuint64_t strides[1] = {32};
         cuuint32_t box[2] = {32, (cuuint32_t)(p.nb * wide::kNt / 2)};
-        if (enc(&bmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, pp.wbias, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+        if (enc(&bmap, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, wbias, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                 CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return PROM_ERR_UNSUPPORTED;
     }
@@ -812,14 +841,20 @@ static prom_status launch_wide(const Conv &c, const DeviceInfo &d, WidePlan &pl)
     }
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    fill_launch_cfg(cfg, attr, blocks * wide::kPrepParts, 256, 0, c.st, true);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, wide::wide_prep_kernel, pp);
-    ++g_launches;
-    if (e != cudaSuccess) return cuda_status(e);
     fill_launch_cfg(cfg, attr, pl.grid, wide::kThreads, pl.smem, c.st, true);
-    e = cudaLaunchKernelEx(&cfg, wide::wide_conv_kernel, xmap, wmap, bmap, ymap, p);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, wide::wide_conv_kernel, xmap, wmap, bmap, ymap, p);
     ++g_launches;
     return cuda_status(e);
+}
+
+static prom_status launch_wide(const Conv &c, WidePlan &pl)
+{
+    if (!encode_tiled_fn()) return PROM_ERR_UNSUPPORTED;
+    bool capturing = false;
+    uint8_t *scratch = wide_scratch_for(c.st, wide_operand_bytes(pl), &capturing);
+    if (!scratch) return capturing ? PROM_ERR_UNSUPPORTED : PROM_ERR_CUDA;
+    const prom_status e = launch_wide_prep(c, pl, scratch);
+    return e != PROM_OK ? e : launch_wide_conv(c, pl, scratch);
 }
 
 static prom_status launch_tc(const Conv &c, int use = kPlanSingle)
@@ -831,7 +866,7 @@ static prom_status launch_tc(const Conv &c, int use = kPlanSingle)
         WidePlan wp;
         bool worth = false;
         if (wide_plan(c, d, wp, worth) && (worth || wide_mode == 2)) {
-            const prom_status e = launch_wide(c, d, wp);
+            const prom_status e = launch_wide(c, wp);
             if (e != PROM_ERR_UNSUPPORTED) return e;
         } else if (wide_mode == 2) {
             return PROM_ERR_UNSUPPORTED;
@@ -1984,9 +2019,23 @@ prom_status prom_pw_conv_i8(const int8_t *x_dev, int64_t m, int cin, const uint8
 }
 
 // ---- one layer with operands prepared ahead of the call --------------------------------------
+static Conv prepared_conv(long long m, int cin, int cout)
+{
+    Conv c;
+    c.m = m; c.cin = cin; c.cout = cout; c.map = RowMap{1, 1, 1, 1, 1}; c.in_rows = m;
+    return c;
+}
 static bool prepared_plan(long long m, int cin, int cout, const DeviceInfo &d, TcPlan &pl)
 {
     return m > 0 && tc_shape_plan(m, cin, cout, RowMap{1, 1, 1, 1, 1}, d, pl, kPlanPrepared);
+}
+// Whether the prepared form of a layer is the row-resident kernel's.
+static bool prepared_wide(const Conv &c, const DeviceInfo &d, WidePlan &pl)
+{
+    const int mode = g_wide_mode.load();
+    bool worth = false;
+    if (mode == 1 || !wide_plan(c, d, pl, worth)) return false;
+    return mode == 2 || wide_prepared_worth(c, d);
 }
 
 size_t prom_pw_prepared_bytes(int64_t m, int cin, int cout)
@@ -1994,6 +2043,8 @@ size_t prom_pw_prepared_bytes(int64_t m, int cin, int cout)
     if (m < 1 || cin < 1 || cin > 4096 || cout < 1 || cout > 4096) return 0;
     DeviceInfo d = device_info();
     if (!d.ok) { d.sms = 148; d.smem_optin = 232448; d.smem_total = 233472; d.ok = true; }
+    WidePlan wp;
+    if (prepared_wide(prepared_conv(m, cin, cout), d, wp)) return wide_operand_bytes(wp);
     TcPlan pl;
     if (!prepared_plan(m, cin, cout, d, pl)) return 0;
     return round256((size_t)pl.p.groups * pl.p.image_stride);
@@ -2009,13 +2060,17 @@ prom_status prom_pw_prepare(int64_t m, int cin, const uint8_t *w_packed_dev, int
     if (!aligned16(w_packed_dev) || !aligned16(prepared_dev)) return PROM_ERR_ALIGN;
     DeviceInfo d = device_info();
     if (!d.ok) return PROM_ERR_CUDA;
+    Conv c = prepared_conv(m, cin, cout);
+    c.w = w_packed_dev; c.rq = *rq; c.st = static_cast<cudaStream_t>(cuda_stream);
+    WidePlan wp;
+    if (prepared_wide(c, d, wp)) {
+        if (prepared_bytes < wide_operand_bytes(wp)) return PROM_ERR_WORKSPACE;
+        return launch_wide_prep(c, wp, static_cast<uint8_t *>(prepared_dev));
+    }
     TcPlan pl;
     if (!prepared_plan(m, cin, cout, d, pl)) return PROM_ERR_UNSUPPORTED;
     if (prepared_bytes < round256((size_t)pl.p.groups * pl.p.image_stride)) return PROM_ERR_WORKSPACE;
     if (tc_set_attr(d) != PROM_OK) return PROM_ERR_CUDA;
-    Conv c;
-    c.x = nullptr; c.m = m; c.cin = cin; c.cout = cout; c.map = RowMap{1, 1, 1, 1, 1}; c.in_rows = m;
-    c.w = w_packed_dev; c.rq = *rq; c.y = nullptr; c.st = static_cast<cudaStream_t>(cuda_stream);
     tc_bind(c, pl, static_cast<uint8_t *>(prepared_dev));
     tc::PrepTable t;
     memset(&t, 0, sizeof(t));
@@ -2040,13 +2095,14 @@ prom_status prom_pw_conv_i8_prepared(const int8_t *x_dev, int64_t m, int cin, in
     if (!aligned16(x_dev) || !aligned16(prepared_dev) || !aligned16(y_dev)) return PROM_ERR_ALIGN;
     DeviceInfo d = device_info();
     if (!d.ok) return PROM_ERR_CUDA;
+    Conv c = prepared_conv(m, cin, cout);
+    c.x = x_dev; c.y = y_dev; c.st = static_cast<cudaStream_t>(cuda_stream);
+    c.rq = prom_requant{nullptr, nullptr, nullptr, act_min, act_max};
+    WidePlan wp;
+    if (prepared_wide(c, d, wp)) return launch_wide_conv(c, wp, const_cast<uint8_t *>(static_cast<const uint8_t *>(prepared_dev)));
     TcPlan pl;
     if (!prepared_plan(m, cin, cout, d, pl)) return PROM_ERR_UNSUPPORTED;
     if (tc_set_attr(d) != PROM_OK) return PROM_ERR_CUDA;
-    Conv c;
-    c.x = x_dev; c.m = m; c.cin = cin; c.cout = cout; c.map = RowMap{1, 1, 1, 1, 1}; c.in_rows = m;
-    c.w = nullptr; c.rq = prom_requant{nullptr, nullptr, nullptr, act_min, act_max}; c.y = y_dev;
-    c.st = static_cast<cudaStream_t>(cuda_stream);
     tc_bind(c, pl, const_cast<uint8_t *>(static_cast<const uint8_t *>(prepared_dev)));
     return tc_launch_planned(c, pl);
 }

@@ -44,7 +44,7 @@ constexpr int kMaxStages = 8;
 constexpr int kAccs = 2;                          // accumulators of up to 256 columns
 constexpr uint32_t kAChunkBytes = 128 * kChunk;   // one resident chunk of a CTA's 128 rows
 constexpr uint32_t kWbiasBytes = kNt * 32;        // bias digits of a block (32-byte swizzled rows)
-// constants of a block: mult[128], {bias, shift}[128], header {shmax, fast, bad, 0}
+// constants of a block: mult[128], {bias, shift}[128], header {shmax, fast, bad, clamp}
 constexpr uint32_t kConstBytes = kNt * 4 + kNt * 8 + 16 + 112;
 constexpr uint32_t kEpiCols = 32;                 // columns an epilogue warp stages per store
 constexpr uint32_t kSlabBytes = 32 * kEpiCols;
@@ -72,6 +72,9 @@ struct PrepParams {
     int8_t *w8;                 // [n_ctiles * 128][k_pad]
     uint8_t *wbias, *consts;
 };
+
+// Operands are for one clamp; the kernel that reads them is told it again.
+__device__ __forceinline__ int clamp_code(int lo, int hi) { return ((lo & 0xFF) << 8) | (hi & 0xFF); }
 
 // The operands of column tile `tile` of one layer; all 256 threads of the CTA take part.  `parts` CTAs share
 // the expansion of the tile's weights (each checks the constants; the first writes them).
@@ -129,7 +132,7 @@ __device__ __forceinline__ void prep_tile(const PrepParams &p, const int tile, c
     }
     if (threadIdx.x == 0 && part == 0) {
         int *hdr = reinterpret_cast<int *>(cst + kNt * 12);
-        hdr[0] = shmax; hdr[1] = fast ? 1 : 0; hdr[2] = bad ? 1 : 0; hdr[3] = 0;
+        hdr[0] = shmax; hdr[1] = fast ? 1 : 0; hdr[2] = bad ? 1 : 0; hdr[3] = clamp_code(p.act_min, p.act_max);
     }
 
     // the tile's rows of the int8 matrix, 16 bytes (16 codes = one 32-bit word) per step
@@ -431,7 +434,9 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
                 const int2 *cbs = reinterpret_cast<const int2 *>(cst + kNt * 4) + (at & (kNt - 1));
                 const int *hdr = reinterpret_cast<const int *>(cst + kNt * 12);
                 const int shmax = hdr[0];
-                const bool fast = hdr[1] != 0, bad = hdr[2] != 0, last = pc + 4 >= pieces;
+                const bool other_clamp = hdr[3] != clamp_code(p.act_min, p.act_max);
+                const bool bad = hdr[2] != 0 || other_clamp, fast = hdr[1] != 0 && !bad, last = pc + 4 >= pieces;
+                if (other_clamp && lane == 0) raise_status(PROM_ERR_BAD_REQUANT);
                 const uint32_t taddr = t_lane + acc * 256u + (uint32_t)at;
                 // the previous store has read the slab
                 ptx::bulk_wait_read0();

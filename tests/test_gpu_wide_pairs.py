@@ -28,3 +28,21 @@ def test_tiles_and_clamps(oracle, m, cin, cout, lo, hi):
     # the rest against the plain kernel
     naive = run_variant(xd, wp, consts, cout, "naive", lo, hi)
     assert np.array_equal(np.asarray(y), np.asarray(naive))
+
+
+@pytest.mark.parametrize("m,cin,cout,lo", [(12001, 320, 528, 0), (5921, 960, 320, -128), (3000, 592, 960, 0)])
+def test_prepared(oracle, m, cin, cout, lo):
+    """Operands prepared ahead where the library takes this kernel for them; another clamp than theirs is refused."""
+    x, lay = make_case(m + cin, m, cin, cout, 0.5, act="i8")
+    xd, wp, consts = to_device(x, lay)
+    prep = binding.pw_prepare(m, cin, wp, cout, binding.make_requant(*consts, lo, 127))
+    assert prep.numel() >= cout * cin                        # int8 weights: the row-resident form
+    naive = run_variant(xd, wp, consts, cout, "naive", lo, 127)
+    for _ in range(2):
+        y = binding.pw_conv_i8_prepared(xd, cout, prep, lo, 127)
+        assert np.array_equal(y.cpu().numpy(), np.asarray(naive))
+    assert binding.last_device_status() == binding.PROM_OK
+    y.fill_(-77)
+    binding.pw_conv_i8_prepared(xd, cout, prep, -5, 90, y=y)
+    assert binding.last_device_status() == binding.PROM_ERR_BAD_REQUANT
+    assert bool((y == -77).all())
