@@ -890,22 +890,22 @@ __device__ __forceinline__ void build_image(const Params &p, const int g, const 
 
     // constants of up to kConstPerThread resident channels per thread, requested early
     constexpr int kConstPerThread = 4;
+    // (the dynamic layer has neither bias nor shift: both pointers are null)
+    auto constants = [&](int i, int &b, int &mu, int &sh) {
+        b = 0; mu = 0; sh = kNoColumn;                      // padding column, or none
+        if (i >= ncols_res) return;
+        const int ls = i / p.nt_pad, c = i - ls * p.nt_pad;
+        const int nfold = (g + ls * p.groups) * p.nt + c;
+        if (c < p.nt && nfold < p.nf) {
+            const int n = nfold % p.n0;
+            mu = __ldg(p.mult + n);
+            b = p.dyn ? 0 : __ldg(p.bias + n);
+            sh = p.dyn ? 0 : (int)__ldg(p.shift + n);
+        }
+    };
     int cb_[kConstPerThread], cm_[kConstPerThread], cs_[kConstPerThread];
 #pragma unroll
-    for (int u = 0; u < kConstPerThread; ++u) {
-        const int i = u * kThreads + (int)threadIdx.x;
-        cb_[u] = 0; cm_[u] = 0; cs_[u] = kNoColumn;         // padding column, or none
-        if (i < ncols_res) {
-            const int ls = i / p.nt_pad, c = i - ls * p.nt_pad;
-            const int nfold = (g + ls * p.groups) * p.nt + c;
-            if (c < p.nt && nfold < p.nf) {
-                const int n = nfold % p.n0;
-                cm_[u] = __ldg(p.mult + n);
-                cb_[u] = p.dyn ? 0 : __ldg(p.bias + n);
-                cs_[u] = p.dyn ? 0 : (int)__ldg(p.shift + n);
-            }
-        }
-    }
+    for (int u = 0; u < kConstPerThread; ++u) constants(u * kThreads + (int)threadIdx.x, cb_[u], cm_[u], cs_[u]);
     __syncthreads();                                        // barriers and flags are set up
 
     // range check, shift span, and whether every channel can take the fast epilogue: with
@@ -931,13 +931,8 @@ __device__ __forceinline__ void build_image(const Params &p, const int g, const 
             if (i < ncols_res) take(i, cb_[u], cm_[u], cs_[u]);
         }
         for (int i = kConstPerThread * kThreads + (int)threadIdx.x; i < ncols_res; i += kThreads) {
-            const int ls = i / p.nt_pad, c = i - ls * p.nt_pad;
-            const int nfold = (g + ls * p.groups) * p.nt + c;
-            int b = 0, mu = 0, sh = kNoColumn;
-            if (c < p.nt && nfold < p.nf) {
-                const int n = nfold % p.n0;
-                b = __ldg(p.bias + n); mu = __ldg(p.mult + n); sh = __ldg(p.shift + n);
-            }
+            int b, mu, sh;
+            constants(i, b, mu, sh);
             take(i, b, mu, sh);
         }
         if (bad) flags[3] = 1;
