@@ -19,12 +19,17 @@ def _sources():
                   + glob.glob(os.path.join(INCLUDE, "*.h")))
 
 
+def _native_sources():
+    # the extension is compiled against the header's structures and signatures
+    return [NATIVE_SOURCE] + sorted(glob.glob(os.path.join(INCLUDE, "*.h")))
+
+
 def _older(target: str, sources) -> bool:
     return not os.path.exists(target) or any(os.path.getmtime(f) > os.path.getmtime(target) for f in sources)
 
 
 def needs_build() -> bool:
-    return _older(LIB, _sources()) or _older(NATIVE, [NATIVE_SOURCE])
+    return _older(LIB, _sources()) or _older(NATIVE, _native_sources())
 
 
 def _build_lib(verbose: bool) -> None:
@@ -63,7 +68,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     """Builds what is older than its sources; returns the path of the C-ABI library."""
     if force or _older(LIB, _sources()):
         _build_lib(verbose)
-    if force or _older(NATIVE, [NATIVE_SOURCE]):
+    if force or _older(NATIVE, _native_sources()):
         _build_native()
     return LIB
 
