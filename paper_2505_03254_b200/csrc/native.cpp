@@ -181,7 +181,7 @@ PyObject *pw_conv_i8_prepared(PyObject *, PyObject *const *a, Py_ssize_t n)
         const int64_t m = x.size(0);
         const int cin = (int)x.size(1), cout = small_int(a[1]), lo = small_int(a[3]), hi = small_int(a[4]);
         const auto *xp = ptr<const int8_t>(x);
-        const void *pp = tensor(a[2], "prepared").data_ptr();
+        const void *pp = ptr<const uint8_t>(dev(a[2], at::kByte, "prepared"));
         auto *yp = ptr<int8_t>(dev(a[5], at::kChar, "y"));
         void *st = stream(a[6]);
         return call([&] { return prom_pw_conv_i8_prepared(xp, m, cin, cout, pp, lo, hi, yp, st); });
