@@ -29,13 +29,16 @@
  *   - Every pointer named *_dev is device memory of the current CUDA device,
  *     owned by the caller; *_host is host memory (pinned for overlap).
  *   - The library allocates nothing the caller must free.  It keeps small
- *     internal caches (tensor-map plans; per device and stream, the index
- *     lists of the add/sub variant and the expanded weight matrix of the
- *     row-resident tensor-core kernel, which single calls with Cin >= 640 and
- *     Cout >= 256 on many rows use: device memory obtained with cudaMalloc on
- *     first use; while a stream is being captured the add/sub variant must
- *     already have its own, and the row-resident kernel gives way to the
- *     weight-resident one when it has not) that prom_shutdown() releases.
+ *     internal caches that prom_shutdown() releases: tensor-map plans, and
+ *     device memory obtained with cudaMalloc on first use.  Per device and
+ *     stream that is the index lists of the add/sub variant (which must exist
+ *     before a call of it is captured) and the expanded weight matrix of the
+ *     row-resident tensor-core kernel, a few MB, which plain single calls with
+ *     many input channels on many rows use (from 320 inputs on).  A call of
+ *     that kernel which is captured into a graph has a matrix of its own; it
+ *     is free for another capture once the graph and what was instantiated
+ *     from it have been destroyed, and prom_shutdown() leaves those of living
+ *     graphs alone.
  *   - `cuda_stream` is a cudaStream_t passed as void* (NULL = default stream).
  *     Convolution calls are asynchronous on that stream.
  *   - Errors are return codes; nothing aborts or traps.  Argument errors are

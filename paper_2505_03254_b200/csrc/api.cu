@@ -619,8 +619,7 @@ static size_t round256(size_t v) { return (v + 255) & ~(size_t)255; }
 static std::atomic<int> g_wide_mode{0};
 static std::atomic<int> g_wide_nb{0};        // 0: the planner's choice; 1 or 2: forced (tests)
 
-// Global scratch of the variant (the expanded weight matrix, bias digits, constants), one buffer
-// per (device, stream), grown on demand and kept until prom_shutdown().
+// Global scratch of the variant: the expanded weight matrix, bias digits, constants.
 struct WideKey {
     int dev;
     cudaStream_t st;
@@ -632,26 +631,36 @@ static std::map<WideKey, WideBuf> g_wide_cache;
 
 static std::vector<uint8_t *> g_wide_retired;
 
-// null: no memory, or (sets *capturing) none yet and the stream is being captured.  A buffer that has become
-// too small is kept until prom_shutdown(): earlier calls and captured graphs may still use it.  Sizes are
-// powers of two, so a stream's buffers add up to less than twice its largest.
-static uint8_t *wide_scratch_for(cudaStream_t st, size_t bytes, bool *capturing)
+// cudaMalloc that neither fails nor spoils a capture because a stream (this one or another thread's) is being captured.
+static cudaError_t malloc_beside_capture(uint8_t **p, size_t bytes)
 {
-    *capturing = false;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaMalloc(reinterpret_cast<void **>(p), bytes);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return e;
+}
+
+static size_t wide_buffer_size(size_t bytes)
+{
+    size_t want = 1 << 20;
+    while (want < bytes) want *= 2;
+    return want;
+}
+
+// A stream's buffer, for calls that run as they are made: in stream order, so that one buffer serves all of them.
+// One that has become too small is kept until prom_shutdown(): earlier calls may still use it.  Sizes are powers of
+// two, so a stream's buffers add up to less than twice its largest.  null: no memory.
+static uint8_t *wide_scratch_for(cudaStream_t st, size_t bytes)
+{
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
     std::lock_guard<std::mutex> lk(g_wide_mu);
     WideBuf &b = g_wide_cache[WideKey{dev, st}];
     if (b.bytes < bytes) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
-            *capturing = true;
-            return nullptr;
-        }
-        size_t want = 1 << 20;
-        while (want < bytes) want *= 2;
+        const size_t want = wide_buffer_size(bytes);
         uint8_t *p = nullptr;
-        if (cudaMalloc(reinterpret_cast<void **>(&p), want) != cudaSuccess) return nullptr;
+        if (malloc_beside_capture(&p, want) != cudaSuccess) return nullptr;
         if (b.p) g_wide_retired.push_back(b.p);
         b.p = p;
         b.bytes = want;
@@ -659,14 +668,71 @@ static uint8_t *wide_scratch_for(cudaStream_t st, size_t bytes, bool *capturing)
     return b.p;
 }
 
+// A captured call runs whenever its graph does, on any stream and beside any other call, so it has a buffer of its own,
+// which belongs to the graph: it becomes idle when the graph and all that was instantiated from it are gone, and serves
+// a later capture.  (Mutex and table are never destroyed: the last graphs may go after this library's static objects.)
+struct GraphBuf { int dev; size_t bytes; uint8_t *p; };
+static std::mutex &graph_mu() { static std::mutex *m = new std::mutex; return *m; }
+static std::vector<GraphBuf> &graph_idle() { static auto *v = new std::vector<GraphBuf>; return *v; }
+
+static void CUDART_CB graph_buffer_idle(void *buf)       // (may call nothing of CUDA)
+{
+    GraphBuf *b = static_cast<GraphBuf *>(buf);
+    std::lock_guard<std::mutex> lk(graph_mu());
+    graph_idle().push_back(*b);
+    delete b;
+}
+
+static uint8_t *graph_scratch_for(cudaStream_t st, size_t bytes)
+{
+    int dev = 0;
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    cudaGraph_t graph = nullptr;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaStreamGetCaptureInfo_v2(st, &status, nullptr, &graph, nullptr, nullptr) != cudaSuccess ||
+        status != cudaStreamCaptureStatusActive || !graph)
+        return nullptr;
+    GraphBuf *b = new GraphBuf{dev, wide_buffer_size(bytes), nullptr};
+    {
+        std::lock_guard<std::mutex> lk(graph_mu());
+        auto &idle = graph_idle();
+        for (size_t i = 0; i < idle.size(); ++i)
+            if (idle[i].dev == dev && idle[i].bytes == b->bytes) {
+                b->p = idle[i].p;
+                idle.erase(idle.begin() + i);
+                break;
+            }
+    }
+    if (!b->p && malloc_beside_capture(&b->p, b->bytes) != cudaSuccess) {
+        delete b;
+        return nullptr;
+    }
+    uint8_t *p = b->p;
+    cudaUserObject_t owner = nullptr;
+    if (cudaUserObjectCreate(&owner, b, graph_buffer_idle, 1, cudaUserObjectNoDestructorSync) != cudaSuccess) {
+        graph_buffer_idle(b);
+        return nullptr;
+    }
+    if (cudaGraphRetainUserObject(graph, owner, 1, cudaGraphUserObjectMove) != cudaSuccess) {
+        cudaUserObjectRelease(owner, 1);
+        return nullptr;
+    }
+    return p;
+}
+
 static void wide_release_cache()
 {
-    std::lock_guard<std::mutex> lk(g_wide_mu);
-    for (auto &kv : g_wide_cache)
-        if (kv.second.p) cudaFree(kv.second.p);
-    g_wide_cache.clear();
-    for (uint8_t *p : g_wide_retired) cudaFree(p);
-    g_wide_retired.clear();
+    {
+        std::lock_guard<std::mutex> lk(g_wide_mu);
+        for (auto &kv : g_wide_cache)
+            if (kv.second.p) cudaFree(kv.second.p);
+        g_wide_cache.clear();
+        for (uint8_t *p : g_wide_retired) cudaFree(p);
+        g_wide_retired.clear();
+    }
+    std::lock_guard<std::mutex> lk(graph_mu());
+    for (const GraphBuf &b : graph_idle()) cudaFree(b.p);
+    graph_idle().clear();
 }
 
 struct WidePlan {
@@ -850,9 +916,14 @@ static prom_status launch_wide_conv(const Conv &c, WidePlan &pl, uint8_t *operan
 static prom_status launch_wide(const Conv &c, WidePlan &pl)
 {
     if (!encode_tiled_fn()) return PROM_ERR_UNSUPPORTED;
-    bool capturing = false;
-    uint8_t *scratch = wide_scratch_for(c.st, wide_operand_bytes(pl), &capturing);
-    if (!scratch) return capturing ? PROM_ERR_UNSUPPORTED : PROM_ERR_CUDA;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c.st, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        return PROM_ERR_UNSUPPORTED;
+    }
+    uint8_t *scratch = cs == cudaStreamCaptureStatusNone ? wide_scratch_for(c.st, wide_operand_bytes(pl))
+                                                         : graph_scratch_for(c.st, wide_operand_bytes(pl));
+    if (!scratch) return PROM_ERR_CUDA;
     const prom_status e = launch_wide_prep(c, pl, scratch);
     return e != PROM_OK ? e : launch_wide_conv(c, pl, scratch);
 }

@@ -1,5 +1,5 @@
-"""The library's own choice of the row-resident kernel: a call captured into a graph before the stream has its
-scratch falls back on the weight-resident kernel, and a later, larger layer leaves a captured graph valid."""
+"""The library's own choice of the row-resident kernel: calls captured into a graph before and after the stream has its
+scratch, and a later, larger layer that leaves the captured graphs valid."""
 import numpy as np
 import pytest
 import torch
