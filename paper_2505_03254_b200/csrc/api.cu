@@ -10,6 +10,7 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <thread>
 #include <unordered_map>
 #include <vector>
 
@@ -620,10 +621,15 @@ static std::atomic<int> g_wide_mode{0};
 static std::atomic<int> g_wide_nb{0};        // 0: the planner's choice; 1 or 2: forced (tests)
 
 // Global scratch of the variant: the expanded weight matrix, bias digits, constants.
+// (The handle of the per-thread default stream names a stream in every thread: the thread is part of the key there.)
 struct WideKey {
     int dev;
     cudaStream_t st;
-    bool operator<(const WideKey &o) const { return dev != o.dev ? dev < o.dev : st < o.st; }
+    std::thread::id thread;
+    bool operator<(const WideKey &o) const
+    {
+        return dev != o.dev ? dev < o.dev : (st != o.st ? st < o.st : thread < o.thread);
+    }
 };
 struct WideBuf { uint8_t *p = nullptr; size_t bytes = 0; };
 static std::mutex g_wide_mu;
@@ -656,7 +662,7 @@ static uint8_t *wide_scratch_for(cudaStream_t st, size_t bytes)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return nullptr;
     std::lock_guard<std::mutex> lk(g_wide_mu);
-    WideBuf &b = g_wide_cache[WideKey{dev, st}];
+    WideBuf &b = g_wide_cache[WideKey{dev, st, st == cudaStreamPerThread ? std::this_thread::get_id() : std::thread::id()}];
     if (b.bytes < bytes) {
         const size_t want = wide_buffer_size(bytes);
         uint8_t *p = nullptr;
@@ -924,6 +930,9 @@ static prom_status launch_wide(const Conv &c, WidePlan &pl)
     uint8_t *scratch = cs == cudaStreamCaptureStatusNone ? wide_scratch_for(c.st, wide_operand_bytes(pl))
                                                          : graph_scratch_for(c.st, wide_operand_bytes(pl));
     if (!scratch) return PROM_ERR_CUDA;
+    // Both launches as one: another thread's call on this stream must not put its operands between them.
+    static std::mutex order;
+    std::lock_guard<std::mutex> lk(order);
     const prom_status e = launch_wide_prep(c, pl, scratch);
     return e != PROM_OK ? e : launch_wide_conv(c, pl, scratch);
 }
