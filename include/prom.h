@@ -34,7 +34,8 @@
  *     stream that is the index lists of the add/sub variant (which must exist
  *     before a call of it is captured) and the expanded weight matrix of the
  *     row-resident tensor-core kernel, a few MB, which plain single calls with
- *     many input channels on many rows use (from 320 inputs on).  A call of
+ *     many input channels on many rows use (from 320 inputs on; without the
+ *     memory they run on the weight-resident kernel, which needs none).  A call of
  *     that kernel which is captured into a graph has a matrix of its own; it
  *     is free for another capture once the graph and what was instantiated
  *     from it have been destroyed, and prom_shutdown() leaves those of living

@@ -929,7 +929,10 @@ static prom_status launch_wide(const Conv &c, WidePlan &pl)
     }
     uint8_t *scratch = cs == cudaStreamCaptureStatusNone ? wide_scratch_for(c.st, wide_operand_bytes(pl))
                                                          : graph_scratch_for(c.st, wide_operand_bytes(pl));
-    if (!scratch) return PROM_ERR_CUDA;
+    if (!scratch) {             // no memory: the weight-resident kernel needs none
+        cudaGetLastError();
+        return PROM_ERR_UNSUPPORTED;
+    }
     // Both launches as one: another thread's call on this stream must not put its operands between them.
     static std::mutex order;
     std::lock_guard<std::mutex> lk(order);
