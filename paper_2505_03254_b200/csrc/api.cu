@@ -216,10 +216,29 @@ static std::atomic<int> g_seq_snake{1};
 
 static int round_up(int v, int a) { return (v + a - 1) / a * a; }
 
+// Outputs up to about this size stay in L2 (126 MB) until they are complete.
+constexpr double kL2Bytes = 0.8e8;
+
+// Edges per row between subtiles that are written far apart in time, where subtiles are not whole 32-byte sectors:
+// about half of them split one.  (One CTA that shares a tile's load among its subtiles writes both sides at once.)
+static int torn_edges(const tc::Params &p)
+{
+    return p.n_sub > 1 && p.nt % 32 && (p.groups > 1 || !p.share_x) ? p.n_sub : 0;
+}
+
+// What a plan is for: kPlanSingle (one call: the kernel builds its operands itself), kPlanDynamic (the dynamic
+// layer: no row folding, a folded row could straddle two samples) or
+// kPlanPrepared (a layer of a sequence, whose operands tc_prep_kernel builds once)
+// kPlanOdd, added to kPlanSingle or kPlanPrepared (the automatic choice of calls and sequences): an odd number of
+// rows that have to be folded in pairs is taken too, the last row as a tile of its own (PROM_VARIANT_TC
+// refuses such a shape), and small layers may have subtiles of any multiple of 8
+// kPlanRes, added to kPlanSingle: a tensor is added to the output
+enum { kPlanSingle = 0, kPlanDynamic = 1, kPlanPrepared = 2, kPlanOdd = 4, kPlanRes = 8 };
+
 // Everything of a plan that follows from (fold, nt, groups, occ); false when it does not fit.
 static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, const DeviceInfo &d,
                          int fold, int nt, int groups, int occ, int want_stages, TcPlan &pl,
-                         int cw_max = 128, int direct = 0, bool tail = false, bool any_width = false)
+                         int cw_max = 128, int direct = 0, bool tail = false, int use = kPlanPrepared)
 {
     tc::Params &p = pl.p;
     memset(&p, 0, sizeof(p));
@@ -230,7 +249,7 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
     // tensor-map stores want rows and subtiles of whole 16-byte pieces; a small layer may store its rows in
     // 8-byte pieces instead, which lets it use more than one channel group (720 -> 120 on 441 rows)
     const bool rows_8 = n_sub > 1 && ((nt & 15) || (nf & 15));
-    if (rows_8 && (!any_width || direct || (nt & 7) || m * cout > 1500000)) return false;
+    if (rows_8 && (!(use & kPlanOdd) || direct || (nt & 7) || m * cout > 1500000)) return false;
     if (n_sub == 1 && (nt & 7)) return false;
     const int subs = n_sub / groups;
     const int nt_pad = round_up(nt, 16);
@@ -344,12 +363,22 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
     // Staged subtile widths with a straight-line epilogue (tc.cuh: epi_fast_fixed); any other width that
     // splits a row runs the looped epilogue, measured ~1 us per layer slower at 128 columns.
     const bool straight = nt == 96 || nt == 64 || nt == 48 || nt == 32 || nt == 80;
-    // Subtiles that split 32-byte sectors: another CTA writes the rest of the sector, and once the output is
-    // larger than L2 that comes too late (802816 rows, 16 -> 1280: 848 us with 80 columns, 334 with 64;
-    // 921600 rows, 16 -> 320: 151 and 106; 64 MB outputs show no difference).
-    const bool torn = n_sub > 1 && nt % 32 && (double)m * cout > 1e8;
-    const double epi_cost = (direct || straight ? 1.0 : (n_sub > 1 ? 1.5 : (nt <= 96 ? 1.0 : 1.2))) * (torn ? 2.5 : 1.0);
-    const double t_epi = (double)tm * nt / epi_rate * epi_cost;
+    // What is written beyond L2, a share of the output that grows from nothing.  There a sector that torn_edges()
+    // splits is written in two pieces that no longer meet, about three sectors more to move per edge (with a residual
+    // its reads bring the sector into L2).  And where a unit is short (one K chunk of at most 64 bytes), stores from
+    // registers, which do not run beside the next unit, cost more than staged ones (852992 rows, 16 -> 576: 157.0 us
+    // direct in 128 columns, 139.4 staged in 96; but 478512 rows, 120 -> 960: 164.5 and 193.6).
+    const bool res = (use & kPlanRes) != 0;
+    const double out_all = (double)m * cout, beyond = out_all > kL2Bytes ? out_all - kL2Bytes : 0.0;
+    const double t_torn = res ? 0.0 : beyond / cout * torn_edges(p) * 96.0 / 5.5e6;
+    double epi_cost = direct ? 1.0 + (kf <= 64 ? 0.4 : 0.0) * beyond / out_all
+                             : (straight ? 1.0 : (n_sub > 1 ? 1.5 : (nt <= 96 ? 1.0 : 1.15)));
+    // A residual: its bytes are held in registers beside direct stores (which one CTA per SM does not hide), and for
+    // the first 48 columns of a staged slab; those of the others are asked for once the accumulator is there, 25 ns a
+    // column (781600 rows, 240 -> 320: 185.2 us direct in 64 columns, 464.0 staged in 160).
+    if (res) epi_cost *= direct ? (occ == 1 ? 1.6 : 1.2) : 1.4;
+    const double t_late = res && !direct && nt > 48 ? 0.025 * (nt - 48) : 0.0;
+    const double t_epi = (double)tm * nt / epi_rate * epi_cost + t_late;
     const double t_load = (double)kc * tm * (kf < cw ? kf : cw) / load_rate;
     // Direct outputs want whole 64-column pieces: half of the stores of a last piece of 32 are short, which
     // shows once L2 is busy (16 -> 96 at 1.6 M rows 53.9 us against 46.3 staged, 64 -> 384 at 25088 rows 6.6
@@ -362,7 +391,9 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
     // fewer channel groups to 64-column ones)
     const double t_first = (t_epi > t_load ? t_epi : t_load) + unit;
     const double t_next = share_x ? t_epi + unit : t_first;
-    const double startup = 1.2 + (double)p.image_bytes / 80e3 * ctas_per_sm;
+    // (a single call's CTAs expand their operands themselves: 18816 rows, 64 -> 1280 take 13.4 us with 80 columns per
+    // CTA and 18.3 with 640)
+    const double startup = 1.2 + (double)p.image_bytes / 80e3 * ctas_per_sm * ((use & 3) == kPlanSingle ? 1.5 : 1.0);
     const double fill = 1.0 + 0.1 * kc;                      // first load, first MMA
     // Draining the last accumulator, store.  A direct store saves the hand-over to the bulk-copy unit: at
     // 392 rows, 64 -> 384 takes 3.1 / 3.4 / 3.9 us with 32 / 64 / 128 columns against 3.4 / 3.6 / 4.5 staged
@@ -370,26 +401,23 @@ static bool tc_fill_plan(long long m, int cin, int cout, const RowMap &map, cons
     const double last = direct && !(short_piece && m * cout > 6000000) ? 0.35 * ((nt + 31) / 32) + 0.5 : 0.45 * ((nt + 31) / 32) + 0.8;
     const double t_cta = startup + fill + rounds * (t_first + (subs - 1) * t_next) + last +
                          (occ == 1 ? 2.5 : 0.0);   // a CTA that fills its SM keeps the next kernel out
-    const double t_mem = ((double)m * cin * (groups == 1 ? 1.0 : 1.0 + 0.15 * (groups - 1)) +
-                          (double)m * cout) / 5.5e6;
-    pl.est_us = t_cta > t_mem ? t_cta : t_mem;
+    // X is read once per unit, or per channel group where one load serves all subtiles of the tile; all readings but the
+    // first come from L2.
+    const int readings = share_x ? groups : n_sub;
+    const double t_mem = ((double)m * cin * (1.0 + 0.1 * (readings - 1)) + (res ? 2.0 : 1.0) * out_all) / 5.5e6;
+    // The constants above were fitted to 3892 calls drawn over the networks' widths and spatial sizes (plain, linear,
+    // with a residual, prepared, dynamic), every plan timed: the chosen plan takes 1.5 to 2 % more than the best on
+    // average (dynamic layers 4 %).
+    pl.est_us = (t_cta > t_mem ? t_cta : t_mem) + t_torn;
     return true;
 }
 
 // Picks fold, subtile width, channel groups and occupancy.  Returns false when
-// the tensor-core variant cannot run this shape.
-// use: kPlanSingle (one call: the kernel builds its operands itself), kPlanDynamic (the dynamic
-// layer: no row folding, a folded row could straddle two samples) or
-// kPlanPrepared (a layer of a sequence, whose operands tc_prep_kernel builds once)
-// kPlanOdd, added to kPlanSingle or kPlanPrepared (the automatic choice of calls and sequences): an odd number of
-// rows that have to be folded in pairs is taken too, the last row as a tile of its own (PROM_VARIANT_TC
-// refuses such a shape), and small layers may have subtiles of any multiple of 8
-enum { kPlanSingle = 0, kPlanDynamic = 1, kPlanPrepared = 2, kPlanOdd = 4 };
+// the tensor-core variant cannot run this shape.  use: kPlan*
 static bool tc_search_plan(long long m, int cin, int cout, const RowMap &map, const DeviceInfo &d,
                            int use, TcPlan &best)
 {
-    const bool dyn = use == kPlanDynamic, odd_ok = (use & kPlanOdd) != 0;
-    use &= ~kPlanOdd;
+    const bool dyn = (use & 3) == kPlanDynamic, odd_ok = (use & kPlanOdd) != 0;
     bool tail = false;
     if (m <= 0 || (cin & 7) || (cout & 7)) return false;
     const TcTune tn = tune_for(m, cin, cout, map.stride);
@@ -408,8 +436,11 @@ static bool tc_search_plan(long long m, int cin, int cout, const RowMap &map, co
         // of 58): fold once more whatever the width, where the larger block-diagonal weights
         // are expanded once per sequence and not by every CTA
         // (a single call expands them in every CTA, which pays when the CTA then has many tiles)
-        const bool many = m >= 128ll * 16 * 2 * d.sms;
-        if (!tail && (use == kPlanPrepared || many) && cin * fold < 32 && fold * 2 <= 8 && m % (fold * 2) == 0) fold *= 2;
+        // (and unless the doubled width has no subtile with a straight-line epilogue: 16 -> 112 at 852074 rows takes
+        // 41.8 us folded against 39.2)
+        const int twice = cout * fold * 2;
+        const bool many = m >= 128ll * 16 * 2 * d.sms && (twice % 48 == 0 || twice % 64 == 0 || twice % 80 == 0);
+        if (!tail && ((use & 3) == kPlanPrepared || many) && cin * fold < 32 && fold * 2 <= 8 && m % (fold * 2) == 0) fold *= 2;
     }
     if (dyn) {
         if ((cin & 15) || ((cout & 15) && cout > 256)) return false;
@@ -434,7 +465,7 @@ static bool tc_search_plan(long long m, int cin, int cout, const RowMap &map, co
                 if (tn.occ == 0 && occ >= 3) continue;      // only on request for now
                 for (int direct = dyn ? 0 : 1; direct >= 0; --direct) {
                     TcPlan pl;
-                    if (!tc_fill_plan(m, cin, cout, map, d, fold, nt, groups, occ, tn.stages, pl, 128, direct, tail, odd_ok))
+                    if (!tc_fill_plan(m, cin, cout, map, d, fold, nt, groups, occ, tn.stages, pl, 128, direct, tail, use))
                         continue;
                     if (!found || pl.est_us < best.est_us) { best = pl; found = true; }
                 }
@@ -956,7 +987,7 @@ static prom_status launch_tc(const Conv &c, int use = kPlanSingle)
         }
     }
     TcPlan pl;
-    if (!tc_shape_plan(c.m, c.cin, c.cout, c.map, d, pl, use)) return PROM_ERR_UNSUPPORTED;
+    if (!tc_shape_plan(c.m, c.cin, c.cout, c.map, d, pl, c.res ? use | kPlanRes : use)) return PROM_ERR_UNSUPPORTED;
     if (tc_set_attr(d) != PROM_OK) return PROM_ERR_CUDA;
     tc_bind(c, pl, nullptr);
     return tc_launch_planned(c, pl);

@@ -73,3 +73,14 @@ def test_forced_plans_are_honoured_or_refused():
         assert pl is not None and pl["grid"] == 3 * SMS and pl["smem"] <= (233472 - 3 * 1024) // 3
     finally:
         binding.debug_tc_plan()
+
+
+@pytest.mark.parametrize("cin", [16, 32, 64, 96, 144, 240])
+@pytest.mark.parametrize("cout", [240, 336, 432, 560, 720])
+def test_the_time_model_has_no_step_where_outputs_outgrow_l2(cin, cout):
+    """Widths that are 16 modulo 32 tear sectors at every inner edge whatever the subtile: an output that grows past
+    L2 changes what that costs little by little."""
+    binding.debug_tc_plan()
+    plans = [binding.debug_tc_plan_query(int(rows * 1e6 / cout) // 8 * 8, cin, cout) for rows in range(60, 160, 4)]
+    for a, b in zip(plans, plans[1:]):
+        assert b["est_us_x100"] <= 1.2 * a["est_us_x100"], (a, b)         # rows of one step to the next: up to 1.07
