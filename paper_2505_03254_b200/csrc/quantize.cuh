@@ -85,7 +85,8 @@ __device__ __forceinline__ void quantize_row(const float *__restrict__ row, int 
     const double mean = sum / (double)cin;
     if (alpha_o && lane == 0) *alpha_o = (float)mean;
     const double guarded = mean < eps ? eps : mean, scale = 1.0 / guarded;
-    const float threshold = zero_threshold(guarded, scale);
+    // (a row with a weight that is not finite has no scale, and the code 0 throughout)
+    const float threshold = isfinite(mean) ? zero_threshold(guarded, scale) : __int_as_float(0x7F800000);
     bool bad = false;
     if (held) {
 #pragma unroll

@@ -41,3 +41,16 @@ def test_what_is_not_finite_is_reported():
         w[1, 7] = bad
         binding.quantize_ternary(w)
         assert binding.last_device_status() == binding.PROM_ERR_BAD_WEIGHT
+
+
+@pytest.mark.parametrize("cin", [63, 64, 2048])                 # row by element, held in registers, read twice
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), float("-inf")])
+def test_a_row_that_is_not_finite_has_code_zero(cin, bad):
+    w = torch.ones((3, cin), device="cuda")
+    w[1, ::2] = -0.25
+    w[1, 7] = bad
+    packed, _ = binding.quantize_ternary(w)
+    assert binding.last_device_status() == binding.PROM_ERR_BAD_WEIGHT
+    one, _ = binding.quantize_ternary(torch.ones((1, cin), device="cuda"))
+    packed, one = packed.view(3, -1), one.view(-1)
+    assert bool((packed[1] == 0).all()) and torch.equal(packed[0], one) and torch.equal(packed[2], one)
