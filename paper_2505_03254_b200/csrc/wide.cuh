@@ -185,6 +185,15 @@ __global__ void __launch_bounds__(256, 1) wide_prep_batch_kernel(const __grid_co
     prep_tile(t.layer[l], (int)blockIdx.x - t.first[l]);
 }
 
+// A loader that has given up must not let its CTA go while its copies are in flight.  They are counted on barriers of the
+// first CTA, together with the other CTA's, which may never be issued, so there is no phase to wait for: it waits for
+// as long as tc::drain_copies would at most.
+__device__ __noinline__ void outwait_copies()
+{
+    const unsigned long long t0 = ptx::globaltimer();
+    while (ptx::globaltimer() - t0 < tc::kWaitLimitNs) {}
+}
+
 // One pair of CTAs per two SMs takes a contiguous range of units (row tile of 256, column tile), column tiles
 // of a row tile one after the other; the range's first unit in a row tile loads the tile's rows, the last one
 // lets go of them.  (Ranges instead of whole row tiles: 98 row tiles on 74 pairs are 1.3 rounds instead of 2.)
@@ -296,11 +305,7 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
                 ok = tc::wait_bar_warp(bar_wempty + 8 * st, ph ^ 1u, flags);
                 if (++st == (uint32_t)p.stages) { st = 0; ph ^= 1u; }
             }
-            if (!ok) {
-                // let the copies in flight land before the CTA goes away
-                const unsigned long long t0 = ptx::globaltimer();
-                while (ptx::globaltimer() - t0 < 20000ull) {}
-            }
+            if (!ok) outwait_copies();
         }
         __syncwarp();
     } else if (warp == kLoader2) {
@@ -336,10 +341,7 @@ wide_conv_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant
             }
             for (int s = 0; s < kASlots && ok; ++s, ++n)
                 ok = tc::wait_bar_warp(bar_aempty + 8 * (n % kASlots), ((n / kASlots) & 1u) ^ 1u, flags);
-            if (!ok) {
-                const unsigned long long t0 = ptx::globaltimer();
-                while (ptx::globaltimer() - t0 < 20000ull) {}
-            }
+            if (!ok) outwait_copies();
         }
         __syncwarp();
     } else if (warp == 1) {
