@@ -177,6 +177,7 @@ def native():
             raise RuntimeError(f"{NATIVE_PATH} is missing: run paper_2505_03254_b200.build.build()")
         lib()
         from . import _native as module
+        module.register_types(PromRequant, PromLayer, PromQuantizeJob)
         _native = module
     return _native
 

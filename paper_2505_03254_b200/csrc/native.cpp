@@ -88,11 +88,29 @@ void *stream(PyObject *o)
     return p;
 }
 
+// The binding's ctypes structures, told by it once (register_types).
+PyObject *requant_type, *layer_type, *job_type;
+
+// A structure of the given type, or an array of them.
+void structure(PyObject *o, PyObject *type, const char *name)
+{
+    if ((PyObject *)Py_TYPE(o) == type) return;
+    PyObject *element = PyObject_GetAttrString((PyObject *)Py_TYPE(o), "_type_");       // of an array type
+    if (!element) PyErr_Clear();
+    const bool ok = element == type || (type && PyObject_IsInstance(o, type) == 1);
+    Py_XDECREF(element);
+    if (!ok) {
+        PyErr_Clear();
+        fail(PyExc_TypeError, "%s must be %s", name, type ? ((PyTypeObject *)type)->tp_name : "a registered structure");
+    }
+}
+
 // The bytes behind a ctypes structure or array (a prom_requant, a layer table, a job table).
 class Buffer {
 public:
-    Buffer(PyObject *o, size_t at_least)
+    Buffer(PyObject *o, size_t at_least, PyObject *type, const char *name)
     {
+        structure(o, type, name);
         if (PyObject_GetBuffer(o, &view_, PyBUF_SIMPLE) != 0) throw ArgError();
         if ((size_t)view_.len < at_least) {
             PyBuffer_Release(&view_);
@@ -146,7 +164,7 @@ PyObject *pw_conv_i8(PyObject *, PyObject *const *a, Py_ssize_t n)
         const auto *xp = ptr<const int8_t>(x);
         const auto *wp = ptr<const uint8_t>(dev(a[1], at::kByte, "w_packed"));
         auto *yp = ptr<int8_t>(dev(a[4], at::kChar, "y"));
-        const Buffer rq(a[3], sizeof(prom_requant));
+        const Buffer rq(a[3], sizeof(prom_requant), requant_type, "rq");
         void *st = stream(a[6]);
         return call([&] { return prom_pw_conv_i8(xp, m, cin, wp, cout, rq.as<prom_requant>(), yp, (prom_variant)variant, st); });
     });
@@ -166,7 +184,7 @@ PyObject *pw_conv_i8_res(PyObject *, PyObject *const *a, Py_ssize_t n)
         const auto *wp = ptr<const uint8_t>(dev(a[1], at::kByte, "w_packed"));
         const auto *rp = ptr<const int8_t>(res);
         auto *yp = ptr<int8_t>(dev(a[5], at::kChar, "y"));
-        const Buffer rq(a[3], sizeof(prom_requant));
+        const Buffer rq(a[3], sizeof(prom_requant), requant_type, "rq");
         void *st = stream(a[7]);
         return call([&] { return prom_pw_conv_i8_res(xp, m, cin, wp, cout, rq.as<prom_requant>(), rp, yp, (prom_variant)variant, st); });
     });
@@ -221,7 +239,7 @@ PyObject *dw_conv3x3_i8(PyObject *, PyObject *const *a, Py_ssize_t n)
         const auto *xp = ptr<const int8_t>(x);
         const auto *wp = ptr<const int8_t>(dev(a[1], at::kChar, "w"));
         auto *yp = ptr<int8_t>(dev(a[4], at::kChar, "y"));
-        const Buffer rq(a[2], sizeof(prom_requant));
+        const Buffer rq(a[2], sizeof(prom_requant), requant_type, "rq");
         void *st = stream(a[5]);
         return call([&] { return prom_dw_conv3x3_i8(xp, b, h, w, c, stride, wp, rq.as<prom_requant>(), yp, st); });
     });
@@ -252,7 +270,7 @@ PyObject *quantize_ternary_batch(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     return guarded(n, 3, [&] {
         const int jobs = small_int(a[1]);
-        const Buffer t(a[0], (size_t)(jobs > 0 ? jobs : 0) * sizeof(prom_quantize_job));
+        const Buffer t(a[0], (size_t)(jobs > 0 ? jobs : 0) * sizeof(prom_quantize_job), job_type, "jobs");
         void *st = stream(a[2]);
         return call([&] { return prom_quantize_ternary_batch(t.as<prom_quantize_job>(), jobs, st); });
     });
@@ -267,7 +285,7 @@ PyObject *pw_layer_seq(PyObject *, PyObject *const *a, Py_ssize_t n)
         dims(x, 4, "x0");
         const int b = (int)x.size(0), h = (int)x.size(1), w = (int)x.size(2);
         const at::Tensor &ws = tensor(a[3], "workspace");
-        const Buffer t(a[0], (size_t)(layers > 0 ? layers : 0) * sizeof(prom_layer));
+        const Buffer t(a[0], (size_t)(layers > 0 ? layers : 0) * sizeof(prom_layer), layer_type, "layers");
         const auto *xp = ptr<const int8_t>(x);
         void *wsp = ws.data_ptr();
         const size_t ws_bytes = (size_t)ws.numel();
@@ -277,10 +295,23 @@ PyObject *pw_layer_seq(PyObject *, PyObject *const *a, Py_ssize_t n)
     });
 }
 
+// (prom_requant, prom_layer, prom_quantize_job as the binding has them); kept for as long as the module
+PyObject *register_types(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    return guarded(n, 3, [&] {
+        for (int i = 0; i < 3; ++i) {
+            if (!PyType_Check(a[i])) fail(PyExc_TypeError, "%s", "types are expected");
+            Py_INCREF(a[i]);
+        }
+        requant_type = a[0]; layer_type = a[1]; job_type = a[2];
+        Py_RETURN_NONE;
+    });
+}
+
 #define ENTRY(name) {#name, (PyCFunction)(void (*)(void))name, METH_FASTCALL, nullptr}
 PyMethodDef methods[] = {ENTRY(pw_conv_i8), ENTRY(pw_conv_i8_res), ENTRY(pw_conv_i8_prepared), ENTRY(pw_conv_i8_dyn),
                          ENTRY(dw_conv3x3_i8), ENTRY(quantize_act_absmax), ENTRY(quantize_ternary_batch),
-                         ENTRY(pw_layer_seq), {nullptr, nullptr, 0, nullptr}};
+                         ENTRY(pw_layer_seq), ENTRY(register_types), {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
 }  // namespace
