@@ -23,13 +23,14 @@ constexpr int kWarps = kThreads / 32;
 
 // The largest |W| whose code is 0: |W| * scale, rounded to binary64, is at most 1/2 up to it and above
 // for every larger float.  (mean / 2 is off by a few units in the last place at most.)
+// A row with a weight that is not finite has no scale: its threshold, infinite or not a number, gives code 0 throughout.
 __device__ __forceinline__ float zero_threshold(double mean, double scale)
 {
     float t = (float)(0.5 * mean);
     for (int i = 0; i < 4 && (double)t * scale > 0.5; ++i) t = __int_as_float(__float_as_int(t) - 1);
     for (int i = 0; i < 4; ++i) {
         const float n = __int_as_float(__float_as_int(t) + 1);
-        if ((double)n * scale > 0.5) break;
+        if (!((double)n * scale <= 0.5)) break;
         t = n;
     }
     return t;
@@ -85,8 +86,7 @@ __device__ __forceinline__ void quantize_row(const float *__restrict__ row, int 
     const double mean = sum / (double)cin;
     if (alpha_o && lane == 0) *alpha_o = (float)mean;
     const double guarded = mean < eps ? eps : mean, scale = 1.0 / guarded;
-    // (a row with a weight that is not finite has no scale, and the code 0 throughout)
-    const float threshold = isfinite(mean) ? zero_threshold(guarded, scale) : __int_as_float(0x7F800000);
+    const float threshold = zero_threshold(guarded, scale);
     bool bad = false;
     if (held) {
 #pragma unroll
