@@ -95,7 +95,8 @@ PyObject *requant_type, *layer_type, *job_type;
 void structure(PyObject *o, PyObject *type, const char *name)
 {
     if ((PyObject *)Py_TYPE(o) == type) return;
-    PyObject *element = PyObject_GetAttrString((PyObject *)Py_TYPE(o), "_type_");       // of an array type
+    static PyObject *const attr = PyUnicode_InternFromString("_type_");
+    PyObject *element = PyObject_GetAttr((PyObject *)Py_TYPE(o), attr);       // of an array type
     if (!element) PyErr_Clear();
     const bool ok = element == type || (type && PyObject_IsInstance(o, type) == 1);
     Py_XDECREF(element);
