@@ -11,8 +11,8 @@
 // Three routes.  Fused: a thread-block cluster per sample; every CTA copies its slice of the
 // sample into shared memory once (bulk copies), the CTAs exchange their maxima through
 // distributed shared memory, and the slice is quantised from shared memory: each float is read
-// from HBM once (5 bytes per element).  Grouped: the maxima of one group of samples beside the codes of
-// the group before, which L2 still holds (samples that do not fit eight SMs' shared memory, and batches
+// from HBM once (5 bytes per element).  Grouped: the codes of one group of samples, which L2 still
+// holds, and then the maxima of the next (samples that do not fit eight SMs' shared memory, and batches
 // of which clusters would take several rounds).  Two-pass, for sizes that are not a multiple of 4: one kernel
 // takes the maxima with atomicMax on the bit pattern, a second one quantises.
 // Measured, calls back to back (floor: 5 bytes per value at the copy bandwidth): [128,112,112,32] 64 us (39; 74.5
@@ -200,11 +200,12 @@ act_quant_cluster_kernel(const float *__restrict__ x, int batch, long long per, 
     if (first_exchange) cluster.barrier_wait();     // a cluster without a sample still pairs its arrive
 }
 
-// Grouped route.  The samples are taken in groups of a few ten megabytes, kernel k of the call takes the
-// maxima of group k and quantises group k - 1, which L2 still holds: HBM reads a float once, every SM works
-// on every group whatever the number and size of the samples, and a kernel's first half needs nothing of the
-// kernel in front, so that it runs beside that kernel's second half (programmatic dependent launch).  A warp
-// takes a contiguous run of pieces of kPiece floats, a piece lies in one sample; per is a multiple of 4.
+// Grouped route.  The samples are taken in groups of up to 64 MB, kernel k of the call quantises group k - 1, whose
+// maxima kernel k - 1 took and which L2 still holds, and then takes the maxima of group k: HBM reads a float once, and
+// every SM works on every group whatever the number and size of the samples.  (The other way round, so that maxima ran
+// beside the codes of the kernel in front, L2 had to hold two groups: 33 samples of 34.5 MB took 469 us in groups of one
+// sample, now 404; 33 of 11.7 MB 139 in groups of 40 MB, now 116.)  A warp takes a contiguous run of pieces of kPiece
+// floats, a piece lies in one sample; per is a multiple of 4.
 constexpr int kGroupThreads = 512;
 constexpr int kPieceVec = 8;                        // float4 loads of a lane in flight
 constexpr int kPiece = 32 * 4 * kPieceVec;
@@ -230,63 +231,82 @@ __device__ __forceinline__ void warp_run(long long total, long long &p, long lon
     end = p + each + (w < more ? 1 : 0);
 }
 
-__global__ void __launch_bounds__(kGroupThreads, 2) act_group_kernel(const GroupArgs a)
+__device__ __forceinline__ void group_maxima(const GroupArgs &a)
 {
-    // The first kernel waits for what wrote x (and for the cleared maxima) before it releases the others; they
-    // wait for the kernel in front only where its maxima are needed.
-    if (a.first) ptx::grid_dep_wait();
-    ptx::grid_dep_launch();
     const int lane = threadIdx.x & 31;
     const long long per4 = a.per >> 2;
     long long p, end;
     warp_run(a.pieces * a.max_count, p, end);
-    if (p < end) {
-        long long s = p / a.pieces, r = p - s * a.pieces;
-        float m = 0.0f;
-        for (; p < end; ++p) {
-            const float4 *src = reinterpret_cast<const float4 *>(a.x + (a.max_first + s) * a.per) + r * (kPiece / 4);
-            const int left = (int)(per4 - r * (kPiece / 4) < kPiece / 4 ? per4 - r * (kPiece / 4) : kPiece / 4);
-            float4 v[kPieceVec];
+    if (p >= end) return;
+    long long s = p / a.pieces, r = p - s * a.pieces;
+    float m = 0.0f;
+    for (; p < end; ++p) {
+        const float4 *src = reinterpret_cast<const float4 *>(a.x + (a.max_first + s) * a.per) + r * (kPiece / 4);
+        const int left = (int)(per4 - r * (kPiece / 4) < kPiece / 4 ? per4 - r * (kPiece / 4) : kPiece / 4);
+        float4 v[kPieceVec];
 #pragma unroll
-            for (int j = 0; j < kPieceVec; ++j)
-                v[j] = lane + 32 * j < left ? __ldg(src + lane + 32 * j) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        for (int j = 0; j < kPieceVec; ++j)
+            v[j] = lane + 32 * j < left ? __ldg(src + lane + 32 * j) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
-            for (int j = 0; j < kPieceVec; ++j)       // (fmaxf drops NaNs)
-                m = fmaxf(fmaxf(m, fmaxf(fabsf(v[j].x), fabsf(v[j].y))), fmaxf(fabsf(v[j].z), fabsf(v[j].w)));
-            if (++r == a.pieces || p + 1 == end) {
-                // non-negative floats are ordered like their bit patterns
-                const uint32_t g = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(m));
-                if (lane == 0 && g) atomicMax(reinterpret_cast<unsigned int *>(a.gamma + a.max_first + s), g);
-                m = 0.0f;
-                if (r == a.pieces) { r = 0; ++s; }
-            }
+        for (int j = 0; j < kPieceVec; ++j)       // (fmaxf drops NaNs)
+            m = fmaxf(fmaxf(m, fmaxf(fabsf(v[j].x), fabsf(v[j].y))), fmaxf(fabsf(v[j].z), fabsf(v[j].w)));
+        if (++r == a.pieces || p + 1 == end) {
+            // non-negative floats are ordered like their bit patterns
+            const uint32_t g = __reduce_max_sync(0xFFFFFFFFu, __float_as_uint(m));
+            if (lane == 0 && g) atomicMax(reinterpret_cast<unsigned int *>(a.gamma + a.max_first + s), g);
+            m = 0.0f;
+            if (r == a.pieces) { r = 0; ++s; }
         }
     }
-    if (!a.first) ptx::grid_dep_wait();
+}
+
+__device__ __forceinline__ void group_codes(const GroupArgs &a)
+{
+    const int lane = threadIdx.x & 31;
+    const long long per4 = a.per >> 2;
+    long long p, end;
     warp_run(a.pieces * a.q_count, p, end);
-    if (p < end) {
-        long long s = p / a.pieces, r = p - s * a.pieces;
-        float sc = 0.0f;
-        bool fresh = true;
-        for (; p < end; ++p) {
-            const long long sample = a.q_first + s, at = r * (kPiece / 4);
-            const float4 *src = reinterpret_cast<const float4 *>(a.x + sample * a.per) + at;
-            uint32_t *dst = reinterpret_cast<uint32_t *>(a.q + sample * a.per) + at;
-            const int left = (int)(per4 - at < kPiece / 4 ? per4 - at : kPiece / 4);
-            float4 v[kPieceVec];
+    if (p >= end) return;
+    long long s = p / a.pieces, r = p - s * a.pieces;
+    float sc = 0.0f;
+    bool fresh = true;
+    for (; p < end; ++p) {
+        const long long sample = a.q_first + s, at = r * (kPiece / 4);
+        const float4 *src = reinterpret_cast<const float4 *>(a.x + sample * a.per) + at;
+        uint32_t *dst = reinterpret_cast<uint32_t *>(a.q + sample * a.per) + at;
+        const int left = (int)(per4 - at < kPiece / 4 ? per4 - at : kPiece / 4);
+        float4 v[kPieceVec];
 #pragma unroll
-            for (int j = 0; j < kPieceVec; ++j)
-                if (lane + 32 * j < left) v[j] = __ldcs(src + lane + 32 * j);
-            if (fresh) {
-                sc = scale_of(__ldcg(a.gamma + sample), a.eps);
-                if (r == 0 && lane == 0) a.scale[sample] = sc;
-                fresh = false;
-            }
-#pragma unroll
-            for (int j = 0; j < kPieceVec; ++j)
-                if (lane + 32 * j < left) __stcs(dst + lane + 32 * j, quantise_four(v[j], sc));
-            if (++r == a.pieces) { r = 0; ++s; fresh = true; }
+        for (int j = 0; j < kPieceVec; ++j)
+            if (lane + 32 * j < left) v[j] = __ldcs(src + lane + 32 * j);
+        if (fresh) {
+            sc = scale_of(__ldcg(a.gamma + sample), a.eps);
+            if (r == 0 && lane == 0) a.scale[sample] = sc;
+            fresh = false;
         }
+#pragma unroll
+        for (int j = 0; j < kPieceVec; ++j)
+            if (lane + 32 * j < left) __stcs(dst + lane + 32 * j, quantise_four(v[j], sc));
+        if (++r == a.pieces) { r = 0; ++s; fresh = true; }
+    }
+}
+
+// SEVERAL: the call has more than one group.  (With one, a kernel does either the one or the other, and the shorter way
+// to the maxima is worth 2 to 4 % of 12 us.)
+template <bool SEVERAL>
+__global__ void __launch_bounds__(kGroupThreads, 2) act_group_kernel(const GroupArgs a)
+{
+    // The first kernel waits for what wrote x and for the cleared maxima, the others for the maxima of the group before.
+    if (a.first) ptx::grid_dep_wait();
+    ptx::grid_dep_launch();
+    if (SEVERAL) {
+        if (!a.first) ptx::grid_dep_wait();
+        group_codes(a);
+        group_maxima(a);
+    } else {
+        group_maxima(a);
+        if (!a.first) ptx::grid_dep_wait();
+        group_codes(a);
     }
 }
 

@@ -1998,7 +1998,7 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
     }
     // Several rounds of clusters run in step, each with its loads exposed; what fits one group of the grouped
     // route below is faster there (192 x 188 KB: 11.3 us against 14.9; 128 x 301 KB: 11.5 against 13.5)
-    constexpr long long kOneGroup = 64ll << 20, kGroup = 40ll << 20;
+    constexpr long long kOneGroup = 64ll << 20, kGroup = kOneGroup;
     if (rounds > 1 && total_bytes > (24ll << 20) && total_bytes <= kOneGroup) cluster = 0;
     if (cluster) {
         const cudaError_t attr_err = raise_smem_limit(actq::act_quant_cluster_kernel, d.smem_optin - 4096);
@@ -2051,14 +2051,14 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
         }
     }
 
-    // groups of samples, maxima of one beside the codes of the one before
+    // groups of samples, the codes of one behind the maxima of the next
     if (per_sample % 4 == 0) {
         actq::GroupArgs a;
         memset(&a, 0, sizeof(a));
         a.x = x_dev; a.per = per_sample; a.pieces = (per_sample + actq::kPiece - 1) / actq::kPiece;
         a.eps = eps; a.q = q_dev; a.gamma = gamma_dev; a.scale = scale_dev;
-        // groups of about 40 MB (32 to 64 are alike, 16 cost 20 % more launches' worth); up to 64 MB in one
-        long long per_group = total_bytes <= kOneGroup ? batch : kGroup / (per_sample * 4);
+        // (groups of up to 64 MB: with 40, or 24, more launches; 6 samples of 23.0 MB 54 us, with 64 47)
+        long long per_group = kGroup / (per_sample * 4);
         if (per_group < 1) per_group = 1;
         const long long groups = (batch + per_group - 1) / per_group;
         per_group = (batch + groups - 1) / groups;
@@ -2077,7 +2077,7 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
             long long blocks = (most + 31) / 32;
             if (blocks > 2 * d.sms) blocks = 2 * d.sms;
             fill_launch_cfg(cfg, attr, (int)blocks, actq::kGroupThreads, 0, st, true);
-            e = cudaLaunchKernelEx(&cfg, actq::act_group_kernel, a);
+            e = cudaLaunchKernelEx(&cfg, groups > 1 ? actq::act_group_kernel<true> : actq::act_group_kernel<false>, a);
             ++g_launches;
         }
         return cuda_status(e);

@@ -1,5 +1,5 @@
-"""The activation quantiser's grouped route (several kernels, maxima of one group of samples beside the codes
-of the one before) and its choice of cluster sizes: codes, gamma and scale bit for bit against the oracle."""
+"""The activation quantiser's grouped route (several kernels, codes of one group of samples and then the maxima of
+the next) and its choice of cluster sizes: codes, gamma and scale bit for bit against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("batch,per", [
     (1, 4), (3, 1004), (70, 1020), (5, 1028),         # not multiples of 16: pieces of 1024 floats and remainders
     (1, 450560), (2, 500004), (19, 460000),           # beyond eight SMs' shared memory, in one group
-    (30, 900004),                                     # 108 MB: three groups
+    (30, 900004), (3, 16800004),                      # 108 MB: two groups; samples larger than a group
     (200, 94080), (297, 47040), (150, 12288), (37, 100352),   # one and several rounds of clusters
 ])
 def test_routes(oracle, batch, per):
