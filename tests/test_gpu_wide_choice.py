@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 def test_capture_before_and_after_the_scratch_exists(oracle):
-    m = 148 * 128                                        # one row tile per SM: the row-resident kernel's smallest
+    m = 148 * 128                                        # well above the 40 rows per SM from which it is the kernel's
     x, lay = make_case(3, m, 640, 256)
     xd, wp, consts = to_device(x, lay)
     rq = binding.make_requant(*consts)
@@ -54,3 +54,50 @@ def test_around_the_choice(oracle, m, cout):
     rows = np.r_[0:300, m // 2:m // 2 + 300, m - 300:m]
     want = oracle.conv_mul(x.numpy()[rows], lay["w"].numpy(), lay["bias"].numpy(), lay["mult"].numpy(), lay["shift"].numpy(), 0, 127)
     assert np.array_equal(y.cpu().numpy()[rows], want)
+
+
+def _rows(per_sm):
+    return per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+
+
+def _launches(m, cin, cout, lo, hi):
+    """How many kernels a plain call launches (1: weight-resident, 2: operands and row-resident kernel), its result
+    checked against the plain kernel."""
+    x, lay = make_case(m + cin + cout, m, cin, cout)
+    xd, wp, consts = to_device(x, lay)
+    rq = binding.make_requant(*consts, lo, hi)
+    want = binding.pw_conv_i8(xd, wp, cout, rq, variant="naive")
+    before = binding.launch_count()
+    y = binding.pw_conv_i8(xd, wp, cout, rq)
+    n = binding.launch_count() - before
+    assert torch.equal(y, want)
+    return n
+
+
+@pytest.mark.parametrize("lo", [0, -128])
+@pytest.mark.parametrize("per_sm,cin,cout", [(80, 320, 256), (80, 960, 64), (40, 512, 240), (40, 576, 160), (20, 576, 320)])
+def test_rules_of_plain_calls(per_sm, cin, cout, lo):
+    m = _rows(per_sm)
+    assert _launches(m, cin, cout, lo, 127) == 2
+    assert _launches(m - 1, cin, cout, lo, 127) == 1
+    assert _launches(m, cin - 16, cout, lo, 127) == 1
+    if cout > 64:                                        # (960 inputs: any width from 64 on)
+        assert _launches(m, cin, cout - 16, lo, 127) == 1
+    assert _launches(m, cin, cout, lo, 126) == 1         # another clamp
+
+
+@pytest.mark.parametrize("per_sm,cin,cout", [(80, 320, 512), (80, 576, 240), (80, 960, 160), (40, 960, 320), (20, 576, 960)])
+def test_rules_of_prepared_calls(per_sm, cin, cout):
+    def kernel(m, k, n):
+        sizes = []
+        for mode in (0, 1, 2):
+            binding.debug_tc_wide(mode)
+            sizes.append(binding.lib().prom_pw_prepared_bytes(m, k, n))
+        binding.debug_tc_wide(0)
+        assert sizes[1] != sizes[2]
+        return "row-resident" if sizes[0] == sizes[2] else "weight-resident"
+    m = _rows(per_sm)
+    assert kernel(m, cin, cout) == "row-resident"
+    assert kernel(m - 1, cin, cout) == "weight-resident"
+    assert kernel(m, cin - 16, cout) == "weight-resident"
+    assert kernel(m, cin, cout - 16) == "weight-resident"
