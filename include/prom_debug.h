@@ -22,7 +22,9 @@ extern "C" {
  * makes TC report PROM_ERR_UNSUPPORTED.  The override is process-wide (one
  * lock guards it; a call that plans while another thread changes it sees the
  * old or the new override, never a mixture).  prom_debug_tc_plan_query writes
- * the plan the library would use for a plain [m][cin] x [cout] layer ({fold,
+ * the plan of the weight-resident kernel for a plain [m][cin] x [cout] layer under
+ * PROM_VARIANT_TC (AUTO also folds an odd number of rows, and cuts small layers
+ * into subtiles of any multiple of 8) ({fold,
  * nt, groups, grid, stages, accumulators, shared bytes, chunk bytes, estimate
  * in 1/100 us}) and returns 1, or returns 0 if TC cannot run it.  Without a
  * CUDA device it plans for a B200's nominal limits (148 SMs, 227 KB of shared
@@ -63,21 +65,23 @@ void prom_debug_seq_chain(int mode);
 void prom_debug_seq_order(int alternate);
 
 /* Which kernel prom_dw_conv3x3_i8 runs: 0 = the library's choice (default: TMA
- * patches and tensor-core taps for stride 1 with a channel count that is a
- * multiple of 16 and images of at least 100 pixels, CUDA cores otherwise), 1 = CUDA cores only, 2 = tensor cores
+ * and tensor-core taps for channel counts that are multiples of 16 and at least
+ * 4 Mi outputs, of either stride, CUDA cores otherwise), 1 = CUDA cores only, 2 = tensor cores
  * or PROM_ERR_UNSUPPORTED.  Results do not depend on it.  Process-wide. */
 void prom_debug_dw_variant(int variant);
 
 /* Which kernel the tensor-core variant of a single pointwise call runs: 0 = the
- * library's choice (the row-resident kernel, which keeps 128 rows with all their
- * input channels in shared memory and streams the weight matrix past them, for
- * layers with Cin >= 640, Cout >= 256 (nearly a multiple of 128, or at least 640), the clamp
- * [0, 127] and at least one tile of 128 rows per SM;
- * the weight-resident kernel otherwise), 1 = the weight-resident kernel only, 2 = the row-resident kernel
+ * library's choice (the row-resident kernel, in which a pair of CTAs keeps 256 rows with all
+ * their input channels in shared memory and streams the weight matrix past them,
+ * by a rule on rows per SM, Cin, Cout and the clamp, which stands in wide_plan and for
+ * prepared operands in wide_prepared_worth; the weight-resident kernel otherwise),
+ * 1 = the weight-resident kernel only, 2 = the row-resident kernel
  * or PROM_ERR_UNSUPPORTED (it takes plain matrices with Cin and Cout multiples
  * of 16, 128 <= Cin <= 1024, Cout >= 64, no residual).  blocks: 128-channel
- * blocks per column tile of that kernel, 1 (MMA N = 128) or 2 (N = 256; on
- * request for Cin <= 512 only), 0 = the planner's choice.  Results do not depend on either.  Process-wide. */
+ * blocks per column tile of that kernel, 1 (MMA N = 128; only here, for tests) or 2 (N = 256, the
+ * library's; asked for by number only up to Cin 512), 0 = the library's choice.  Results do not depend on
+ * either, but the layout of prepared operands does: they are used under the setting they were made under.
+ * Process-wide. */
 void prom_debug_tc_wide(int mode, int blocks);
 
 /* Where layer `layer`'s output ([rows][cout] int8) sits in the workspace of a

@@ -815,7 +815,7 @@ static bool wide_plan(const Conv &c, const DeviceInfo &d, WidePlan &pl, bool &wo
     p.ksteps_last = (c.cin - (p.kc - 1) * wide::kChunk + 31) / 32;
     p.n_mtiles = (int)((c.m + 255) / 256);
     pl.k_pad = p.kc * wide::kChunk;
-    // 256-channel column tiles; the tests ask for 128, or for 256 where a CTA of its own could hold them
+    // 256-channel column tiles; 128 (and 256 by number, up to Cin 512) only through prom_debug_tc_wide, for tests
     const int forced = g_wide_nb.load();
     if (forced == 2 && c.cin > 512) return false;
     const int nb = forced ? forced : 2;
@@ -862,7 +862,8 @@ static bool wide_plan(const Conv &c, const DeviceInfo &d, WidePlan &pl, bool &wo
 // 401408): Cin 960, Cout 160: 0.76 0.92 0.87, 1280: 0.57 0.56 0.51; Cin 576, Cout 240: 0.85 0.74 0.49, but 160: 0.81
 // 0.95 1.06; Cin 320, Cout 576: 0.99 0.95 0.97, 1280: 0.92 0.91 0.83, but 384: 1.11 1.06 0.91; Cin 192, Cout 1280:
 // 1.01 0.99 1.00.  On 6272 rows Cin 960, Cout 320 0.99, 576 0.85, but Cin 576: 1.02 1.07; on 3136 rows Cin 576,
-// Cout 960 0.97, 1280 0.82.
+// Cout 960 0.97, 1280 0.82.  Other clamps, the 64-bit epilogue in both kernels: 0.67 to 1.0 from 25088 rows on (576 ->
+// 240 1.15), on 6272 and 12544 rows 0.76 to 1.15.  (The size of the buffer is asked for without the clamp.)
 static bool wide_prepared_worth(const Conv &c, const DeviceInfo &d)
 {
     const long long rows_per_sm = c.m / d.sms;

@@ -10,7 +10,7 @@
 // by one comparison: clip(round(v), -1, 1) is 0 for |v| <= 1/2 (ties go to the even 0) and the sign
 // otherwise, |W| * scale is monotone in |W|, so the row has one float threshold, found from the
 // binary64 definition at the floats around mean / 2.  All 34 matrices of MobileNetV2 (9.1 MB, floor
-// 1.4 us at the copy bandwidth), calls back to back: 10.3 us with two reads and binary64 decisions, 8.0 us now.
+// 1.4 us at the copy bandwidth), calls back to back: 10.3 us with two reads and binary64 decisions, 7.3 us now.
 #pragma once
 
 #include "common.cuh"

@@ -10,10 +10,10 @@
 // 256 x 256 x 32): each CTA holds half of a column tile's weights, so that per 128 clocks of the tensor
 // pipe a CTA's shared memory is read for 4 KB of rows and 4 KB of weights and written with 4 KB, 96 of the
 // 128 bytes per clock that it can take, and 32 bytes per clock come from L2.  (One CTA alone with 128 x 128 x 32
-// MMAs needs 128 + 64 bytes per clock, and 64 of the 61.5 measured from L2.)
+// MMAs needs 128 + 64 bytes per clock, and 64 from L2, of which 58 to 61 were measured.)
 // 1.6 M x 960 -> 1280: 1615-1670 us with single CTAs, 1460-1480 with pairs, under the power cap in both.
 //
-// wide_prep_kernel (one CTA per column tile) expands the 2-bit weights into an int8 matrix
+// wide_prep_kernel (kPrepParts CTAs per 128 channels) expands the 2-bit weights into an int8 matrix
 // [Cout padded to 128][Cin padded to 128] in global scratch, scaled for the one-multiply
 // epilogue of tc.cuh where the tile's constants allow it, and writes the tile's bias digits
 // and requantisation constants beside it.  The convolution kernel reads that matrix through a
