@@ -64,6 +64,15 @@ void prom_debug_seq_chain(int mode);
  * from the first to the last.  Results do not depend on it.  Process-wide. */
 void prom_debug_seq_order(int alternate);
 
+/* Blocks inside prom_pw_layer_seq (an expanding pointwise layer and the layer with a
+ * depthwise convolution behind it, channel counts multiples of 8) in one launch each, the
+ * tensors between them kept in shared memory: 0 = where the library's rule finds it faster
+ * (default), 1 = never, 2 = wherever the shape allows it.  rows: output rows per band, split: CTAs
+ * per cluster that share a band's channels (0 = the planner's; a combination that does not fit leaves
+ * the block to one launch per layer).  Results do not depend on it; the workspace size does.
+ * prom_debug_layer_seq_output_offset returns -2 for the expanding layer.  Process-wide. */
+void prom_debug_seq_block(int mode, int rows, int split);
+
 /* Which kernel prom_dw_conv3x3_i8 runs: 0 = the library's choice (default: TMA
  * and tensor-core taps for channel counts that are multiples of 16 and at least
  * 4 Mi outputs, of either stride, CUDA cores otherwise), 1 = CUDA cores only, 2 = tensor cores

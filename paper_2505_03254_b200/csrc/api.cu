@@ -28,6 +28,7 @@
 #include "depthwise.cuh"
 #include "dwtc.cuh"
 #include "wide.cuh"
+#include "block.cuh"
 #include "stack.cuh"
 #include "quantize.cuh"
 #include "peak.cuh"
@@ -1319,6 +1320,228 @@ static bool make_y_map(CUtensorMap *map, int8_t *y, int nf, long long rows, int 
 }
 
 // Where everything of a sequence sits in the caller's workspace.
+// ---- depthwise kernels: which one, for the layers and for the rule on blocks ----------------------
+// 0: the library's choice, 1: CUDA cores only, 2: tensor cores or PROM_ERR_UNSUPPORTED
+static std::atomic<int> g_dw_variant{0};
+// Outputs from which the tensor-core kernel (dwtc.cuh) is the better one: a call of it costs about 6 us whatever its
+// size (tensor memory and weight blocks to set up, one CTA of 190 KB per SM, so that little of this
+// overlaps the kernel in front) against 3 us, and then 0.4 us per million outputs against 1.0 (stride 1)
+// and 0.8 against 1.8 (stride 2).  Measured alone the lines cross at 3.3 to 5.6 million, inside the
+// network's body at 3 to 6 million.
+constexpr long long kDwTcOutputs = 4ll << 20;
+
+// ---- whole blocks of a sequence in one launch (block.cuh) ------------------------------------------
+// g_block_mode: 0: the library's choice, 1: never, 2: wherever a block qualifies; with a band height and a number of
+// CTAs per cluster for tests (0: the planner's)
+static std::atomic<int> g_block_mode{0}, g_block_rows{0}, g_block_split{0};
+
+struct BlockPlan {
+    block::Params p;
+    int grid = 0;
+    size_t smem = 0, image_bytes = 0;
+    double est_us = 0;
+};
+
+// Clusters of block_kernel that a GPU holds at once (a cluster lies within one of its processing clusters).
+static int block_resident(int csize, const DeviceInfo &d)
+{
+    static const int b200[block::kMaxCluster + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+    const int n = d.sms >= 148 ? b200[csize] : d.sms / csize * 9 / 10;
+    return n > 0 ? n : 1;
+}
+
+// The geometry of one candidate: `rows` output rows per band, `ipi` images per item, `per_cta` slices per CTA.
+static bool block_fill(int c0, int ce, int co, int batch, int h, int w, int stride, int rows, int ipi, int per_cta,
+                       const DeviceInfo &d, BlockPlan &pl)
+{
+    block::Params &p = pl.p;
+    memset(&p, 0, sizeof(p));
+    p.batch = batch; p.h = h; p.w = w; p.stride = stride;
+    p.ho = (h - 1) / stride + 1; p.wo = (w - 1) / stride + 1;
+    p.c0 = c0; p.co = co; p.npad = round_up(co, 16);
+    p.rows = rows; p.rin = stride == 1 ? rows + 2 : 2 * rows + 1;
+    p.bands = (p.ho + rows - 1) / rows; p.ipi = ipi;
+    if (ipi > 1 && p.bands != 1) return false;
+    const long long items = (long long)((batch + ipi - 1) / ipi) * p.bands;
+    if (items >= (1 << 30) || (long long)batch * h >= (1ll << 31) || p.rin > 255 || ipi > 255) return false;
+    p.items = (int)items;
+    p.pitch = p.wo + 1;
+    p.qlen = stride == 1 ? p.rin * p.pitch : (rows + 1) * p.pitch;
+    const long long last = (long long)(ipi - 1) * p.qlen + (rows - 1) * p.pitch + p.wo;       // outputs in the buffer's order
+    const long long pixels = (long long)ipi * p.rin * w;
+    if (last > 128 * 16 || pixels > 128 * 24) return false;
+    p.t1 = (int)((pixels + 127) / 128); p.t2 = (int)((last + 127) / 128);
+    p.ks = (c0 + 31) / 32;
+    p.slices = (ce + block::kSlice - 1) / block::kSlice;
+    p.per_cta = per_cta;
+    p.csize = (p.slices + per_cta - 1) / per_cta;
+    if (p.csize > block::kMaxCluster) return false;
+    // pixel buffer: what the last output block's taps reach, and where the expanded pixels go
+    int reach = stride == 1 ? 128 * p.t2 + 2 * p.pitch + 3 : 128 * p.t2 + p.pitch + 2;
+    const int held = ipi * p.qlen + 2;
+    p.plane = round_up(reach > held ? reach : held, 8);
+    const int len = stride == 1 ? p.plane : 4 * p.plane;
+    if (len > 65535) return false;
+    p.e_bytes = (uint32_t)round_up(len * block::kSlice, 1024);
+    p.last_half = (ce - 1) % block::kSlice < block::kHalf;
+    for (int dy = 0; dy < 3; ++dy)
+        for (int dx = 0; dx < 3; ++dx)
+            p.tap[3 * dy + dx] = (stride == 1 ? dy * p.pitch + dx
+                                              : ((dy & 1) * 2 + (dx & 1)) * p.plane + (dy >> 1) * p.pitch + (dx >> 1)) *
+                                 block::kSlice / 16;
+    p.px = (c0 & 15) ? c0 / 8 : c0 / 16;
+    p.px_magic = (uint32_t)(((1ull << 32) + p.px - 1) / p.px);
+    if (pixels * p.px >= (1 << 20) || (long long)ipi * h * w * c0 >= (1ll << 31)) return false;
+    p.x_bytes = (uint32_t)(p.t1 * p.ks) * block::kStepBytes;
+    p.slice_bytes = block::slice_bytes(p.ks, p.npad);
+    pl.image_bytes = (size_t)p.slices * p.slice_bytes;
+    p.rpc = (ipi * rows * p.wo + p.csize - 1) / p.csize;
+    p.xpitch = co + 4;
+    auto magic = [](int v) { return v > 1 ? (uint32_t)(((1ull << 32) + v - 1) / v) : 0u; };
+    p.per_img_magic = magic(p.rin * w); p.w_magic = magic(w); p.qlen_magic = magic(p.qlen); p.pitch_magic = magic(p.pitch);
+    // tensor memory
+    const int d3 = p.t2 * p.npad, cols = 512;
+    p.n1 = 4; p.n2 = 4;
+    p.chunks = p.t2 * ((co + 31) / 32);
+    while (block::kSlice * (p.n1 + p.n2) + d3 > cols && p.n1 + p.n2 > 2) { if (p.n2 >= p.n1) p.n2 /= 2; else p.n1 /= 2; }
+    if (block::kSlice * (p.n1 + p.n2) + d3 > cols) return false;
+    p.d2_col = block::kSlice * p.n1; p.d3_col = p.d2_col + block::kSlice * p.n2;
+    p.tmem_cols = cols;
+    // (a read of 32 columns may go past the sums' last ones)
+    const int used = p.d3_col + (p.t2 - 1) * p.npad + round_up(p.npad, 32);
+    if (used > cols) return false;
+    while (p.tmem_cols > 32 && used <= p.tmem_cols / 2) p.tmem_cols /= 2;
+    // shared memory: rings as deep as fit
+    auto layout = [&](int ne, int ns, int np, int nx) {
+        p.ne = ne; p.ns = ns; p.np = np; p.nx = nx;
+        uint32_t o = (uint32_t)nx * p.x_bytes;
+        p.off_e = o; o += (uint32_t)ne * p.e_bytes;
+        p.off_p = o; o += (uint32_t)np * block::kUnitBytes;
+        p.off_w = (o + 1023u) & ~1023u; o = p.off_w + (uint32_t)ns * p.slice_bytes;
+        const uint32_t exch = (uint32_t)(p.csize > 1 ? p.csize * p.rpc * p.xpitch * 4 : 0);
+        if (o < exch) o = exch;
+        p.off_aconst = (o + 1023u) & ~1023u; o = p.off_aconst + tc::kAConstBytes;
+        p.off_etab = o; o += 512u * (uint32_t)p.t1;
+        p.off_otab = o; o += 512u * (uint32_t)p.t2;
+        p.off_pc = o; o += 16u * (uint32_t)p.npad;
+        p.off_bars = (o + 15u) & ~15u; o = p.off_bars + block::kBarBytes + 32u;
+        return (size_t)o + 1024;
+    };
+    const bool one_item = p.csize > 1;
+    static const int rings[][4] = {{4, 5, 4, 2}, {4, 4, 4, 2}, {4, 4, 4, 1}, {4, 4, 2, 1}, {2, 4, 4, 2}, {2, 3, 4, 2}, {2, 3, 2, 2}, {2, 3, 4, 1}, {2, 3, 2, 1}, {2, 2, 2, 1}};
+    bool fits = false;
+    for (const auto &r : rings) {
+        int ns = r[1], nx = one_item ? 1 : r[3], ne = r[0], np = r[2];
+        if (p.items <= d.sms) nx = 1;          // one item per CTA
+        if (one_item && ns > per_cta) ns = per_cta;
+        if (one_item) while (ne > per_cta) ne /= 2;
+        p.ahead = ne > 1 ? ne - 1 : 1;
+        pl.smem = layout(ne, ns, np, nx);
+        if ((fits = pl.smem <= (size_t)d.smem_optin)) break;
+    }
+    if (!fits) return false;
+    // a cluster takes one item; single CTAs stay and take one after the other
+    const long long room = d.sms;
+    p.clusters = p.csize > 1 ? p.items : (int)(p.items < room ? p.items : room);
+    pl.grid = p.clusters * p.csize;
+    // Time model, in cycles, fitted to 18 thousand timings (3297 shapes of the networks in several geometries; standard
+    // error 8 %, the chosen geometry within 1 % of the best timed one on average).  What counts are the tensor pipe's
+    // reads of shared memory (an MMA of 32 columns reads 5 KB, beside the epilogue's traffic), slices that are not asked
+    // for early enough, what surrounds an item, and the rounds of resident clusters.
+    const double tensor = 1.88 * (p.t1 * 48.0 * (p.ks + 1) + p.t2 * (800.0 + (p.npad > 80 ? p.npad : 80))) *
+                          (p.slices - 0.5 * p.last_half) / p.slices;
+    const int mine = p.csize > 1 ? 1 : (p.items + p.clusters - 1) / p.clusters;
+    const int resident = block_resident(p.csize, d);
+    const int waves = p.csize > 1 ? (p.items + resident - 1) / resident : 1;
+    const bool late = p.ns < p.ahead + 2 && p.per_cta * mine > p.ns;
+    const double slice = tensor + 680.0 / p.ahead + (late ? 540.0 + p.slice_bytes / 640.0 : 0.0);
+    const double around = 4440.0 + tensor + (p.csize > 1 ? 7540.0 + 10.8 * p.t2 * p.npad : 0.0);
+    const double item = 777.0 * p.t1 + (p.csize > 1 ? 0.0 : 4090.0 * ((p.chunks + block::kGroups - 1) / block::kGroups));
+    pl.est_us = (8625.0 + waves * (around + (double)p.per_cta * mine * slice) + mine * item) / 1900.0;
+    return true;
+}
+
+// Whether layers l[0], l[1] (rows of batch images of h x w pixels) are a block that block_kernel takes.
+static bool block_layers_ok(const prom_layer *l)
+{
+    const prom_layer &e = l[0], &q = l[1];
+    return !e.dw_w && e.in_stride == 1 && !e.add_block_input && q.dw_w && (e.cin & 7) == 0 && (e.cout & 7) == 0 &&
+           (q.cout & 7) == 0 && q.cout <= 384 && e.cin <= 512 && e.cout >= 32;
+}
+
+// Whether one launch is expected to beat one per layer, whose time (us) is a fit to the same shapes (standard error
+// 9 %).  Inside a sequence a block saves about 1.2 us more than calls of its own show, whose preparation is not shared.
+// With this margin 43 % of the shapes run as blocks, in 0.88 of the layers' time; 4 % of all are slower by more than 3 %
+// (with a margin of 1: 77 %, 0.92 and 13 %).  Mostly they are planes of 10 to 60 thousand pixels, batch included:
+// larger ones are bound by the requantiser and the taps either way, and their units leave gaps here.
+static bool block_worth(const BlockPlan &pl, int ce)
+{
+    const block::Params &p = pl.p;
+    const double in = (double)p.batch * p.h * p.w * ce * 1e-6, out = (double)p.batch * p.ho * p.wo * ce * 1e-6;
+    const bool tensor_taps = (ce & 15) == 0 && out * 1e6 >= (double)kDwTcOutputs;
+    const double layers = 12.5 + 0.28 * in + (tensor_taps ? 5.7 + 0.39 * out : 2.04 * out) + 0.22e-4 * p.c0 * ce +
+                          0.014e-4 * ce * p.co + 1.34 * out * p.co / ce + (p.c0 & 15 ? 1.5 + 0.13 * in : 0.0);
+    return pl.est_us - 1.2 < 0.9 * layers;
+}
+
+typedef std::array<int, 10> BlockKey;
+static bool block_plan(int c0, int ce, int co, int batch, int h, int w, int stride, const DeviceInfo &d, BlockPlan &best)
+{
+    const int f_rows = g_block_rows.load(), f_split = g_block_split.load();
+    const BlockKey key = {c0, ce, co, batch, h, w, stride, d.dev, f_rows, f_split};
+    static std::mutex mu;
+    static std::map<BlockKey, std::pair<bool, BlockPlan>> cache;
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = cache.find(key);
+    if (it == cache.end()) {
+        bool found = false;
+        BlockPlan top;
+        const int ho = (h - 1) / stride + 1, slices = (ce + block::kSlice - 1) / block::kSlice;
+        for (int bands = 1; bands <= ho; ++bands) {
+            const int rows = (ho + bands - 1) / bands;
+            if (bands > 1 && rows == (ho + bands - 2) / (bands - 1)) continue;
+            if (f_rows > 0 && rows != (f_rows < ho ? f_rows : ho)) continue;
+            for (int ipi = 1; ipi <= (bands == 1 ? 8 : 1) && ipi <= batch; ++ipi)
+                for (int c = 1; c <= block::kMaxCluster && c <= slices; ++c) {
+                    const int per = (slices + c - 1) / c;
+                    if ((slices + per - 1) / per != c) continue;
+                    if (f_split > 0 && c != f_split) continue;
+                    BlockPlan pl;
+                    if (!block_fill(c0, ce, co, batch, h, w, stride, rows, ipi, per, d, pl)) continue;
+                    if (!found || pl.est_us < top.est_us) { top = pl; found = true; }
+                }
+        }
+        if (cache.size() > 4096) cache.clear();
+        it = cache.emplace(key, std::make_pair(found, top)).first;
+    }
+    if (it->second.first) best = it->second.second;
+    return it->second.first;
+}
+
+static prom_status launch_block(BlockPlan &pl, const int8_t *x, int8_t *y, const int8_t *res, const uint8_t *image,
+                                const prom_layer *l, int pdl, cudaStream_t st)
+{
+    block::Params &p = pl.p;
+    p.x = x; p.y = y; p.res = res; p.image = image;
+    p.bias = l[1].rq.bias; p.mult = l[1].rq.mult; p.shift = l[1].rq.shift;
+    p.lo_e = l[0].rq.act_min; p.hi_e = l[0].rq.act_max;
+    p.lo_d = l[1].dw_rq.act_min; p.hi_d = l[1].dw_rq.act_max;
+    p.lo_p = l[1].rq.act_min; p.hi_p = l[1].rq.act_max;
+    p.pdl = pdl;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    fill_launch_cfg(cfg, attr, pl.grid, block::kThreads, pl.smem, st, true);
+    if (p.csize > 1) {
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = (unsigned)p.csize;
+        attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+        cfg.numAttrs = 2;
+    }
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, block::block_kernel, p);
+    ++g_launches;
+    return cuda_status(e);
+}
+
 struct SeqLayout {
     size_t ra = 0, rb = 0, dw_off = 0;     // the two ping-pong regions (b ends with the depthwise buffer)
     std::vector<size_t> img_off;           // per layer: prepared image of a one-launch layer, or -1
@@ -1327,24 +1550,73 @@ struct SeqLayout {
     std::vector<int> chain_of;             // per layer: its chain, or -1
     std::vector<size_t> cimg_off, cbuf_off;   // per chain layer: images, output buffer
     size_t cimg_total = 0, cbuf_total = 0;
+    std::vector<BlockPlan> blocks;         // layers taken two at a time by one launch
+    std::vector<int> block_of;             // per layer: its block, or -1
+    std::vector<size_t> bimg_off;          // per block: its slices' operands
+    size_t bimg_total = 0;
+    std::vector<char> region;              // per layer: the region its output goes to
+    size_t plain_base = 0;                 // regions of one launch per layer (what a workspace must hold at least)
     size_t base() const { return ra + rb; }
     size_t with_images() const { return round256(base()) + img_total; }
+    size_t with_blocks() const { return round256(with_images()) + bimg_total; }
     size_t with_chains() const { return round256(with_images()) + cimg_total + cbuf_total; }
 };
 
+// The blocks of a sequence: an expanding pointwise layer and, behind it, a layer with a depthwise convolution.
+// What lies between them is not written, so the two regions take the outputs of what is left in turn.
+static void find_blocks(const prom_layer *layers, int n, const SeqShape &s, const DeviceInfo &d, SeqLayout &L)
+{
+    const int mode = g_block_mode.load();
+    if (mode == 1 || g_dw_variant.load() != 0) return;
+    for (int i = 0; i + 1 < n; ++i) {
+        if (L.block_of[i] >= 0 || !block_layers_ok(layers + i) || s.m[i + 1] <= 0) continue;
+        BlockPlan pl;
+        const int batch = (int)(s.m[i] / ((long long)s.h[i] * s.w[i]));
+        if (!block_plan(layers[i].cin, layers[i].cout, layers[i + 1].cout, batch, s.h[i], s.w[i], layers[i + 1].in_stride, d, pl))
+            continue;
+        if (mode == 0 && !block_worth(pl, layers[i].cout)) continue;
+        L.block_of[i] = L.block_of[i + 1] = (int)L.blocks.size();
+        L.blocks.push_back(pl);
+        L.bimg_off.push_back(L.bimg_total);
+        L.bimg_total += round256(pl.image_bytes);
+    }
+    if (L.blocks.empty()) return;
+    size_t r[2] = {0, 0}, c = 0;
+    int side = 1;
+    for (int i = 0; i < n; ++i) {
+        const bool in_block = L.block_of[i] >= 0;
+        if (in_block && i + 1 < n && L.block_of[i + 1] == L.block_of[i]) continue;         // has no output
+        side ^= 1;
+        L.region[i] = (char)side;
+        const size_t bytes = round256((size_t)s.m[i] * layers[i].cout);
+        if (i + 1 < n && bytes > r[side]) r[side] = bytes;
+        if (layers[i].dw_w && !in_block) {
+            const size_t b = round256((size_t)s.m[i] * layers[i].cin);
+            if (b > c) c = b;
+        }
+    }
+    L.ra = r[0]; L.rb = r[1] + c; L.dw_off = r[0] + r[1];
+}
+
 static void seq_layout(const prom_layer *layers, int n, const SeqShape &s, const DeviceInfo &d, bool want_tc,
-                       SeqLayout &L, bool allow_chains = true)
+                       SeqLayout &L, bool allow_chains = true, bool allow_blocks = true)
 {
     seq_regions(layers, n, s, L.ra, L.rb, &L.dw_off);
+    L.plain_base = L.base();
     L.chain_of.assign(n, -1);
+    L.block_of.assign(n, -1);
+    L.region.assign(n, 0);
+    for (int i = 0; i < n; ++i) L.region[i] = (char)(i & 1);
     L.img_off.assign(n, (size_t)-1);
     L.cimg_off.assign(n, 0);
     L.cbuf_off.assign(n, 0);
     if (!want_tc || !d.ok) return;
     if (allow_chains) find_chains(layers, n, s, d, L.chains);
+    if (allow_blocks && L.chains.empty()) find_blocks(layers, n, s, d, L);
     for (size_t c = 0; c < L.chains.size(); ++c)
         for (int i = L.chains[c].first; i <= L.chains[c].last; ++i) L.chain_of[i] = (int)c;
     for (int i = 0; i < n; ++i) {
+        if (L.block_of[i] >= 0) continue;
         if (L.chain_of[i] >= 0) {
             const ChainPlan &c = L.chains[L.chain_of[i]];
             L.cimg_off[i] = L.cimg_total;
@@ -1374,14 +1646,6 @@ static void seq_layout(const prom_layer *layers, int n, const SeqShape &s, const
 
 
 // ---- depthwise 3x3 on the tensor cores (dwtc.cuh) ---------------------------------------------
-// 0: the library's choice, 1: CUDA cores only, 2: tensor cores or PROM_ERR_UNSUPPORTED
-static std::atomic<int> g_dw_variant{0};
-// Outputs from which the tensor-core kernel is the better one: a call of it costs about 6 us whatever its
-// size (tensor memory and weight blocks to set up, one CTA of 190 KB per SM, so that little of this
-// overlaps the kernel in front) against 3 us, and then 0.4 us per million outputs against 1.0 (stride 1)
-// and 0.8 against 1.8 (stride 2).  Measured alone the lines cross at 3.3 to 5.6 million, inside the
-// network's body at 3 to 6 million.
-constexpr long long kDwTcOutputs = 4ll << 20;
 
 template <int STRIDE>
 static prom_status launch_dw_tc(const int8_t *x, int batch, int h, int w, int c, const int8_t *wt,
@@ -1596,6 +1860,8 @@ static prom_status launch_stack(const prom_layer *layers, const SeqShape &s, con
     return cuda_status(e);
 }
 
+static bool seq_overlap(const int8_t *a, size_t na, const int8_t *b, size_t nb) { return a < b + nb && b < a + na; }
+
 static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, int batch, int h0,
                            int w0, void *ws, size_t ws_bytes, int8_t *y_out, prom_variant variant,
                            cudaStream_t st)
@@ -1620,14 +1886,20 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
     const bool want_tc = variant == PROM_VARIANT_TC || variant == PROM_VARIANT_AUTO;
     SeqLayout lay;
     seq_layout(layers, n, s, d, want_tc, lay);
-    const size_t ra = lay.ra, rb = lay.rb;
-    if (ra + rb > 0) {
+    if (lay.plain_base > 0) {
         if (!ws) return PROM_ERR_NULL;
         if (!aligned16(ws)) return PROM_ERR_ALIGN;
-        if (ws_bytes < ra + rb) return PROM_ERR_WORKSPACE;
+        if (ws_bytes < lay.plain_base) return PROM_ERR_WORKSPACE;
     }
     if (!d.ok) return PROM_ERR_CUDA;
-    int8_t *reg[2] = {static_cast<int8_t *>(ws), static_cast<int8_t *>(ws) + ra};
+    // A block reads rows of its input that other CTAs' outputs stand for, so the two may not overlap; and
+    // its operands need room.  One launch per layer takes any workspace of the plain size.
+    if (!lay.blocks.empty() && (ws_bytes < lay.with_blocks() ||
+                                seq_overlap(x0, (size_t)batch * h0 * w0 * layers[0].cin, y_out, (size_t)s.m[n - 1] * layers[n - 1].cout))) {
+        lay = SeqLayout();
+        seq_layout(layers, n, s, d, want_tc, lay, true, false);
+    }
+    int8_t *reg[2] = {static_cast<int8_t *>(ws), static_cast<int8_t *>(ws) + lay.ra};
     int8_t *dw_buf = static_cast<int8_t *>(ws) + lay.dw_off;      // depthwise outputs
 
     // The images and the chains are optimisations: a workspace without room for them still works.
@@ -1639,7 +1911,7 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
     if (!chain_base && !lay.chains.empty()) {
         // no room: plan again without chains (their layers then want one-launch images)
         lay = SeqLayout();
-        seq_layout(layers, n, s, d, want_tc, lay, false);
+        seq_layout(layers, n, s, d, want_tc, lay, false, false);
         img_base = nullptr;
         if (ws && lay.img_total > 0 && ws_bytes >= lay.with_images())
             img_base = static_cast<uint8_t *>(ws) + round256(lay.base());
@@ -1650,17 +1922,20 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
     std::vector<TcPlan> plan(n);
     std::vector<char> is_tc(n, 0);
     std::vector<uint8_t *> chain_img(n, nullptr);
+    std::vector<const int8_t *> input(n, nullptr);
+    uint8_t *block_base = lay.blocks.empty() ? nullptr : static_cast<uint8_t *>(ws) + round256(lay.with_images());
     const int8_t *cur = x0;
     long long in_rows = (long long)batch * h0 * w0;
     for (int i = 0; i < n; ++i) {
         Conv &c = conv[i];
-        const bool chained = lay.chain_of[i] >= 0;
+        const bool chained = lay.chain_of[i] >= 0, in_block = lay.block_of[i] >= 0;
+        input[i] = cur;
         // behind a depthwise convolution the pointwise layer reads that convolution's output
         c.x = layers[i].dw_w ? dw_buf : cur; c.m = s.m[i]; c.cin = layers[i].cin; c.cout = layers[i].cout;
         c.map = s.map[i]; c.in_rows = layers[i].dw_w ? s.m[i] : in_rows;
         c.w = layers[i].w_packed; c.rq = layers[i].rq;
         c.y = (i == n - 1) ? y_out
-              : (chained ? reinterpret_cast<int8_t *>(chain_base + lay.cbuf_off[i]) : reg[i & 1]);
+              : (chained ? reinterpret_cast<int8_t *>(chain_base + lay.cbuf_off[i]) : reg[(int)lay.region[i]]);
         c.st = st;
         // the first kernel waits before it reads anything (the operands prepared below included) and
         // before it releases its successor, so every later link finds weights and operands complete
@@ -1668,8 +1943,13 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
         c.pdl_next = true;
         // The block's input is the output of layer i-2, which sits where this layer's output
         // goes (unless a chain wrote it to a buffer of its own: then the sum reads from there).
-        if (layers[i].add_block_input) c.res = i == 1 ? x0 : conv[i - 2].y;
-        if (chained) {
+        if (layers[i].add_block_input) c.res = input[i - 1];
+        if (in_block) {
+            // (what one launch per layer refuses stays refused)
+            TcPlan tmp;
+            if (variant == PROM_VARIANT_TC && !tc_shape_plan(c.m, c.cin, c.cout, c.map, d, tmp, kPlanPrepared)) return PROM_ERR_UNSUPPORTED;
+            if (i + 1 < n && lay.block_of[i + 1] == lay.block_of[i]) continue;         // has no output: the next layer's input is this one's
+        } else if (chained) {
             chain_img[i] = chain_base + lay.cimg_off[i];
         } else if (want_tc && c.m > 0 && tc_shape_plan(c.m, c.cin, c.cout, c.map, d, plan[i],
                                                                variant == PROM_VARIANT_AUTO ? kPlanPrepared | kPlanOdd : kPlanPrepared)) {
@@ -1688,6 +1968,7 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
         bool writer_rev = true;             // the first layer walks forwards
         for (int i = 0; i < n; ++i) {
             if (layers[i].dw_w) writer_rev = false;
+            if (lay.block_of[i] >= 0) continue;
             const bool rev = is_tc[i] && lay.chain_of[i] < 0 && !writer_rev;
             if (is_tc[i]) plan[i].p.reverse = rev ? 1 : 0;
             writer_rev = rev;
@@ -1695,6 +1976,7 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
     }
 
     // one launch prepares the operands of every tensor-core layer (of a chain: one image per subtile)
+    bool prepared = false;              // such a launch of this call is in front
     if (img_base || chain_base) {
         int i = 0;
         while (i < n) {
@@ -1718,10 +2000,42 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
             cudaLaunchAttribute attr[1];
             fill_launch_cfg(cfg, attr, ctas, tc::kPrepThreads, smem, st, true);
             const cudaError_t e = cudaLaunchKernelEx(&cfg, tc::tc_prep_kernel, t);
+            prepared = true;
             ++g_launches;
             if (e != cudaSuccess) return PROM_ERR_CUDA;
         }
     }
+
+    // ... one launch those of the blocks
+    for (size_t k = 0; k < lay.blocks.size();) {
+        block::PrepTable t;
+        memset(&t, 0, sizeof(t));
+        t.behind = prepared ? 1 : 0;
+        prepared = true;
+        int ctas = 0;
+        for (; k < lay.blocks.size() && t.n < block::kMaxPrep; ++k) {
+            int i = 0;
+            while (lay.block_of[i] != (int)k) ++i;
+            const block::Params &p = lay.blocks[k].p;
+            const prom_layer &e = layers[i], &q = layers[i + 1];
+            block::PrepBlock &b = t.b[t.n++];
+            b.we = e.w_packed; b.wp = q.w_packed; b.wd = q.dw_w;
+            b.bias_e = e.rq.bias; b.mult_e = e.rq.mult; b.shift_e = e.rq.shift;
+            b.bias_d = q.dw_rq.bias; b.mult_d = q.dw_rq.mult; b.shift_d = q.dw_rq.shift;
+            b.image = block_base + lay.bimg_off[k];
+            b.c0 = e.cin; b.ce = e.cout; b.co = q.cout; b.npad = p.npad; b.ks = p.ks;
+            b.lo_e = e.rq.act_min; b.hi_e = e.rq.act_max; b.lo_d = q.dw_rq.act_min; b.hi_d = q.dw_rq.act_max;
+            b.first = ctas;
+            ctas += p.slices;
+        }
+        cudaLaunchConfig_t cfg;
+        cudaLaunchAttribute attr[1];
+        fill_launch_cfg(cfg, attr, ctas, block::kPrepThreads, 0, st, true);
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, block::block_prep_kernel, t);
+        ++g_launches;
+        if (e != cudaSuccess) return cuda_status(e);
+    }
+    if (!lay.blocks.empty() && raise_smem_limit(block::block_kernel, d.smem_optin) != cudaSuccess) return PROM_ERR_CUDA;
 
     // ... and one launch the operands of the runs that stay in shared memory
     if (chain_base) {
@@ -1762,9 +2076,17 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
             i = c.last;
             continue;
         }
+        if (lay.block_of[i] >= 0) {
+            const int k = lay.block_of[i];
+            const prom_status e = launch_block(lay.blocks[k], input[i], conv[i + 1].y, conv[i + 1].res, block_base + lay.bimg_off[k],
+                                               layers + i, i > 0 ? tc::kPdlChain : tc::kPdlWait, st);
+            if (e != PROM_OK) return e;
+            ++i;
+            continue;
+        }
         if (layers[i].dw_w && s.m[i] > 0) {
             const int stride = layers[i].in_stride;
-            const int8_t *src = i == 0 ? x0 : conv[i - 1].y;
+            const int8_t *src = input[i];
             // chained like the pointwise kernels: behind layer i-1's kernel (which releases its
             // dependents at entry) and in front of layer i's, which waits for it before its loads
             prom_status de = dw_conv3x3(src, batch, s.h[i] * stride, s.w[i] * stride, layers[i].cin, stride,
@@ -2291,7 +2613,13 @@ size_t prom_layer_seq_workspace_bytes(const prom_layer *layers, int n, int batch
     SeqLayout lay;
     seq_layout(layers, n, s, d, true, lay);
     if (!lay.chains.empty()) return lay.with_chains();
-    return lay.img_total ? lay.with_images() : lay.base();
+    const size_t blocks = lay.blocks.empty() ? 0 : lay.with_blocks();
+    if (blocks) {                 // room for one launch per layer too: what the call falls back on
+        lay = SeqLayout();
+        seq_layout(layers, n, s, d, true, lay, true, false);
+    }
+    const size_t plain = lay.img_total ? lay.with_images() : lay.base();
+    return blocks > plain ? blocks : plain;
 }
 
 prom_status prom_pw_layer_seq(const prom_layer *layers, int n, const int8_t *x0_dev, int batch,
@@ -2518,6 +2846,12 @@ prom_status prom_debug_mma_beside(int mode, int iters, int nwarps, int stages, c
 void prom_debug_seq_order(int alternate) { g_seq_snake.store(alternate ? 1 : 0); }
 void prom_debug_seq_chain(int mode) { g_seq_chain.store(mode == 2 ? 2 : (mode ? 1 : 0)); }
 
+void prom_debug_seq_block(int mode, int rows, int split)
+{
+    g_block_mode.store(mode < 0 || mode > 2 ? 0 : mode);
+    g_block_rows.store(rows);
+    g_block_split.store(split);
+}
 void prom_debug_dw_variant(int variant) { g_dw_variant.store(variant < 0 || variant > 2 ? 0 : variant); }
 
 void prom_debug_tc_wide(int mode, int blocks)
@@ -2541,7 +2875,11 @@ int64_t prom_debug_layer_seq_output_offset(const prom_layer *layers, int n, int 
         if (c.kind == 1 && layer != c.last) return -2;      // never written: it stays in shared memory
         return (int64_t)(round256(lay.with_images()) + lay.cbuf_off[layer]);
     }
-    return (layer & 1) ? (int64_t)lay.ra : 0;
+    if (lay.block_of[layer] >= 0 && lay.block_of[layer + 1] == lay.block_of[layer]) {
+        if (chained) *chained = 1;
+        return -2;                                          // a block's expanded tensor is never written
+    }
+    return lay.region[layer] ? (int64_t)lay.ra : 0;
 }
 
 int prom_debug_once_per_device(int device, int key)

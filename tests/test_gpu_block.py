@@ -1,0 +1,136 @@
+"""A block of a sequence (expand, depthwise 3x3, project with its skip connection) in one launch: bytes equal
+to the oracle's at the edges of its bands, units, slices, rings and clusters."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2505_03254_b200 import binding, synth
+from gpu_util import Guarded
+
+pytestmark = pytest.mark.gpu
+
+
+def _layer(rng, seed, cin, cout, stride=1, **kw):
+    d = synth.make_layer(seed, cin, cout, 0.5)
+    h = dict(cin=cin, cout=cout, in_stride=stride, w=d["w"].numpy(), bias=d["bias"].numpy(), mult=d["mult"].numpy(),
+             shift=d["shift"].numpy(), act_min=kw.get("act_min", 0), skip=kw.get("skip", False))
+    if "shift" in kw:
+        h["shift"] = kw["shift"].astype(np.int8)
+    if kw.get("dw"):
+        h["dw_w"] = rng.integers(-128, 128, size=(cin, 3, 3)).astype(np.int8)
+        h["dw_bias"] = rng.integers(-3000, 3001, size=cin).astype(np.int32)
+        h["dw_mult"] = rng.integers(1 << 30, (1 << 31) - 1, size=cin).astype(np.int32)
+        h["dw_shift"] = rng.integers(*kw.get("dw_shift", (8, 11)), size=cin).astype(np.int8)
+    dev = {k: v for k, v in h.items() if k not in ("w", "skip")}
+    dev = {k: torch.from_numpy(v).cuda() if isinstance(v, np.ndarray) else v for k, v in dev.items()}
+    dev["w_packed"] = binding.pack_ternary(d["w"].cuda())
+    dev["add_block_input"] = h["skip"]
+    return h, dev
+
+
+def _want(oracle, e, q, x):
+    b, h, w, c = x.shape
+    t = oracle.conv_mul(x.reshape(-1, c), e["w"], e["bias"], e["mult"], e["shift"], e["act_min"], 127).reshape(b, h, w, -1)
+    t = oracle.dw3x3(t, q["dw_w"], q["dw_bias"], q["dw_mult"], q["dw_shift"], stride=q["in_stride"], act_min=0, act_max=127)
+    b, h, w, c = t.shape
+    y = oracle.conv_mul(t.reshape(-1, c), q["w"], q["bias"], q["mult"], q["shift"], q["act_min"], 127).reshape(b, h, w, -1)
+    return oracle.residual_add(y, x) if q["skip"] else y
+
+
+def _run(dev, x, rows=0, split=0, mode=2):
+    binding.debug_seq_block(mode, rows, split)
+    try:
+        seq = binding.LayerSeq(dev)
+        b, h, w, _ = x.shape
+        fused = binding.debug_layer_seq_output_offset(seq, b, h, w, 0)[0] == -2
+        ws = Guarded(seq.workspace_bytes(b, h, w), dtype=torch.uint8, fill=0)
+        s = seq.total_stride
+        y = Guarded(b * (h // s) * (w // s) * dev[-1]["cout"])
+        binding.pw_layer_seq(seq, x, ws.t, y.view(b, h // s, w // s, dev[-1]["cout"]))
+        ws.check("workspace"); y.check("output")
+        assert binding.last_device_status() == binding.PROM_OK
+        return y.view(b, h // s, w // s, dev[-1]["cout"]).cpu().numpy(), fused
+    finally:
+        binding.debug_seq_block()
+
+
+CASES = [
+    # batch, h, w, cin, expanded, cout, stride, skip, rows, split
+    (1, 7, 7, 160, 960, 160, 1, True, 0, 0),
+    (5, 7, 7, 160, 960, 320, 1, False, 0, 8),          # two images per item, project sums of 320 columns
+    (3, 14, 14, 64, 384, 64, 1, True, 7, 1),
+    (2, 14, 14, 72, 432, 72, 1, True, 0, 3),           # channel counts that are 8 modulo 16, a half-empty last slice
+    (2, 14, 14, 96, 576, 160, 2, False, 0, 0),
+    (2, 28, 28, 32, 192, 32, 1, True, 5, 1),           # a ragged last band
+    (3, 28, 20, 32, 192, 64, 2, False, 3, 2),
+    (2, 56, 56, 24, 144, 24, 1, True, 0, 0),
+    (1, 56, 56, 24, 144, 32, 2, False, 4, 1),
+    (1, 112, 112, 16, 96, 24, 2, False, 2, 1),
+    (1, 5, 3, 8, 72, 8, 1, False, 1, 2),               # one row per band, planes of a few pixels
+    (4, 2, 2, 8, 32, 16, 2, False, 0, 0),
+    (1, 1, 1, 16, 96, 24, 1, False, 0, 0),
+    (40, 14, 14, 16, 64, 16, 1, True, 2, 1),           # more items than CTAs: several per CTA
+    (700, 7, 7, 16, 32, 16, 1, True, 0, 1),            # ... of one slice each
+    (9, 10, 6, 24, 96, 48, 1, False, 0, 2),
+]
+
+
+@pytest.mark.parametrize("b,h,w,cin,mid,cout,stride,skip,rows,split", CASES)
+def test_block(oracle, b, h, w, cin, mid, cout, stride, skip, rows, split):
+    rng = np.random.default_rng(b * 1000 + h * 10 + cin)
+    e, de = _layer(rng, 3, cin, mid)
+    q, dq = _layer(rng, 4, mid, cout, stride, dw=True, act_min=-128, skip=skip)
+    x = synth.act_post_relu6(9 + h, (b, h, w, cin))
+    got, fused = _run([de, dq], x.cuda(), rows, split)
+    assert fused
+    assert np.array_equal(got, _want(oracle, e, q, x.numpy()))
+
+
+@pytest.mark.parametrize("what", ["wide_shifts", "signed_expand", "dw_shift_0", "clamped_project"])
+def test_block_exact_epilogues(oracle, what):
+    """Constants and clamps that the one-multiply epilogues do not take."""
+    rng = np.random.default_rng(17)
+    cin, mid, cout = 24, 72, 24
+    kw = {}
+    if what == "wide_shifts":
+        kw["shift"] = rng.integers(6, 14, size=mid)
+    if what == "signed_expand":
+        kw["act_min"] = -128
+    e, de = _layer(rng, 5, cin, mid, **kw)
+    q, dq = _layer(rng, 6, mid, cout, dw=True, skip=True, act_min=-20 if what == "clamped_project" else -128,
+                   dw_shift=(0, 14) if what == "dw_shift_0" else (8, 11))
+    x = synth.act_post_relu6(2, (3, 14, 14, cin))
+    got, fused = _run([de, dq], x.cuda())
+    assert fused
+    assert np.array_equal(got, _want(oracle, e, q, x.numpy()))
+
+
+def test_block_falls_back(oracle):
+    """A workspace of the plain size, and an output that overlaps the input: one launch per layer, the same bytes."""
+    rng = np.random.default_rng(19)
+    e, de = _layer(rng, 7, 32, 192)
+    q, dq = _layer(rng, 8, 192, 32, dw=True, act_min=-128, skip=True)
+    x = synth.act_post_relu6(3, (2, 14, 14, 32))
+    want = _want(oracle, e, q, x.numpy())
+    binding.debug_seq_block(1)
+    try:
+        plain = binding.LayerSeq([de, dq]).workspace_bytes(2, 14, 14)
+    finally:
+        binding.debug_seq_block()
+    binding.debug_seq_block(2)
+    try:
+        seq = binding.LayerSeq([de, dq])
+        need = seq.workspace_bytes(2, 14, 14)
+        assert need >= plain
+        before = binding.launch_count()
+        y = binding.pw_layer_seq(seq, x.cuda(), torch.empty((need,), dtype=torch.uint8, device="cuda"))
+        fused = binding.launch_count() - before
+        xy = x.cuda()
+        before = binding.launch_count()
+        binding.pw_layer_seq(seq, xy, torch.empty((need,), dtype=torch.uint8, device="cuda"), xy)
+        assert binding.launch_count() - before > fused
+    finally:
+        binding.debug_seq_block()
+    torch.cuda.synchronize()
+    assert np.array_equal(y.cpu().numpy(), want)
+    assert np.array_equal(xy.cpu().numpy(), want)
