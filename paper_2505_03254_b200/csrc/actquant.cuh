@@ -15,8 +15,8 @@
 // holds, and then the maxima of the next (samples that do not fit eight SMs' shared memory, and batches
 // of which clusters would take several rounds).  Two-pass, for sizes that are not a multiple of 4: one kernel
 // takes the maxima with atomicMax on the bit pattern, a second one quantises.
-// Measured, calls back to back (floor: 5 bytes per value at the copy bandwidth): [128,112,112,32] 64 us (39; 74.5
-// before, when a lane quantised 64 neighbouring bytes and met four-way bank conflicts); [1,112,112,320] 8 us
+// Measured, calls back to back (floor: 5 bytes per value at the copy bandwidth): [128,112,112,32] 58 us (39; 64
+// before chunks were held in registers, 74.5 when a lane quantised 64 neighbouring bytes and met four-way bank conflicts); [1,112,112,320] 8 us
 // (3; 60 on one cluster); [60,112,112,96] 96 us (55; 107); [192,7,7,960] 11 us (7; 19).
 #pragma once
 
@@ -90,7 +90,12 @@ __device__ __forceinline__ float block_absmax(float m, float *part)
 // each of them; slice is a multiple of 16 and slice * 4 bytes fit the dynamic shared memory.
 // The slice arrives in chunks of kCopyBytes, one mbarrier each: the maximum of a chunk is taken
 // while later chunks are on their way, and as soon as a chunk has been quantised its place is
-// filled with the same chunk of the cluster's next sample, so the copies never stop.
+// filled with the same chunk of the cluster's next sample.
+// HOLD: the first chunks of a sample stay in registers once their maximum is taken, 16 floats per thread and chunk,
+// and their places are filled at once.  Without that no copy is on its way from the last chunk's arrival over the
+// exchange to the first code, about 2 of the 8 us that a round of samples took.  It costs 64 registers for the four
+// chunks (128 KB) that cover the gap, so it is for slices that fill an SM; smaller ones share it.
+template <int HOLD>
 __global__ void __launch_bounds__(kThreads, 1)
 act_quant_cluster_kernel(const float *__restrict__ x, int batch, long long per, int slice, float eps,
                          int8_t *__restrict__ q, float *__restrict__ gamma, float *__restrict__ scale)
@@ -139,18 +144,43 @@ act_quant_cluster_kernel(const float *__restrict__ x, int batch, long long per, 
     bool ok = true;
     bool first_exchange = true;
     uint32_t parity = 0;
+    constexpr int kPer = (int)(kCopyBytes / 16) / kThreads;       // 16-byte words of a chunk per thread
+    float4 held[HOLD > 0 ? HOLD * kPer : 1];
     for (int sample = cid, it = 0; sample < batch; sample += nclusters, ++it, parity ^= 1u) {
+        const int next = sample + nclusters;
         // ---- this CTA's maximum, chunk by chunk as the copies land (bounded waits) --------
         float m = 0.0f;
-        for (int c = 0; c < nchunks && ok; ++c) {
+        auto landed = [&](int c) {
             unsigned long long t0 = 0;
             for (uint32_t i = 1; !ptx::mbar_try_wait(bar_addr + 8 * c, parity); ++i) {
                 if ((i & 255u) == 0) {
                     const unsigned long long now = ptx::globaltimer();
                     if (t0 == 0) t0 = now;
-                    else if (now - t0 > kWaitLimitNs) { ok = false; break; }
+                    else if (now - t0 > kWaitLimitNs) return false;
                 }
             }
+            return true;
+        };
+#pragma unroll
+        for (int c = 0; c < HOLD; ++c) {
+            if (c >= nchunks) break;
+            ok = ok && landed(c);
+            const int lo = c * (int)(kCopyBytes / 16), hi = min((int)(count >> 2), lo + (int)(kCopyBytes / 16));
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+                const int i = lo + (int)threadIdx.x + j * kThreads;
+                const float4 v = ok && i < hi ? b4[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                held[kPer * c + j] = v;
+                float a = fabsf(v.x); m = a > m ? a : m;
+                a = fabsf(v.y); m = a > m ? a : m;
+                a = fabsf(v.z); m = a > m ? a : m;
+                a = fabsf(v.w); m = a > m ? a : m;
+            }
+            __syncthreads();              // the chunk has been read by everyone
+            if (threadIdx.x == 0 && ok && next < batch) load_chunk(next, c);
+        }
+        for (int c = HOLD; c < nchunks && ok; ++c) {
+            ok = landed(c);
             if (!ok) break;
             const int lo = c * (int)(kCopyBytes / 16);
             const int hi = min((int)(count >> 2), lo + (int)(kCopyBytes / 16));
@@ -183,8 +213,18 @@ act_quant_cluster_kernel(const float *__restrict__ x, int batch, long long per, 
 
         // ---- quantise from shared memory; refill each chunk at once ----
         int8_t *dst = q + (long long)sample * per + first;
-        const int next = sample + nclusters;
-        for (int c = 0; c < nchunks; ++c) {
+#pragma unroll
+        for (int c = 0; c < HOLD; ++c) {
+            if (!ok || c >= nchunks) break;
+            const int lo = c * (int)(kCopyBytes / 16), hi = min((int)(count >> 2), lo + (int)(kCopyBytes / 16));
+            uint32_t *dst4 = reinterpret_cast<uint32_t *>(dst);
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+                const int i = lo + (int)threadIdx.x + j * kThreads;
+                if (i < hi) dst4[i] = quantise_four(held[kPer * c + j], sc);
+            }
+        }
+        for (int c = HOLD; c < nchunks; ++c) {
             if (ok) {
                 // (four codes per thread: neighbouring lanes on neighbouring 16-byte words, no bank conflicts)
                 const int lo = c * (int)(kCopyBytes / 16);
@@ -198,6 +238,10 @@ act_quant_cluster_kernel(const float *__restrict__ x, int batch, long long per, 
         }
     }
     if (first_exchange) cluster.barrier_wait();     // a cluster without a sample still pairs its arrive
+    if (HOLD > 0 && threadIdx.x == 0 && failed) {   // copies may be on their way for a sample that is not awaited any more
+        const unsigned long long t0 = ptx::globaltimer();
+        while (ptx::globaltimer() - t0 < kWaitLimitNs) {}
+    }
 }
 
 // Grouped route.  The samples are taken in groups of up to 64 MB, kernel k of the call quantises group k - 1, whose

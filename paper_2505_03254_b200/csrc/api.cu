@@ -2324,7 +2324,10 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
     constexpr long long kOneGroup = 64ll << 20, kGroup = kOneGroup;
     if (rounds > 1 && total_bytes > (24ll << 20) && total_bytes <= kOneGroup) cluster = 0;
     if (cluster) {
-        const cudaError_t attr_err = raise_smem_limit(actq::act_quant_cluster_kernel, d.smem_optin - 4096);
+        // (whether an SM holds one such CTA or several does not depend on the registers of either form)
+        auto *kernel = (size_t)slice * 4 > (size_t)d.smem_total / 2 && rounds > 1 ? actq::act_quant_cluster_kernel<4>
+                                                                                    : actq::act_quant_cluster_kernel<0>;
+        const cudaError_t attr_err = raise_smem_limit(kernel, d.smem_optin - 4096);
         if (attr_err != cudaSuccess) return cuda_status(attr_err);
         cudaLaunchConfig_t cfg;
         memset(&cfg, 0, sizeof(cfg));
@@ -2351,7 +2354,7 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
             const std::array<long long, 3> key = {dev, cluster, slice};
             auto it = known.find(key);
             if (it == known.end()) {
-                if (cudaOccupancyMaxActiveClusters(&resident, actq::act_quant_cluster_kernel, &cfg) !=
+                if (cudaOccupancyMaxActiveClusters(&resident, kernel, &cfg) !=
                     cudaSuccess)
                     resident = 0;
                 cudaGetLastError();
@@ -2366,7 +2369,7 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
             attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
             attr[1].val.programmaticStreamSerializationAllowed = 1;
             cfg.numAttrs = 2;
-            cudaError_t e = cudaLaunchKernelEx(&cfg, actq::act_quant_cluster_kernel, x_dev, batch,
+            cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, x_dev, batch,
                                                (long long)per_sample, slice, eps, q_dev, gamma_dev,
                                                scale_dev);
             ++g_launches;
