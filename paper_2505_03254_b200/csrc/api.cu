@@ -1342,10 +1342,12 @@ struct BlockPlan {
     double est_us = 0;
 };
 
-// Clusters of block_kernel that a GPU holds at once (a cluster lies within one of its processing clusters).
+// Clusters of block_kernel that can be counted on to run at once.  A GPU holds 74, 45, 33, 26, 22, 15 and 15 of them
+// (a cluster lies within one of its processing clusters), but behind a kernel that leaves its SMs one by one they do not
+// pack like that: 45 clusters of three, 88 -> 528 -> 88 on 45 images of 12 x 12, took 16 us or 29 inside a sequence.
 static int block_resident(int csize, const DeviceInfo &d)
 {
-    static const int b200[block::kMaxCluster + 1] = {0, 148, 74, 45, 33, 26, 22, 15, 15};
+    static const int b200[block::kMaxCluster + 1] = {0, 148, 66, 40, 29, 23, 19, 13, 13};
     const int n = d.sms >= 148 ? b200[csize] : d.sms / csize * 9 / 10;
     return n > 0 ? n : 1;
 }
@@ -1470,10 +1472,12 @@ static bool block_layers_ok(const prom_layer *l)
 }
 
 // Whether one launch is expected to beat one per layer, whose time (us) is a fit to the same shapes (standard error
-// 9 %).  Inside a sequence a block saves about 1.2 us more than calls of its own show, whose preparation is not shared.
-// With this margin 43 % of the shapes run as blocks, in 0.88 of the layers' time; 4 % of all are slower by more than 3 %
-// (with a margin of 1: 77 %, 0.92 and 13 %).  Mostly they are planes of 10 to 60 thousand pixels, batch included:
-// larger ones are bound by the requantiser and the taps either way, and their units leave gaps here.
+// 9 %).  Inside a sequence a block saves about 1.2 us more than calls of its own show, whose preparation is not shared;
+// its own estimate is low where the project layer is wide (more sums to exchange and to requantise) and with stride 2.
+// With this margin a third of the shapes run as blocks, in 0.85 of the layers' time; 1 % of all are slower by more than
+// 3 % (without the corrections, at a margin of 0.9: 45 %, 0.88 and 4.5 %).  Over 189 bodies of the network (ten widths and
+// sizes, batch 1 to 150) a call takes 0.96 of the time on average, 0.84 to 1.02.  Mostly blocks are planes of 10 to 60
+// thousand pixels, batch included: larger ones are bound by the requantiser and the taps either way, and units leave gaps.
 static bool block_worth(const BlockPlan &pl, int ce)
 {
     const block::Params &p = pl.p;
@@ -1481,7 +1485,8 @@ static bool block_worth(const BlockPlan &pl, int ce)
     const bool tensor_taps = (ce & 15) == 0 && out * 1e6 >= (double)kDwTcOutputs;
     const double layers = 12.5 + 0.28 * in + (tensor_taps ? 5.7 + 0.39 * out : 2.04 * out) + 0.22e-4 * p.c0 * ce +
                           0.014e-4 * ce * p.co + 1.34 * out * p.co / ce + (p.c0 & 15 ? 1.5 + 0.13 * in : 0.0);
-    return pl.est_us - 1.2 < 0.9 * layers;
+    const int wide = p.co < 48 ? 0 : p.co - 48;
+    return pl.est_us * (1.0 + 0.0011 * wide + (p.stride == 1 ? 0.0 : p.csize == 1 ? 0.12 : 0.03)) - 1.2 < 0.92 * layers;
 }
 
 typedef std::array<int, 10> BlockKey;
