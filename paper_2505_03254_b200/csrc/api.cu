@@ -1472,21 +1472,23 @@ static bool block_layers_ok(const prom_layer *l)
 }
 
 // Whether one launch is expected to beat one per layer, whose time (us) is a fit to the same shapes (standard error
-// 9 %).  Inside a sequence a block saves about 1.2 us more than calls of its own show, whose preparation is not shared;
+// 7 %).  Inside a sequence a block saves about 1.2 us more than calls of its own show, whose preparation is not shared;
 // its own estimate is low where the project layer is wide (more sums to exchange and to requantise) and with stride 2.
-// With this margin a third of the shapes run as blocks, in 0.85 of the layers' time; 1 % of all are slower by more than
-// 3 % (without the corrections, at a margin of 0.9: 45 %, 0.88 and 4.5 %).  Over 189 bodies of the network (ten widths and
-// sizes, batch 1 to 150) a call takes 0.96 of the time on average, 0.84 to 1.02.  Mostly blocks are planes of 10 to 60
-// thousand pixels, batch included: larger ones are bound by the requantiser and the taps either way, and units leave gaps.
+// With this margin two fifths of the shapes run as blocks, in 0.85 of the layers' time; 0.7 % of all are slower by more
+// than 3 % (at 0.92: 28 %, 0.83 and 0.2 %).  Over 189 bodies of the network (ten widths and sizes, batch 1 to 150) a call
+// takes 0.945 of the time of one launch per layer on average, 0.84 to 1.005.  Mostly blocks are planes of 10 to 60 thousand pixels, batch included: larger
+// ones are bound by the requantiser and the taps either way, and units leave gaps.
 static bool block_worth(const BlockPlan &pl, int ce)
 {
     const block::Params &p = pl.p;
     const double in = (double)p.batch * p.h * p.w * ce * 1e-6, out = (double)p.batch * p.ho * p.wo * ce * 1e-6;
     const bool tensor_taps = (ce & 15) == 0 && out * 1e6 >= (double)kDwTcOutputs;
-    const double layers = 12.5 + 0.28 * in + (tensor_taps ? 5.7 + 0.39 * out : 2.04 * out) + 0.22e-4 * p.c0 * ce +
-                          0.014e-4 * ce * p.co + 1.34 * out * p.co / ce + (p.c0 & 15 ? 1.5 + 0.13 * in : 0.0);
+    const double weights = 1e-4 * p.c0 * ce;
+    const double layers = 12.4 + 0.27 * in + 2.26 * (out < 2.0 ? out : 2.0) + (tensor_taps ? 1.7 + 0.35 * out : 0.45 * out) +
+                          0.19 * weights + 1.5 * out * p.co / ce + (p.c0 & 15 ? 0.15 * in + 0.26 * weights : 0.0) +
+                          (p.co & 15 ? 0.13 + 0.083 * out : 0.0);
     const int wide = p.co < 48 ? 0 : p.co - 48;
-    return pl.est_us * (1.0 + 0.0011 * wide + (p.stride == 1 ? 0.0 : p.csize == 1 ? 0.12 : 0.03)) - 1.2 < 0.92 * layers;
+    return pl.est_us * (1.0 + 0.0011 * wide + (p.stride == 1 ? 0.0 : p.csize == 1 ? 0.12 : 0.03)) - 1.2 < 0.96 * layers;
 }
 
 typedef std::array<int, 10> BlockKey;
