@@ -70,7 +70,8 @@ void prom_debug_seq_order(int alternate);
  * (default), 1 = never, 2 = wherever the shape allows it.  rows: output rows per band, split: CTAs
  * per cluster that share a band's channels (0 = the planner's; a combination that does not fit leaves
  * the block to one launch per layer).  Results do not depend on it; the workspace size does.
- * prom_debug_layer_seq_output_offset returns -2 for the expanding layer.  Process-wide. */
+ * prom_debug_layer_seq_output_offset returns -2 for the expanding layer.  While prom_debug_dw_variant or
+ * prom_debug_seq_chain asks for a kernel of its own no block is taken.  Process-wide. */
 void prom_debug_seq_block(int mode, int rows, int split);
 
 /* Which kernel prom_dw_conv3x3_i8 runs: 0 = the library's choice (default: TMA

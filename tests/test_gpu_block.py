@@ -134,3 +134,46 @@ def test_block_falls_back(oracle):
     torch.cuda.synchronize()
     assert np.array_equal(y.cpu().numpy(), want)
     assert np.array_equal(xy.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("seed", range(6))
+def test_random_blocks_match_one_launch_per_layer(seed):
+    """Sequences of random blocks (odd planes, any multiple of 8 channels, both strides, clamps of every kind), in whatever
+    geometry the planner takes, live and from a captured graph: the bytes of one launch per layer."""
+    rng = np.random.default_rng(100 + seed)
+    for _ in range(4):
+        b = int(rng.integers(1, 12)) if rng.random() < 0.8 else int(rng.integers(150, 320))
+        h, w = int(rng.integers(1, 40)), int(rng.integers(1, 40))
+        cin, dev = 8 * int(rng.integers(1, 25)), []
+        x = synth.act_post_relu6(seed, (b, h, w, cin)).cuda()
+        for i in range(int(rng.integers(1, 4))):
+            stride = 2 if h % 2 == 0 and w % 2 == 0 and rng.random() < 0.4 else 1
+            mid = 8 * int(rng.integers(4, 90))
+            skip = stride == 1 and rng.random() < 0.5
+            cout = cin if skip else 8 * int(rng.integers(1, 40))
+            fast = rng.random() < 0.7
+            _, e = _layer(rng, seed * 10 + i, cin, mid, act_min=0 if fast else -128)
+            _, q = _layer(rng, seed * 10 + i + 5, mid, cout, stride, dw=True, skip=skip, act_min=int(rng.choice([-128, -40, 0])),
+                          dw_shift=(8, 11) if fast else (0, 14))
+            dev += [e, q]
+            h, w, cin = h // stride, w // stride, cout
+        want, _ = _run(dev, x, mode=1)
+        got, _ = _run(dev, x)
+        assert np.array_equal(got, want), (b, x.shape, [(d["cin"], d["cout"], d["in_stride"]) for d in dev])
+    binding.debug_seq_block(2)
+    try:
+        seq = binding.LayerSeq(dev)
+        ws = torch.empty((seq.workspace_bytes(*x.shape[:3]),), dtype=torch.uint8, device="cuda")
+        y = torch.zeros(want.shape, dtype=torch.int8, device="cuda")
+        s = torch.cuda.Stream()
+        with torch.cuda.stream(s):
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=s):
+                binding.pw_layer_seq(seq, x, ws, y)
+                binding.pw_layer_seq(seq, x, ws, y)
+        g.replay()
+        torch.cuda.synchronize()
+        assert np.array_equal(y.cpu().numpy(), want)
+        assert binding.last_device_status() == binding.PROM_OK
+    finally:
+        binding.debug_seq_block()
