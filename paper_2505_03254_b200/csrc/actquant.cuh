@@ -93,8 +93,9 @@ __device__ __forceinline__ float block_absmax(float m, float *part)
 // filled with the same chunk of the cluster's next sample.
 // HOLD: the first chunks of a sample stay in registers once their maximum is taken, 16 floats per thread and chunk,
 // and their places are filled at once.  Without that no copy is on its way from the last chunk's arrival over the
-// exchange to the first code, about 2 of the 8 us that a round of samples took.  It costs 64 registers for the four
-// chunks (128 KB) that cover the gap, so it is for slices that fill an SM; smaller ones share it.
+// exchange to the first code, about 2 of the 8 us that a round of samples took.  It costs 48 registers for the three
+// chunks (96 KB) that cover the gap, so it is for slices that fill an SM; smaller ones share it.  (128 samples of 1.6 MB:
+// 64.0 us without, 61.4, 59.3, 58.0, 58.4 and 60.6 with one to five chunks.)
 template <int HOLD>
 __global__ void __launch_bounds__(kThreads, 1)
 act_quant_cluster_kernel(const float *__restrict__ x, int batch, long long per, int slice, float eps,

@@ -2332,7 +2332,7 @@ prom_status prom_quantize_act_absmax(const float *x_dev, int batch, int64_t per_
     if (rounds > 1 && total_bytes > (24ll << 20) && total_bytes <= kOneGroup) cluster = 0;
     if (cluster) {
         // (whether an SM holds one such CTA or several does not depend on the registers of either form)
-        auto *kernel = (size_t)slice * 4 > (size_t)d.smem_total / 2 && rounds > 1 ? actq::act_quant_cluster_kernel<4>
+        auto *kernel = (size_t)slice * 4 > (size_t)d.smem_total / 2 && rounds > 1 ? actq::act_quant_cluster_kernel<3>
                                                                                     : actq::act_quant_cluster_kernel<0>;
         const cudaError_t attr_err = raise_smem_limit(kernel, d.smem_optin - 4096);
         if (attr_err != cudaSuccess) return cuda_status(attr_err);

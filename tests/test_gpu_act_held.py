@@ -10,9 +10,9 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("batch,per", [
-    (76, 8 * 29600),           # four chunks, the last of them short: all in registers
+    (76, 8 * 29600),           # four chunks, the last of them short
     (70, 8 * 32768),           # four whole chunks
-    (70, 8 * 32768 + 16),      # the last CTA has less, and its last chunk is not held
+    (70, 8 * 32768 + 16),      # a fifth chunk of a few floats
     (47, 8 * 50176),           # seven chunks
     (42, 8 * 55808 - 112),     # as much as shared memory holds, a ragged last CTA
 ])
