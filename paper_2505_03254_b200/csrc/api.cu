@@ -1577,6 +1577,8 @@ static void find_blocks(const prom_layer *layers, int n, const SeqShape &s, cons
     if (mode == 1 || g_dw_variant.load() != 0) return;
     for (int i = 0; i + 1 < n; ++i) {
         if (L.block_of[i] >= 0 || !block_layers_ok(layers + i) || s.m[i + 1] <= 0) continue;
+        // a skip connection into layer i + 2 reads the expanded tensor, which must exist
+        if (i + 2 < n && layers[i + 2].add_block_input) continue;
         BlockPlan pl;
         const int batch = (int)(s.m[i] / ((long long)s.h[i] * s.w[i]));
         if (!block_plan(layers[i].cin, layers[i].cout, layers[i + 1].cout, batch, s.h[i], s.w[i], layers[i + 1].in_stride, d, pl))
@@ -1948,8 +1950,8 @@ static prom_status run_seq(const prom_layer *layers, int n, const int8_t *x0, in
         // before it releases its successor, so every later link finds weights and operands complete
         c.pdl = i > 0 || layers[i].dw_w ? tc::kPdlChain : tc::kPdlWait;
         c.pdl_next = true;
-        // The block's input is the output of layer i-2, which sits where this layer's output
-        // goes (unless a chain wrote it to a buffer of its own: then the sum reads from there).
+        // The input of layer i-1, often in the region that this layer's output goes to (a chain's layers write buffers
+        // of their own).  It is always a tensor in memory: find_blocks and find_chains see to that.
         if (layers[i].add_block_input) c.res = input[i - 1];
         if (in_block) {
             // (what one launch per layer refuses stays refused)

@@ -37,6 +37,19 @@ def _want(oracle, e, q, x):
     return oracle.residual_add(y, x) if q["skip"] else y
 
 
+def _want_sequence(oracle, layers, x):
+    """One layer after the other; a skip connection adds the input of the layer before."""
+    before = None
+    for l in layers:
+        t = x
+        if "dw_w" in l:
+            t = oracle.dw3x3(x, l["dw_w"], l["dw_bias"], l["dw_mult"], l["dw_shift"], stride=l["in_stride"], act_min=0, act_max=127)
+        b, h, w, c = t.shape
+        y = oracle.conv_mul(t.reshape(-1, c), l["w"], l["bias"], l["mult"], l["shift"], l["act_min"], 127).reshape(b, h, w, -1)
+        before, x = x, oracle.residual_add(y, before) if l["skip"] else y
+    return x
+
+
 def _run(dev, x, rows=0, split=0, mode=2):
     binding.debug_seq_block(mode, rows, split)
     try:
@@ -84,6 +97,34 @@ def test_block(oracle, b, h, w, cin, mid, cout, stride, skip, rows, split):
     got, fused = _run([de, dq], x.cuda(), rows, split)
     assert fused
     assert np.array_equal(got, _want(oracle, e, q, x.numpy()))
+
+
+@pytest.mark.parametrize("mode", [0, 2])
+@pytest.mark.parametrize("third", ["pointwise", "depthwise", "more_behind"])
+def test_skip_connection_behind_a_block(oracle, third, mode):
+    """A layer that adds the expanded tensor of the two layers in front of it: that tensor has to be written."""
+    rng = np.random.default_rng(23)
+    b, side, cin, mid = 64, 14, 64, 384
+    layers = [_layer(rng, 11, cin, mid), _layer(rng, 12, mid, cin, dw=True, act_min=-128, skip=True),
+              _layer(rng, 13, cin, mid, skip=True, dw=third == "depthwise")]
+    if third == "more_behind":
+        layers += [_layer(rng, 14, mid, cin, dw=True, act_min=-128), _layer(rng, 15, cin, mid),
+                   _layer(rng, 16, mid, cin, dw=True, act_min=-128, skip=True)]
+    host, dev = [h for h, _ in layers], [d for _, d in layers]
+    x = synth.act_post_relu6(31, (b, side, side, cin))
+    binding.debug_seq_block(mode)
+    try:
+        pair = binding.LayerSeq(dev[:2])
+        assert binding.debug_layer_seq_output_offset(pair, b, side, side, 0)[0] == -2      # a block, on its own
+        seq = binding.LayerSeq(dev)
+        offsets = [binding.debug_layer_seq_output_offset(seq, b, side, side, i)[0] for i in range(len(dev) - 1)]
+    finally:
+        binding.debug_seq_block()
+    assert [i for i, o in enumerate(offsets) if o == -2] == ([4] if third == "more_behind" else [])
+    xg = Guarded(x.numel())
+    xg.t.copy_(x.reshape(-1))
+    got, _ = _run(dev, xg.view(*x.shape), mode=mode)
+    assert np.array_equal(got, _want_sequence(oracle, host, x.numpy()))
 
 
 @pytest.mark.parametrize("what", ["wide_shifts", "signed_expand", "dw_shift_0", "clamped_project"])
