@@ -55,8 +55,8 @@ constexpr int kThreads = 32 * (kFirstEpi + kEpiWarps);
 
 // A slice's prepared operands: expand weights (ks blocks of 64 rows x 32), bias digits (64 x 32), for each half
 // nine depthwise taps (32 x 32) and bias digits, project weights (npad rows x 64), then constants as 32-bit
-// words: four of a header {shift of E, or -1: exact epilogue; the same of D; halves with channels; 0} and
-// per channel as below.
+// words: four of a header {shift of E, or -1: exact epilogue; the same of D; halves with channels; whether a constant of E or D
+// is out of range} and per channel as below.
 enum { kMultE = 4, kMultD = kMultE + kSlice, kUpD = kMultD + kSlice, kBiasE = kUpD + kSlice, kShiftE = kBiasE + kSlice,
        kBiasD = kShiftE + kSlice, kShiftD = kBiasD + kSlice, kConstWords = kShiftD + kSlice };
 __host__ __device__ constexpr uint32_t off_taps(int ks) { return (uint32_t)(ks + 1) * 2 * kTapBytes; }
@@ -112,6 +112,10 @@ __device__ __forceinline__ void cp_async_8(uint32_t dst, const void *src)
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void st_cluster_32(uint32_t addr, uint32_t v)
+{
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
 __device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
 {
     asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
@@ -256,7 +260,8 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
     auto bar = [&](int kind, uint32_t i) { return bar0 + 8u * (uint32_t)(kind * kRing) + 8u * i; };
     volatile uint32_t *tmem_slot = reinterpret_cast<volatile uint32_t *>(smem + p.off_bars + kBarBytes);
     volatile int *flags = reinterpret_cast<volatile int *>(smem + p.off_bars + kBarBytes) + 2;     // [0] abort
-    int *pspan = reinterpret_cast<int *>(smem + p.off_bars + kBarBytes) + 4;     // project layer: smallest, largest shift, largest |bias|
+    int *pspan = reinterpret_cast<int *>(smem + p.off_bars + kBarBytes) + 4;     // project layer: smallest shift (-1: a constant of
+                                                                                 // the block is out of range), largest, largest |bias|
     uint32_t *etab = reinterpret_cast<uint32_t *>(smem + p.off_etab), *otab = reinterpret_cast<uint32_t *>(smem + p.off_otab);
     int *pc = reinterpret_cast<int *>(smem + p.off_pc);
 
@@ -277,7 +282,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
             ptx::mbar_init(bar(kBarD2Full, i), 1); ptx::mbar_init(bar(kBarD2Empty, i), 4);
             ptx::mbar_init(bar(kBarEFull, i), 4 * p.t1); ptx::mbar_init(bar(kBarEEmpty, i), 1);
             ptx::mbar_init(bar(kBarPFull, i), 4); ptx::mbar_init(bar(kBarPEmpty, i), 1);
-            ptx::mbar_init(bar(kBarD3Full, i), 1); ptx::mbar_init(bar(kBarD3Empty, i), 4 * p.chunks);
+            ptx::mbar_init(bar(kBarD3Full, i), 2); ptx::mbar_init(bar(kBarD3Empty, i), 4 * p.chunks);
             ptx::mbar_init(bar(kBarDrain, i), 1);
         }
         if (lane == 0) flags[0] = 0;
@@ -451,6 +456,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
         const bool leader = ptx::elect_one();
         Ring w;
         uint32_t v = 0;
+        int bad = 0;
         const int n_a = min(p.npad, 256), n_b = p.npad - n_a;      // an MMA is at most 256 columns wide
         const uint32_t i_a = kI0 | ((uint32_t)(n_a >> 3) << 17), i_b = kI0 | ((uint32_t)(n_b >> 3) << 17);
         for (int j = 0; j < n_items && ok; ++j) {
@@ -458,6 +464,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
             for (int s = 0; s < nsl && ok; ++s) {
                 const bool two = !(p.last_half && s_first + s == p.slices - 1);
                 if (!tc::wait_bar_warp(bar(kBarWFull, w.i), w.ph, flags)) { ok = false; break; }
+                bad |= *reinterpret_cast<const volatile int *>(smem + p.off_w + w.i * p.slice_bytes + off_consts(p.ks, p.npad) + 12);
                 const uint64_t b = d64 | (uint64_t)(w_lo + w.i * w_step + (off_project(p.ks) >> 4));
                 for (int t = 0; t < p.t2; ++t, ++v) {
                     if (!tc::wait_bar_warp(bar(kBarPFull, at8(v)), phase8(v), flags)) { ok = false; break; }
@@ -477,7 +484,11 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                 if (leader) ptx::mma_commit(bar(kBarWEmpty, w.i));
                 w.next(p.ns);
             }
-            if (leader) ptx::mma_commit(bar(kBarD3Full, 0));
+            if (leader) {
+                if (bad) atomicMin(pspan, -1);
+                ptx::mbar_arrive(bar(kBarD3Full, 0));
+                ptx::mma_commit(bar(kBarD3Full, 0));
+            }
         }
     } else {
         // ---- epilogue -----------------------------------------------------------------------------------
@@ -487,12 +498,13 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
         load_pixels(p, item_of(p, cluster), base, etab, etid, kEpiThreads, p.ipi * p.rin * p.w * p.px);
         // beside those loads, the project layer's constants.  Common shift: |sum| <= 4096 * 128 plus the bias, times
         // 2^10, stays within 31 bits for a bias below 2^20
+        // (a constant out of range: a smallest shift of -1, and no output is written)
         int mn = 31, mx = 0, ab = 0;
         for (int c = etid; c < p.npad; c += kEpiThreads) {
             int b = 0, mu = 0, sh = -1;
             if (c < p.co) {
                 b = __ldg(p.bias + c); mu = __ldg(p.mult + c); sh = __ldg(p.shift + c);
-                if (!requant_ok(b, mu, sh)) { raise_status(PROM_ERR_BAD_REQUANT); b = 0; mu = 0; sh = 0; }
+                if (!requant_ok(b, mu, sh)) { raise_status(PROM_ERR_BAD_REQUANT); b = 0; mu = 0; sh = 0; mn = -1; }
                 mn = min(mn, sh); mx = max(mx, sh); ab = max(ab, abs(b));
             }
             pc[c] = mu; pc[p.npad + c] = b; pc[3 * p.npad + c] = sh;
@@ -523,7 +535,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
         const int per_px = p.chunks / p.t2;
         auto finish = [&](int j) {
             const Item it = item_of(p, cluster + j * p.clusters);
-            bool waited = false;
+            bool waited = false, write = false;
             for (int i = grp; i < p.chunks; i += kGroups) {
                 const int t = i / per_px, c0 = 32 * (i - t * per_px);
                 const uint32_t o = otab[128 * t + 32 * quarter + lane];
@@ -539,6 +551,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                     if (!wait(bar(kBarD3Full, 0), (uint32_t)j & 1u)) return false;
                     ptx::tc_fence_after_sync();
                     waited = true;
+                    write = *reinterpret_cast<volatile int *>(pspan) >= 0;
                 }
                 __syncwarp();
                 const uint32_t sums = t_lane + (uint32_t)(p.d3_col + t * p.npad + c0);
@@ -552,7 +565,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                     const int a[8] = {(int)z[0], (int)z[1], (int)z[2], (int)z[3], (int)z[4], (int)z[5], (int)z[6], (int)z[7]};
                     uint2 out = project_8(prj, a, c0 + e);
                     if (add) { out.x = __vaddss4(out.x, r[0].x); out.y = __vaddss4(out.y, r[0].y); }
-                    if (valid) *reinterpret_cast<uint2 *>(p.y + at + e) = out;
+                    if (valid && write) *reinterpret_cast<uint2 *>(p.y + at + e) = out;
                     r[0] = r[1]; r[1] = r[2]; r[2] = r[3];
                     __syncwarp();
                 }
@@ -734,6 +747,8 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                 }
             }
         }
+        // (a constant out of range in one CTA's slices: no CTA writes)
+        if (warp == kFirstEpi && lane < p.csize && pspan[0] < 0) st_cluster_32(ptx::map_to_rank(ptx::smem_u32(pspan), (uint32_t)lane), 0xFFFFFFFFu);
         // this thread's outputs: eight channels of pixel rr of the CTA's share, then every kEpiThreads-th such piece
         const int etid = (int)threadIdx.x - 32 * kFirstEpi, c8 = p.co >> 3, plane = p.rows * p.wo;
         const int share = min(p.rpc, p.ipi * plane - rank * p.rpc) * c8;
@@ -752,7 +767,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
         if (mine) {
             const int top = max(pspan[1], 2);
             const Project prj = {pc, p.npad, top - pspan[0] <= 10 && pspan[2] < (1 << 20) ? top : 0, p.lo_p, p.hi_p};
-            for (int i = etid; i < share; i += kEpiThreads) {
+            for (int i = pspan[0] < 0 ? share : etid; i < share; i += kEpiThreads) {
                 if (i != etid) {
                     at = place(i, rr, c);
                     if (p.res && at >= 0) rs = __ldcg(reinterpret_cast<const uint2 *>(p.res + at));
@@ -820,7 +835,7 @@ __global__ void __launch_bounds__(kPrepThreads) block_prep_kernel(const __grid_c
 {
     __shared__ int cst[kConstWords];
     __shared__ int scale_e[kSlice];              // the expand weights are +-2^this
-    __shared__ int span[6];
+    __shared__ int span[7];
     const int tid = (int)threadIdx.x;
     int l = 0;
     while (l + 1 < t.n && (int)blockIdx.x >= t.b[l + 1].first) ++l;
@@ -830,7 +845,7 @@ __global__ void __launch_bounds__(kPrepThreads) block_prep_kernel(const __grid_c
     if (!t.behind) ptx::grid_dep_wait();
     ptx::grid_dep_launch();
 
-    if (tid == 0) { span[0] = 31; span[1] = 0; span[2] = 0; span[3] = 2; span[4] = 0; span[5] = 31; }
+    if (tid == 0) { span[0] = 31; span[1] = 0; span[2] = 0; span[3] = 2; span[4] = 0; span[5] = 31; span[6] = 0; }
     __syncthreads();
     int be = 0, me = 0, se = 0, bd = 0, md = 0, sd = 0;
     const bool mine = tid < kSlice && ch0 + tid < p.ce;
@@ -840,8 +855,8 @@ __global__ void __launch_bounds__(kPrepThreads) block_prep_kernel(const __grid_c
         if (mine) {
             be = __ldg(p.bias_e + ch); me = __ldg(p.mult_e + ch); se = __ldg(p.shift_e + ch);
             bd = __ldg(p.bias_d + ch); md = __ldg(p.mult_d + ch); sd = __ldg(p.shift_d + ch);
-            if (!requant_ok(be, me, se)) { raise_status(PROM_ERR_BAD_REQUANT); be = 0; me = 0; se = 0; }
-            if (!requant_ok(bd, md, sd)) { raise_status(PROM_ERR_BAD_REQUANT); bd = 0; md = 0; sd = 0; }
+            if (!requant_ok(be, me, se)) { raise_status(PROM_ERR_BAD_REQUANT); be = 0; me = 0; se = 0; span[6] = 1; }
+            if (!requant_ok(bd, md, sd)) { raise_status(PROM_ERR_BAD_REQUANT); bd = 0; md = 0; sd = 0; span[6] = 1; }
             atomicMin(&span[0], se); atomicMax(&span[1], se);
             const long long ab = be < 0 ? -(long long)be : be;
             if ((((long long)128 * p.c0 + ab) << 6) >= (1ll << 31) || (ab << 6) > tc::kBiasMax) span[2] = 1;
@@ -853,7 +868,7 @@ __global__ void __launch_bounds__(kPrepThreads) block_prep_kernel(const __grid_c
     if (tid < kSlice) {
         const bool e_ok = span[2] == 0 && p.lo_e == 0 && p.hi_e == 127 && span[1] - span[0] <= 4 && span[1] <= 24;
         const bool d_ok = span[4] == 0 && p.lo_d == 0 && p.hi_d == 127 && span[3] - span[5] <= 10;
-        if (tid < 4) cst[tid] = tid == 0 ? (e_ok ? span[1] : -1) : (tid == 1 ? (d_ok ? span[3] - 2 : -1) : (tid == 2 ? (p.ce - ch0 > kHalf ? 2 : 1) : 0));
+        if (tid < 4) cst[tid] = tid == 0 ? (e_ok ? span[1] : -1) : (tid == 1 ? (d_ok ? span[3] - 2 : -1) : (tid == 2 ? (p.ce - ch0 > kHalf ? 2 : 1) : span[6]));
         cst[kMultE + tid] = me; cst[kMultD + tid] = md; cst[kUpD + tid] = mine && d_ok ? 1 << (span[3] - sd) : 1;
         cst[kBiasE + tid] = be; cst[kShiftE + tid] = se; cst[kBiasD + tid] = bd; cst[kShiftD + tid] = sd;
         scale_e[tid] = e_ok && mine ? 2 + span[1] - se : 0;

@@ -146,6 +146,48 @@ def test_block_exact_epilogues(oracle, what):
     assert np.array_equal(got, _want(oracle, e, q, x.numpy()))
 
 
+@pytest.mark.parametrize("split", [1, 3])
+@pytest.mark.parametrize("layer,name,value", [(0, "mult", -1), (1, "dw_bias", (1 << 28) + 1), (1, "shift", 32)])
+def test_block_with_bad_constants(layer, name, value, split):
+    """A constant out of range in any of the block's layers, one channel of one slice: reported, and no output written."""
+    rng = np.random.default_rng(29)
+    dev = [_layer(rng, 9, 32, 192)[1], _layer(rng, 10, 192, 32, dw=True, act_min=-128, skip=True)[1]]
+    x = synth.act_post_relu6(5, (3, 14, 14, 32)).cuda()
+    for channel in (0, dev[layer][name].numel() - 1):
+        was = dev[layer][name][channel].item()
+        dev[layer][name][channel] = value
+        binding.debug_seq_block(2, 5, split)
+        try:
+            seq = binding.LayerSeq(dev)
+            assert binding.debug_layer_seq_output_offset(seq, 3, 14, 14, 0)[0] == -2
+            y = Guarded(x.numel())
+            binding.pw_layer_seq(seq, x, torch.empty((seq.workspace_bytes(3, 14, 14),), dtype=torch.uint8, device="cuda"), y.view(*x.shape))
+        finally:
+            binding.debug_seq_block()
+        assert binding.last_device_status() == binding.PROM_ERR_BAD_REQUANT
+        y.check("output")
+        assert bool((y.t == -77).all()), (channel, split)
+        dev[layer][name][channel] = was
+    got, fused = _run(dev, x, 5, split)
+    assert fused and (got != -77).any()
+
+
+@pytest.mark.parametrize("layer", [0, 1])
+def test_block_with_an_invalid_weight_code(layer):
+    rng = np.random.default_rng(31)
+    dev = [_layer(rng, 9, 32, 192)[1], _layer(rng, 10, 192, 32, dw=True, act_min=-128)[1]]
+    dev[layer]["w_packed"][-1, -1] = 0b10000000           # code 10 in the last place of the last row
+    binding.debug_seq_block(2)
+    try:
+        seq = binding.LayerSeq(dev)
+        assert binding.debug_layer_seq_output_offset(seq, 2, 14, 14, 0)[0] == -2
+        x = synth.act_post_relu6(5, (2, 14, 14, 32)).cuda()
+        binding.pw_layer_seq(seq, x, torch.empty((seq.workspace_bytes(2, 14, 14),), dtype=torch.uint8, device="cuda"))
+    finally:
+        binding.debug_seq_block()
+    assert binding.last_device_status() == binding.PROM_ERR_BAD_WEIGHT
+
+
 def test_block_falls_back(oracle):
     """A workspace of the plain size, and an output that overlaps the input: one launch per layer, the same bytes."""
     rng = np.random.default_rng(19)
