@@ -55,10 +55,12 @@ constexpr int kThreads = 32 * (kFirstEpi + kEpiWarps);
 
 // A slice's prepared operands: expand weights (ks blocks of 64 rows x 32), bias digits (64 x 32), for each half
 // nine depthwise taps (32 x 32) and bias digits, project weights (npad rows x 64), then constants as 32-bit
-// words: four of a header {shift of E, or -1: exact epilogue; the same of D; halves with channels; whether a constant of E or D
-// is out of range} and per channel as below.
-enum { kMultE = 4, kMultD = kMultE + kSlice, kUpD = kMultD + kSlice, kBiasE = kUpD + kSlice, kShiftE = kBiasE + kSlice,
-       kBiasD = kShiftE + kSlice, kShiftD = kBiasD + kSlice, kConstWords = kShiftD + kSlice };
+// words: four of a header {shift of E, or -1: any_constants; the same of D; halves with channels; whether a constant of E or D
+// is out of range} and per channel as below (biases times four where any_constants takes them so).
+enum { kMultE = 4, kMultD = kMultE + kSlice, kUpD = kMultD + kSlice, kBiasE = kUpD + kSlice, kBiasD = kBiasE + kSlice,
+       kShiftE = kBiasD + kSlice, kShiftD = kShiftE + kSlice, kConstWords = kShiftD + kSlice };
+constexpr int kToBias = kBiasE - kMultE, kToShift = kShiftE - kMultE;      // (the same for E and D)
+static_assert(kToBias == kBiasD - kMultD && kToShift == kShiftD - kMultD, "one way from a multiplier to its bias and shift");
 __host__ __device__ constexpr uint32_t off_taps(int ks) { return (uint32_t)(ks + 1) * 2 * kTapBytes; }
 __host__ __device__ constexpr uint32_t off_project(int ks) { return off_taps(ks) + 2 * kHalfTaps; }
 __host__ __device__ constexpr uint32_t off_consts(int ks, int npad) { return off_project(ks) + (uint32_t)npad * kSlice; }
@@ -146,10 +148,35 @@ __device__ __forceinline__ void requant_32(const uint32_t (&v)[32], uint32_t mul
     }
 }
 
-// The 64-bit definition (any clamp, shift and bias) of a whole slice.
-__device__ __noinline__ void exact_64(uint32_t taddr, const int *mult, const int *bias, const int *shift, int lo, int hi,
-                                      uint32_t at, uint32_t swz, bool store, bool zero)
+// A whole slice of one pixel with constants or clamps that requant_32 does not take.  Clamp [0, 127]: requant_floor with the
+// bias (times four) and shift of every channel, 7 instructions per output against 4 (E) and 5 (D): slices in which a channel
+// lies far from the others, a batch normalisation that has all but switched it off, say.  Any other clamp: the 64-bit definition.
+// (A function of its own: inlined, bodies of the network whose constants do not need it took 2 % longer at batch 9, since the
+// kernel's loops wait for their instructions.)
+__device__ __noinline__ void any_constants(uint32_t taddr, const int *mult, int lo, int hi, int halves, uint32_t at, uint32_t swz, bool store, bool zero)
 {
+    if (lo == 0 && hi == 127) {
+#pragma unroll 1
+        for (int h = 0; h < halves; ++h) {
+            uint32_t v[32], out[8];
+            ptx::tmem_ld_x32(taddr + h * kHalf, v);
+            ptx::tmem_wait_ld();
+#pragma unroll
+            for (int c = 0; c < 32; c += 4) {
+                const uint32_t o = ptx::smem_u32(mult + h * kHalf + c);
+                const int4 mu = ptx::lds_128(o), bi = ptx::lds_128(o + 4 * kToBias), sh = ptx::lds_128(o + 4 * kToShift);
+                const int q0 = (__mulhi((int)(4u * v[c]) + bi.x, mu.x) >> sh.x) + 1, q1 = (__mulhi((int)(4u * v[c + 1]) + bi.y, mu.y) >> sh.y) + 1;
+                const int q2 = (__mulhi((int)(4u * v[c + 2]) + bi.z, mu.z) >> sh.z) + 1, q3 = (__mulhi((int)(4u * v[c + 3]) + bi.w, mu.w) >> sh.w) + 1;
+                out[c / 4] = zero ? 0u : (ptx::pack_sat_u8(q1, q0, ptx::pack_sat_u8(q3, q2, 0u)) >> 1) & 0x7F7F7F7Fu;
+            }
+            if (store) {
+                sts_128(at + ((32u * h) ^ swz), out[0], out[1], out[2], out[3]);
+                sts_128(at + ((32u * h + 16u) ^ swz), out[4], out[5], out[6], out[7]);
+            }
+            __syncwarp();
+        }
+        return;
+    }
     for (int h = 0; h < kSlice / 16; ++h) {
         uint32_t v[16];
         ptx::tmem_ld_x16(taddr + 16 * h, v);
@@ -158,7 +185,7 @@ __device__ __noinline__ void exact_64(uint32_t taddr, const int *mult, const int
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
             const int c = 16 * h + i;
-            const int q = zero ? 0 : requant_exact((int)v[i] + bias[c], mult[c], shift[c], lo, hi);
+            const int q = zero ? 0 : requant_exact((int)v[i] + mult[kToBias + c], mult[c], mult[kToShift + c], lo, hi);
             o[i >> 2] |= ((uint32_t)q & 0xFFu) << (8 * (i & 3));
         }
         if (store) sts_128(at + (((uint32_t)h << 4) ^ swz), o[0], o[1], o[2], o[3]);
@@ -535,7 +562,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
         const int per_px = p.chunks / p.t2;
         auto finish = [&](int j) {
             const Item it = item_of(p, cluster + j * p.clusters);
-            bool waited = false, write = false;
+            bool waited = false;
             for (int i = grp; i < p.chunks; i += kGroups) {
                 const int t = i / per_px, c0 = 32 * (i - t * per_px);
                 const uint32_t o = otab[128 * t + 32 * quarter + lane];
@@ -551,9 +578,9 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                     if (!wait(bar(kBarD3Full, 0), (uint32_t)j & 1u)) return false;
                     ptx::tc_fence_after_sync();
                     waited = true;
-                    write = *reinterpret_cast<volatile int *>(pspan) >= 0;
                 }
                 __syncwarp();
+                const bool write = valid && *reinterpret_cast<volatile int *>(pspan) >= 0;
                 const uint32_t sums = t_lane + (uint32_t)(p.d3_col + t * p.npad + c0);
                 const int n = min(p.co - c0, 32);
                 // (rolled: straight-line code for a few outputs per thread waits for its instructions)
@@ -565,7 +592,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                     const int a[8] = {(int)z[0], (int)z[1], (int)z[2], (int)z[3], (int)z[4], (int)z[5], (int)z[6], (int)z[7]};
                     uint2 out = project_8(prj, a, c0 + e);
                     if (add) { out.x = __vaddss4(out.x, r[0].x); out.y = __vaddss4(out.y, r[0].y); }
-                    if (valid && write) *reinterpret_cast<uint2 *>(p.y + at + e) = out;
+                    if (write) *reinterpret_cast<uint2 *>(p.y + at + e) = out;
                     r[0] = r[1]; r[1] = r[2]; r[2] = r[3];
                     __syncwarp();
                 }
@@ -614,8 +641,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                     __syncwarp();
                 }
             } else {
-                const int *c = reinterpret_cast<const int *>(smem + off_c);
-                exact_64(acc, c + kMultE, c + kBiasE, c + kShiftE, p.lo_e, p.hi_e, at, swz, store, zero);
+                any_constants(acc, reinterpret_cast<const int *>(smem + off_c) + kMultE, p.lo_e, p.hi_e, hdr.z, at, swz, store, zero);
                 tc::release_acc(bar(kBarD1Empty, at8(u)));
             }
             ptx::fence_proxy_async_smem();
@@ -645,8 +671,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                     sts_128(at + ((32u * h + 16u) ^ swz), out[4], out[5], out[6], out[7]);
                 }
             } else {
-                const int *c = reinterpret_cast<const int *>(smem + off_c);
-                exact_64(acc, c + kMultD, c + kBiasD, c + kShiftD, p.lo_d, p.hi_d, at, swz, true, false);
+                any_constants(acc, reinterpret_cast<const int *>(smem + off_c) + kMultD, p.lo_d, p.hi_d, hdr.z, at, swz, true, false);
                 tc::release_acc(bar(kBarD2Empty, at8(v)));
             }
             ptx::fence_proxy_async_smem();
@@ -866,11 +891,13 @@ __global__ void __launch_bounds__(kPrepThreads) block_prep_kernel(const __grid_c
     }
     __syncthreads();
     if (tid < kSlice) {
-        const bool e_ok = span[2] == 0 && p.lo_e == 0 && p.hi_e == 127 && span[1] - span[0] <= 4 && span[1] <= 24;
-        const bool d_ok = span[4] == 0 && p.lo_d == 0 && p.hi_d == 127 && span[3] - span[5] <= 10;
+        const bool relu_e = p.lo_e == 0 && p.hi_e == 127, relu_d = p.lo_d == 0 && p.hi_d == 127;
+        const bool e_ok = span[2] == 0 && relu_e && span[1] - span[0] <= 4 && span[1] <= 24;
+        const bool d_ok = span[4] == 0 && relu_d && span[3] - span[5] <= 10;
         if (tid < 4) cst[tid] = tid == 0 ? (e_ok ? span[1] : -1) : (tid == 1 ? (d_ok ? span[3] - 2 : -1) : (tid == 2 ? (p.ce - ch0 > kHalf ? 2 : 1) : span[6]));
         cst[kMultE + tid] = me; cst[kMultD + tid] = md; cst[kUpD + tid] = mine && d_ok ? 1 << (span[3] - sd) : 1;
-        cst[kBiasE + tid] = be; cst[kShiftE + tid] = se; cst[kBiasD + tid] = bd; cst[kShiftD + tid] = sd;
+        cst[kShiftE + tid] = se; cst[kShiftD + tid] = sd;
+        cst[kBiasE + tid] = relu_e && !e_ok ? 4 * be : be; cst[kBiasD + tid] = relu_d && !d_ok ? 4 * bd : bd;
         scale_e[tid] = e_ok && mine ? 2 + span[1] - se : 0;
     }
     __syncthreads();

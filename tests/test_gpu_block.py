@@ -99,6 +99,29 @@ def test_block(oracle, b, h, w, cin, mid, cout, stride, skip, rows, split):
     assert np.array_equal(got, _want(oracle, e, q, x.numpy()))
 
 
+@pytest.mark.parametrize("cin,mid,cout", [(24, 72, 24), (64, 192, 40)])
+@pytest.mark.parametrize("what", ["expand", "depthwise", "both"])
+def test_block_with_constants_far_apart(oracle, what, cin, mid, cout):
+    """Shifts, multipliers and biases at the ends of their documented ranges beside ordinary ones of the same slice."""
+    rng = np.random.default_rng(mid)
+    e, de = _layer(rng, 35, cin, mid)
+    q, dq = _layer(rng, 36, mid, cout, dw=True, act_min=-128, skip=cin == cout)
+    for h, dev, pre, mine in ((e, de, "", what != "depthwise"), (q, dq, "dw_", what != "expand")):
+        if not mine:
+            continue
+        for name, values in (("shift", [0, 1, 15, 30, 31]), ("mult", [0, 1, 1 << 30, (1 << 31) - 1]),
+                             ("bias", [-(1 << 28), -(1 << 20), 467000, 1 << 20, 1 << 28])):
+            a = h[pre + name].copy()
+            at = rng.random(mid) < 0.2
+            a[at] = rng.choice(values, size=int(at.sum()))
+            h[pre + name] = a
+            dev[pre + name] = torch.from_numpy(a).cuda()
+    x = synth.act_post_relu6(37, (3, 14, 14, cin))
+    got, fused = _run([de, dq], x.cuda())
+    assert fused
+    assert np.array_equal(got, _want(oracle, e, q, x.numpy()))
+
+
 @pytest.mark.parametrize("mode", [0, 2])
 @pytest.mark.parametrize("third", ["pointwise", "depthwise", "more_behind"])
 def test_skip_connection_behind_a_block(oracle, third, mode):
