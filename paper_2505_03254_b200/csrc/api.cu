@@ -1471,6 +1471,15 @@ static bool block_layers_ok(const prom_layer *l)
            (q.cout & 7) == 0 && q.cout <= 384 && e.cin <= 512 && e.cout >= 32;
 }
 
+// Whether the expanding layer and the depthwise convolution have the clamp that block_kernel's fast epilogues take.  With any
+// other it computes by the 64-bit definition, the separate kernels mostly do not: with -128 in the expanding layer three blocks
+// of 64 x 28 x 28, 32 -> 192 -> 32, took 125 us against 67, with an upper limit of 100 in the depthwise one 149 against 115;
+// 32 x 14 x 14, 96 -> 576 -> 96, 93 against 55 and 100 against 57.
+static bool block_clamps_fast(const prom_layer *l)
+{
+    return l[0].rq.act_min == 0 && l[0].rq.act_max == 127 && l[1].dw_rq.act_min == 0 && l[1].dw_rq.act_max == 127;
+}
+
 // Whether one launch is expected to beat one per layer, whose time (us) is a fit to the same shapes (standard error
 // 7 %).  Inside a sequence a block saves about 1.2 us more than calls of its own show, whose preparation is not shared;
 // its own estimate is low where the project layer is wide (more sums to exchange and to requantise) and with stride 2.
@@ -1583,7 +1592,7 @@ static void find_blocks(const prom_layer *layers, int n, const SeqShape &s, cons
         const int batch = (int)(s.m[i] / ((long long)s.h[i] * s.w[i]));
         if (!block_plan(layers[i].cin, layers[i].cout, layers[i + 1].cout, batch, s.h[i], s.w[i], layers[i + 1].in_stride, d, pl))
             continue;
-        if (mode == 0 && !block_worth(pl, layers[i].cout)) continue;
+        if (mode == 0 && !(block_clamps_fast(layers + i) && block_worth(pl, layers[i].cout))) continue;
         L.block_of[i] = L.block_of[i + 1] = (int)L.blocks.size();
         L.blocks.push_back(pl);
         L.bimg_off.push_back(L.bimg_total);

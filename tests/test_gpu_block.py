@@ -99,6 +99,32 @@ def test_block(oracle, b, h, w, cin, mid, cout, stride, skip, rows, split):
     assert np.array_equal(got, _want(oracle, e, q, x.numpy()))
 
 
+@pytest.mark.parametrize("e_clamp,d_clamp,fused", [((0, 127), (0, 127), True), ((-128, 127), (0, 127), False), ((0, 100), (0, 127), False),
+                                                   ((0, 127), (-128, 127), False), ((0, 127), (0, 100), False), ((1, 127), (5, 127), False)])
+def test_clamps_that_the_library_takes_as_a_block(oracle, e_clamp, d_clamp, fused):
+    rng = np.random.default_rng(41)
+    e, de = _layer(rng, 43, 32, 192)
+    q, dq = _layer(rng, 44, 192, 32, dw=True, act_min=-128, skip=True)
+    x = synth.act_post_relu6(45, (16, 28, 28, 32))
+    seq = binding.LayerSeq([de, dq])
+    seq.array[0].rq.act_min, seq.array[0].rq.act_max = e_clamp
+    seq.array[1].dw_rq.act_min, seq.array[1].dw_rq.act_max = d_clamp
+    t = oracle.conv_mul(x.numpy().reshape(-1, 32), e["w"], e["bias"], e["mult"], e["shift"], *e_clamp).reshape(16, 28, 28, 192)
+    t = oracle.dw3x3(t, q["dw_w"], q["dw_bias"], q["dw_mult"], q["dw_shift"], stride=1, act_min=d_clamp[0], act_max=d_clamp[1])
+    y = oracle.conv_mul(t.reshape(-1, 192), q["w"], q["bias"], q["mult"], q["shift"], -128, 127).reshape(x.shape)
+    want = oracle.residual_add(y, x.numpy())
+    for mode in (0, 2):                                 # by the library's rule, and wherever possible
+        binding.debug_seq_block(mode)
+        try:
+            taken = binding.debug_layer_seq_output_offset(seq, 16, 28, 28, 0)[0] == -2
+            got = binding.pw_layer_seq(seq, x.cuda(), torch.empty((seq.workspace_bytes(16, 28, 28),), dtype=torch.uint8, device="cuda"))
+            assert np.array_equal(got.cpu().numpy(), want), mode
+        finally:
+            binding.debug_seq_block()
+        assert taken == (fused or mode == 2)
+    assert binding.last_device_status() == binding.PROM_OK
+
+
 @pytest.mark.parametrize("cin,mid,cout", [(24, 72, 24), (64, 192, 40)])
 @pytest.mark.parametrize("what", ["expand", "depthwise", "both"])
 def test_block_with_constants_far_apart(oracle, what, cin, mid, cout):
