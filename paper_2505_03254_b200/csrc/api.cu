@@ -1339,7 +1339,8 @@ struct BlockPlan {
     block::Params p;
     int grid = 0;
     size_t smem = 0, image_bytes = 0;
-    double est_us = 0;
+    double est_us = 0;                      // of the geometry: what block_plan ranks by
+    double block_us = 0, layers_us = 0;     // block_estimate
 };
 
 // Clusters of block_kernel that can be counted on to run at once.  A GPU holds 74, 45, 33, 26, 22, 15 and 15 of them
@@ -1480,6 +1481,31 @@ static bool block_clamps_fast(const prom_layer *l)
     return l[0].rq.act_min == 0 && l[0].rq.act_max == 127 && l[1].dw_rq.act_min == 0 && l[1].dw_rq.act_max == 127;
 }
 
+// What a call of one block alone is expected to take, in one launch and in one per layer (us).  Fits to 4942 shapes, blocks of
+// the networks and others, standard errors 6.3 and 7.0 %, no worse on a third that a fit has not seen.  The planners' own
+// figures go into both: that of the geometry here, those of the two pointwise layers there.
+static void block_estimate(const prom_layer *l, const DeviceInfo &d, BlockPlan &pl)
+{
+    const block::Params &p = pl.p;
+    const int ce = l[0].cout;
+    const int more = p.csize > 1 ? 0 : (p.items + p.clusters - 1) / p.clusters - 1;      // items after a CTA's first
+    const double e0 = pl.est_us - 4.54, pieces = 0.128 * p.t1 * p.px, sums = 0.01 * p.t2 * p.npad;
+    pl.block_us = 4.83 + 0.7275 * e0 + (0.243 + 2.49 * more) * pieces + 0.523 * p.per_cta +
+                  (p.csize > 1 ? 1.937 * sums
+                               : 0.475 * more * sums + 0.133 * p.t1 + 0.0112 * (p.co < 48 ? 0 : p.co - 48) + (p.stride == 2 ? 0.052 * e0 : 0.0));
+    TcPlan e, q;
+    const int use = kPlanPrepared | kPlanOdd;
+    pl.layers_us = 1e9;                     // not on the tensor cores: several times slower
+    if (!tc_shape_plan((long long)p.batch * p.h * p.w, p.c0, ce, RowMap{1, 1, 1, 1, 1}, d, e, use) ||
+        !tc_shape_plan((long long)p.batch * p.ho * p.wo, ce, p.co, RowMap{1, 1, 1, 1, 1}, d, q, use))
+        return;
+    const double out = (double)p.batch * p.ho * p.wo * ce * 1e-6;
+    const bool odd_e = (p.c0 & 15) != 0, odd_p = ((ce | p.co) & 15) != 0, tensor_taps = (ce & 15) == 0 && out * 1e6 >= (double)kDwTcOutputs;
+    pl.layers_us = 2.35 + (odd_e ? 0.722 : 0.64) * e.est_us + (odd_p ? 1.727 + 1.013 * q.est_us : 1.439 * q.est_us) +
+                   2.007 * (out < 2.0 ? out : 2.0) + (tensor_taps ? 2.58 + 0.3 * out : (odd_p ? 0.997 : 0.66) * out) +
+                   0.04 * (e.p.groups + q.p.groups);
+}
+
 // Whether one launch is expected to beat one per layer, whose time (us) is a fit to the same shapes (standard error
 // 7 %).  Inside a sequence a block saves about 1.2 us more than calls of its own show, whose preparation is not shared;
 // its own estimate is low where the project layer is wide (more sums to exchange and to requantise) and with stride 2.
@@ -1500,9 +1526,17 @@ static bool block_worth(const BlockPlan &pl, int ce)
     return pl.est_us * (1.0 + 0.0011 * wide + (p.stride == 1 ? 0.0 : p.csize == 1 ? 0.12 : 0.03)) - 1.2 < 0.96 * layers;
 }
 
+// What a call's blocks have to gain together.  By block_estimate every block beside the first gains kBlockBeside more than
+// alone: the blocks' operands take one launch, and kernels of different layers wait for their instructions where block_kernel
+// finds its own (fit to 70 bodies of the network, which all but one keep their blocks).  So a call of one block needs 1.3 us.  Of
+// 4942 calls of one block 0.6 % are slower than one launch per layer by more than 3 % (without this rule 4.7, up to 1.45
+// times for wide inputs in many items), of 2850 of three alike 1.1 % (2.2).
+constexpr double kBlockBeside = 1.6, kBlocksGain = 1.3;
+
 typedef std::array<int, 10> BlockKey;
-static bool block_plan(int c0, int ce, int co, int batch, int h, int w, int stride, const DeviceInfo &d, BlockPlan &best)
+static bool block_plan(const prom_layer *l, int batch, int h, int w, const DeviceInfo &d, BlockPlan &best)
 {
+    const int c0 = l[0].cin, ce = l[0].cout, co = l[1].cout, stride = l[1].in_stride;
     const int f_rows = g_block_rows.load(), f_split = g_block_split.load();
     const BlockKey key = {c0, ce, co, batch, h, w, stride, d.dev, f_rows, f_split};
     static std::mutex mu;
@@ -1527,6 +1561,7 @@ static bool block_plan(int c0, int ce, int co, int batch, int h, int w, int stri
                     if (!found || pl.est_us < top.est_us) { top = pl; found = true; }
                 }
         }
+        if (found) block_estimate(l, d, top);
         if (cache.size() > 4096) cache.clear();
         it = cache.emplace(key, std::make_pair(found, top)).first;
     }
@@ -1584,19 +1619,24 @@ static void find_blocks(const prom_layer *layers, int n, const SeqShape &s, cons
 {
     const int mode = g_block_mode.load();
     if (mode == 1 || g_dw_variant.load() != 0) return;
+    double gain = 0.0;                  // of all blocks, the first one's share of kBlockBeside too
     for (int i = 0; i + 1 < n; ++i) {
         if (L.block_of[i] >= 0 || !block_layers_ok(layers + i) || s.m[i + 1] <= 0) continue;
         // a skip connection into layer i + 2 reads the expanded tensor, which must exist
         if (i + 2 < n && layers[i + 2].add_block_input) continue;
         BlockPlan pl;
         const int batch = (int)(s.m[i] / ((long long)s.h[i] * s.w[i]));
-        if (!block_plan(layers[i].cin, layers[i].cout, layers[i + 1].cout, batch, s.h[i], s.w[i], layers[i + 1].in_stride, d, pl))
-            continue;
+        if (!block_plan(layers + i, batch, s.h[i], s.w[i], d, pl)) continue;
         if (mode == 0 && !(block_clamps_fast(layers + i) && block_worth(pl, layers[i].cout))) continue;
+        gain += pl.layers_us - pl.block_us + kBlockBeside;
         L.block_of[i] = L.block_of[i + 1] = (int)L.blocks.size();
         L.blocks.push_back(pl);
         L.bimg_off.push_back(L.bimg_total);
         L.bimg_total += round256(pl.image_bytes);
+    }
+    if (mode == 0 && gain < kBlocksGain + kBlockBeside) {
+        L.blocks.clear(); L.bimg_off.clear(); L.bimg_total = 0;
+        L.block_of.assign(n, -1);
     }
     if (L.blocks.empty()) return;
     size_t r[2] = {0, 0}, c = 0;

@@ -125,6 +125,26 @@ def test_clamps_that_the_library_takes_as_a_block(oracle, e_clamp, d_clamp, fuse
     assert binding.last_device_status() == binding.PROM_OK
 
 
+@pytest.mark.parametrize("b,h,w,cin,mid,cout,stride,blocks,taken", [
+    (16, 28, 28, 32, 192, 32, 1, 1, True),
+    (2, 20, 20, 32, 192, 32, 1, 1, False),             # 13.6 us against 11.7
+    (2, 33, 9, 184, 672, 200, 1, 1, False),            # 20.5 against 16.4
+    (149, 10, 10, 256, 200, 112, 1, 1, False),         # 32.9 against 23.8: wide inputs, two items per CTA
+    (64, 14, 14, 64, 384, 64, 1, 1, True),
+    (58, 20, 20, 232, 32, 232, 1, 3, False),
+    (9, 28, 28, 24, 144, 24, 1, 3, True),
+])
+def test_blocks_that_the_library_takes(b, h, w, cin, mid, cout, stride, blocks, taken):
+    """By the rule: blocks that save too little in their call have one launch per layer."""
+    rng = np.random.default_rng(47)
+    dev = []
+    for i in range(blocks):
+        dev += [_layer(rng, 48, cin, mid)[1], _layer(rng, 49, mid, cout, stride, dw=True, act_min=-128)[1]]
+    seq = binding.LayerSeq(dev)
+    got = [binding.debug_layer_seq_output_offset(seq, b, h, w, 2 * i)[0] == -2 for i in range(blocks)]
+    assert got == [taken] * blocks
+
+
 @pytest.mark.parametrize("cin,mid,cout", [(24, 72, 24), (64, 192, 40)])
 @pytest.mark.parametrize("what", ["expand", "depthwise", "both"])
 def test_block_with_constants_far_apart(oracle, what, cin, mid, cout):
