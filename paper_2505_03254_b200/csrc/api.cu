@@ -1410,10 +1410,7 @@ static bool block_fill(int c0, int ce, int co, int batch, int h, int w, int stri
     if (block::kSlice * (p.n1 + p.n2) + d3 > cols) return false;
     p.d2_col = block::kSlice * p.n1; p.d3_col = p.d2_col + block::kSlice * p.n2;
     p.tmem_cols = cols;
-    // (a read of 32 columns may go past the sums' last ones)
-    const int used = p.d3_col + (p.t2 - 1) * p.npad + round_up(p.npad, 32);
-    if (used > cols) return false;
-    while (p.tmem_cols > 32 && used <= p.tmem_cols / 2) p.tmem_cols /= 2;
+    while (p.tmem_cols > 32 && p.d3_col + d3 <= p.tmem_cols / 2) p.tmem_cols /= 2;
     // shared memory: rings as deep as fit
     auto layout = [&](int ne, int ns, int np, int nx) {
         p.ne = ne; p.ns = ns; p.np = np; p.nx = nx;

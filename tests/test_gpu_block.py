@@ -85,6 +85,9 @@ CASES = [
     (40, 14, 14, 16, 64, 16, 1, True, 2, 1),           # more items than CTAs: several per CTA
     (700, 7, 7, 16, 32, 16, 1, True, 0, 1),            # ... of one slice each
     (9, 10, 6, 24, 96, 48, 1, False, 0, 2),
+    (2, 16, 30, 24, 96, 80, 1, False, 16, 1),          # sums that end with tensor memory
+    (2, 16, 30, 24, 96, 72, 1, False, 16, 2),
+    (2, 30, 30, 16, 96, 16, 1, True, 30, 2),
 ]
 
 
