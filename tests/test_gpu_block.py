@@ -102,9 +102,10 @@ def test_block(oracle, b, h, w, cin, mid, cout, stride, skip, rows, split):
     assert np.array_equal(got, _want(oracle, e, q, x.numpy()))
 
 
+@pytest.mark.parametrize("p_clamp", [(-128, 127), (-128, 60), (-30, 60)])
 @pytest.mark.parametrize("e_clamp,d_clamp,fused", [((0, 127), (0, 127), True), ((-128, 127), (0, 127), False), ((0, 100), (0, 127), False),
                                                    ((0, 127), (-128, 127), False), ((0, 127), (0, 100), False), ((1, 127), (5, 127), False)])
-def test_clamps_that_the_library_takes_as_a_block(oracle, e_clamp, d_clamp, fused):
+def test_clamps_that_the_library_takes_as_a_block(oracle, e_clamp, d_clamp, fused, p_clamp):
     rng = np.random.default_rng(41)
     e, de = _layer(rng, 43, 32, 192)
     q, dq = _layer(rng, 44, 192, 32, dw=True, act_min=-128, skip=True)
@@ -112,9 +113,10 @@ def test_clamps_that_the_library_takes_as_a_block(oracle, e_clamp, d_clamp, fuse
     seq = binding.LayerSeq([de, dq])
     seq.array[0].rq.act_min, seq.array[0].rq.act_max = e_clamp
     seq.array[1].dw_rq.act_min, seq.array[1].dw_rq.act_max = d_clamp
+    seq.array[1].rq.act_min, seq.array[1].rq.act_max = p_clamp
     t = oracle.conv_mul(x.numpy().reshape(-1, 32), e["w"], e["bias"], e["mult"], e["shift"], *e_clamp).reshape(16, 28, 28, 192)
     t = oracle.dw3x3(t, q["dw_w"], q["dw_bias"], q["dw_mult"], q["dw_shift"], stride=1, act_min=d_clamp[0], act_max=d_clamp[1])
-    y = oracle.conv_mul(t.reshape(-1, 192), q["w"], q["bias"], q["mult"], q["shift"], -128, 127).reshape(x.shape)
+    y = oracle.conv_mul(t.reshape(-1, 192), q["w"], q["bias"], q["mult"], q["shift"], *p_clamp).reshape(x.shape)
     want = oracle.residual_add(y, x.numpy())
     for mode in (0, 2):                                 # by the library's rule, and wherever possible
         binding.debug_seq_block(mode)
@@ -260,75 +262,143 @@ def test_block_with_an_invalid_weight_code(layer):
     assert binding.last_device_status() == binding.PROM_ERR_BAD_WEIGHT
 
 
+def _mixed(rng):
+    """Blocks between layers that are none: a depthwise + project layer without an expanding one, twice, and a last pointwise layer."""
+    return [_layer(rng, 51, 32, 32, dw=True, act_min=-128), _layer(rng, 52, 32, 192), _layer(rng, 53, 192, 32, dw=True, act_min=-128, skip=True),
+            _layer(rng, 54, 32, 48, dw=True, act_min=-128), _layer(rng, 55, 48, 288), _layer(rng, 56, 288, 64, 2, dw=True, act_min=-128),
+            _layer(rng, 57, 64, 96)]
+
+
 def test_block_falls_back(oracle):
-    """A workspace of the plain size, and an output that overlaps the input: one launch per layer, the same bytes."""
-    rng = np.random.default_rng(19)
-    e, de = _layer(rng, 7, 32, 192)
-    q, dq = _layer(rng, 8, 192, 32, dw=True, act_min=-128, skip=True)
-    x = synth.act_post_relu6(3, (2, 14, 14, 32))
-    want = _want(oracle, e, q, x.numpy())
+    """A workspace without room for the blocks' operands: one launch per layer in the regions of that layout, the same bytes,
+    and the same least size as without blocks."""
+    # (few pixels: the operands then outweigh the expanded tensors that need no room)
+    layers = _mixed(np.random.default_rng(19))
+    host, dev = [h for h, _ in layers], [d for _, d in layers]
+    x = synth.act_post_relu6(3, (1, 6, 6, 32))
+    want = _want_sequence(oracle, host, x.numpy())
+    seq, xd = binding.LayerSeq(dev), x.cuda()
+
+    def call(nbytes):
+        ws = Guarded(nbytes, dtype=torch.uint8, fill=0x33)
+        y = Guarded(want.size)
+        before = binding.launch_count()
+        binding.pw_layer_seq(seq, xd, ws.t, y.view(*want.shape))
+        launches = binding.launch_count() - before
+        ws.check("workspace"); y.check("output")
+        assert np.array_equal(y.view(*want.shape).cpu().numpy(), want), nbytes
+        return launches
+
+    def least():                                        # the smallest workspace that is not refused
+        lo, hi = 0, 1 << 22
+        while lo + 16 < hi:
+            mid = (lo + hi) // 32 * 16
+            try:
+                call(mid)
+                hi = mid
+            except binding.PromError as err:
+                assert err.code == binding.PROM_ERR_WORKSPACE
+                lo = mid
+        return hi
+
     binding.debug_seq_block(1)
     try:
-        plain = binding.LayerSeq([de, dq]).workspace_bytes(2, 14, 14)
+        plain, least_plain = seq.workspace_bytes(1, 6, 6), least()
+        one_per_layer = call(plain)
     finally:
         binding.debug_seq_block()
     binding.debug_seq_block(2)
     try:
+        need = seq.workspace_bytes(1, 6, 6)
+        assert [binding.debug_layer_seq_output_offset(seq, 1, 6, 6, i)[0] == -2 for i in range(6)] == [False, True, False, False, True, False]
+        assert need > plain
+        assert call(need) == one_per_layer - 4 + 1      # two launches fewer per block, one more for their operands
+        assert call(plain) == one_per_layer and call(need - 1) == one_per_layer
+        assert least() == least_plain
+    finally:
+        binding.debug_seq_block()
+    assert binding.last_device_status() == binding.PROM_OK
+
+
+def test_block_with_an_output_that_overlaps_its_input(oracle):
+    rng = np.random.default_rng(19)
+    e, de = _layer(rng, 7, 32, 192)
+    q, dq = _layer(rng, 8, 192, 32, dw=True, act_min=-128, skip=True)
+    x = synth.act_post_relu6(3, (2, 14, 14, 32))
+    binding.debug_seq_block(2)
+    try:
         seq = binding.LayerSeq([de, dq])
-        need = seq.workspace_bytes(2, 14, 14)
-        assert need >= plain
+        ws = torch.empty((seq.workspace_bytes(2, 14, 14),), dtype=torch.uint8, device="cuda")
         before = binding.launch_count()
-        y = binding.pw_layer_seq(seq, x.cuda(), torch.empty((need,), dtype=torch.uint8, device="cuda"))
+        y = binding.pw_layer_seq(seq, x.cuda(), ws)
         fused = binding.launch_count() - before
         xy = x.cuda()
         before = binding.launch_count()
-        binding.pw_layer_seq(seq, xy, torch.empty((need,), dtype=torch.uint8, device="cuda"), xy)
+        binding.pw_layer_seq(seq, xy, ws, xy)
         assert binding.launch_count() - before > fused
     finally:
         binding.debug_seq_block()
     torch.cuda.synchronize()
-    assert np.array_equal(y.cpu().numpy(), want)
-    assert np.array_equal(xy.cpu().numpy(), want)
+    want = _want(oracle, e, q, x.numpy())
+    assert np.array_equal(y.cpu().numpy(), want) and np.array_equal(xy.cpu().numpy(), want)
 
 
 @pytest.mark.parametrize("seed", range(6))
 def test_random_blocks_match_one_launch_per_layer(seed):
-    """Sequences of random blocks (odd planes, any multiple of 8 channels, both strides, clamps of every kind), in whatever
-    geometry the planner takes, live and from a captured graph: the bytes of one launch per layer."""
+    """Sequences of random blocks (odd planes, any multiple of 8 channels, both strides, ordinary and other clamps on each of the
+    three layers), in whatever geometry the planner takes, live and from a captured graph: the bytes of one launch per layer."""
     rng = np.random.default_rng(100 + seed)
+    pairs = taken = most = 0
     for _ in range(4):
         b = int(rng.integers(1, 12)) if rng.random() < 0.8 else int(rng.integers(150, 320))
         h, w = int(rng.integers(1, 40)), int(rng.integers(1, 40))
-        cin, dev = 8 * int(rng.integers(1, 25)), []
+        cin, dev, clamps = 8 * int(rng.integers(1, 25)), [], []
         x = synth.act_post_relu6(seed, (b, h, w, cin)).cuda()
-        for i in range(int(rng.integers(1, 4))):
+        n = int(rng.integers(1, 4))
+        for i in range(n):
             stride = 2 if h % 2 == 0 and w % 2 == 0 and rng.random() < 0.4 else 1
             mid = 8 * int(rng.integers(4, 90))
             skip = stride == 1 and rng.random() < 0.5
             cout = cin if skip else 8 * int(rng.integers(1, 40))
             fast = rng.random() < 0.7
-            _, e = _layer(rng, seed * 10 + i, cin, mid, act_min=0 if fast else -128)
-            _, q = _layer(rng, seed * 10 + i + 5, mid, cout, stride, dw=True, skip=skip, act_min=int(rng.choice([-128, -40, 0])),
-                          dw_shift=(8, 11) if fast else (0, 14))
+            _, e = _layer(rng, seed * 10 + i, cin, mid)
+            _, q = _layer(rng, seed * 10 + i + 5, mid, cout, stride, dw=True, skip=skip, dw_shift=(8, 11) if fast else (0, 14))
             dev += [e, q]
+            clamps += [[(0, 127)] if fast else [(-128, 127), (0, 101), (-60, 55)], [(0, 127)] if fast else [(-128, 90), (0, 127), (3, 127)],
+                       [(-128, 127), (-40, 127), (-128, 70), (0, 127)]]
             h, w, cin = h // stride, w // stride, cout
-        want, _ = _run(dev, x, mode=1)
-        got, _ = _run(dev, x)
-        assert np.array_equal(got, want), (b, x.shape, [(d["cin"], d["cout"], d["in_stride"]) for d in dev])
-    binding.debug_seq_block(2)
-    try:
         seq = binding.LayerSeq(dev)
-        ws = torch.empty((seq.workspace_bytes(*x.shape[:3]),), dtype=torch.uint8, device="cuda")
-        y = torch.zeros(want.shape, dtype=torch.int8, device="cuda")
-        s = torch.cuda.Stream()
-        with torch.cuda.stream(s):
-            g = torch.cuda.CUDAGraph()
-            with torch.cuda.graph(g, stream=s):
-                binding.pw_layer_seq(seq, x, ws, y)
-                binding.pw_layer_seq(seq, x, ws, y)
-        g.replay()
-        torch.cuda.synchronize()
-        assert np.array_equal(y.cpu().numpy(), want)
+        for i in range(n):
+            for rq, of in ((seq.array[2 * i].rq, 0), (seq.array[2 * i + 1].dw_rq, 1), (seq.array[2 * i + 1].rq, 2)):
+                choice = clamps[3 * i + of]
+                rq.act_min, rq.act_max = choice[int(rng.integers(len(choice)))]
+        shape = (b, h, w, cin)
+        out = {}
+        for mode in (1, 2):
+            binding.debug_seq_block(mode)
+            try:
+                ws = Guarded(seq.workspace_bytes(*x.shape[:3]), dtype=torch.uint8, fill=0)
+                y = Guarded(int(np.prod(shape)))
+                fused = [binding.debug_layer_seq_output_offset(seq, *x.shape[:3], 2 * i)[0] == -2 for i in range(n)]
+                binding.pw_layer_seq(seq, x, ws.t, y.view(*shape))
+                ws.check("workspace"); y.check("output")
+                out[mode] = y.t.cpu().numpy()
+                if mode == 1:
+                    assert not any(fused)
+                    continue
+                pairs += n; taken += sum(fused); most = max(most, sum(fused))
+                y.t.fill_(-77)
+                s = torch.cuda.Stream()
+                with torch.cuda.stream(s):
+                    g = torch.cuda.CUDAGraph()
+                    with torch.cuda.graph(g, stream=s):
+                        binding.pw_layer_seq(seq, x, ws.t, y.view(*shape))
+                        binding.pw_layer_seq(seq, x, ws.t, y.view(*shape))
+                g.replay()
+                ws.check("workspace"); y.check("output")
+                assert np.array_equal(y.t.cpu().numpy(), out[1])
+            finally:
+                binding.debug_seq_block()
+        assert np.array_equal(out[2], out[1]), (x.shape, [(d["cin"], d["cout"], d["in_stride"]) for d in dev], fused)
         assert binding.last_device_status() == binding.PROM_OK
-    finally:
-        binding.debug_seq_block()
+    assert 2 * taken >= pairs and most >= 2, (taken, pairs, most)
