@@ -105,28 +105,6 @@ struct Params {
 };
 
 // ---- device helpers -----------------------------------------------------------------------------
-__device__ __forceinline__ void cp_async_16(uint32_t dst, const void *src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_8(uint32_t dst, const void *src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-__device__ __forceinline__ void st_cluster_32(uint32_t addr, uint32_t v)
-{
-    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-__device__ __forceinline__ void sts_128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-
 // 32 accumulator columns of one pixel, clamp [0, 127], bias in the sum: the high word of a 64-bit
 // multiply-add (rounding term in the addend), one shift, saturating pack, halve.  UP: the sums are first
 // brought to the slice's common shift by a power of two per channel.
@@ -170,8 +148,8 @@ __device__ __noinline__ void any_constants(uint32_t taddr, const int *mult, int 
                 out[c / 4] = zero ? 0u : (ptx::pack_sat_u8(q1, q0, ptx::pack_sat_u8(q3, q2, 0u)) >> 1) & 0x7F7F7F7Fu;
             }
             if (store) {
-                sts_128(at + ((32u * h) ^ swz), out[0], out[1], out[2], out[3]);
-                sts_128(at + ((32u * h + 16u) ^ swz), out[4], out[5], out[6], out[7]);
+                ptx::sts_128(at + ((32u * h) ^ swz), out[0], out[1], out[2], out[3]);
+                ptx::sts_128(at + ((32u * h + 16u) ^ swz), out[4], out[5], out[6], out[7]);
             }
             __syncwarp();
         }
@@ -188,7 +166,7 @@ __device__ __noinline__ void any_constants(uint32_t taddr, const int *mult, int 
             const int q = zero ? 0 : requant_exact((int)v[i] + mult[kToBias + c], mult[c], mult[kToShift + c], lo, hi);
             o[i >> 2] |= ((uint32_t)q & 0xFFu) << (8 * (i & 3));
         }
-        if (store) sts_128(at + (((uint32_t)h << 4) ^ swz), o[0], o[1], o[2], o[3]);
+        if (store) ptx::sts_128(at + (((uint32_t)h << 4) ^ swz), o[0], o[1], o[2], o[3]);
     }
 }
 
@@ -258,8 +236,8 @@ __device__ __forceinline__ void load_pixels(const Params &p, const Item &it, uin
         const int8_t *src = origin + (q * img_step + m * p.c0 + (int)b);
         const uint32_t d = dst + ((uint32_t)(m >> 7) * p.ks + (b >> 5)) * kStepBytes + tc::swz_offset(row, (b >> 4) & 1u, 32u) + (b & 15u);
         if ((unsigned)y < (unsigned)p.h && it.img + q < p.batch) {
-            if (wide) cp_async_16(d, src);
-            else cp_async_8(d, src);
+            if (wide) ptx::cp_async_16(d, src);
+            else ptx::cp_async_8(d, src);
         }
     }
 }
@@ -348,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                                                             : kNoPixel;
         }
         for (uint32_t i = threadIdx.x; i < (uint32_t)p.ne * p.e_bytes / 16; i += kThreads)
-            sts_128(base + p.off_e + 16 * i, 0u, 0u, 0u, 0u);
+            ptx::sts_128(base + p.off_e + 16 * i, 0u, 0u, 0u, 0u);
         tc::build_aconst(smem + p.off_aconst, (int)threadIdx.x, kThreads);
         if (threadIdx.x == 64) { pspan[0] = 31; pspan[1] = 0; pspan[2] = 0; }
     }
@@ -391,7 +369,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                     load_pixels(p, item_of(p, cluster + j * p.clusters), base + x.i * p.x_bytes, etab, at + lane, 32, end);
                     at = end;
                     if (at == pieces) {
-                        cp_async_wait_all();
+                        ptx::cp_async_wait_all();
                         ptx::fence_proxy_async_smem();
                         __syncwarp();
                         if (leader) ptx::mbar_arrive_n(bar(kBarXFull, x.i), kEpiWarps);
@@ -406,7 +384,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                 if (__any_sync(0xFFFFFFFFu, t0 == tc::kWaitGiveUp)) { ok = false; break; }
             }
         }
-        cp_async_wait_all();
+        ptx::cp_async_wait_all();
         if (leader) tc::drain_copies(bar(kBarWFull, 0), (uint32_t)p.ns, (uint32_t)issued);
         __syncwarp();
     } else if (warp == 1) {
@@ -536,7 +514,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
             }
             pc[c] = mu; pc[p.npad + c] = b; pc[3 * p.npad + c] = sh;
         }
-        cp_async_wait_all();
+        ptx::cp_async_wait_all();
         ptx::fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(bar(kBarXFull, 0));
@@ -635,8 +613,8 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                         for (int i = 0; i < 8; ++i) out[i] = 0u;
                     }
                     if (store) {
-                        sts_128(at + ((32u * h) ^ swz), out[0], out[1], out[2], out[3]);
-                        sts_128(at + ((32u * h + 16u) ^ swz), out[4], out[5], out[6], out[7]);
+                        ptx::sts_128(at + ((32u * h) ^ swz), out[0], out[1], out[2], out[3]);
+                        ptx::sts_128(at + ((32u * h + 16u) ^ swz), out[4], out[5], out[6], out[7]);
                     }
                     __syncwarp();
                 }
@@ -667,8 +645,8 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                     ptx::tmem_wait_ld();
                     if (h + 1 == hdr.z) tc::release_acc(bar(kBarD2Empty, at8(v)));
                     requant_32<true>(acc_v, base + off_c + 4 * (kMultD + h * kHalf), base + off_c + 4 * (kUpD + h * kHalf), hdr.y, out);
-                    sts_128(at + ((32u * h) ^ swz), out[0], out[1], out[2], out[3]);
-                    sts_128(at + ((32u * h + 16u) ^ swz), out[4], out[5], out[6], out[7]);
+                    ptx::sts_128(at + ((32u * h) ^ swz), out[0], out[1], out[2], out[3]);
+                    ptx::sts_128(at + ((32u * h + 16u) ^ swz), out[4], out[5], out[6], out[7]);
                 }
             } else {
                 any_constants(acc, reinterpret_cast<const int *>(smem + off_c) + kMultD, p.lo_d, p.hi_d, hdr.z, at, swz, true, false);
@@ -764,8 +742,8 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
 #pragma unroll
                         for (int e = 0; e < 16; e += 8) {
                             if (c0 + e >= p.co) break;
-                            st_cluster_v4(to + 4 * (c0 + e), z[e], z[e + 1], z[e + 2], z[e + 3]);
-                            st_cluster_v4(to + 4 * (c0 + e) + 16, z[e + 4], z[e + 5], z[e + 6], z[e + 7]);
+                            ptx::st_cluster_v4(to + 4 * (c0 + e), z[e], z[e + 1], z[e + 2], z[e + 3]);
+                            ptx::st_cluster_v4(to + 4 * (c0 + e) + 16, z[e + 4], z[e + 5], z[e + 6], z[e + 7]);
                         }
                     }
                     __syncwarp();
@@ -773,7 +751,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
             }
         }
         // (a constant out of range in one CTA's slices: no CTA writes)
-        if (warp == kFirstEpi && lane < p.csize && pspan[0] < 0) st_cluster_32(ptx::map_to_rank(ptx::smem_u32(pspan), (uint32_t)lane), 0xFFFFFFFFu);
+        if (warp == kFirstEpi && lane < p.csize && pspan[0] < 0) ptx::st_cluster_32(ptx::map_to_rank(ptx::smem_u32(pspan), (uint32_t)lane), 0xFFFFFFFFu);
         // this thread's outputs: eight channels of pixel rr of the CTA's share, then every kEpiThreads-th such piece
         const int etid = (int)threadIdx.x - 32 * kFirstEpi, c8 = p.co >> 3, plane = p.rows * p.wo;
         const int share = min(p.rpc, p.ipi * plane - rank * p.rpc) * c8;
@@ -838,22 +816,6 @@ struct PrepTable {
     int behind;                                 // the kernel in front is this call's own and reads nothing written here
     PrepBlock b[kMaxPrep];
 };
-
-// Four bias digits (word w of a column's eight): the first of weight 1, the second unused, the others 127.
-__device__ __forceinline__ uint32_t bias_word(int v, int w)
-{
-    const int h = (v >= 0 ? v + 63 : v - 63) / 127;
-    uint32_t wd = 0;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const int d = 4 * w + e - 2;
-        int dig = 0;
-        if (d == -2) dig = v - 127 * h;
-        else if (d >= 0) dig = h >= 0 ? min(127, max(0, h - 127 * d)) : max(-127, min(0, h + 127 * d));
-        wd |= ((uint32_t)dig & 0xFFu) << (8 * e);
-    }
-    return wd;
-}
 
 // One CTA per slice.
 __global__ void __launch_bounds__(kPrepThreads) block_prep_kernel(const __grid_constant__ PrepTable t)
@@ -921,7 +883,7 @@ __global__ void __launch_bounds__(kPrepThreads) block_prep_kernel(const __grid_c
         const int w = i & 7, n = (i >> 3) & (kSlice - 1), d = i / (kSlice * 8);
         const int v = d ? (fast_d ? cst[kBiasD + n] : 0) : (fast_e ? cst[kBiasE + n] << scale_e[n] : 0);
         uint8_t *blk = image + (d ? off_taps(p.ks) + (n / kHalf) * kHalfTaps + 9 * kTapBytes : (uint32_t)p.ks * 2 * kTapBytes);
-        *reinterpret_cast<uint32_t *>(blk + tc::swz_offset((uint32_t)(d ? n & (kHalf - 1) : n), (uint32_t)w >> 2, 32u) + 4 * (w & 3)) = bias_word(v, w);
+        *reinterpret_cast<uint32_t *>(blk + tc::swz_offset((uint32_t)(d ? n & (kHalf - 1) : n), (uint32_t)w >> 2, 32u) + 4 * (w & 3)) = tc::bias_word(v, w);
     }
 #pragma unroll 4
     for (int i = tid; i < 2 * 9 * kHalf * 2; i += kPrepThreads) {

@@ -230,18 +230,8 @@ dw3x3_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant_
         for (int i = tid; i < kBlock * 8; i += kBuilders) {
             const int col = i >> 3, w = i & 7, s = col / kSlice;
             const int b = in_sum ? cst[s * kSlice + channel_of(col & 31)] : 0;
-            const int h = (b >= 0 ? b + 63 : b - 63) / 127;
-            uint32_t wd = 0;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int d = 4 * w + e - 2;             // digit of weight 127, or below 0
-                int dig = 0;
-                if (d == -2) dig = b - 127 * h;
-                else if (d >= 0) dig = h >= 0 ? min(127, max(0, h - 127 * d)) : max(-127, min(0, h + 127 * d));
-                wd |= ((uint32_t)dig & 0xFFu) << (8 * e);
-            }
             uint8_t *bb = smem + off_b(STRIDE) + (size_t)s * kSliceB + 3 * kTapBytes;
-            *reinterpret_cast<uint32_t *>(bb + tc::swz_offset((uint32_t)(col & 31), (uint32_t)w >> 2, 32u) + 4 * (w & 3)) = wd;
+            *reinterpret_cast<uint32_t *>(bb + tc::swz_offset((uint32_t)(col & 31), (uint32_t)w >> 2, 32u) + 4 * (w & 3)) = tc::bias_word(b, w);
         }
         ptx::fence_proxy_async_smem();
         ptx::tc_fence_before_sync();

@@ -155,6 +155,21 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *gsrc, uint32
                  : "memory");
 }
 
+// ---- copies of a few bytes per thread into shared memory, and 16-byte stores --------------------------
+__device__ __forceinline__ void cp_async_16(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_8(uint32_t dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void sts_128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+
 // ---- pairs of CTAs (clusters of two, cta_group::2) ------------------------------------------------
 __device__ __forceinline__ uint32_t cluster_rank()
 {
@@ -172,6 +187,15 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank)
 __device__ __forceinline__ void cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// Into the shared memory of a CTA of the cluster (an address that map_to_rank gave).
+__device__ __forceinline__ void st_cluster_32(uint32_t addr, uint32_t v)
+{
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 // An arrival on a barrier of either CTA.  It hands over tensor memory whose reads have completed, no shared or
 // global memory: with release.cluster it waits for all of the thread's earlier stores (half of a read-out).

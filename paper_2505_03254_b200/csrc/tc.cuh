@@ -817,6 +817,22 @@ __device__ __forceinline__ void build_aconst(uint8_t *aconst_smem, int tid, int 
     }
 }
 
+// Four bias digits of a column, word w of its eight: the first of weight 1, the second unused, the others of weight 127.
+__device__ __forceinline__ uint32_t bias_word(int v, int w)
+{
+    const int h = (v >= 0 ? v + 63 : v - 63) / 127;        // nearest multiple of 127
+    uint32_t wd = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int d = 4 * w + e - 2;                        // digit of weight 127, or below 0
+        int dig = 0;
+        if (d == -2) dig = v - 127 * h;
+        else if (d >= 0) dig = h >= 0 ? min(127, max(0, h - 127 * d)) : max(-127, min(0, h + 127 * d));
+        wd |= ((uint32_t)dig & 0xFFu) << (8 * e);
+    }
+    return wd;
+}
+
 // Code tables: byte of four 2-bit codes -> four int8 of magnitude 1, 4, 8, .., 64.
 __device__ __forceinline__ void build_luts(uint32_t *lut, int tid, int nthreads)
 {
@@ -1681,18 +1697,8 @@ __global__ void __launch_bounds__(kPrepThreads) tc_prep_kernel(const __grid_cons
             const int col = i >> 3, w = i & 7, ls = col / p.nt_pad, c = col - ls * p.nt_pad;
             const int2 bs = prep_bs[p.direct ? ls * p.nt_pad + channel_of(c, p.nt) : col];
             const int v = fast ? bs.x << (2 + shmax - bs.y) : 0;
-            const int h = (v >= 0 ? v + 63 : v - 63) / 127;        // nearest multiple of 127
-            uint32_t wd = 0;
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int d = 4 * w + e - 2;                        // digit of weight 127, or below 0
-                int dig = 0;
-                if (d == -2) dig = v - 127 * h;
-                else if (d >= 0) dig = h >= 0 ? min(127, max(0, h - 127 * d)) : max(-127, min(0, h + 127 * d));
-                wd |= ((uint32_t)dig & 0xFFu) << (8 * e);
-            }
             uint8_t *blk = image + p.off_wbias + (size_t)ls * p.nt_pad * 32;
-            *reinterpret_cast<uint32_t *>(blk + swz_offset((uint32_t)c, (uint32_t)w >> 2, 32u) + 4 * (w & 3)) = wd;
+            *reinterpret_cast<uint32_t *>(blk + swz_offset((uint32_t)c, (uint32_t)w >> 2, 32u) + 4 * (w & 3)) = bias_word(v, w);
         }
         if (tid == 0) {
             int *hdr = reinterpret_cast<int *>(image + p.off_hdr);
