@@ -1319,7 +1319,6 @@ static bool make_y_map(CUtensorMap *map, int8_t *y, int nf, long long rows, int 
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Where everything of a sequence sits in the caller's workspace.
 // ---- depthwise kernels: which one, for the layers and for the rule on blocks ----------------------
 // 0: the library's choice, 1: CUDA cores only, 2: tensor cores or PROM_ERR_UNSUPPORTED
 static std::atomic<int> g_dw_variant{0};
@@ -1538,32 +1537,40 @@ static bool block_plan(const prom_layer *l, int batch, int h, int w, const Devic
     const BlockKey key = {c0, ce, co, batch, h, w, stride, d.dev, f_rows, f_split};
     static std::mutex mu;
     static std::map<BlockKey, std::pair<bool, BlockPlan>> cache;
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = cache.find(key);
-    if (it == cache.end()) {
-        bool found = false;
-        BlockPlan top;
-        const int ho = (h - 1) / stride + 1, slices = (ce + block::kSlice - 1) / block::kSlice;
-        for (int bands = 1; bands <= ho; ++bands) {
-            const int rows = (ho + bands - 1) / bands;
-            if (bands > 1 && rows == (ho + bands - 2) / (bands - 1)) continue;
-            if (f_rows > 0 && rows != (f_rows < ho ? f_rows : ho)) continue;
-            for (int ipi = 1; ipi <= (bands == 1 ? 8 : 1) && ipi <= batch; ++ipi)
-                for (int c = 1; c <= block::kMaxCluster && c <= slices; ++c) {
-                    const int per = (slices + c - 1) / c;
-                    if ((slices + per - 1) / per != c) continue;
-                    if (f_split > 0 && c != f_split) continue;
-                    BlockPlan pl;
-                    if (!block_fill(c0, ce, co, batch, h, w, stride, rows, ipi, per, d, pl)) continue;
-                    if (!found || pl.est_us < top.est_us) { top = pl; found = true; }
-                }
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        const auto it = cache.find(key);
+        if (it != cache.end()) {
+            if (it->second.first) best = it->second.second;
+            return it->second.first;
         }
-        if (found) block_estimate(l, d, top);
-        if (cache.size() > 4096) cache.clear();
-        it = cache.emplace(key, std::make_pair(found, top)).first;
     }
-    if (it->second.first) best = it->second.second;
-    return it->second.first;
+    // (not under the lock: other threads' known shapes need not wait for it)
+    bool found = false;
+    BlockPlan top;
+    const int ho = (h - 1) / stride + 1, slices = (ce + block::kSlice - 1) / block::kSlice;
+    for (int bands = 1; bands <= ho; ++bands) {
+        const int rows = (ho + bands - 1) / bands;
+        if (bands > 1 && rows == (ho + bands - 2) / (bands - 1)) continue;
+        if (f_rows > 0 && rows != (f_rows < ho ? f_rows : ho)) continue;
+        for (int ipi = 1; ipi <= (bands == 1 ? 8 : 1) && ipi <= batch; ++ipi)
+            for (int c = 1; c <= block::kMaxCluster && c <= slices; ++c) {
+                const int per = (slices + c - 1) / c;
+                if ((slices + per - 1) / per != c) continue;
+                if (f_split > 0 && c != f_split) continue;
+                BlockPlan pl;
+                if (!block_fill(c0, ce, co, batch, h, w, stride, rows, ipi, per, d, pl)) continue;
+                if (!found || pl.est_us < top.est_us) { top = pl; found = true; }
+            }
+    }
+    if (found) {
+        block_estimate(l, d, top);
+        best = top;
+    }
+    std::lock_guard<std::mutex> lk(mu);
+    if (cache.size() > 4096) cache.clear();
+    cache.emplace(key, std::make_pair(found, top));
+    return found;
 }
 
 static prom_status launch_block(BlockPlan &pl, const int8_t *x, int8_t *y, const int8_t *res, const uint8_t *image,
@@ -1590,6 +1597,7 @@ static prom_status launch_block(BlockPlan &pl, const int8_t *x, int8_t *y, const
     return cuda_status(e);
 }
 
+// Where everything of a sequence sits in the caller's workspace.
 struct SeqLayout {
     size_t ra = 0, rb = 0, dw_off = 0;     // the two ping-pong regions (b ends with the depthwise buffer)
     std::vector<size_t> img_off;           // per layer: prepared image of a one-launch layer, or -1
@@ -1699,9 +1707,7 @@ static void seq_layout(const prom_layer *layers, int n, const SeqShape &s, const
         }
 }
 
-
 // ---- depthwise 3x3 on the tensor cores (dwtc.cuh) ---------------------------------------------
-
 template <int STRIDE>
 static prom_status launch_dw_tc(const int8_t *x, int batch, int h, int w, int c, const int8_t *wt,
                                 const prom_requant *rq, int8_t *y, const DeviceInfo &d, cudaStream_t st, int pdl)
