@@ -86,7 +86,10 @@ typedef enum {
  * |bias| <= 2^28, -128 <= act_min <= act_max <= 127.  The clamp is checked on
  * the host; the arrays are checked on the device by the kernels that read
  * them (a violation sets PROM_ERR_BAD_REQUANT in the device status word and
- * the affected output tile is left unwritten). */
+ * the affected output tile is left unwritten; where a sequence runs an
+ * expanding layer, a depthwise convolution and a project layer in one launch,
+ * a violation in any of the three leaves the project layer's whole output
+ * unwritten). */
 typedef struct {
     const int32_t *bias;
     const int32_t *mult;
@@ -330,9 +333,16 @@ prom_status prom_pw_conv_i8_host(const int8_t *x_host, int64_t m, int cin,
  * the start of every call, so the call stays stateless);
  * prom_layer_seq_workspace_bytes gives the size needed (0 on a shape error).
  * A workspace that only holds the two activation regions still works, more
- * slowly.  `variant` applies to every layer (AUTO picks per layer).  The
- * kernels of one call are chained with programmatic dependent launch and can
- * be captured into a CUDA graph. */
+ * slowly.  Under AUTO and TC an expanding layer and the layer with a depthwise
+ * convolution behind it may run in one launch, where the library expects that
+ * to be faster; the expanded tensor is then never written, the workspace holds
+ * that launch's operands too, and prom_layer_seq_workspace_bytes covers this
+ * form as well as one launch per layer.  The bytes of the result are the same.
+ * A call whose y_out_dev overlaps x0_dev, or whose workspace has no room for
+ * those operands, has a launch per layer.
+ * `variant` applies to every layer (AUTO picks per layer).  The kernels of one
+ * call are chained with programmatic dependent launch and can be captured into
+ * a CUDA graph. */
 size_t prom_layer_seq_workspace_bytes(const prom_layer *layers, int n,
                                       int batch, int h0, int w0);
 prom_status prom_pw_layer_seq(const prom_layer *layers, int n,

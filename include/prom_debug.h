@@ -69,7 +69,8 @@ void prom_debug_seq_order(int alternate);
  * tensors between them kept in shared memory: 0 = where the library's rule finds it faster
  * (default), 1 = never, 2 = wherever the shape allows it.  rows: output rows per band, split: CTAs
  * per cluster that share a band's channels (0 = the planner's; a combination that does not fit leaves
- * the block to one launch per layer).  Results do not depend on it; the workspace size does.
+ * the block to one launch per layer).  Mode 2 takes clamps too that mode 0 leaves to one launch
+ * per layer.  Results do not depend on it; the workspace size does.
  * prom_debug_layer_seq_output_offset returns -2 for the expanding layer.  While prom_debug_dw_variant or
  * prom_debug_seq_chain asks for a kernel of its own no block is taken.  Process-wide. */
 void prom_debug_seq_block(int mode, int rows, int split);
@@ -98,10 +99,12 @@ void prom_debug_tc_wide(int mode, int blocks);
  * prom_pw_layer_seq call whose workspace has prom_layer_seq_workspace_bytes
  * bytes, with AUTO or TC as the variant: the byte offset from the workspace's
  * start, -1 for the last layer (its output is y_out_dev) or a bad argument,
- * -2 for a layer inside a shared-memory run (prom_debug_seq_chain(2)) that is
- * not the run's last: it writes no tensor.  *chained (may be NULL) receives 1
- * when the layer runs inside a multi-layer launch.  A layer's output stays intact until the layer two further on has
- * run (ping-pong regions) or, inside a depth-first launch, until the next
+ * -2 for a layer that writes no tensor: the expanding layer of a block (in the
+ * default mode too) and a layer inside a shared-memory run
+ * (prom_debug_seq_chain(2)) that is not the run's last.  *chained (may be NULL)
+ * receives 1 for these and for a layer inside a depth-first launch.  A layer's
+ * output stays intact until the second of the later layers that write a tensor
+ * has run (ping-pong regions) or, inside a depth-first launch, until the next
  * call. */
 int64_t prom_debug_layer_seq_output_offset(const prom_layer *layers, int n, int batch, int h0,
                                            int w0, int layer, int *chained);

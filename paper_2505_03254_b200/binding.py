@@ -315,8 +315,8 @@ def debug_seq_order(alternate: bool = True) -> None:
 
 def debug_layer_seq_output_offset(seq: "LayerSeq", batch: int, h0: int, w0: int, layer: int):
     """prom_debug_layer_seq_output_offset: (byte offset of the layer's output in the workspace, -1
-    for a bad argument or -2 for a layer inside a shared-memory run, which writes no tensor;
-    whether the layer runs inside a multi-layer launch)."""
+    for a bad argument or -2 for a layer that writes no tensor, the expanding layer of a block or one
+    inside a shared-memory run; whether the layer is one of these or runs inside a depth-first launch)."""
     chained = C.c_int(0)
     off = lib().prom_debug_layer_seq_output_offset(seq.array, seq.n, batch, h0, w0, layer, C.byref(chained))
     return int(off), bool(chained.value)

@@ -1502,13 +1502,12 @@ static void block_estimate(const prom_layer *l, const DeviceInfo &d, BlockPlan &
                    0.04 * (e.p.groups + q.p.groups);
 }
 
-// Whether one launch is expected to beat one per layer, whose time (us) is a fit to the same shapes (standard error
-// 7 %).  Inside a sequence a block saves about 1.2 us more than calls of its own show, whose preparation is not shared;
-// its own estimate is low where the project layer is wide (more sums to exchange and to requantise) and with stride 2.
-// With this margin two fifths of the shapes run as blocks, in 0.85 of the layers' time; 0.7 % of all are slower by more
-// than 3 % (at 0.92: 28 %, 0.83 and 0.2 %).  Over 189 bodies of the network (ten widths and sizes, batch 1 to 150) a call
-// takes 0.945 of the time of one launch per layer on average, 0.84 to 1.005.  Mostly blocks are planes of 10 to 60 thousand pixels, batch included: larger
-// ones are bound by the requantiser and the taps either way, and units leave gaps.
+// Whether one launch is expected to beat one per layer beside other blocks; the layers' time (us) is a fit to the shapes that
+// the geometry's model was fitted to (standard error 7 %).  Inside a sequence a block saves about 1.2 us more than calls of its
+// own show, whose preparation is not shared; its own estimate is low where the project layer is wide (more sums to exchange
+// and to requantise) and with stride 2.  Mostly blocks are planes of 10 to 60 thousand pixels, batch included: larger ones
+// are bound by the requantiser and the taps either way, and units leave gaps.  67 bodies of the network (five widths, four
+// sizes, batch 1 to 151) take 0.963 of the time of one launch per layer on average, 0.88 to 1.009.
 static bool block_worth(const BlockPlan &pl, int ce)
 {
     const block::Params &p = pl.p;
@@ -1524,7 +1523,7 @@ static bool block_worth(const BlockPlan &pl, int ce)
 
 // What a call's blocks have to gain together.  By block_estimate every block beside the first gains kBlockBeside more than
 // alone: the blocks' operands take one launch, and kernels of different layers wait for their instructions where block_kernel
-// finds its own (fit to 70 bodies of the network, which all but one keep their blocks).  So a call of one block needs 1.3 us.  Of
+// finds its own (fit to those bodies, all but two of which keep their blocks).  So a call of one block needs 1.3 us.  Of
 // 4942 calls of one block 0.6 % are slower than one launch per layer by more than 3 % (without this rule 4.7, up to 1.45
 // times for wide inputs in many items), of 2850 of three alike 1.1 % (2.2).
 constexpr double kBlockBeside = 1.6, kBlocksGain = 1.3;
