@@ -751,7 +751,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
             }
         }
         // (a constant out of range in one CTA's slices: no CTA writes)
-        if (warp == kFirstEpi && lane < p.csize && pspan[0] < 0) ptx::st_cluster_32(ptx::map_to_rank(ptx::smem_u32(pspan), (uint32_t)lane), 0xFFFFFFFFu);
+        if (warp == 3 && lane < p.csize && pspan[0] < 0) ptx::st_cluster_32(ptx::map_to_rank(ptx::smem_u32(pspan), (uint32_t)lane), 0xFFFFFFFFu);
         // this thread's outputs: eight channels of pixel rr of the CTA's share, then every kEpiThreads-th such piece
         const int etid = (int)threadIdx.x - 32 * kFirstEpi, c8 = p.co >> 3, plane = p.rows * p.wo;
         const int share = min(p.rpc, p.ipi * plane - rank * p.rpc) * c8;
@@ -770,7 +770,8 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
         if (mine) {
             const int top = max(pspan[1], 2);
             const Project prj = {pc, p.npad, top - pspan[0] <= 10 && pspan[2] < (1 << 20) ? top : 0, p.lo_p, p.hi_p};
-            for (int i = pspan[0] < 0 ? share : etid; i < share; i += kEpiThreads) {
+            const bool write = pspan[0] >= 0;
+            for (int i = etid; i < share; i += kEpiThreads) {
                 if (i != etid) {
                     at = place(i, rr, c);
                     if (p.res && at >= 0) rs = __ldcg(reinterpret_cast<const uint2 *>(p.res + at));
@@ -785,7 +786,7 @@ __global__ void __launch_bounds__(kThreads, 1) block_kernel(const __grid_constan
                 }
                 uint2 out = project_8(prj, sum, c);
                 if (p.res) { out.x = __vaddss4(out.x, rs.x); out.y = __vaddss4(out.y, rs.y); }
-                *reinterpret_cast<uint2 *>(p.y + at) = out;
+                if (write) *reinterpret_cast<uint2 *>(p.y + at) = out;
             }
         }
     }
