@@ -1506,8 +1506,8 @@ static void block_estimate(const prom_layer *l, const DeviceInfo &d, BlockPlan &
 // the geometry's model was fitted to (standard error 7 %).  Inside a sequence a block saves about 1.2 us more than calls of its
 // own show, whose preparation is not shared; its own estimate is low where the project layer is wide (more sums to exchange
 // and to requantise) and with stride 2.  Mostly blocks are planes of 10 to 60 thousand pixels, batch included: larger ones
-// are bound by the requantiser and the taps either way, and units leave gaps.  67 bodies of the network (five widths, four
-// sizes, batch 1 to 151) take 0.963 of the time of one launch per layer on average, 0.88 to 1.009.
+// are bound by the requantiser and the taps either way, and units leave gaps.  123 bodies of the network (five widths,
+// four sizes, batch 1 to 151) take 0.944 of the time of one launch per layer on average, 0.85 to 1.014.
 static bool block_worth(const BlockPlan &pl, int ce)
 {
     const block::Params &p = pl.p;
@@ -1521,12 +1521,15 @@ static bool block_worth(const BlockPlan &pl, int ce)
     return pl.est_us * (1.0 + 0.0011 * wide + (p.stride == 1 ? 0.0 : p.csize == 1 ? 0.12 : 0.03)) - 1.2 < 0.96 * layers;
 }
 
-// What a call's blocks have to gain together.  By block_estimate every block beside the first gains kBlockBeside more than
-// alone: the blocks' operands take one launch, and kernels of different layers wait for their instructions where block_kernel
-// finds its own (fit to those bodies, all but two of which keep their blocks).  So a call of one block needs 1.3 us.  Of
-// 4942 calls of one block 0.6 % are slower than one launch per layer by more than 3 % (without this rule 4.7, up to 1.45
-// times for wide inputs in many items), of 2850 of three alike 1.1 % (2.2).
-constexpr double kBlockBeside = 1.6, kBlocksGain = 1.3;
+// What a call's blocks have to gain together, by block_estimate.  A block beside others, or beside other layers, gains
+// kBlockBeside more than one whose call is nothing else (launches follow one another closer, the kernels of different layers
+// wait for their instructions, the operands take one launch: 1.8 to 2.5 us per block in 130 bodies of the network).  So calls of
+// one block alone need 0.5 us, and the bodies keep theirs.  Of 3391 such calls 0.2 % are slower than one launch per layer by
+// more than 3 %, from a captured graph 0.7 % (without this rule, over the shapes of the fit, 1.7 and 4.7 %, up to 1.45 times).
+// A block that block_estimate finds slower by more than 1.3 us is left to its layers where these are long enough for its figure
+// to be the better one: 120 -> 720 -> 120 on 6 x 6 in a body of 86 images (425 us with it, 422 without, one launch per layer 417).
+constexpr double kBlockBeside = 2.4, kBlocksGain = 0.5;
+static bool block_slow(const BlockPlan &pl) { return pl.layers_us > 21.0 && pl.block_us > pl.layers_us + 1.3; }
 
 typedef std::array<int, 10> BlockKey;
 static bool block_plan(const prom_layer *l, int batch, int h, int w, const DeviceInfo &d, BlockPlan &best)
@@ -1623,7 +1626,7 @@ static void find_blocks(const prom_layer *layers, int n, const SeqShape &s, cons
 {
     const int mode = g_block_mode.load();
     if (mode == 1 || g_dw_variant.load() != 0) return;
-    double gain = 0.0;                  // of all blocks, the first one's share of kBlockBeside too
+    double gain = 0.0;
     for (int i = 0; i + 1 < n; ++i) {
         if (L.block_of[i] >= 0 || !block_layers_ok(layers + i) || s.m[i + 1] <= 0) continue;
         // a skip connection into layer i + 2 reads the expanded tensor, which must exist
@@ -1631,14 +1634,15 @@ static void find_blocks(const prom_layer *layers, int n, const SeqShape &s, cons
         BlockPlan pl;
         const int batch = (int)(s.m[i] / ((long long)s.h[i] * s.w[i]));
         if (!block_plan(layers + i, batch, s.h[i], s.w[i], d, pl)) continue;
-        if (mode == 0 && !(block_clamps_fast(layers + i) && block_worth(pl, layers[i].cout))) continue;
+        if (mode == 0 && !(block_clamps_fast(layers + i) && block_worth(pl, layers[i].cout) && !block_slow(pl))) continue;
         gain += pl.layers_us - pl.block_us + kBlockBeside;
         L.block_of[i] = L.block_of[i + 1] = (int)L.blocks.size();
         L.blocks.push_back(pl);
         L.bimg_off.push_back(L.bimg_total);
         L.bimg_total += round256(pl.image_bytes);
     }
-    if (mode == 0 && gain < kBlocksGain + kBlockBeside) {
+    if (n == 2 * (int)L.blocks.size()) gain -= kBlockBeside;       // nothing else in the call
+    if (mode == 0 && gain < kBlocksGain) {
         L.blocks.clear(); L.bimg_off.clear(); L.bimg_total = 0;
         L.block_of.assign(n, -1);
     }
